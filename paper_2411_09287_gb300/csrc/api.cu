@@ -49,17 +49,18 @@ inline void counted(int k, F f, A... a) {
 #define launch_gr_lincomb(...) counted(1, mpc3::launch_gr_lincomb, __VA_ARGS__)
 #define launch_gr_mulmat2(...) counted(1, mpc3::launch_gr_mulmat2, __VA_ARGS__)
 #define launch_gr_inverses(...) counted(1, mpc3::launch_gr_inverses, __VA_ARGS__)
-#define launch_gr_lagrange(...) counted(1, mpc3::launch_gr_lagrange, __VA_ARGS__)
 #define launch_gr_fold_reduce(...) counted(1, mpc3::launch_gr_fold_reduce, __VA_ARGS__)
-#define launch_gr_combine_z(...) counted(1, mpc3::launch_gr_combine_z, __VA_ARGS__)
 #define launch_gr_scale_rows(...) counted(1, mpc3::launch_gr_scale_rows, __VA_ARGS__)
 #define launch_gr_lift(...) counted(1, mpc3::launch_gr_lift, __VA_ARGS__)
 #define launch_gram_lifted(...) counted(1, mpc3::launch_gram_lifted, __VA_ARGS__)
 #define launch_fold_lifted(...) counted(1, mpc3::launch_fold_lifted, __VA_ARGS__)
 #define launch_neg_copy(...) counted(1, mpc3::launch_neg_copy, __VA_ARGS__)
-#define launch_gr_check_zero(...) counted(1, mpc3::launch_gr_check_zero, __VA_ARGS__)
+#define launch_round_tail(...) counted(1, mpc3::launch_round_tail, __VA_ARGS__)
+#define launch_reveal(...) counted(1, mpc3::launch_reveal, __VA_ARGS__)
+#define launch_delta(...) counted(1, mpc3::launch_delta, __VA_ARGS__)
+#define launch_rec_hash(...) counted(1, mpc3::launch_rec_hash, __VA_ARGS__)
+#define launch_trunc_round_sums(...) counted(1, mpc3::launch_trunc_round_sums, __VA_ARGS__)
 #define launch_trunc_u(...) counted(1, mpc3::launch_trunc_u, __VA_ARGS__)
-#define launch_trunc_round_h(...) counted(1, mpc3::launch_trunc_round_h, __VA_ARGS__)
 #define launch_trunc_update_vw(...) counted(1, mpc3::launch_trunc_update_vw, __VA_ARGS__)
 #define launch_trunc_materialize(...) counted(1, mpc3::launch_trunc_materialize, __VA_ARGS__)
 #define launch_gr_mul_rows(...) counted(1, mpc3::launch_gr_mul_rows, __VA_ARGS__)
@@ -68,10 +69,6 @@ inline void counted(int k, F f, A... a) {
 #define launch_gr_mulmat_batch(...) counted(1, mpc3::launch_gr_mulmat_batch, __VA_ARGS__)
 #define launch_word_transpose(...) counted(1, mpc3::launch_word_transpose, __VA_ARGS__)
 #define launch_scalar_gr_sum(...) counted(1, mpc3::launch_scalar_gr_sum, __VA_ARGS__)
-#define launch_gr_rec1(...) counted(1, mpc3::launch_gr_rec1, __VA_ARGS__)
-#define launch_gr_inner_finish_all(...) counted(1, mpc3::launch_gr_inner_finish_all, __VA_ARGS__)
-#define launch_gr_quad_combine(...) counted(1, mpc3::launch_gr_quad_combine, __VA_ARGS__)
-#define launch_mode_consts(...) counted(1, mpc3::launch_mode_consts, __VA_ARGS__)
 #define launch_prf_words(...) counted(1, mpc3::launch_prf_words, __VA_ARGS__)
 #define launch_prf_words_keyed(...) counted(1, mpc3::launch_prf_words_keyed, __VA_ARGS__)
 #define launch_trunc_limb_table(...) counted(1, mpc3::launch_trunc_limb_table, __VA_ARGS__)
@@ -86,10 +83,9 @@ constexpr u32 ST_TIMEOUT = 4u;  // a bounded device wait expired
 
 // device constants block (words)
 constexpr int CST_INV = 0;      // 192: x^-1, (1-x)^-1, (x(x-1))^-1
-constexpr int CST_LAM = 192;    // 128: 1 - p2, p2
-constexpr int CST_ONE = 320;    // 64: the element 1
-constexpr int CST_MONE = 384;   // 64: the element -1
-constexpr int CST_WORDS = 448;
+constexpr int CST_ONE = 192;    // 64: the element 1
+constexpr int CST_MONE = 256;   // 64: the element -1
+constexpr int CST_WORDS = 320;
 
 constexpr int TRACE_ROUND = 832;  // words per round in a verification trace
 
@@ -427,65 +423,39 @@ int party_sums(mpc_ctx* ctx, const View& u, const View& v, long long count, u64*
   return cuda_check(ctx, "party_sums");
 }
 
-// Secure GR inner-product finish (P0's Gamma, P1/P2 cross terms, one exchange); 3 messages.
-void inner_finish(mpc_ctx* ctx, const u64* S, u32 purpose, u64 obj, u64* h6) {
-  launch_gr_inner_finish_all(ctx->st, S, ctx->k01, ctx->k02, purpose, obj, h6);
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);
-}
-
-// Pi_Rec of one shared GR element (3 shares + 3 hashes); an armed REC_MSG fault corrupts the
-// P0 -> P1 share, as for any other Pi_Rec.
-void rec1(mpc_ctx* ctx, const u64* s6, u64* out) {
-  u64 mask = 0;
-  int idx = -1;
-  Fault& f = ctx->fault[MPC_SITE_REC_MSG];
-  if (f.armed) {
-    mask = f.mask;
-    idx = (int)(f.index % 64);
-    f.armed = false;
-  }
-  launch_gr_rec1(ctx->st, s6, mask, idx, out, ctx->status, ST_ABORT);
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 32);
-}
-
-// <v> random GR element, revealed with Pi_Rec.
-void reveal(mpc_ctx* ctx, u32 purpose, u64 obj, u64* tmp6, u64* out) {
-  launch_gr_random_shared(ctx->st, 1, ctx->k01, ctx->k02, ctx->k12, purpose, obj, tmp6);
-  rec1(ctx, tmp6, out);
-}
-
 // ---- verification state ---------------------------------------------------------------------
 struct Small {   // per-verification small scratch (all device, from the workspace)
   u64* Pmat;     // 4 x 3 x 4096
-  u64* S;        // 5 x 192: S00, S01, S10, S11, Sh2
-  u64* h0;       // 384
-  u64* h2;       // 384
+  u64* S;        // 4 x 192: S00, S01, S10, S11 (reduced; u64 path)
+  u64* U;        // 2 x 12 x 128: a round's party sums ee, S01, S10, oo (3 parties each), the other
+                 // half cleared for the next round (sums_begin, next_sums)
+  u64* rec;      // REC_SLOTS records of opened single elements, hashed by flush_recs
   u64* z[2];     // 384 each
-  u64* coef;     // 448
+  u64* coef;     // 448: the fold element f at 0, 1 - f at 384
   u64* zp;       // 64
   u64* r;        // 64
-  u64* tmp6;     // 384
   u64* MM;       // 128 x 64
   u64* MA;       // 5 x 4096 (multiplication matrices of alpha components)
   u64* alpha;    // 384
   u64* aux;      // 4 x 64
   u64* Sfull;    // 192
   u64* zinit;    // 384: the claim entering the first round (never round scratch)
+  mutable int nrec = 0, uc = 0;   // records not hashed yet; half of U in use
 };
+constexpr int REC_SLOTS = 40;
+constexpr int SUMS_WORDS = 12 * 128;
 
 Small plan_small(Arena& a) {
   Small s;
   s.Pmat = a.take<u64>(4 * 3 * 4096);
-  s.S = a.take<u64>(5 * 192);
-  s.h0 = a.take<u64>(384);
-  s.h2 = a.take<u64>(384);
+  s.S = a.take<u64>(4 * 192);
+  s.U = a.take<u64>(2 * SUMS_WORDS);
+  s.rec = a.take<u64>(REC_SLOTS * REC_WORDS);
   s.z[0] = a.take<u64>(384);
   s.z[1] = a.take<u64>(384);
   s.coef = a.take<u64>(448);
   s.zp = a.take<u64>(64);
   s.r = a.take<u64>(64);
-  s.tmp6 = a.take<u64>(384);
   s.MM = a.take<u64>(128 * 64);
   s.MA = a.take<u64>(5 * 4096);
   s.alpha = a.take<u64>(384);
@@ -536,27 +506,81 @@ IVBuf plan_iv(Arena& a, long long D) {
   return b;
 }
 
-void trace_round(mpc_ctx* ctx, u64* trace, int k, const Small& s) {
-  if (!trace) return;
-  u64* t = trace + (long long)(k - 1) * TRACE_ROUND;
-  cudaMemcpyAsync(t, s.zp, 64 * 8, cudaMemcpyDeviceToDevice, ctx->st);
-  cudaMemcpyAsync(t + 64, s.h0, 384 * 8, cudaMemcpyDeviceToDevice, ctx->st);
-  cudaMemcpyAsync(t + 448, s.h2, 384 * 8, cudaMemcpyDeviceToDevice, ctx->st);
+// The hash comparisons of the Pi_Rec calls recorded since the last flush; each batch flushes
+// before its Delta is read.
+void flush_recs(mpc_ctx* ctx, const Small& s) {
+  if (!s.nrec) return;
+  launch_rec_hash(ctx->st, s.rec, s.nrec, ctx->status, ST_ABORT);
+  s.nrec = 0;
 }
 
-// The part of a Pi_Reduce round after its party sums (in s.S: S00, S01 + S10 (with S10), S11):
-// h(0) and h(p2) by secure GR inner products, zeta revealed, the Lagrange weights, the next claim
-// zo, and M_zeta (s.MM) for the folds; the fold element is s.coef[0..63].
-void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, const Small& s) {
-  cudaStream_t st = ctx->st;
-  launch_gr_quad_combine(st, ctx->cst + CST_LAM, s.S, s.S + 192, s.S + 384, s.S + 576, s.S + 768);
-  const u64 obj = make_obj(vid, batch, (u32)k);
-  inner_finish(ctx, s.S, P_VER_H0, obj, s.h0);
-  inner_finish(ctx, s.S + 768, P_VER_H2, obj, s.h2);
-  reveal(ctx, P_VER_ZETA, obj, s.tmp6, s.zp);
-  launch_gr_lagrange(st, s.zp, ctx->reduce_mode, ctx->cst + CST_INV, s.coef);
-  launch_gr_combine_z(st, s.coef, s.h0, s.h2, z, zo);
-  launch_gr_mulmat2(st, s.coef, nullptr, s.MM);   // M_zeta
+// Pi_Rec of one shared GR element (3 shares + 3 hashes): the record its messages go to, and an
+// armed REC_MSG fault, which corrupts the P0 -> P1 share, as for any other Pi_Rec.
+struct Rec1 {
+  u64* rec;
+  u64 mask = 0;
+  int idx = -1;
+};
+Rec1 begin_rec(mpc_ctx* ctx, const Small& s) {
+  if (s.nrec == REC_SLOTS) flush_recs(ctx, s);
+  Rec1 r;
+  r.rec = s.rec + (long long)s.nrec++ * REC_WORDS;
+  Fault& f = ctx->fault[MPC_SITE_REC_MSG];
+  if (f.armed) {
+    r.mask = f.mask;
+    r.idx = (int)(f.index % 64);
+    f.armed = false;
+  }
+  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);
+  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 32);
+  return r;
+}
+
+// <v> random GR element, revealed with Pi_Rec.
+void reveal(mpc_ctx* ctx, u32 purpose, u64 obj, const Small& s, u64* out) {
+  const Rec1 r = begin_rec(ctx, s);
+  launch_reveal(ctx->st, ctx->k01, ctx->k02, ctx->k12, purpose, obj, r.mask, r.idx, out, r.rec);
+}
+
+// Clears both halves of the round sums; a round adds into cur_sums, and its tail clears the other
+// half for the next round.
+int sums_begin(mpc_ctx* ctx, const Small& s) {
+  s.uc = 0;
+  CK(cudaMemsetAsync(s.U, 0, 2 * SUMS_WORDS * 8, ctx->st));
+  return MPC_OK;
+}
+u64* cur_sums(const Small& s) { return s.U + s.uc * SUMS_WORDS; }
+
+// The part of a Pi_Reduce round after its party sums (sums: 12 blocks S00, S01, S10, S11 of three
+// parties, ld words apart: 64 reduced, 128 unreduced coefficients): h(0) and h(p2) by secure GR
+// inner products, zeta revealed, the next claim zo, and M_zeta (s.MM) for the folds; the fold
+// element is s.coef[0..63].
+void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, const Small& s,
+                const u64* sums, int ld, u64* trace) {
+  RoundTail a;
+  a.sums = sums;
+  a.ld = ld;
+  a.mode = ctx->reduce_mode;
+  a.k01 = ctx->k01;
+  a.k02 = ctx->k02;
+  a.k12 = ctx->k12;
+  a.obj = make_obj(vid, batch, (u32)k);
+  a.inv = ctx->cst + CST_INV + 128;
+  a.z = z;
+  a.zo = zo;
+  a.coef = s.coef;
+  a.MM = s.MM;
+  a.zp = s.zp;
+  a.zero = s.U + (s.uc ^ 1) * SUMS_WORDS;
+  a.nzero = SUMS_WORDS;
+  a.trace = trace ? trace + (long long)(k - 1) * TRACE_ROUND : nullptr;
+  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 6, 512);   // two secure inner products
+  const Rec1 r = begin_rec(ctx, s);
+  a.rec = r.rec;
+  a.xmask = r.mask;
+  a.xidx = r.idx;
+  launch_round_tail(ctx->st, a);
+  s.uc ^= 1;
 }
 
 // One Pi_Reduce round on a dense claim (Fig. Reduce).  x, y: current vectors (D elements, with
@@ -593,32 +617,33 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
   // [r]_2 (P0, P2 copies), so P1's and P2's cross terms vanish and P0's sums are single Grams.
   const bool bit_form = !ys && x.c[0] && !x.c[1] && !x.c[2] && x.c[3] && !x.c[4] && !x.c[5] &&
                         !y.c[0] && y.c[1] && !y.c[2] && !y.c[3] && !y.c[4] && y.c[5];
+  u64* U = cur_sums(s);
+  const u64* sums = s.S;   // reduced sums of the CUDA-core Grams unless set below
+  int ld = 64;
   if (ys) {
-    CK(cudaMemsetAsync(s.S, 0, 4 * 192 * 8, st));
-    launch_gram_lifted(st, x.c, ys->c, Dh, D, s.S);   // S00 | S01 + S10 | 0 | S11
+    launch_gram_lifted(st, x.c, ys->c, Dh, D, U);   // S00 | S01 + S10 | 0 | S11
+    sums = U;
   } else if (bit_form) {
-    // G00, G11 and G(x0 + x1, y0 + y1); G01 + G10 = G(x0 + x1, y0 + y1) - G00 - G11
-    CK(cudaMemsetAsync(s.Pmat, 0, 3 * 4096 * 8, st));
-    CK(cudaMemsetAsync(s.S, 0, 4 * 192 * 8, st));
     bool done = false;
     if (ctx->gemm_path == MPC_GEMM_LIMB_TC) {
       // tensor cores: G00, G11 and the cross sum G01 + G10 directly
       g_launches += 1;
       {
         Phase kp(ctx, MPC_PROF_K_GRAM, 4.0 * Dh * 4096);
-        done = gram3_tc(st, Dh, x.c[0], y.c[1], s.Pmat, ctx->status, ST_TIMEOUT,
+        done = gram3_tc(st, Dh, x.c[0], y.c[1], U, ctx->status, ST_TIMEOUT,
                         ctx->tune.gram_split) == 0;
       }
       if (done) {
-        launch_gr_fold_reduce(st, s.Pmat, 3, s.aux);
-        CK(cudaMemcpyAsync(S00, s.aux, 512, cudaMemcpyDeviceToDevice, st));
-        CK(cudaMemcpyAsync(S11, s.aux + 64, 512, cudaMemcpyDeviceToDevice, st));
-        CK(cudaMemcpyAsync(S01, s.aux + 128, 512, cudaMemcpyDeviceToDevice, st));
+        sums = U;
+        ld = 128;
       } else {
         g_launches -= 1;
       }
     }
     if (!done) {
+      // G00, G11 and G(x0 + x1, y0 + y1); G01 + G10 = G(x0 + x1, y0 + y1) - G00 - G11
+      CK(cudaMemsetAsync(s.Pmat, 0, 3 * 4096 * 8, st));
+      CK(cudaMemsetAsync(s.S, 0, 4 * 192 * 8, st));
       gram(ctx, s.Pmat, x.c[0], nullptr, 1, 128, y.c[1], nullptr, 1, 128, Dh, 1);
       gram(ctx, s.Pmat + 4096, x.c[0] + 64, nullptr, 1, 128, y.c[1] + 64, nullptr, 1, 128, Dh, 1);
       gram(ctx, s.Pmat + 8192, x.c[0], x.c[0] + 64, 1, 128, y.c[1], y.c[1] + 64, 1, 128, Dh, 1);
@@ -637,21 +662,20 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       // scale into its sign; a term with an absent side is zero.
       const u64 M1 = ~0ull;
       GramJobs jobs{};
-      jobs.off_x = 3 * 4096;
-      jobs.off_oo = 9 * 4096;
+      jobs.off_x = 3 * 128;
+      jobs.off_oo = 9 * 128;
       auto add = [&](int party, const u64* a0, const u64* a1, u64 sa1, const u64* b0,
                      const u64* b1, u64 sb1, u64 sign) {
         if (!a0) { a0 = a1; a1 = nullptr; sign *= sa1; }
         if (!b0) { b0 = b1; b1 = nullptr; sign *= sb1; }
         if (!a0 || !b0) return;
-        jobs.j[jobs.n++] = GramJob{a0, a1, sa1, b0, b1, sb1, s.Pmat + party * 4096, sign};
+        jobs.j[jobs.n++] = GramJob{a0, a1, sa1, b0, b1, sb1, U + party * 128, sign};
       };
       add(0, x.c[0], x.c[1], 1, y.c[0], y.c[1], 1, 1);
       add(1, x.c[2], nullptr, 0, y.c[3], nullptr, 0, M1);
       add(1, y.c[2], nullptr, 0, x.c[3], nullptr, 0, M1);
       add(2, x.c[4], nullptr, 0, y.c[4], y.c[5], M1, 1);
       add(2, y.c[4], nullptr, 0, x.c[5], nullptr, 0, M1);
-      CK(cudaMemsetAsync(s.Pmat, 0, 12 * 4096 * 8, st));
       int nl = 0;
       for (int q = 0; q < jobs.n; ++q) nl |= (jobs.j[q].a1 || jobs.j[q].b1) ? 2 : 1;
       nl = (nl & 1) + (nl >> 1);   // one launch for the single-source jobs, one for the others
@@ -661,7 +685,8 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
         done = gram_jobs_tc(st, Dh, jobs, ctx->status, ST_TIMEOUT, ctx->tune.gram_split) == 0;
       }
       if (done) {
-        launch_gr_fold_reduce(st, s.Pmat, 12, s.S);   // S00 | S01 + S10 | 0 | S11
+        sums = U;   // S00 | S01 + S10 | 0 | S11
+        ld = 128;
       } else {
         g_launches -= nl;
       }
@@ -673,7 +698,7 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       if ((rc = party_sums(ctx, f[1], g[1], Dh, s.Pmat + 9 * 4096, S11))) return rc;
     }
   }
-  round_tail(ctx, vid, batch, k, z, zo, s);
+  round_tail(ctx, vid, batch, k, z, zo, s, sums, ld, trace);
   // f(zeta) = f(0) + zeta (f(1) - f(0)): rows [x_{2i+1} - x_{2i}] times M_zeta, plus x_{2i}.
   // Vectors that sit at one stride (the dense plans put a slot's x vectors, then its y vectors,
   // one after another) go through one launch: segment s of Dh rows (padded to whole tiles); all
@@ -728,7 +753,6 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
   if (ys)   // the fold element is the first GR element of the Lagrange coefficients
     for (int c = 0; c < 6; ++c)
       if (ys->c[c]) launch_fold_lifted(st, ys->c[c], Dh, D, s.coef, yo.c[c]);
-  trace_round(ctx, trace, k, s);
   return cuda_check(ctx, "reduce_round");
 }
 
@@ -814,11 +838,11 @@ int inner_verify_dense(mpc_ctx* ctx, u64 vid, u32 batch, const Vec& x, const Vec
   u.ld = 64;
   v.ld = 64;
   if ((rc = party_sums(ctx, u, v, D + 1, s.Pmat, s.Sfull))) return rc;
-  inner_finish(ctx, s.Sfull, P_VER_DELTA, obj, s.tmp6);
-  rec1(ctx, s.tmp6, b.delta);
-  launch_gr_check_zero(st, b.delta, ctx->status, ST_VERIFY);
-  if (trace)
-    CK(cudaMemcpyAsync(trace + (long long)R * TRACE_ROUND, b.delta, 512, cudaMemcpyDeviceToDevice, st));
+  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);
+  const Rec1 r = begin_rec(ctx, s);
+  launch_delta(st, s.Sfull, ctx->k01, ctx->k02, obj, r.mask, r.idx, r.rec, b.delta,
+               trace ? trace + (long long)R * TRACE_ROUND : nullptr, ctx->status, ST_VERIFY);
+  flush_recs(ctx, s);
   return cuda_check(ctx, "inner_verify");
 }
 
@@ -1028,7 +1052,7 @@ struct TruncPlan {
   int R1 = 0, kd = 0;
   long long Dt = 0;
   long long L = 0, Epad = 0, nhi = 0;   // S = sum over e_hi < nhi of T_hi (x) (sum over e_lo < L ...)
-  u64 *b1, *b2, *Rtab, *S, *Zpq, *V, *W, *hsum, *S3, *zt, *S_hi, *Pst, *Thi, *Mhi;
+  u64 *b1, *b2, *Rtab, *S, *Zpq, *V, *W, *zt, *S_hi, *Pst, *Thi, *Mhi;
   u64 *B1T, *B2T;   // bit-transposed b1, b2: [j][e / 64]
   unsigned char* TL8;
   // tensor-core materialisation with r^(2e) = r^(2 Lm e_hi) r^(2 e_lo), e = e_hi Lm + e_lo:
@@ -1151,8 +1175,6 @@ TruncPlan plan_trunc(Arena& a, long long E, int R1, bool tc, bool chunked, const
   p.Zpq = a.take<u64>(12 * 64);
   p.V = a.take<u64>(4096);
   p.W = a.take<u64>(4096);
-  p.hsum = a.take<u64>(128);
-  p.S3 = a.take<u64>(2 * 192);
   p.zt = a.take<u64>(2 * 384);
   if (chunked) p.pqc = a.take<u64>(12 * E);
   if (h.Lm) {
@@ -1270,7 +1292,8 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
     CK(cudaMemcpy2DAsync(p.pqc, (size_t)E * 8, pq_all + e0, (size_t)E_all * 8, (size_t)E * 8, 12,
                          cudaMemcpyDeviceToDevice, st));
   const u64* pq = p.pqc ? p.pqc : pq_all;
-  reveal(ctx, P_VER_R, make_obj(verify_id, batch, 0), s.tmp6, s.r);
+  if ((rc = sums_begin(ctx, s))) return rc;
+  reveal(ctx, P_VER_R, make_obj(verify_id, batch, 0), s, s.r);
   launch_trunc_u(st, s.r, trunc_bits, p.V);                         // V_j = u_j
   for (int j = 0; j < 64; ++j)
     CK(cudaMemcpyAsync(p.W + j * 64, ctx->cst + CST_ONE, 512, cudaMemcpyDeviceToDevice, st));
@@ -1365,21 +1388,12 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
   u64* zbuf[2] = {s.z[0], s.z[1]};
   int zi = 0;
   for (int k = 1; k <= p.kd; ++k) {   // rounds folding the 64 bits of each output
-    const u64 obj = make_obj(verify_id, batch, (u32)k);
-    CK(cudaMemsetAsync(p.hsum, 0, 128 * 8, st));
-    launch_trunc_round_h(st, p.V, p.W, p.S, k, ctx->cst + CST_LAM, p.hsum);
-    CK(cudaMemsetAsync(p.S3, 0, 2 * 192 * 8, st));
-    CK(cudaMemcpyAsync(p.S3, p.hsum, 512, cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpyAsync(p.S3 + 192, p.hsum + 64, 512, cudaMemcpyDeviceToDevice, st));
-    inner_finish(ctx, p.S3, P_VER_H0, obj, s.h0);
-    inner_finish(ctx, p.S3 + 192, P_VER_H2, obj, s.h2);
-    reveal(ctx, P_VER_ZETA, obj, s.tmp6, s.zp);
-    launch_gr_lagrange(st, s.zp, ctx->reduce_mode, ctx->cst + CST_INV, s.coef);
-    launch_gr_combine_z(st, s.coef, s.h0, s.h2, z, zbuf[zi]);
+    u64* sums = cur_sums(s);
+    launch_trunc_round_sums(st, p.V, p.W, p.S, k, sums);
+    round_tail(ctx, verify_id, batch, k, z, zbuf[zi], s, sums, 64, tr);
     z = zbuf[zi];
     zi ^= 1;
     launch_trunc_update_vw(st, p.V, p.W, k, s.coef);
-    trace_round(ctx, tr, k, s);
   }
   delete phase;
   phase = new Phase(ctx, MPC_PROF_TRUNC_MATERIALIZE);
@@ -1566,7 +1580,6 @@ int mpc_create(const mpc_config* cfg, mpc_ctx** out) {
   std::memcpy(master.k, cfg->seed, 32);
   k_derive_keys<<<1, 32, 0, ctx->st>>>(master, keys_dev);
   launch_gr_inverses(ctx->st, ctx->cst + CST_INV);
-  launch_mode_consts(ctx->st, ctx->reduce_mode, ctx->cst + CST_LAM);
   k_init_consts<<<1, 64, 0, ctx->st>>>(ctx->reduce_mode, ctx->cst);
   e = cudaMemsetAsync(ctx->status, 0, sizeof(u32), ctx->st);
   if (e != cudaSuccess) return bail("cudaMemset", e);
@@ -2015,8 +2028,9 @@ int verify_mult_body(mpc_ctx* ctx, uint64_t verify_id, const u64* xs, const u64*
   cudaStream_t st = ctx->st;
   const Small& s = p.s;
   // Pi_Tran (Fig. MTP): reveal r; x'_i = r^i x_i; y lifted; z = sum r^i z_i
-  reveal(ctx, P_VER_R, make_obj(verify_id, 0, 0), s.tmp6, s.r);
   int rc;
+  if ((rc = sums_begin(ctx, s))) return rc;
+  reveal(ctx, P_VER_R, make_obj(verify_id, 0, 0), s, s.r);
   if ((rc = power_table(ctx, s.r, p.pp, p.pw, s.aux))) return rc;
   Vec& x = p.dv.x[0];
   Vec ylift;   // y stays in ring words until the first round folds it
@@ -2126,7 +2140,8 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
   const long long MK = M * K, KN = K * N;
   // ---- batch 0: the M N inner products of Z = X W, rank-1 consolidation ----
   Phase* phase = new Phase(ctx, MPC_PROF_VERIFY_GEMM);
-  reveal(ctx, P_VER_R, make_obj(verify_id, 0, 0), s.tmp6, s.r);
+  if ((rc = sums_begin(ctx, s))) return rc;
+  reveal(ctx, P_VER_R, make_obj(verify_id, 0, 0), s, s.r);
   launch_gr_powers(st, s.r, N, p.Q);                       // r^b
   launch_gr_mul1(st, p.Q + (N - 1) * 64, s.r, s.aux);      // rho = r^N
   launch_gr_powers(st, s.aux, M, p.P);                     // rho^a
@@ -2938,7 +2953,8 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     VMultPlan& v = p.vm;
     const Small& s = v.s;
     const long long n = p.nm;
-    reveal(ctx, P_VER_R, make_obj(vid, 0, 0), s.tmp6, s.r);
+    if ((rc = sums_begin(ctx, s))) return rc;
+    reveal(ctx, P_VER_R, make_obj(vid, 0, 0), s, s.r);
     if ((rc = power_table(ctx, s.r, v.pp, v.pw, s.aux))) return rc;
     Vec& x = v.dv.x[0];
     Vec ylift;
@@ -2955,7 +2971,8 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
   // ---- batch 1: the edaBit inner products, weight r^e on row e (e over all stages)
   {
     const Small& s = p.s1;
-    reveal(ctx, P_VER_R, make_obj(vid, 1, 0), s.tmp6, s.r);
+    if ((rc = sums_begin(ctx, s))) return rc;
+    reveal(ctx, P_VER_R, make_obj(vid, 1, 0), s, s.r);
     launch_gr_powers(st, s.r, p.ne, p.pw1);
     Vec ylift;
     for (int c = 0; c < 6; ++c) ylift.c[c] = p.Ye + c * p.D1;
@@ -2972,7 +2989,7 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     // Round 1 from the bits: x = r^g <m_i> pairs the bits 2k, 2k + 1 of one element, so the
     // party sums are sum_g r^g s(g) over per-element words (rows P1, P2 of each block; P0's are
     // zero) and the folded x is a selection among 0, r^g - r^g f, r^g f and r^g.
-    CK(cudaMemsetAsync(s.S, 0, 4 * 192 * 8, st));
+    u64* U = cur_sums(s);
     e0 = 0;
     for (int q = 0; q < p.nst; ++q) {
       CSPlan& c = p.cs[q];
@@ -2980,10 +2997,10 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
       g_launches += 1;
       e0 += c.np;
     }
-    launch_scalar_gr_sum(st, p.ne, p.S6, p.ne, 2, p.pw1, s.S + 64);                   // S00
-    launch_scalar_gr_sum(st, p.ne, p.S6 + 2 * p.ne, p.ne, 2, p.pw1, s.S + 192 + 64);  // S01 + S10
-    launch_scalar_gr_sum(st, p.ne, p.S6 + 4 * p.ne, p.ne, 2, p.pw1, s.S + 576 + 64);  // S11
-    round_tail(ctx, vid, 1, 1, s.zinit, s.z[1], s);
+    launch_scalar_gr_sum(st, p.ne, p.S6, p.ne, 2, p.pw1, U + 64);                   // S00
+    launch_scalar_gr_sum(st, p.ne, p.S6 + 2 * p.ne, p.ne, 2, p.pw1, U + 192 + 64);  // S01 + S10
+    launch_scalar_gr_sum(st, p.ne, p.S6 + 4 * p.ne, p.ne, 2, p.pw1, U + 576 + 64);  // S11
+    round_tail(ctx, vid, 1, 1, s.zinit, s.z[1], s, U, 64, tr1);
     Vec& xo = p.d1.x[1];
     Vec& yo = p.d1.y[1];
     if ((rc = gr_matmul(ctx, p.ne, p.pw1, nullptr, 1, 64, s.MM, nullptr, 0, p.A1, 64))) return rc;
@@ -2996,7 +3013,6 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     }
     const long long Dh = p.D1 / 2;
     for (int c = 0; c < 6; ++c) launch_fold_lifted(st, ylift.c[c], Dh, p.D1, s.coef, yo.c[c]);
-    trace_round(ctx, tr1, 1, s);
     if ((rc = cuda_check(ctx, "edaBit first round"))) return rc;
     p.d1.cur = 1;
     if ((rc = run_dense(ctx, vid, 1, p.d1, Dh, s.z[1], 2, p.R1, s, p.iv1, tr1))) return rc;
@@ -3025,7 +3041,8 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
   // single-Gram form
   {
     const Small& s = p.sb;
-    reveal(ctx, P_VER_R, make_obj(vid, 3, 0), s.tmp6, s.r);
+    if ((rc = sums_begin(ctx, s))) return rc;
+    reveal(ctx, P_VER_R, make_obj(vid, 3, 0), s, s.r);
     if ((rc = power_table(ctx, s.r, p.ppb, p.pwb, s.aux))) return rc;
     Vec& x = p.db.x[0];
     Vec ylift{};   // components 1 and 5 of the b2 bits, as ring words

@@ -1,0 +1,99 @@
+// Block-cooperative products in GR(2^64, 64) by 64 P threads, for the single-element steps of the
+// verification (challenges, claims, weights), which are chains of dependent products: their time
+// is the latency of one product, so a product is spread over P threads per coefficient.
+#pragma once
+#include "common.cuh"
+
+namespace mpc3 {
+
+// Coefficient c of the reduction mod f of a 127-coefficient product (lo: coefficients 0..63, hi:
+// 64..126, hi[63] ignored).
+__device__ __forceinline__ u64 gr_reduce_at(const u64* lo, const u64* hi, int c) {
+  u64 v = lo[c] - gr_hg(hi, c);
+  if (c < 7) {
+    u64 h2[3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) h2[m] = gr_hg(hi, 64 + m);
+    u64 g = 0;
+    if (c < 3) g += h2[c];
+    if (c - 1 >= 0 && c - 1 < 3) g += h2[c - 1];
+    if (c - 3 >= 0 && c - 3 < 3) g += h2[c - 3];
+    if (c - 4 >= 0 && c - 4 < 3) g += h2[c - 4];
+    v += g;
+  }
+  return v;
+}
+
+// lo += product terms of coefficient t, hi += those of coefficient 64 + t, over the factors
+// a_i, i0 <= i < i0 + N.
+template <int N>
+__device__ __forceinline__ void gr_mac_part(const u64* a, const u64* b, int t, int i0, u64& lo,
+                                            u64& hi) {
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const int i = i0 + k;
+    const u64 pr = a[i] * b[(t - i) & 63];
+    if (i <= t) lo += pr; else hi += pr;
+  }
+}
+
+// The sum of the P parts' (lo, hi) and its reduction: every thread of the block calls it (sub =
+// the thread's index in its group of 64 P, scr = the group's 128 P words); returns coefficient
+// sub of the result to the threads sub < 64.  A thread whose group has no product passes zeros.
+template <int P>
+__device__ __forceinline__ u64 gr_finish(u64 lo, u64 hi, u64* scr, int sub) {
+  const int t = sub & 63, part = sub >> 6;
+  scr[part * 128 + t] = lo;
+  scr[part * 128 + 64 + t] = hi;
+  __syncthreads();
+  if (P > 1) {
+    if (sub < 128) {
+      u64 v = scr[sub];
+#pragma unroll
+      for (int p = 1; p < P; ++p) v += scr[p * 128 + sub];
+      scr[sub] = v;
+    }
+    __syncthreads();
+  }
+  const u64 r = sub < 64 ? gr_reduce_at(scr, scr + 64, sub) : 0ull;
+  __syncthreads();
+  return r;
+}
+
+// a * b by a group of 64 P threads; all threads of the block call it (a, b in shared memory).
+template <int P>
+__device__ __forceinline__ u64 gr_mul_par(const u64* a, const u64* b, u64* scr, int sub) {
+  u64 lo = 0, hi = 0;
+  gr_mac_part<64 / P>(a, b, sub & 63, (sub >> 6) * (64 / P), lo, hi);
+  return gr_finish<P>(lo, hi, scr, sub);
+}
+
+// Coefficient t of x v and of x^2 v (x^64 = -(x^4 + x^3 + x + 1)).
+__device__ __forceinline__ u64 gr_x_at(const u64* v, int t) {
+  u64 r = t > 0 ? v[t - 1] : 0ull;
+  if (t == 0 || t == 1 || t == 3 || t == 4) r -= v[63];
+  return r;
+}
+__device__ __forceinline__ u64 gr_x2_at(const u64* v, int t) {
+  u64 r = t > 1 ? v[t - 2] : 0ull;
+  if (t == 0 || t == 1 || t == 3 || t == 4) r -= v[62];
+  if (t == 1 || t == 2 || t == 4 || t == 5) r -= v[63];
+  return r;
+}
+
+// Entry (i, t) of the multiplication matrix of a: coefficient t of a x^i, 0 <= i < 64.
+__device__ __forceinline__ u64 gr_mulmat_at(const u64* a, int i, int t) {
+  // a x^i = sum_m a_m x^(m + i); coefficient 64 + m of the unreduced product is a_(64 + m - i)
+  // for m < i, else 0
+  auto h = [&](int m) -> u64 { return (m >= 0 && m < i) ? a[64 + m - i] : 0ull; };
+  auto hg = [&](int s) -> u64 { return h(s) + h(s - 1) + h(s - 3) + h(s - 4); };
+  u64 v = (t >= i ? a[t - i] : 0ull) - hg(t);
+  if (t < 7) {
+    const u64 h0 = hg(64), h1 = hg(65), h2 = hg(66);
+    auto q = [&](int m) -> u64 { return m == 0 ? h0 : m == 1 ? h1 : m == 2 ? h2 : 0ull; };
+    v += q(t) + q(t - 1) + q(t - 3) + q(t - 4);
+  }
+  return v;
+}
+
+}  // namespace mpc3

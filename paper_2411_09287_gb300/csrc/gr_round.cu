@@ -1,0 +1,381 @@
+// The single-element steps of the batched verification over GR(2^64, 64), one launch per protocol
+// round: everything of a Pi_Reduce round between its party sums and its folds (k_round_tail), the
+// revealed challenges, the opened Delta, and the hashes of their Pi_Rec calls.
+//
+// These steps are chains of products of single GR elements: they move a few KB and are bound by
+// latency alone.  As separate launches (reduction of the Gram blocks, quadratic combination, two
+// inner-product finishes, the random sharing, Pi_Rec with its SHA-256, Lagrange weights, the next
+// claim, the fold matrix, three trace copies) a round took about 95 us of kernel time, 20 us of it
+// SHA-256 on one thread per digest.  Fused, with the products by the interpolation points x and
+// 1 - x as shifts, the Lagrange weights from one square and one product, and the hash comparisons
+// of all of a batch's Pi_Rec calls in one launch at its end, a round's tail is one launch.
+#include "gr_mul.cuh"
+#include "kernels.h"
+
+namespace mpc3 {
+
+namespace {
+
+// The 64 words (8 ChaCha20 blocks) of a stream into w; threads lane = 0..7 each write 8 words.
+__device__ __forceinline__ void stream64(const Key& k, u32 tag, u64 obj, int lane, u64* w) {
+  u64 o[8];
+  prf_block8(k, tag, obj, (u64)lane, o);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) w[lane * 8 + j] = o[j];
+}
+
+// The messages of Pi_Rec of a shared element with streams (r1, r2, m), for the batch's hash
+// comparison: rows of 64 words: the three values as their senders hold them ([r]_1, [r]_2, m at
+// P0, P0, P1), as their hashers hold them ([r]_1 at P1, [r]_2 at P2, m at P2), and [r]_2 as it
+// arrived at P1.
+constexpr int REC_ROWS = 7;
+
+// One Pi_Reduce round after its party sums (Fig. Reduce): h(0) and h(p2) by secure GR inner
+// products, zeta' drawn and opened, the next claim z' = L0 h(0) + L1 (z - h(0)) + L2 h(p2), the
+// fold element f and its multiplication matrix.  Block c < 6 computes component c of h(0), h(p2)
+// and z'; block 6 the matrix, the Pi_Rec messages and the next round's cleared sums.  Every block
+// derives zeta' from its streams, so that no block waits for another.
+//
+// L0 + L1 + L2 = 1 in both readings of the third point, hence z' = h(0) + L1 (z - 2 h(0)) +
+// L2 (h(p2) - h(0)), with (points 0, 1, x) L2 = (z^2 - z) / (x (x - 1)), L1 = z - (z^2 - z) / x -
+// L2, z = zeta'; (points 0, 1, 2) L2 = 2 z^2 - z, L1 = 4 z - 4 z^2, zeta = 2 zeta'.
+__global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
+  __shared__ u64 st[9][64];       // streams: H0 (r1, r2, g1), H2 (r1, r2, g1), zeta (r1, r2, m)
+  __shared__ u64 zt[64], sq[64], L1[64], L2[64], inv[64], va[64], vb[64];
+  __shared__ u64 S[9][64];        // reduced party sums: ee (3 parties), cross, oo
+  __shared__ u64 scr[2][4 * 128];
+  const int tid = threadIdx.x, blk = blockIdx.x;
+  const int t = tid & 63;
+  if (tid < 72) {
+    const int s = tid >> 3, q = s % 3, g = s / 3;
+    const u32 purpose = g == 0 ? P_VER_H0 : g == 1 ? P_VER_H2 : P_VER_ZETA;
+    const Key& key = q == 0 ? a.k01 : q == 1 ? a.k02 : (g == 2 ? a.k12 : a.k01);
+    const u32 comp = q == 0 ? C_R1 : q == 1 ? C_R2 : (g == 2 ? C_M12 : C_G1);
+    stream64(key, make_tag(purpose, comp), a.obj, tid & 7, st[s]);
+  } else if (tid >= 128 && tid < 192) {
+    inv[t] = a.inv[t];
+  }
+  const bool msg = blk == 2 || blk == 4;   // the components m, which take the party sums
+  if (msg && tid >= 192) {
+    for (int i = tid - 192; i < 9 * 64; i += 320) {
+      const int q = i >> 6, c = i & 63;
+      const u64* s0 = a.sums + (q < 3 ? q : q < 6 ? q : q + 3) * a.ld;   // ee, S01, oo
+      u64 v = a.ld == 128 ? gr_reduce_at(s0, s0 + 64, c) : s0[c];
+      if (q >= 3 && q < 6) {   // cross: S01 + S10
+        const u64* s1 = a.sums + (q + 3) * a.ld;
+        v += a.ld == 128 ? gr_reduce_at(s1, s1 + 64, c) : s1[c];
+      }
+      S[q][c] = v;
+    }
+  }
+  __syncthreads();
+  if (tid < 64) {   // P1's opening: m - [r]_1 - [r]_2 as received
+    const u64 r2 = st[7][t] ^ (t == a.xidx ? a.xmask : 0ull);
+    zt[t] = st[8][t] - st[6][t] - r2;
+  }
+  __syncthreads();
+  if (blk == 6) {
+    __shared__ u64 fe[64];
+    if (tid < 64) {
+      const u64 f = a.mode == 1 ? 2 * zt[t] : zt[t];
+      fe[t] = f;
+      a.coef[t] = f;
+      a.coef[384 + t] = (t == 0 ? 1ull : 0ull) - f;
+      a.zp[t] = zt[t];
+      if (a.trace) a.trace[t] = zt[t];
+    } else if (tid < 128) {
+      u64* l = a.rec;
+      l[t] = st[6][t];             // [r]_1 sent by P0
+      l[64 + t] = st[7][t];        // [r]_2 sent by P0
+      l[128 + t] = st[8][t];       // m sent by P1
+      l[192 + t] = st[6][t];       // [r]_1 held by P1
+      l[256 + t] = st[7][t];       // [r]_2 held by P2
+      l[320 + t] = st[8][t];       // m held by P2
+      l[384 + t] = st[7][t] ^ (t == a.xidx ? a.xmask : 0ull);   // [r]_2 received by P1
+    }
+    __syncthreads();
+    for (int i = tid; i < 4096; i += 512) a.MM[i] = gr_mulmat_at(fe, i >> 6, i & 63);
+    for (long long i = tid; i < a.nzero; i += 512) a.zero[i] = 0ull;
+    return;
+  }
+  const int sub = tid & 255, grp = tid >> 8;
+  // z^2 (the second group idles), then L2
+  u64 r = gr_mul_par<4>(zt, zt, scr[grp], sub);
+  if (tid < 64) sq[t] = a.mode == 1 ? r : r - zt[t];   // z^2, or z^2 - z
+  __syncthreads();
+  if (a.mode == 1) {
+    if (tid < 64) {
+      L2[t] = 2 * sq[t] - zt[t];
+      L1[t] = 4 * zt[t] - 4 * sq[t];
+    }
+  } else {
+    r = gr_mul_par<4>(inv, sq, scr[grp], sub);
+    if (tid < 64) {
+      // (z^2 - z) / x: the coefficients move down one, the constant term times
+      // x^-1 = -(x^63 + x^3 + x^2 + 1)
+      u64 u = t < 63 ? sq[t + 1] : 0ull;
+      if (t == 0 || t == 2 || t == 3 || t == 63) u -= sq[0];
+      L2[t] = r;
+      L1[t] = zt[t] - u - r;
+    }
+  }
+  u64 h0 = 0, z = 0;
+  if (tid < 64) {
+    u64 h2;
+    if (msg) {
+      // P0: Gamma = S0 + r1 + r2, sends Gamma - g1 to P2; P1: S1 + g1; P2: S2 + (received)
+      u64 q[3], e[3];
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        const u64 *s00 = S[p], *sx = S[3 + p], *s11 = S[6 + p];
+        e[p] = s00[t];
+        if (a.mode == 1) {   // p2 = 2: (1 - p2)^2 = 1, (1 - p2) p2 = -2, p2^2 = 4
+          q[p] = s00[t] - 2 * sx[t] + 4 * s11[t];
+        } else {             // p2 = x: S00 + x (Sx - 2 S00) + x^2 (S00 - Sx + S11)
+          q[p] = s00[t] + gr_x_at(sx, t) - 2 * gr_x_at(s00, t) + gr_x2_at(s00, t) -
+                 gr_x2_at(sx, t) + gr_x2_at(s11, t);
+        }
+      }
+      const u64 g20 = e[0] + st[0][t] + st[1][t] - st[2][t];
+      h0 = (e[1] + st[2][t]) + (e[2] + g20);
+      const u64 g22 = q[0] + st[3][t] + st[4][t] - st[5][t];
+      h2 = (q[1] + st[5][t]) + (q[2] + g22);
+    } else {
+      const int s = (blk == 0 || blk == 3) ? 0 : 1;   // [r]_1 or [r]_2
+      h0 = st[s][t];
+      h2 = st[3 + s][t];
+    }
+    z = a.z[blk * 64 + t];
+    va[t] = z - 2 * h0;
+    vb[t] = h2 - h0;
+    if (a.trace) {
+      a.trace[64 + blk * 64 + t] = h0;
+      a.trace[448 + blk * 64 + t] = h2;
+    }
+  }
+  __syncthreads();
+  r = gr_mul_par<4>(grp ? L2 : L1, grp ? vb : va, scr[grp], sub);
+  if (grp == 1 && sub < 64) sq[t] = r;
+  __syncthreads();
+  if (tid < 64) a.zo[blk * 64 + t] = h0 + r + sq[t];
+}
+
+// <v> random GR element (streams of `purpose`), opened with Pi_Rec; its messages go to rec.
+__global__ void __launch_bounds__(64)
+k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u64* __restrict__ out,
+         u64* __restrict__ rec) {
+  __shared__ u64 st[3][64];
+  const int t = threadIdx.x;
+  if (t < 24) {
+    const int s = t >> 3;
+    stream64(s == 0 ? k01 : s == 1 ? k02 : k12,
+             make_tag(purpose, s == 0 ? C_R1 : s == 1 ? C_R2 : C_M12), obj, t & 7, st[s]);
+  }
+  __syncthreads();
+  const u64 r1 = st[0][t], r2 = st[1][t], m = st[2][t];
+  const u64 r2in = r2 ^ (t == xidx ? xmask : 0ull);
+  rec[t] = r1;
+  rec[64 + t] = r2;
+  rec[128 + t] = m;
+  rec[192 + t] = r1;
+  rec[256 + t] = r2;
+  rec[320 + t] = m;
+  rec[384 + t] = r2in;
+  out[t] = m - r1 - r2in;
+}
+
+// Delta of Pi_InnerVerify from its party sums S (3 x 64, reduced): the secure inner product's
+// finish, Pi_Rec of the result (messages to rec), and `flag` in *status unless it is zero.
+__global__ void __launch_bounds__(64)
+k_delta(const u64* __restrict__ S, Key k01, Key k02, u64 obj, u64 xmask, int xidx,
+        u64* __restrict__ rec, u64* __restrict__ out, u64* __restrict__ trace, u32* status,
+        u32 flag) {
+  __shared__ u64 st[3][64];
+  const int t = threadIdx.x;
+  if (t < 24) {
+    const int s = t >> 3;
+    stream64(s == 1 ? k02 : k01, make_tag(P_VER_DELTA, s == 0 ? C_R1 : s == 1 ? C_R2 : C_G1), obj,
+             t & 7, st[s]);
+  }
+  __syncthreads();
+  const u64 r1 = st[0][t], r2 = st[1][t], g1 = st[2][t];
+  const u64 g2 = S[t] + r1 + r2 - g1;                       // P0 -> P2
+  const u64 m1 = (S[64 + t] + g1) + (S[128 + t] + g2);      // P1: own + received
+  const u64 m2 = m1;                                        // P2: received + own
+  const u64 r2in = r2 ^ (t == xidx ? xmask : 0ull);
+  rec[t] = r1;
+  rec[64 + t] = r2;
+  rec[128 + t] = m1;
+  rec[192 + t] = r1;
+  rec[256 + t] = r2;
+  rec[320 + t] = m2;
+  rec[384 + t] = r2in;
+  const u64 d = m1 - r1 - r2in;
+  out[t] = d;
+  if (trace) trace[t] = d;
+  if (d != 0ull) atomicOr(status, flag);
+}
+
+// The hash comparisons of n Pi_Rec calls of single GR elements (one block each): P1 sends H([r]_1)
+// to P2, P2 sends H(m) to P0 and H([r]_2) to P1, and every receiver hashes what it received; a
+// mismatch sets `flag` in *status.  Six digests of 512 bytes: the message schedules (plus round
+// constants) of all 6 x 9 blocks first, by one thread each, then six threads run the rounds, whose
+// dependent chain is what the launch takes.
+__global__ void __launch_bounds__(64)
+k_rec_hash(const u64* __restrict__ log, u32* status, u32 flag) {
+  constexpr int LD = 55;             // words of one schedule step, 54 used
+  __shared__ u32 wk[64 * LD];
+  __shared__ u32 dig[6][8];
+  const u64* rec = log + (long long)blockIdx.x * (REC_ROWS * 64);
+  const int tid = threadIdx.x;
+  if (tid < 54) {
+    const int hsh = tid / 9, b = tid % 9;
+    // P1's [r]_1, P2's m, P2's [r]_2; received: [r]_1 at P2, m at P0, [r]_2 at P1
+    const int row = hsh == 0 ? 3 : hsh == 1 ? 5 : hsh == 2 ? 4 : hsh == 3 ? 0 : hsh == 4 ? 2 : 6;
+    u32 w[16];
+    if (b < 8) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const u64 v = rec[row * 64 + b * 8 + q];
+        w[2 * q] = bswap32((u32)v);
+        w[2 * q + 1] = bswap32((u32)(v >> 32));
+      }
+    } else {   // padding of a 512-byte message
+#pragma unroll
+      for (int q = 0; q < 16; ++q) w[q] = 0;
+      w[0] = 0x80000000u;
+      w[15] = 4096u;
+    }
+#pragma unroll
+    for (int i = 0; i < 64; ++i) {
+      u32 v = w[i & 15];
+      if (i >= 16) {
+        const u32 w15 = w[(i - 15) & 15], w2 = w[(i - 2) & 15];
+        v += (rotr32(w15, 7) ^ rotr32(w15, 18) ^ (w15 >> 3)) + w[(i - 7) & 15] +
+             (rotr32(w2, 17) ^ rotr32(w2, 19) ^ (w2 >> 10));
+        w[i & 15] = v;
+      }
+      wk[i * LD + tid] = v + SHA_K[i];
+    }
+  }
+  __syncthreads();
+  if (tid < 6) {
+    u32 h[8];
+    sha256_init(h);
+#pragma unroll 1
+    for (int b = 0; b < 9; ++b) {
+      const u32* W = wk + tid * 9 + b;
+      u32 s[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s[q] = h[q];
+#pragma unroll 16
+      for (int i = 0; i < 64; ++i) {
+        const u32 S1 = rotr32(s[4], 6) ^ rotr32(s[4], 11) ^ rotr32(s[4], 25);
+        const u32 ch = (s[4] & s[5]) ^ (~s[4] & s[6]);
+        const u32 t1 = (s[7] + W[i * LD]) + S1 + ch;
+        const u32 S0 = rotr32(s[0], 2) ^ rotr32(s[0], 13) ^ rotr32(s[0], 22);
+        const u32 mj = (s[0] & s[1]) ^ (s[0] & s[2]) ^ (s[1] & s[2]);
+        s[7] = s[6]; s[6] = s[5]; s[5] = s[4]; s[4] = s[3] + t1;
+        s[3] = s[2]; s[2] = s[1]; s[1] = s[0]; s[0] = t1 + S0 + mj;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) h[q] += s[q];
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) dig[tid][q] = h[q];
+  }
+  __syncthreads();
+  if (tid < 8 && (dig[0][tid] != dig[3][tid] || dig[1][tid] != dig[4][tid] ||
+                  dig[2][tid] != dig[5][tid]))
+    atomicOr(status, flag);
+}
+
+// One round of the first rounds of the truncation batch (index i = 64 e + j, so that round k
+// folds bit k - 1 of j): with V_j, W_j the accumulated public weights of the x- and y-side bit j
+// and S_{j,j'} = sum_e r^(2e) b1_{e,j} b2_{e,j'}, the sums over the pairs (j, j') of one 2^k-block
+//   out[2 a + b] += sum_{bit k-1 of j = a, of j' = b} V_j W_j' S_{j,j'},  64 words at 192 (2 a + b)
+// (P0's S00, S01, S10, S11 of the round; out must be zero on entry).  Block (j, c) takes the c-th
+// eight j' of j's 2^k-block: the eight products share one reduction, so a block runs three
+// dependent products' latency.  One thread group per j ran 2^k + 5 products one after another:
+// 201 us for k = 6, 461 us for the six rounds.
+__global__ void __launch_bounds__(256)
+k_trunc_round_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64* __restrict__ S,
+                   int k, u64* __restrict__ out) {
+  __shared__ u64 w[8][64], s[8][64], T[2][64], v[64], scr[4 * 128];
+  const int tid = threadIdx.x, t = tid & 63, part = tid >> 6;
+  const int j = blockIdx.x, sh = k - 1, bs = 1 << k;
+  const int n = bs < 8 ? bs : 8;
+  const int j0 = (j & ~(bs - 1)) + blockIdx.y * 8;
+  for (int i = tid; i < n * 64; i += 256) {
+    w[i >> 6][i & 63] = W[(j0 + (i >> 6)) * 64 + (i & 63)];
+    s[i >> 6][i & 63] = S[((long long)j * 64 + j0 + (i >> 6)) * 64 + (i & 63)];
+  }
+  if (tid < 64) v[t] = V[j * 64 + t];
+  __syncthreads();
+  // halves of the block: with eight j' of a larger block they all lie in one half
+  u64 lo[2] = {0, 0}, hi[2] = {0, 0};
+  for (int q = 0; q < n; ++q) {
+    u64 l = 0, h = 0;
+    gr_mac_part<16>(w[q], s[q], t, part * 16, l, h);
+    if (((j0 + q) >> sh) & 1) { lo[1] += l; hi[1] += h; }
+    else { lo[0] += l; hi[0] += h; }
+  }
+  const int aj = (j >> sh) & 1;
+  for (int b = 0; b < 2; ++b) {
+    if (n == 8 && bs > 8 && (((j0 >> sh) & 1) != b)) continue;   // uniform over the block
+    const u64 r = gr_finish<4>(lo[b], hi[b], scr, tid);
+    if (tid < 64) T[b][t] = r;
+    __syncthreads();
+    const u64 y = gr_mul_par<4>(v, T[b], scr, tid);
+    if (tid < 64)
+      atomicAdd(reinterpret_cast<unsigned long long*>(out + 192 * (2 * aj + b) + t),
+                (unsigned long long)y);
+  }
+}
+
+// After round k: V_j <- w(j) V_j and W_j <- w(j) W_j with w = 1 - f or f by bit k-1 of j
+// (coef: f at 0, 1 - f at 384).
+__global__ void __launch_bounds__(256)
+k_trunc_update_vw(u64* __restrict__ V, u64* __restrict__ W, int k, const u64* __restrict__ coef) {
+  __shared__ u64 a[64], b[64], scr[4 * 128];
+  const int j = blockIdx.x & 63;
+  u64* X = (blockIdx.x < 64) ? V : W;
+  const int t = threadIdx.x;
+  if (t < 64) a[t] = ((j >> (k - 1)) & 1) ? coef[t] : coef[384 + t];
+  else if (t < 128) b[t - 64] = X[j * 64 + t - 64];
+  __syncthreads();
+  const u64 r = gr_mul_par<4>(a, b, scr, t);
+  if (t < 64) X[j * 64 + t] = r;
+}
+
+}  // namespace
+
+void launch_round_tail(cudaStream_t st, const RoundTail& a) { k_round_tail<<<7, 512, 0, st>>>(a); }
+
+void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
+                   int xidx, u64* out, u64* rec) {
+  k_reveal<<<1, 64, 0, st>>>(k01, k02, k12, purpose, obj, xmask, xidx, out, rec);
+}
+
+void launch_delta(cudaStream_t st, const u64* S, Key k01, Key k02, u64 obj, u64 xmask, int xidx,
+                  u64* rec, u64* out, u64* trace, u32* status, u32 flag) {
+  k_delta<<<1, 64, 0, st>>>(S, k01, k02, obj, xmask, xidx, rec, out, trace, status, flag);
+}
+
+void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 flag) {
+  if (n <= 0) return;
+  static_assert(REC_ROWS * 64 == REC_WORDS, "record size");
+  k_rec_hash<<<n, 64, 0, st>>>(log, status, flag);
+}
+
+void launch_trunc_round_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int k,
+                             u64* out) {
+  const int bs = 1 << k;
+  k_trunc_round_sums<<<dim3(64, bs < 8 ? 1 : bs / 8), 256, 0, st>>>(V, W, S, k, out);
+}
+
+void launch_trunc_update_vw(cudaStream_t st, u64* V, u64* W, int k, const u64* coef) {
+  k_trunc_update_vw<<<128, 256, 0, st>>>(V, W, k, coef);
+}
+
+}  // namespace mpc3

@@ -104,8 +104,8 @@ int gr_matmul_tc_ex(cudaStream_t st, const GrMMArgs& a, unsigned* err, unsigned 
 // One job of a batched tensor-core Gram launch.  u = a0 + sa1 a1 and v = b0 + sb1 b1 (a1, b1 may
 // be null; every pointer 16-byte aligned) are vectors of GR elements (rows of 64 words,
 // contiguous); over their Dh element pairs (2i, 2i + 1) the job adds, mod 2^64,
-//   P[0] += sign G(u_e, v_e),  P[off_oo] += sign G(u_o, v_o),  P[off_x] += sign (G(u_e, v_o) + G(u_o, v_e))
-// with G(u, v)[a][b] = sum_i u_i[a] v_i[b] a 64 x 64 block.
+//   P[0] += sign C(u_e, v_e),  P[off_oo] += sign C(u_o, v_o),  P[off_x] += sign (C(u_e, v_o) + C(u_o, v_e))
+// with C(u, v) = sum_i u_i v_i as its 127 unreduced product coefficients (a block of 128 words).
 struct GramJob {
   const u64* a0;
   const u64* a1;
@@ -127,11 +127,47 @@ struct GramJobs {
 // bad job (null or misaligned pointers), 0 otherwise.
 int gram_jobs_tc(cudaStream_t st, long long Dh, const GramJobs& jobs, unsigned* err,
                  unsigned err_flag, int nsplit = 0);
-// P[0..2] (3 x 4096 words, accumulated mod 2^64) += the Gram sums G(x_e, y_e), G(x_o, y_o),
-// G(x_e, y_o) + G(x_o, y_e) over the Dh element pairs (x_{2i}, x_{2i+1}) of x and y (rows of 64
-// words, contiguous).  Exact, on the tensor cores; returns -1 for misaligned inputs.
+// The single-source job of x and y with P = party 0's blocks of a round's sums (S00 at 0, the
+// cross sum at 3 * 128, S11 at 9 * 128).  Returns -1 for misaligned inputs.
 int gram3_tc(cudaStream_t st, long long Dh, const u64* x, const u64* y, u64* P, unsigned* err,
              unsigned err_flag, int nsplit = 0);
+
+// ---- single-element steps of the verification (gr_round.cu) ---------------------------------
+// Words of one opened element's record: the copies that Pi_Rec's hashes compare.
+constexpr int REC_WORDS = 7 * 64;
+struct RoundTail {
+  const u64* sums;      // 12 blocks of party sums (S00, S01, S10, S11; three parties each)
+  int ld;               // words per block: 64 (reduced) or 128 (unreduced coefficients)
+  int mode;             // MPC_REDUCE_POINT_X or MPC_REDUCE_POINT_2
+  Key k01, k02, k12;
+  u64 obj;              // the round's stream object
+  const u64* inv;       // (x (x - 1))^-1
+  const u64* z;         // the claim entering the round, 6 x 64
+  u64* zo;              // the next claim (not z)
+  u64* coef;            // the fold element f at 0, 1 - f at 384
+  u64* MM;              // the multiplication matrix of f
+  u64* zp;              // the opened zeta'
+  u64* rec;             // this Pi_Rec's record (REC_WORDS)
+  u64 xmask;            // fault: word xidx of the P0 -> P1 message is XORed with xmask
+  int xidx;
+  u64* zero;            // nzero words cleared for the next round
+  long long nzero;
+  u64* trace;           // zeta' | h(0) | h(p2) of the round, or null
+};
+void launch_round_tail(cudaStream_t st, const RoundTail& a);
+// A random GR element of the streams of (purpose, obj), opened into out; record in rec.
+void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
+                   int xidx, u64* out, u64* rec);
+// Delta from the party sums S (3 x 64, reduced), opened into out (and trace when not null); `flag`
+// in *status unless it is zero.
+void launch_delta(cudaStream_t st, const u64* S, Key k01, Key k02, u64 obj, u64 xmask, int xidx,
+                  u64* rec, u64* out, u64* trace, u32* status, u32 flag);
+// The hash comparisons of n records: `flag` in *status on a mismatch.
+void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 flag);
+// Round k's sums S00, S01, S10, S11 (192 words apart, added into out) of the bit rounds.
+void launch_trunc_round_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int k,
+                             u64* out);
+void launch_trunc_update_vw(cudaStream_t st, u64* V, u64* W, int k, const u64* coef);
 
 // ---- elementwise protocol kernels (prf_kernels.cu) ------------------------------------------
 void launch_share_input(cudaStream_t st, const u64* x, long long n, Key k01, Key k02, u64 obj,
@@ -186,11 +222,7 @@ void launch_gr_lincomb(cudaStream_t st, const u64* ca, const u64* a, const u64* 
                        u64* out);
 void launch_gr_mulmat2(cudaStream_t st, const u64* a, const u64* b, u64* M);
 void launch_gr_inverses(cudaStream_t st, u64* out);
-void launch_gr_lagrange(cudaStream_t st, const u64* zeta_prime, int mode, const u64* inv,
-                        u64* coef);
 void launch_gr_fold_reduce(cudaStream_t st, const u64* P, int n, u64* out);
-void launch_gr_combine_z(cudaStream_t st, const u64* coef, const u64* h0, const u64* h2,
-                         const u64* z, u64* znew);
 void launch_gr_scale_rows(cudaStream_t st, const u64* pw, const u64* s, long long n, u64* out);
 void launch_gr_lift(cudaStream_t st, const u64* s, long long n, u64* out);
 // First-round party sums and folds of a claim whose y vectors are lifted ring words (one word per
@@ -202,11 +234,7 @@ void launch_gram_lifted(cudaStream_t st, const u64* const x[6], const u64* const
 void launch_fold_lifted(cudaStream_t st, const u64* Y, long long Dh, long long D, const u64* f,
                         u64* out);
 void launch_neg_copy(cudaStream_t st, const u64* a, long long n, u64* out);
-void launch_gr_check_zero(cudaStream_t st, const u64* v, u32* status, u32 flag);
 void launch_trunc_u(cudaStream_t st, const u64* r, int t, u64* u);
-void launch_trunc_round_h(cudaStream_t st, const u64* V, const u64* W, const u64* S, int k,
-                          const u64* lam, u64* out);
-void launch_trunc_update_vw(cudaStream_t st, u64* V, u64* W, int k, const u64* coef);
 // out[c] += sum_{e < n} A[c * lda + e] * R[e] (R: n GR elements), c < nrows <= 16, atomically
 void launch_scalar_gr_sum(cudaStream_t st, long long n, const u64* A, long long lda, int nrows,
                           const u64* R, u64* out);
@@ -226,13 +254,6 @@ void launch_word_transpose(cudaStream_t st, long long rows, long long cols, long
                            const u64* in, u64* out);
 void launch_trunc_materialize(cudaStream_t st, long long E, const u64* words, const u64* VW,
                               const u64* R, int kd, u64* out);
-void launch_gr_rec1(cudaStream_t st, const u64* s6, u64 xor_mask, int xor_idx, u64* out,
-                    u32* status, u32 flag);
-void launch_gr_inner_finish_all(cudaStream_t st, const u64* S, Key k01, Key k02, u32 purpose,
-                                u64 obj, u64* h6);
-void launch_gr_quad_combine(cudaStream_t st, const u64* lam, const u64* S00, const u64* S01,
-                            const u64* S10, const u64* S11, u64* out);
-void launch_mode_consts(cudaStream_t st, int mode, u64* cst);
 // PRF words off .. off + n - 1 of one stream into out[0 .. n) (e.g. the truncation bits b1, b2
 // of the outputs of one verification chunk)
 void launch_prf_words(cudaStream_t st, long long n, Key key, u32 tag, u64 obj, u64* out,

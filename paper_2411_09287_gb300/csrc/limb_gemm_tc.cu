@@ -1478,12 +1478,12 @@ k_gr_matmul_tm(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ 
 
 // ---- Gram sums of the dense Pi_Reduce rounds -------------------------------------------------
 // For vectors u, v of n = 2 Dh GR elements (rows of 64 words, element i at row i) a job adds
-//   P[ee] += s G(u_even, v_even), P[oo] += s G(u_odd, v_odd), P[x] += s (G(u_even, v_odd) + G(u_odd, v_even))
-// with G(u, v)[a][b] = sum_i u_i[a] v_i[b] (each block a 64 x 64 matrix, mod 2^64) and s the job's
-// sign; u = a0 + sa1 a1 and v = b0 + sb1 b1 (a1, b1 may be absent).  The MMA tile is M = 128
+//   P[ee] += s C(u_even, v_even), P[oo] += s C(u_odd, v_odd), P[x] += s (C(u_even, v_odd) + C(u_odd, v_even))
+// with G(u, v)[a][b] = sum_i u_i[a] v_i[b] (a 64 x 64 matrix, mod 2^64), C its 127 anti-diagonal
+// sums (the coefficients of sum_i u_i v_i before the reduction mod f) and s the job's sign; u = a0 + sa1 a1 and v = b0 + sb1 b1 (a1, b1 may be absent).  The MMA tile is M = 128
 // (rows a: u_even coefficients, then u_odd) x N = 64 (v of one parity, blockIdx.y) with K = the
-// element pairs i, split across blockIdx.x; blockIdx.z is the job; each CTA adds its partial tile
-// atomically.  Producers combine and split the rows into digit planes transposed to K-major; MMA
+// element pairs i, split across blockIdx.x; blockIdx.z is the job; each CTA adds its partial
+// coefficients atomically.  Producers combine and split the rows into digit planes transposed to K-major; MMA
 // issue and drains as in k_limb_gemm_tc; the drain warps accumulate over all of the CTA's chunks.
 constexpr size_t GR_SMEM = (size_t)NSTAGE * STAGE + 1024;   // 2 x (64 KB A + 32 KB B)
 
@@ -1683,18 +1683,31 @@ k_gram_tc(long long Dh, const GramJobs jobs, unsigned* __restrict__ err, unsigne
         if (lane == 0) mbar_arrive(&acce_bar[g]);
       }
     }
-    if (ok && !*abort && nunits > 0) {
-      const int a = q4 * 32 + lane;                // tile row: x parity a / 64, coefficient a % 64
-      const int xpar = a >> 6;
-      // (x parity, y parity) -> P block: (0,0) -> ee, (1,1) -> oo, mixed -> cross
-      const long long blk = xpar != par ? jobs.off_x : (xpar ? jobs.off_oo : 0);
-      u64* dst = J.P + blk + (a & 63) * 64 + h * GM_DC;
-      const u64 sg = J.sign;
+    if (!ok && lane == 0) fail();
+    // The tile through shared memory (the stages are idle: every MMA has completed), then the
+    // sums along its anti-diagonals, the product's 127 coefficients: 254 atomic adds a CTA in
+    // place of 8192, and the consumer reads 1 KB a block in place of 32 KB.
+    u64* tile = reinterpret_cast<u64*>(base);
+    constexpr int TLD = 65;                        // words of a tile row: conflict-free both ways
+    if (ok) {
+      const int r = q4 * 32 + lane;                // tile row: x parity r / 64, coefficient r % 64
 #pragma unroll
-      for (int c = 0; c < GM_DC; ++c)
-        atomicAdd(reinterpret_cast<unsigned long long*>(dst + c), (unsigned long long)(sg * acc[c]));
-    } else if (!ok && lane == 0) {
-      fail();
+      for (int c = 0; c < GM_DC; ++c) tile[r * TLD + h * GM_DC + c] = acc[c];
+    }
+    asm volatile("bar.sync 1, %0;\n" ::"n"(GM_NDRAIN * 32) : "memory");
+    if (nunits > 0 && !*abort) {
+      const int xpar = tid >> 7, d = tid & 127;    // x parity, coefficient (127: none)
+      u64 v = 0;
+#pragma unroll 8
+      for (int a = 0; a < 64; ++a) {
+        const int b = d - a;
+        if (b >= 0 && b < 64) v += tile[(xpar * 64 + a) * TLD + b];
+      }
+      // (x parity, y parity): (0,0) -> ee, (1,1) -> oo, mixed -> cross
+      const long long blk = xpar != par ? jobs.off_x : (xpar ? jobs.off_oo : 0);
+      if (d < 127)
+        atomicAdd(reinterpret_cast<unsigned long long*>(J.P + blk + d),
+                  (unsigned long long)(J.sign * v));
     }
   }
   tc_fence_before();
@@ -1914,8 +1927,8 @@ int gram3_tc(cudaStream_t st, long long Dh, const u64* x, const u64* y, u64* P, 
              unsigned err_flag, int nsplit) {
   GramJobs jobs{};
   jobs.n = 1;
-  jobs.off_oo = 4096;
-  jobs.off_x = 2 * 4096;
+  jobs.off_oo = 9 * 128;
+  jobs.off_x = 3 * 128;
   jobs.j[0] = GramJob{x, nullptr, 0ull, y, nullptr, 0ull, P, 1ull};
   return gram_jobs_tc(st, Dh, jobs, err, err_flag, nsplit);
 }
