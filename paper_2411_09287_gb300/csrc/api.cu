@@ -65,6 +65,7 @@ inline void counted(int k, F f, A... a) {
 #define launch_trunc_materialize(...) counted(1, mpc3::launch_trunc_materialize, __VA_ARGS__)
 #define launch_gr_mul_rows(...) counted(1, mpc3::launch_gr_mul_rows, __VA_ARGS__)
 #define launch_gather_rows_affine(...) counted(1, mpc3::launch_gather_rows_affine, __VA_ARGS__)
+#define launch_sum_blocks(...) counted(1, mpc3::launch_sum_blocks, __VA_ARGS__)
 #define launch_block_rowsum(...) counted(1, mpc3::launch_block_rowsum, __VA_ARGS__)
 #define launch_gr_mulmat_batch(...) counted(1, mpc3::launch_gr_mulmat_batch, __VA_ARGS__)
 #define launch_word_transpose(...) counted(1, mpc3::launch_word_transpose, __VA_ARGS__)
@@ -73,7 +74,6 @@ inline void counted(int k, F f, A... a) {
 #define launch_prf_words_keyed(...) counted(1, mpc3::launch_prf_words_keyed, __VA_ARGS__)
 #define launch_trunc_limb_table(...) counted(1, mpc3::launch_trunc_limb_table, __VA_ARGS__)
 #define launch_trunc_bit_transpose(...) counted(1, mpc3::launch_trunc_bit_transpose, __VA_ARGS__)
-#define launch_fold_reduce_strided(...) counted(1, mpc3::launch_fold_reduce_strided, __VA_ARGS__)
 
 namespace {
 
@@ -1052,7 +1052,8 @@ struct TruncPlan {
   int R1 = 0, kd = 0;
   long long Dt = 0;
   long long L = 0, Epad = 0, nhi = 0;   // S = sum over e_hi < nhi of T_hi (x) (sum over e_lo < L ...)
-  u64 *b1, *b2, *Rtab, *S, *Zpq, *V, *W, *zt, *S_hi, *Pst, *Thi, *Mhi;
+  u64 *b1, *b2, *Rtab, *S, *Zpq, *V, *W, *zt, *S_hi, *Thi, *Mhi;
+  PowPlan pow;          // the table r^(2 e_lo), e_lo < L
   u64 *B1T, *B2T;   // bit-transposed b1, b2: [j][e / 64]
   unsigned char* TL8;
   // tensor-core materialisation with r^(2e) = r^(2 Lm e_hi) r^(2 e_lo), e = e_hi Lm + e_lo:
@@ -1064,7 +1065,6 @@ struct TruncPlan {
   // sum_e r^(2e) pq_c[e] = sum_{e_hi} T_hi[e_hi] (sum_{e_lo} pq_c[e] r^(2 e_lo)) (a limb GEMM over
   // the first block, then 12 nhi GR products), and the rows r^(2 Lm e_hi) come from T_hi x r^(2 e_lo)
   bool compact = false;
-  bool tc_combine = false;   // sum_{e_hi} T_hi (x) S_hi on the tensor cores
   u64 *Zhi = nullptr, *Zrep = nullptr, *Zprod = nullptr, *Prow = nullptr;
   u64* pqc = nullptr;        // the chunk's 12 rows of <p>, <q> gathered (chunked batches only)
   Dense dt;
@@ -1080,6 +1080,7 @@ struct TruncBatch {
 struct VMatPlan {
   Small s;
   u64 *Q, *P, *T, *Pz;
+  PowPlan powQ, powP;
   Dense dv;
   IVBuf iv;
   int R0;
@@ -1092,7 +1093,7 @@ struct VMatPlan {
 struct TruncShape {
   long long L, Epad, nhi, Lm = 0, nhm = 0;
   int R1, kd;
-  bool compact = false, tc_combine = false, blocked = false;
+  bool compact = false, blocked = false;
 };
 
 TruncShape trunc_shape(long long E, int R1, bool tc, const mpc_tuning& tu) {
@@ -1105,7 +1106,6 @@ TruncShape trunc_shape(long long E, int R1, bool tc, const mpc_tuning& tu) {
   h.Epad = ((E + h.L - 1) / h.L) * h.L;
   h.nhi = h.Epad / h.L;
   h.compact = tc && h.kd == 6 && h.blocked && E % h.L == 0;
-  h.tc_combine = tc && h.nhi >= tu.tc_combine_min;
   if (tc && h.kd == 6 && h.blocked) {
     if (tu.row_split > 0) {
       // at most E rounded up to a tile: the row-split table reads r^(2 e_lo) for e_lo < Lm
@@ -1140,13 +1140,10 @@ TruncShape trunc_shape(long long E, int R1, bool tc, const mpc_tuning& tu) {
   return h;
 }
 
-// tensor-core scratch of a truncation chunk: the S_hi combination (64 x 262144 x nhi) and the
-// compact table's sum over the first block (12 nhi x 64 x L)
+// tensor-core scratch of a truncation chunk: the compact table's sum over the first block
+// (12 nhi x 64 x L)
 size_t trunc_tc_scratch(const TruncShape& h) {
-  size_t b = 0;
-  if (h.tc_combine) b = std::max(b, limb_tc_scratch_bytes(64, 262144, h.nhi, 1));
-  if (h.compact) b = std::max(b, limb_tc_scratch_bytes(12 * h.nhi, 64, h.L, 1));
-  return b;
+  return h.compact ? limb_tc_scratch_bytes(12 * h.nhi, 64, h.L, 1) : 0;
 }
 
 TruncPlan plan_trunc(Arena& a, long long E, int R1, bool tc, bool chunked, const mpc_tuning& tu) {
@@ -1160,16 +1157,15 @@ TruncPlan plan_trunc(Arena& a, long long E, int R1, bool tc, bool chunked, const
   p.Epad = h.Epad;
   p.nhi = h.nhi;
   p.compact = h.compact;
-  p.tc_combine = h.tc_combine;
   p.b1 = a.take<u64>(p.Epad);
   p.b2 = a.take<u64>(p.Epad);
   p.Rtab = a.take<u64>((p.compact ? p.L : p.Epad) * 64);
-  p.S = a.take<u64>(4096 * 64);
   p.TL8 = a.take<unsigned char>(1024 * p.L);
   p.B1T = a.take<u64>(p.Epad);
   p.B2T = a.take<u64>(p.Epad);
   p.S_hi = a.take<u64>(p.nhi * 4096 * 64);
-  p.Pst = a.take<u64>(64ll * 262144);
+  p.S = p.nhi > 1 ? a.take<u64>(4096 * 64) : p.S_hi;   // one block: T_hi[0] = 1
+  p.pow = plan_pow(a, p.L);
   p.Thi = a.take<u64>(p.nhi * 64);
   p.Mhi = a.take<u64>(std::max<long long>(1, p.nhi - 1) * 4096);
   p.Zpq = a.take<u64>(12 * 64);
@@ -1252,6 +1248,8 @@ bool plan_vmat(Arena& a, long long M, long long N, long long K, int t, int R0, i
              : nullptr;
   p.Q = a.take<u64>(N * 64);
   p.P = a.take<u64>(M * 64);
+  p.powQ = plan_pow(a, N);
+  p.powP = plan_pow(a, M);
   p.T = a.take<u64>(6 * M * 64);
   p.Pz = a.take<u64>(6 * 4096);
   const bool all[6] = {true, true, true, true, true, true};
@@ -1311,10 +1309,11 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
   launch_gr_mul1(st, s.r, s.r, s.aux + 64);                          // r^2
   // r^(2e) for e < Epad: r^(2 e_lo) for e_lo < L by repeated multiplication, then every further
   // block of L rows is that block times the constant r^(2 L e_hi) (a 64 x 64 matrix product)
-  launch_gr_powers(st, s.aux + 64, p.L, p.Rtab);
+  if ((rc = power_table(ctx, s.aux + 64, p.pow, p.Rtab, s.aux + 192))) return rc;
   if (p.compact) {
     launch_gr_mul1(st, p.Rtab + (p.L - 1) * 64, s.aux + 64, s.aux + 128);   // r^(2L)
     launch_gr_powers(st, s.aux + 128, p.nhi, p.Thi);
+    launch_gr_mulmat_batch(st, p.nhi - 1, p.Thi + 64, 64, p.Mhi);
   } else if (p.nhi > 1) {
     launch_gr_mul1(st, p.Rtab + (p.L - 1) * 64, s.aux + 64, s.aux + 128);   // r^(2L)
     launch_gr_powers(st, s.aux + 128, p.nhi, p.Thi);
@@ -1373,14 +1372,34 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
                             ST_TIMEOUT))
         return fail(ctx, MPC_ERR_CUDA, "verify_matmul: tensor map of the limb table");
     }
-    GemmTerm T;
-    // A[a][e_hi] = coefficient a of r^(2 L e_hi)
-    T.A = p.compact ? op(p.Thi, 64, 1) : op(p.Rtab, p.L * 64, 1);
-    T.B = op(p.S_hi, 262144);            // B[e_hi][(p, b)]
-    if ((rc = dense_gemm(ctx, 64, 262144, p.nhi, T, epi_store(p.Pst, 262144),
-                         p.tc_combine ? tcs : nullptr)))
-      return rc;
-    launch_fold_reduce_strided(st, p.Pst, 262144, 4096, p.S);
+    // S = sum_{e_hi} T_hi S_hi: the blocks h >= 1 times r^(2 L h) (matrix h - 1) in place, then the
+    // sum over the blocks
+    if (p.nhi > 1) {
+      bool done = false;
+      u64* blk1 = p.S_hi + 262144;
+      if (ctx->gemm_path == MPC_GEMM_LIMB_TC) {
+        GrMMArgs g = grargs(ctx);
+        g.R = (p.nhi - 1) * 4096;
+        g.p0 = blk1;
+        g.in = GrRowMap{0, 64, 0};
+        g.Mmat = p.Mhi;
+        g.mrows = 4096;
+        g.out = blk1;
+        g.om = GrRowMap{0, 64, 0};
+        g_launches += 1;
+        Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)g.R * 4096);
+        done = gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT) == 0;
+        if (!done) g_launches -= 1;
+      }
+      for (long long h = 1; h < p.nhi && !done; ++h) {
+        // block h into S (used as scratch), then back: the CUDA-core product is not in place
+        if ((rc = gr_matmul(ctx, 4096, p.S_hi + h * 262144, nullptr, 1, 64, p.Mhi + (h - 1) * 4096,
+                            nullptr, 0, p.S, 64)))
+          return rc;
+        CK(cudaMemcpyAsync(p.S_hi + h * 262144, p.S, 262144 * 8, cudaMemcpyDeviceToDevice, st));
+      }
+      launch_sum_blocks(st, 262144, p.nhi, 262144, p.S_hi, p.S);
+    }
   }
   delete phase;
   phase = new Phase(ctx, MPC_PROF_TRUNC_ROUNDS);
@@ -2040,10 +2059,7 @@ int verify_mult_body(mpc_ctx* ctx, uint64_t verify_id, const u64* xs, const u64*
   }
   CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
   {  // z_c = sum_i z_c[i] r^i for the 6 components at once: (6 x n) . (n x 64)
-    GemmTerm T;
-    T.A = op(zs, n);
-    T.B = op(p.pw, 64);
-    gemm_u64(st, 6, 64, n, 1, &T, epi_atomic(s.zinit, 64), nsplit_for(n));
+    launch_scalar_gr_sum(st, n, zs, n, 6, p.pw, s.zinit);
   }
   p.dv.cur = 0;
   return run_dense(ctx, verify_id, 0, p.dv, n, s.zinit, 1, p.R, s, p.iv, trace, &ylift);
@@ -2142,9 +2158,9 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
   Phase* phase = new Phase(ctx, MPC_PROF_VERIFY_GEMM);
   if ((rc = sums_begin(ctx, s))) return rc;
   reveal(ctx, P_VER_R, make_obj(verify_id, 0, 0), s, s.r);
-  launch_gr_powers(st, s.r, N, p.Q);                       // r^b
-  launch_gr_mul1(st, p.Q + (N - 1) * 64, s.r, s.aux);      // rho = r^N
-  launch_gr_powers(st, s.aux, M, p.P);                     // rho^a
+  if ((rc = power_table(ctx, s.r, p.powQ, p.Q, s.aux + 64))) return rc;   // r^b
+  launch_gr_mul1(st, p.Q + (N - 1) * 64, s.r, s.aux);                     // rho = r^N
+  if ((rc = power_table(ctx, s.aux, p.powP, p.P, s.aux + 64))) return rc; // rho^a
   Vec& x = p.dv.x[0];
   Vec& y = p.dv.y[0];
   for (int c = 0; c < 6; ++c) {
@@ -2163,8 +2179,11 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
     T.B = op(p.Q, 64);
     if ((rc = dense_gemm(ctx, 6 * M, 64, N, T, epi_store(p.T, 64), p.tcs))) return rc;
     CK(cudaMemsetAsync(p.Pz, 0, 6 * 4096 * 8, st));
+    GramBatch gb;
     for (int c = 0; c < 6; ++c)
-      gram(ctx, p.Pz + c * 4096, p.P, nullptr, 1, 64, p.T + c * M * 64, nullptr, 1, 64, M, 1);
+      gb.add(p.Pz + c * 4096, p.P, nullptr, 1, 64, p.T + c * M * 64, nullptr, 1, 64, 1);
+    g_launches += 1;
+    gemm_u64_gram_batch(st, M, gb.n, gb.T, gb.e, nsplit_for(M));
     launch_gr_fold_reduce(st, p.Pz, 6, s.zinit);
   }
   p.dv.cur = 0;
@@ -2862,6 +2881,7 @@ struct NLPlan {
   int R1;
   Small s1;
   u64* pw1;
+  PowPlan pp1;
   Dense d1;
   IVBuf iv1;
   u64* Ye;                       // 6 x D1 ring words: the y side before its first fold
@@ -2902,6 +2922,7 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2]) {
   p.R1 = default_R(p.D1);
   p.s1 = plan_small(a);
   p.pw1 = a.take<u64>(p.ne * 64);
+  p.pp1 = plan_pow(a, p.ne);
   const bool xc[6] = {false, false, true, false, true, false};
   const bool yc[6] = {true, true, true, true, true, true};
   p.d1 = plan_dense(a, p.D1, xc, yc, p.R1, true);
@@ -2973,7 +2994,7 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     const Small& s = p.s1;
     if ((rc = sums_begin(ctx, s))) return rc;
     reveal(ctx, P_VER_R, make_obj(vid, 1, 0), s, s.r);
-    launch_gr_powers(st, s.r, p.ne, p.pw1);
+    if ((rc = power_table(ctx, s.r, p.pp1, p.pw1, s.aux))) return rc;
     Vec ylift;
     for (int c = 0; c < 6; ++c) ylift.c[c] = p.Ye + c * p.D1;
     CK(cudaMemcpyAsync(p.ydev, ylift.c, 6 * sizeof(u64*), cudaMemcpyHostToDevice, st));

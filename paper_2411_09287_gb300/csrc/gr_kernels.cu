@@ -4,6 +4,7 @@
 //   materialisation of the folded vectors).  The steps on single elements are in gr_round.cu.
 // A GR element is 64 consecutive u64 coefficients.  A <.>^{l[x]}-shared vector of D elements uses
 // the 6-component layout with component c at [c*D*64, (c+1)*D*64).
+#include "gr_mul.cuh"
 #include "kernels.h"
 
 namespace mpc3 {
@@ -45,25 +46,48 @@ __global__ void k_gr_random_shared(long long nwords, Key k01, Key k02, Key k12, 
 }
 
 // ---- powers ---------------------------------------------------------------------------------
-// Block b writes table[64 b .. 64 b + 63] = a^(64 b) ... ; 64 threads.
-__global__ void k_gr_powers(const u64* __restrict__ a, long long n, u64* __restrict__ table) {
-  __shared__ u64 acc[64], base[64], av[64], scr[128];
-  const int t = threadIdx.x;
-  const long long start = (long long)blockIdx.x * 64;
-  if (start >= n) return;
-  av[t] = a[t];
-  base[t] = a[t];
-  acc[t] = (t == 0) ? 1ull : 0ull;
+// Block b writes table[16 b .. 16 b + 15]: the squares a^(2^k) by one half of the block while the
+// other multiplies the ones of 16 b's bits into a^(16 b), then four doublings of the row count
+// (row 2^k + i = row i a^(2^k)).  A block is a chain of about log2(n) + 5 products, so its time is
+// their latency: 64 rows a block, one product after another on 64 threads, took 186 to 305 us.
+constexpr int POW_ROWS = 16, POW_LG = 4;
+__global__ void __launch_bounds__(256)
+k_gr_powers(const u64* __restrict__ a, long long n, u64* __restrict__ table) {
+  __shared__ u64 rows[POW_ROWS][64], P[64], Pk[POW_LG][64], scr[4 * 128];
+  const int tid = threadIdx.x, t = tid & 63;
+  const long long start = (long long)blockIdx.x * POW_ROWS;
+  if (tid < 64) {
+    P[t] = a[t];
+    rows[0][t] = t == 0 ? 1ull : 0ull;
+  }
   __syncthreads();
-  for (long long e = start; e; e >>= 1) {
-    if (e & 1) gr_mul_block(acc, base, acc, scr);
-    if (e >> 1) gr_mul_block(base, base, base, scr);
-  }
-  for (int i = 0; i < 64 && start + i < n; ++i) {
-    table[(start + i) * 64 + t] = acc[t];
+  const int half = tid >> 7, sub = tid & 127;
+  for (int k = 0; k < POW_LG || (start >> k); ++k) {   // P = a^(2^k)
+    const bool bit = (start >> k) & 1;
+    if (k < POW_LG && tid < 64) Pk[k][t] = P[t];
+    const u64 r = gr_mul_par<2>(half ? rows[0] : P, P, scr + half * 256, sub);
+    if (sub < 64) {
+      if (!half) P[t] = r;
+      else if (bit) rows[0][t] = r;
+    }
     __syncthreads();
-    gr_mul_block(acc, av, acc, scr);
   }
+  u64 r = gr_mul_par<4>(rows[0], Pk[0], scr, tid);
+  if (tid < 64) rows[1][t] = r;
+  __syncthreads();
+  r = gr_mul_par<2>(rows[half], Pk[1], scr + half * 256, sub);
+  if (sub < 64) rows[2 + half][t] = r;
+  __syncthreads();
+  const int g = tid >> 6;
+  r = gr_mul_par<1>(rows[g], Pk[2], scr + g * 128, t);
+  rows[4 + g][t] = r;
+  __syncthreads();
+  for (int q = 0; q < 8; q += 4) {
+    r = gr_mul_par<1>(rows[q + g], Pk[3], scr + g * 128, t);
+    rows[8 + q + g][t] = r;
+  }
+  __syncthreads();
+  for (int i = g; i < POW_ROWS && start + i < n; i += 4) table[(start + i) * 64 + t] = rows[i][t];
 }
 
 __global__ void k_gr_mul1(const u64* a, const u64* b, u64* out) {
@@ -90,19 +114,22 @@ __global__ void k_gr_lincomb(const u64* ca, const u64* a, const u64* cb, const u
 }
 
 // [M_a; M_b]: rows 0..63 the multiplication matrix of a, rows 64..127 that of b.
-__global__ void k_gr_mulmat2(const u64* a, const u64* b, u64* M) {
-  __shared__ u64 buf[64 * 64];
-  const u64* src = (blockIdx.x == 0) ? a : b;
-  gr_mulmat_block(src, buf);
-  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) M[blockIdx.x * 4096 + i] = buf[i];
+__global__ void __launch_bounds__(256) k_gr_mulmat2(const u64* a, const u64* b, u64* M) {
+  __shared__ u64 e[64];
+  if (threadIdx.x < 64) e[threadIdx.x] = (blockIdx.x == 0 ? a : b)[threadIdx.x];
+  __syncthreads();
+  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x)
+    M[blockIdx.x * 4096 + i] = gr_mulmat_at(e, i >> 6, i & 63);
 }
 
 // M[i] = multiplication matrix of the GR element src + i * stride, for i < n (one block each).
-__global__ void k_gr_mulmat_batch(const u64* src, long long stride, u64* M) {
-  __shared__ u64 buf[64 * 64];
-  gr_mulmat_block(src + blockIdx.x * stride, buf);
+__global__ void __launch_bounds__(256)
+k_gr_mulmat_batch(const u64* src, long long stride, u64* M) {
+  __shared__ u64 e[64];
+  if (threadIdx.x < 64) e[threadIdx.x] = src[blockIdx.x * stride + threadIdx.x];
+  __syncthreads();
   u64* dst = M + (long long)blockIdx.x * 4096;
-  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) dst[i] = buf[i];
+  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) dst[i] = gr_mulmat_at(e, i >> 6, i & 63);
 }
 
 // out[c * rows + r] = in[r * cols + c] for r < rows, c < cols; entries with r * cols + c >= n
@@ -134,10 +161,23 @@ __global__ void k_gather_rows_affine(long long n, const u64* __restrict__ src, l
   }
 }
 
+// out[i] = sum_{h < n} in[h ld + i] for i < m words.
+__global__ void __launch_bounds__(256)
+k_sum_blocks(long long m, long long n, long long ld, const u64* __restrict__ in,
+             u64* __restrict__ out) {
+  const long long i = blockIdx.x * 256ll + threadIdx.x;
+  if (i >= m) return;
+  u64 v = 0;
+#pragma unroll 8
+  for (long long h = 0; h < n; ++h) v += in[h * ld + i];
+  out[i] = v;
+}
+
 // out[c] = sum_{h < nper} in[c nper + h] for c < ncomp (rows of 64 words).
 __global__ void k_block_rowsum(long long nper, const u64* __restrict__ in, u64* __restrict__ out) {
   const long long c = blockIdx.x;
   u64 v = 0;
+#pragma unroll 8
   for (long long h = 0; h < nper; ++h) v += in[(c * nper + h) * 64 + threadIdx.x];
   out[c * 64 + threadIdx.x] = v;
 }
@@ -463,11 +503,13 @@ k_gr_mul_rows(long long n, const u64* __restrict__ a, const u64* __restrict__ b,
   }
 }
 
-// out[c] += sum_{e < n} A[c][e] * R[e] for c < nrows <= 16: GR elements R[e] (rows of 64 words)
+// out[c] += sum_{e < n} A[c][e] * R[e] for c < nrows <= NR: GR elements R[e] (rows of 64 words)
 // scaled by ring scalars and summed (e.g. sum_e r^(2e) p_c[e] for the truncation batch).  Each
 // block takes a contiguous slice of e, 256 e at a time: the slice of A is staged in shared memory
-// as [e][c] (a broadcast read per e), and each 64-thread group takes 64 of the 256 e, thread t
-// coefficient t of every row c; partial sums are added atomically at the end.
+// as [e][c] (a broadcast read per e), and the four 64-thread groups take every fourth e, thread t
+// coefficient t of every row c; the groups' sums are added in shared memory, then atomically.
+// Bound by the rows of R (512 bytes an e) once the grid fills the GPU; 4096 e a block left one
+// block for the smallest batches and 256 for 2^20 (361 and 413 us).
 template <int NR>
 __global__ void __launch_bounds__(256)
 k_scalar_gr_sum(long long n, const u64* __restrict__ A, long long lda, int nrows,
@@ -481,29 +523,33 @@ k_scalar_gr_sum(long long n, const u64* __restrict__ A, long long lda, int nrows
 #pragma unroll
   for (int c = 0; c < NR; ++c) acc[c] = 0;
   for (long long eb = e0; eb < e1; eb += 256) {
+    const int cnt = (int)(e1 - eb < 256 ? e1 - eb : 256);
     __syncthreads();
     for (int i = threadIdx.x; i < NR * 256; i += 256) {
       const int c = i >> 8, k = i & 255;
-      as[k][c] = (c < nrows && eb + k < e1) ? A[c * lda + eb + k] : 0ull;
+      as[k][c] = (c < nrows && k < cnt) ? A[c * lda + eb + k] : 0ull;
     }
     __syncthreads();
-    const int kmax = (int)((e1 - eb - grp * 64 < 64) ? e1 - eb - grp * 64 : 64);
-#pragma unroll 2
-    for (int k = 0; k < kmax; ++k) {
-      const int kk = grp * 64 + k;
-      const u64 r = R[(eb + kk) * 64 + t];
+#pragma unroll 4
+    for (int k = grp; k < cnt; k += 4) {
+      const u64 r = R[(eb + k) * 64 + t];
 #pragma unroll
       for (int c = 0; c < NR; c += 2) {
-        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&as[kk][c]);
+        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&as[k][c]);
         acc[c] += w.x * r;
         acc[c + 1] += w.y * r;
       }
     }
   }
+  __syncthreads();
+  u64* red = &as[0][0];   // [grp][c][t]: 4 x NR x 64 of the 256 x NR words
 #pragma unroll
-  for (int c = 0; c < NR; ++c)
-    if (c < nrows)
-      atomicAdd(reinterpret_cast<unsigned long long*>(out + c * 64 + t), (unsigned long long)acc[c]);
+  for (int c = 0; c < NR; ++c) red[(grp * NR + c) * 64 + t] = acc[c];
+  __syncthreads();
+  for (int i = threadIdx.x; i < nrows * 64; i += 256) {
+    const u64 v = red[i] + red[NR * 64 + i] + red[2 * NR * 64 + i] + red[3 * NR * 64 + i];
+    atomicAdd(reinterpret_cast<unsigned long long*>(out + i), (unsigned long long)v);
+  }
 }
 
 }  // namespace
@@ -519,7 +565,7 @@ void launch_gr_random_shared(cudaStream_t st, long long n, Key k01, Key k02, Key
 
 void launch_gr_powers(cudaStream_t st, const u64* a, long long n, u64* table) {
   if (n <= 0) return;
-  k_gr_powers<<<(unsigned)((n + 63) / 64), 64, 0, st>>>(a, n, table);
+  k_gr_powers<<<(unsigned)((n + POW_ROWS - 1) / POW_ROWS), 256, 0, st>>>(a, n, table);
 }
 
 void launch_gr_mul1(cudaStream_t st, const u64* a, const u64* b, u64* out) {
@@ -532,13 +578,13 @@ void launch_gr_lincomb(cudaStream_t st, const u64* ca, const u64* a, const u64* 
 }
 
 void launch_gr_mulmat2(cudaStream_t st, const u64* a, const u64* b, u64* M) {
-  k_gr_mulmat2<<<b ? 2 : 1, 64, 0, st>>>(a, b, M);
+  k_gr_mulmat2<<<b ? 2 : 1, 256, 0, st>>>(a, b, M);
 }
 
 void launch_gr_mulmat_batch(cudaStream_t st, long long n, const u64* src, long long stride,
                             u64* M) {
   if (n <= 0) return;
-  k_gr_mulmat_batch<<<(unsigned)n, 64, 0, st>>>(src, stride, M);
+  k_gr_mulmat_batch<<<(unsigned)n, 256, 0, st>>>(src, stride, M);
 }
 
 void launch_word_transpose(cudaStream_t st, long long rows, long long cols, long long n,
@@ -557,6 +603,12 @@ void launch_gather_rows_affine(cudaStream_t st, long long n, const u64* src, lon
 void launch_block_rowsum(cudaStream_t st, int ncomp, long long nper, const u64* in, u64* out) {
   if (ncomp <= 0) return;
   k_block_rowsum<<<(unsigned)ncomp, 64, 0, st>>>(nper, in, out);
+}
+
+void launch_sum_blocks(cudaStream_t st, long long m, long long n, long long ld, const u64* in,
+                       u64* out) {
+  if (m <= 0) return;
+  k_sum_blocks<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(m, n, ld, in, out);
 }
 
 void launch_gr_inverses(cudaStream_t st, u64* out) { k_gr_inverses<<<1, 64, 0, st>>>(out); }
@@ -633,12 +685,14 @@ void launch_gr_mul_rows(cudaStream_t st, long long n, const u64* a, const u64* b
 void launch_scalar_gr_sum(cudaStream_t st, long long n, const u64* A, long long lda, int nrows,
                           const u64* R, u64* out) {
   if (n <= 0 || nrows <= 0) return;
-  long long g = (n + 4095) / 4096;
+  // 64 e a block while the batch is small, then eight blocks an SM
+  long long g = (n + 63) / 64;
   if (g > 152 * 8) g = 152 * 8;
-  if (nrows <= 12)
-    k_scalar_gr_sum<12><<<(unsigned)g, 256, 0, st>>>(n, A, lda, nrows, R, out);
-  else
-    k_scalar_gr_sum<16><<<(unsigned)g, 256, 0, st>>>(n, A, lda, nrows, R, out);
+  auto go = [&](auto kern) { kern<<<(unsigned)g, 256, 0, st>>>(n, A, lda, nrows, R, out); };
+  if (nrows <= 2) go(k_scalar_gr_sum<2>);
+  else if (nrows <= 6) go(k_scalar_gr_sum<6>);
+  else if (nrows <= 12) go(k_scalar_gr_sum<12>);
+  else go(k_scalar_gr_sum<16>);
 }
 
 }  // namespace mpc3

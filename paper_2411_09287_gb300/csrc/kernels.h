@@ -245,6 +245,9 @@ void launch_gather_rows_affine(cudaStream_t st, long long n, const u64* src, lon
                                long long div, long long m, u64* out);
 // out[c] = sum over h < nper of in[c nper + h] (rows of 64 words), c < ncomp.
 void launch_block_rowsum(cudaStream_t st, int ncomp, long long nper, const u64* in, u64* out);
+// out[i] = sum over h < n of in[h ld + i], i < m words.
+void launch_sum_blocks(cudaStream_t st, long long m, long long n, long long ld, const u64* in,
+                       u64* out);
 // M + 4096 i = multiplication matrix (M[b][c] = coefficient c of g x^b) of g = src + i stride,
 // i < n.
 void launch_gr_mulmat_batch(cudaStream_t st, long long n, const u64* src, long long stride,
@@ -271,7 +274,6 @@ void launch_trunc_bit_transpose(cudaStream_t st, const u64* words, long long Epa
 int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long Epad,
                       const unsigned char* TL8, long long L, long long nhi, u64* S_hi,
                       unsigned* err, unsigned err_flag);
-void launch_fold_reduce_strided(cudaStream_t st, const u64* P, long long ld, int npairs, u64* out);
 
 // ---- non-linear layers: Boolean sharings, AND gates, GF(2^64) (nonlinear.cu) ------------------
 void launch_and_offline(cudaStream_t st, const u64* xs, const u64* ys, long long nw, Key k01, Key k02,

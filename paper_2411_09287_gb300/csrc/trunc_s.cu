@@ -252,36 +252,6 @@ k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* __restrict__ B1
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// out[p][c] = reduce(sum_{a+b=s} P[a*ld + p*64 + b]) for n pairs.
-__global__ void k_fold_reduce_strided(const u64* __restrict__ P, long long ld, u64* __restrict__ out) {
-  __shared__ u64 prod[128];
-  const long long p = blockIdx.x;
-  const int s = threadIdx.x;
-  u64 v = 0;
-  if (s < 127) {
-    const int a0 = (s < 64) ? 0 : s - 63;
-    const int a1 = (s < 64) ? s : 63;
-    for (int a = a0; a <= a1; ++a) v += P[a * ld + p * 64 + (s - a)];
-  }
-  prod[s] = (s < 127) ? v : 0ull;
-  __syncthreads();
-  if (s < 64) {
-    const u64* h = prod + 64;
-    u64 r = prod[s] - gr_hg(h, s);
-    if (s < 7) {
-      u64 h2[3];
-      for (int m = 0; m < 3; ++m) h2[m] = gr_hg(h, 64 + m);
-      u64 g = 0;
-      if (s < 3) g += h2[s];
-      if (s - 1 >= 0 && s - 1 < 3) g += h2[s - 1];
-      if (s - 3 >= 0 && s - 3 < 3) g += h2[s - 3];
-      if (s - 4 >= 0 && s - 4 < 3) g += h2[s - 4];
-      r += g;
-    }
-    out[p * 64 + s] = r;
-  }
-}
-
 }  // namespace
 
 void launch_trunc_limb_table(cudaStream_t st, const u64* Tlo, long long L, unsigned char* TL8) {
@@ -315,10 +285,6 @@ int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long
   dim3 grid(4096 / S_TPAIRS, 1024 / S_TCOLS, (unsigned)nhi);
   k_trunc_s_tc<<<grid, S_THREADS, S_SMEM, st>>>(mb, B1T, B2T, Epad / 64, L, S_hi, err, err_flag);
   return 0;
-}
-
-void launch_fold_reduce_strided(cudaStream_t st, const u64* P, long long ld, int npairs, u64* out) {
-  k_fold_reduce_strided<<<npairs, 128, 0, st>>>(P, ld, out);
 }
 
 }  // namespace mpc3
