@@ -50,18 +50,19 @@ inline void counted(int k, F f, A... a) {
 #define launch_gr_mulmat2(...) counted(1, mpc3::launch_gr_mulmat2, __VA_ARGS__)
 #define launch_gr_inverses(...) counted(1, mpc3::launch_gr_inverses, __VA_ARGS__)
 #define launch_gr_fold_reduce(...) counted(1, mpc3::launch_gr_fold_reduce, __VA_ARGS__)
-#define launch_gr_scale_rows(...) counted(1, mpc3::launch_gr_scale_rows, __VA_ARGS__)
-#define launch_gr_lift(...) counted(1, mpc3::launch_gr_lift, __VA_ARGS__)
-#define launch_gram_lifted(...) counted(1, mpc3::launch_gram_lifted, __VA_ARGS__)
-#define launch_fold_lifted(...) counted(1, mpc3::launch_fold_lifted, __VA_ARGS__)
 #define launch_neg_copy(...) counted(1, mpc3::launch_neg_copy, __VA_ARGS__)
 #define launch_round_tail(...) counted(1, mpc3::launch_round_tail, __VA_ARGS__)
 #define launch_reveal(...) counted(1, mpc3::launch_reveal, __VA_ARGS__)
 #define launch_delta(...) counted(1, mpc3::launch_delta, __VA_ARGS__)
 #define launch_rec_hash(...) counted(1, mpc3::launch_rec_hash, __VA_ARGS__)
-#define launch_trunc_round_sums(...) counted(1, mpc3::launch_trunc_round_sums, __VA_ARGS__)
+#define launch_weighted_sums(...) counted(1, mpc3::launch_weighted_sums, __VA_ARGS__)
+#define launch_update_vw(...) counted(1, mpc3::launch_update_vw, __VA_ARGS__)
+#define launch_blk_sums(...) counted(1, mpc3::launch_blk_sums, __VA_ARGS__)
+#define launch_words_sums(...) counted(1, mpc3::launch_words_sums, __VA_ARGS__)
+#define launch_blk_claim(...) counted(1, mpc3::launch_blk_claim, __VA_ARGS__)
+#define launch_blk_combine(...) counted(1, mpc3::launch_blk_combine, __VA_ARGS__)
+#define launch_ones(...) counted(1, mpc3::launch_ones, __VA_ARGS__)
 #define launch_trunc_u(...) counted(1, mpc3::launch_trunc_u, __VA_ARGS__)
-#define launch_trunc_update_vw(...) counted(1, mpc3::launch_trunc_update_vw, __VA_ARGS__)
 #define launch_trunc_materialize(...) counted(1, mpc3::launch_trunc_materialize, __VA_ARGS__)
 #define launch_gr_mul_rows(...) counted(1, mpc3::launch_gr_mul_rows, __VA_ARGS__)
 #define launch_gather_rows_affine(...) counted(1, mpc3::launch_gather_rows_affine, __VA_ARGS__)
@@ -585,18 +586,15 @@ void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, 
 
 // One Pi_Reduce round on a dense claim (Fig. Reduce).  x, y: current vectors (D elements, with
 // capacity for D+1), z: current claim; writes the folded vectors into xo, yo and z into zo.
-// ys (optional): the y vectors are lifted ring words, one word per element (Fig. MTP's y side
-// before any fold); y is then not read, the party sums are scalar-weighted row sums and the y
-// folds scalar times GR element.
 int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, const Vec& y,
                        long long D, const u64* z, Vec& xo, Vec& yo, u64* zo, const Small& s,
-                       u64* trace, const Vec* ys = nullptr) {
+                       u64* trace) {
   cudaStream_t st = ctx->st;
   const long long Dh = (D + 1) / 2;
   if (D & 1) {
     for (int c = 0; c < 6; ++c) {
       if (x.c[c]) CK(cudaMemsetAsync(x.c[c] + D * 64, 0, 512, st));
-      if (y.c[c] && !ys) CK(cudaMemsetAsync(y.c[c] + D * 64, 0, 512, st));
+      if (y.c[c]) CK(cudaMemsetAsync(y.c[c] + D * 64, 0, 512, st));
     }
   }
   View f[2], g[2];
@@ -615,15 +613,12 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
   int rc;
   // Shape of the truncation batch's dense rounds: x holds only [r]_1 (P0, P1 copies), y only
   // [r]_2 (P0, P2 copies), so P1's and P2's cross terms vanish and P0's sums are single Grams.
-  const bool bit_form = !ys && x.c[0] && !x.c[1] && !x.c[2] && x.c[3] && !x.c[4] && !x.c[5] &&
+  const bool bit_form = x.c[0] && !x.c[1] && !x.c[2] && x.c[3] && !x.c[4] && !x.c[5] &&
                         !y.c[0] && y.c[1] && !y.c[2] && !y.c[3] && !y.c[4] && y.c[5];
   u64* U = cur_sums(s);
   const u64* sums = s.S;   // reduced sums of the CUDA-core Grams unless set below
   int ld = 64;
-  if (ys) {
-    launch_gram_lifted(st, x.c, ys->c, Dh, D, U);   // S00 | S01 + S10 | 0 | S11
-    sums = U;
-  } else if (bit_form) {
+  if (bit_form) {
     bool done = false;
     if (ctx->gemm_path == MPC_GEMM_LIMB_TC) {
       // tensor cores: G00, G11 and the cross sum G01 + G10 directly
@@ -733,7 +728,7 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
   const u64* ins[12];
   u64* outs[12];
   int nx = 0, n = 0;
-  for (int side = 0; side < (ys ? 1 : 2); ++side)
+  for (int side = 0; side < 2; ++side)
     for (int c = 0; c < 6; ++c) {
       const u64* in = side ? y.c[c] : x.c[c];
       if (!in) continue;
@@ -743,16 +738,13 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       if (!side) ++nx;
     }
   bool done_all = fold_batched(ins, outs, n);
-  for (int side = 0; side < (ys ? 1 : 2) && !done_all; ++side) {
+  for (int side = 0; side < 2 && !done_all; ++side) {
     const int i0 = side ? nx : 0, i1 = side ? n : nx;
     if (fold_batched(ins + i0, outs + i0, i1 - i0)) continue;
     for (int i = i0; i < i1; ++i)
       if ((rc = gr_matmul(ctx, Dh, ins[i] + 64, ins[i], ~0ull, 128, s.MM, ins[i], 128, outs[i], 64)))
         return rc;
   }
-  if (ys)   // the fold element is the first GR element of the Lagrange coefficients
-    for (int c = 0; c < 6; ++c)
-      if (ys->c[c]) launch_fold_lifted(st, ys->c[c], Dh, D, s.coef, yo.c[c]);
   return cuda_check(ctx, "reduce_round");
 }
 
@@ -847,11 +839,8 @@ int inner_verify_dense(mpc_ctx* ctx, u64 vid, u32 batch, const Vec& x, const Vec
 }
 
 // Dense rounds k = k0..R followed by Pi_InnerVerify.
-// ylift (optional): the y vectors entering round k0 are lifted ring words (one word per element
-// and present component); they are folded into dv.y's GR rows by the first round, or lifted there
-// when no round is left.
 int run_dense(mpc_ctx* ctx, u64 vid, u32 batch, Dense& dv, long long D, const u64* z0, int k0,
-              int R, const Small& s, const IVBuf& ivb, u64* trace, const Vec* ylift = nullptr) {
+              int R, const Small& s, const IVBuf& ivb, u64* trace) {
   int rc;
   const u64* z = z0;
   int zi = 0;
@@ -861,17 +850,12 @@ int run_dense(mpc_ctx* ctx, u64 vid, u32 batch, Dense& dv, long long D, const u6
     Vec& xo = dv.x[dv.cur ^ 1];
     Vec& yo = dv.y[dv.cur ^ 1];
     u64* zo = s.z[zi];
-    if ((rc = reduce_round_dense(ctx, vid, batch, k, x, y, D, z, xo, yo, zo, s, trace,
-                                 k == k0 ? ylift : nullptr)))
-      return rc;
+    if ((rc = reduce_round_dense(ctx, vid, batch, k, x, y, D, z, xo, yo, zo, s, trace))) return rc;
     z = zo;
     zi ^= 1;
     dv.cur ^= 1;
     D = (D + 1) / 2;
   }
-  if (ylift && k0 > R)
-    for (int c = 0; c < 6; ++c)
-      if (ylift->c[c]) launch_gr_lift(ctx->st, ylift->c[c], D, dv.y[dv.cur].c[c]);
   return inner_verify_dense(ctx, vid, batch, dv.x[dv.cur], dv.y[dv.cur], D, z, s, ivb, trace, R);
 }
 
@@ -880,24 +864,16 @@ long long dim_after(long long D, int R) {
   return D;
 }
 
-// Allocate ping-pong vectors for a dense claim of dimension D over the present components.  With
-// ylifted_R >= 1 the y side enters in ring words (run_dense's ylift) and the first round writes
-// slot 1, so slot 0 of y only ever holds the outputs of round 2 and later (at most cap[1] rows).
-// With x_from_bits the first round writes x's slot 1 without reading slot 0 (the edaBit
-// inner-product batch), so x's slot 0 is half size as well.
-Dense plan_dense(Arena& a, long long D, const bool xc[6], const bool yc[6], int ylifted_R = 0,
-                 bool x_from_bits = false) {
+// Allocate ping-pong vectors for a dense claim of dimension D over the present components: a
+// slot's x vectors, then its y vectors, each side's present vectors at one stride (the batched
+// folds use that).
+Dense plan_dense(Arena& a, long long D, const bool xc[6], const bool yc[6]) {
   Dense d;
   d.cap[0] = D + 1;
   d.cap[1] = (D + 1) / 2 + 1;
-  const long long ycap0 = ylifted_R >= 1 ? d.cap[1] : d.cap[0];
-  const long long xcap0 = x_from_bits && ylifted_R >= 1 ? d.cap[1] : d.cap[0];
-  // a slot's x vectors, then its y vectors: each side's present vectors sit at one stride (the
-  // batched folds use that)
   for (int i = 0; i < 2; ++i) {
-    for (int c = 0; c < 6; ++c) d.x[i].c[c] = xc[c] ? a.take<u64>((i ? d.cap[1] : xcap0) * 64) : nullptr;
-    for (int c = 0; c < 6; ++c)
-      d.y[i].c[c] = yc[c] ? a.take<u64>((i ? d.cap[1] : ycap0) * 64) : nullptr;
+    for (int c = 0; c < 6; ++c) d.x[i].c[c] = xc[c] ? a.take<u64>(d.cap[i] * 64) : nullptr;
+    for (int c = 0; c < 6; ++c) d.y[i].c[c] = yc[c] ? a.take<u64>(d.cap[i] * 64) : nullptr;
   }
   return d;
 }
@@ -1010,12 +986,126 @@ int power_table(mpc_ctx* ctx, const u64* r, const PowPlan& p, u64* table, u64* a
   return MPC_OK;
 }
 
-struct VMultPlan {
-  Small s;
-  u64* pw;
+// A batch of weighted ring words (gr_block.cu): x_i = R_{b >> sh} T_j X_i, y_i = lift(Y_i), i =
+// B b + j < D, whose first kap = log2(B) rounds need no GR vectors.
+constexpr int BLK_ROUNDS = 3;
+struct BlkPlan {
+  long long D, nb;        // words, blocks
+  long long nw, nwp;      // weight rows R, rounded up to whole tiles
+  int R, kap, B, sh;
+  bool full;              // all components and the claim's sums; else x has 2 and 4 only
   PowPlan pp;
+  u64 *T, *Rw, *S, *V, *W, *Vm, *G;
   Dense dv;
   IVBuf iv;
+};
+
+// wlog: log2 of the words per weight step (0: weights r^i; 6: r^(i / 64), T_j = 1)
+BlkPlan plan_blk(Arena& a, long long D, int R, int wlog, bool full, const bool xc[6],
+                 const bool yc[6]) {
+  BlkPlan p;
+  p.D = D;
+  p.R = R;
+  p.kap = std::min(R, BLK_ROUNDS);
+  p.B = 1 << p.kap;
+  p.nb = (D + p.B - 1) / p.B;
+  p.sh = wlog > p.kap ? wlog - p.kap : 0;
+  p.nw = ((p.nb - 1) >> p.sh) + 1;
+  p.nwp = (p.nw + 127) / 128 * 128;
+  p.full = full;
+  p.pp = plan_pow(a, p.nw);
+  p.T = a.take<u64>((p.B + 1) * 64);
+  p.Rw = a.take<u64>(p.nwp * 64);
+  p.S = a.take<u64>(blk_rows(p.B, full) * 64);
+  p.V = a.take<u64>(p.B * 64);
+  p.W = a.take<u64>(p.B * 64);
+  p.Vm = a.take<u64>(p.B * 4096);
+  p.G = a.take<u64>(p.nwp * p.B * 64);
+  p.dv = plan_dense(a, p.nb, xc, yc);
+  p.iv = plan_iv(a, dim_after(p.nb, R - p.kap));
+  return p;
+}
+
+// T_j = r^j (j <= B) and the weights R_b = r^(B b) of a batch with weights r^i.
+int blk_tables(mpc_ctx* ctx, BlkPlan& p, const u64* r, u64* aux) {
+  launch_gr_powers(ctx->st, r, p.B + 1, p.T);
+  return power_table(ctx, p.T + p.B * 64, p.pp, p.Rw, aux);
+}
+
+// The batch from its weights (T, Rw), words (xw, yw: component pointers) and claim (zw: 6 x D
+// words, full batches; else s.zinit holds the claim): the first kap rounds from the block sums,
+// the vectors after them, and the dense rounds.
+int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const Vec& yw,
+            const u64* zw, const Small& s, u64* trace) {
+  cudaStream_t st = ctx->st;
+  const int B = p.B;
+  int rc;
+  CK(cudaMemsetAsync(p.S, 0, (size_t)blk_rows(B, p.full) * 512, st));
+  BlkIn in;
+  for (int c = 0; c < 6; ++c) {
+    in.x[c] = xw.c[c];
+    in.y[c] = yw.c[c];
+  }
+  in.z = zw;
+  in.ldz = p.D;
+  in.D = p.D;
+  // parties 1 and 2 only: their matrices sit where those of a full batch's first two would
+  const int np = p.full ? 3 : 2, p0 = p.full ? 0 : 1;
+  if (p.full || p.kap > 0) launch_blk_sums(st, in, B, p.full, p.nb, p.sh, p.Rw, p.S);
+  if (p.full) {
+    CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
+    launch_blk_claim(st, p.T, p.S + 3ll * B * B * 64, B, s.zinit);
+  }
+  CK(cudaMemcpyAsync(p.V, p.T, (size_t)B * 512, cudaMemcpyDeviceToDevice, st));
+  launch_ones(st, B, p.W);
+  const u64* z = s.zinit;
+  for (int k = 1; k <= p.kap; ++k) {
+    u64* sums = cur_sums(s);
+    launch_weighted_sums(st, p.V, p.W, p.S, B, k, np, sums + 64 * p0);
+    u64* zo = s.z[k & 1];
+    round_tail(ctx, vid, batch, k, z, zo, s, sums, 64, trace);
+    z = zo;
+    launch_update_vw(st, p.V, p.W, B, k, s.coef);
+  }
+  // G row b B + j = R_b V_j
+  bool done = false;
+  launch_gr_mulmat_batch(st, B, p.V, 64, p.Vm);
+  if (ctx->gemm_path == MPC_GEMM_LIMB_TC) {
+    GrMMArgs g = grargs(ctx);
+    g.R = B * p.nwp;   // rows j nwp + b read R_b, matrix j
+    g.p0 = p.Rw;
+    g.in = GrRowMap{p.nwp, 64, 0};
+    g.Mmat = p.Vm;
+    g.mrows = p.nwp;
+    g.out = p.G;
+    g.om = GrRowMap{p.nwp, 64ll * B, 64};
+    g_launches += 1;
+    Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)g.R * 4096);
+    done = gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT) == 0;
+    if (!done) g_launches -= 1;
+  }
+  for (int j = 0; j < B && !done; ++j)
+    if ((rc = gr_matmul(ctx, p.nw, p.Rw, nullptr, 1, 64, p.Vm + j * 4096, nullptr, 0, p.G + j * 64,
+                        64ll * B)))
+      return rc;
+  BlkVec vi;
+  BlkOut vo;
+  for (int side = 0; side < 2; ++side) {
+    for (int c = 0; c < 6; ++c) {
+      vi.c[c] = side ? yw.c[c] : xw.c[c];
+      vo.c[c] = side ? p.dv.y[0].c[c] : p.dv.x[0].c[c];
+    }
+    launch_blk_combine(st, vi, vo, B, side == 0, p.D, p.nb, side ? 0 : p.sh, side ? p.W : p.G);
+  }
+  if (z != s.zinit) CK(cudaMemcpyAsync(s.zinit, z, 384 * 8, cudaMemcpyDeviceToDevice, st));
+  p.dv.cur = 0;
+  if ((rc = cuda_check(ctx, "block rounds"))) return rc;
+  return run_dense(ctx, vid, batch, p.dv, p.nb, s.zinit, p.kap + 1, p.R, s, p.iv, trace);
+}
+
+struct VMultPlan {
+  Small s;
+  BlkPlan b;
   int R;
 };
 
@@ -1023,11 +1113,8 @@ VMultPlan plan_vmult(Arena& a, long long n, int R) {
   VMultPlan p;
   p.R = R < 0 ? default_R(n) : R;
   p.s = plan_small(a);
-  p.pw = a.take<u64>(n * 64);
-  p.pp = plan_pow(a, n);
   const bool all[6] = {true, true, true, true, true, true};
-  p.dv = plan_dense(a, n, all, all, p.R);
-  p.iv = plan_iv(a, dim_after(n, p.R));
+  p.b = plan_blk(a, n, p.R, 0, true, all, all);
   return p;
 }
 
@@ -1146,9 +1233,12 @@ size_t trunc_tc_scratch(const TruncShape& h) {
   return h.compact ? limb_tc_scratch_bytes(12 * h.nhi, 64, h.L, 1) : 0;
 }
 
-TruncPlan plan_trunc(Arena& a, long long E, int R1, bool tc, bool chunked, const mpc_tuning& tu) {
+// whole_table: every power rho^e is kept (the caller reads them)
+TruncPlan plan_trunc(Arena& a, long long E, int R1, bool tc, bool chunked, const mpc_tuning& tu,
+                     bool whole_table = false) {
   TruncPlan p;
-  const TruncShape h = trunc_shape(E, R1, tc, tu);
+  TruncShape h = trunc_shape(E, R1, tc, tu);
+  if (whole_table) h.compact = false;
   p.E = E;
   p.R1 = h.R1;
   p.kd = h.kd;
@@ -1275,49 +1365,30 @@ bool plan_vtrunc(Arena& a, long long n, int R, bool tc, const mpc_tuning& tu, VT
   return true;
 }
 
-// One chunk of batch 1 of Pi_BIVerify (Fig. PBDP): the 2 E inner products of the truncation pairs
-// of outputs e0 .. e0 + E - 1 (E = p.E) of a layer of E_all outputs, with the challenge and round
-// streams of batch `batch`.  pq_all: the layer's 12 rows of <p>, <q> (stride E_all).
-int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, const u64* pq_all,
-                       long long E_all, long long e0, int trunc_bits, u64 verify_id, u32 batch,
-                       u64 matmul_call_id, u64* tr, const u64* row_keys, long long N) {
+// ---- batches of bit pairs -----------------------------------------------------------------------
+// A batch whose 64-element blocks are bit words: x_{64 e + j} = -rho^e V_j b1_{e,j} (held by P0 and
+// P1), y_{64 e + j} = -W_j b2_{e,j} (P0 and P2): the truncation pairs (rho = r^2, V_j = u_j, W_j =
+// 1) and the edaBit bit products (rho = r^64, V_j = r^j, W_j = 1).  The weights first.
+int bit_tables(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* rho) {
   cudaStream_t st = ctx->st;
-  Phase* phase = new Phase(ctx, MPC_PROF_TRUNC_SETUP);
-  const u64 mobj = make_obj(matmul_call_id, 0, 0);
   const long long E = p.E;
   int rc;
-  if (p.pqc)   // this chunk's outputs of the 12 rows of <p>, <q>, gathered to a stride of E
-    CK(cudaMemcpy2DAsync(p.pqc, (size_t)E * 8, pq_all + e0, (size_t)E_all * 8, (size_t)E * 8, 12,
-                         cudaMemcpyDeviceToDevice, st));
-  const u64* pq = p.pqc ? p.pqc : pq_all;
-  if ((rc = sums_begin(ctx, s))) return rc;
-  reveal(ctx, P_VER_R, make_obj(verify_id, batch, 0), s, s.r);
-  launch_trunc_u(st, s.r, trunc_bits, p.V);                         // V_j = u_j
-  for (int j = 0; j < 64; ++j)
-    CK(cudaMemcpyAsync(p.W + j * 64, ctx->cst + CST_ONE, 512, cudaMemcpyDeviceToDevice, st));
+  launch_ones(st, 64, p.W);
   if (p.Epad > E) {
     CK(cudaMemsetAsync(p.b1 + E, 0, (size_t)(p.Epad - E) * 8, st));
     CK(cudaMemsetAsync(p.b2 + E, 0, (size_t)(p.Epad - E) * 8, st));
   }
-  if (row_keys) {
-    launch_prf_words_keyed(st, E, ctx->k01, make_tag(P_TRUNC_BITS, C_TB1), row_keys, N, p.b1, e0);
-    launch_prf_words_keyed(st, E, ctx->k02, make_tag(P_TRUNC_BITS, C_TB2), row_keys, N, p.b2, e0);
-  } else {
-    launch_prf_words(st, E, ctx->k01, make_tag(P_TRUNC_BITS, C_TB1), mobj, p.b1, e0);
-    launch_prf_words(st, E, ctx->k02, make_tag(P_TRUNC_BITS, C_TB2), mobj, p.b2, e0);
-  }
-  launch_gr_mul1(st, s.r, s.r, s.aux + 64);                          // r^2
-  // r^(2e) for e < Epad: r^(2 e_lo) for e_lo < L by repeated multiplication, then every further
-  // block of L rows is that block times the constant r^(2 L e_hi) (a 64 x 64 matrix product)
-  if ((rc = power_table(ctx, s.aux + 64, p.pow, p.Rtab, s.aux + 192))) return rc;
+  // rho^e for e < Epad: rho^e_lo for e_lo < L by repeated multiplication, then every further
+  // block of L rows is that block times the constant rho^(L e_hi) (a 64 x 64 matrix product)
+  if ((rc = power_table(ctx, rho, p.pow, p.Rtab, s.aux + 192))) return rc;
   if (p.compact) {
-    launch_gr_mul1(st, p.Rtab + (p.L - 1) * 64, s.aux + 64, s.aux + 128);   // r^(2L)
+    launch_gr_mul1(st, p.Rtab + (p.L - 1) * 64, rho, s.aux + 128);   // rho^L
     launch_gr_powers(st, s.aux + 128, p.nhi, p.Thi);
     launch_gr_mulmat_batch(st, p.nhi - 1, p.Thi + 64, 64, p.Mhi);
   } else if (p.nhi > 1) {
-    launch_gr_mul1(st, p.Rtab + (p.L - 1) * 64, s.aux + 64, s.aux + 128);   // r^(2L)
+    launch_gr_mul1(st, p.Rtab + (p.L - 1) * 64, rho, s.aux + 128);   // rho^L
     launch_gr_powers(st, s.aux + 128, p.nhi, p.Thi);
-    // rows h L + e_lo (h >= 1) = r^(2 L h) r^(2 e_lo): one grouped product, matrix h - 1 for
+    // rows h L + e_lo (h >= 1) = rho^(L h) rho^e_lo: one grouped product, matrix h - 1 for
     // the rows (h - 1) L .. h L - 1 of the block, each reading row e_lo of the first block
     launch_gr_mulmat_batch(st, p.nhi - 1, p.Thi + 64, 64, p.Mhi);
     bool done = false;
@@ -1340,27 +1411,18 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
                           p.Rtab + h * p.L * 64, 64)))
         return rc;
   }
-  CK(cudaMemsetAsync(p.Zpq, 0, 12 * 64 * 8, st));
-  // sum_e r^(2e) p_c[e], sum_e r^(2e) q_c[e]: (12 x E) . (E x 64)
-  if (p.compact) {
-    // Zhi[c nhi + h] = sum_{e_lo} pq_c[h L + e_lo] r^(2 e_lo) (E = nhi L: one strided view)
-    GemmTerm T;
-    T.A = op(pq, p.L);
-    T.B = op(p.Rtab, 64);
-    if ((rc = dense_gemm(ctx, 12 * p.nhi, 64, p.L, T, epi_store(p.Zhi, 64), tcs))) return rc;
-    launch_gather_rows_affine(st, 12 * p.nhi, p.Thi, 1, 1, p.nhi, p.Zrep);   // T_hi[h]
-    launch_gr_mul_rows(st, 12 * p.nhi, p.Zhi, p.Zrep, p.Zprod);
-    launch_block_rowsum(st, 12, p.nhi, p.Zprod, p.Zpq);
-  } else {
-    launch_scalar_gr_sum(st, E, pq, E, 12, p.Rtab, p.Zpq);
-  }
-  u64* z0 = p.zt + 384;
-  for (int c = 0; c < 6; ++c)   // z_c = sum r^(2e) p_c + r sum r^(2e) q_c
-    launch_gr_lincomb(st, ctx->cst + CST_ONE, p.Zpq + c * 64, s.r, p.Zpq + (6 + c) * 64,
-                      z0 + c * 64);
-  delete phase;
-  phase = new Phase(ctx, MPC_PROF_TRUNC_S);
-  {  // S_{j,j'} = sum_e r^(2e) b1_{e,j} b2_{e,j'} (P0), with r^(2e) = r^(2 L e_hi) r^(2 e_lo):
+  return MPC_OK;
+}
+
+// The batch from its weights (bit_tables), bit words (p.b1, p.b2), V and claim z0: the matrix S,
+// the rounds that fold the 64 bits, the folded vectors and the dense rounds.
+int bit_batch(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* z0, u64 verify_id, u32 batch,
+              u64* tr) {
+  cudaStream_t st = ctx->st;
+  const long long E = p.E;
+  int rc;
+  Phase* phase = new Phase(ctx, MPC_PROF_TRUNC_S);
+  {  // S_{j,j'} = sum_e rho^e b1_{e,j} b2_{e,j'} (P0), with rho^e = rho^(L e_hi) rho^e_lo:
      // tensor cores for the inner sums over e_lo, then sum_{e_hi} T_hi (x) S_hi as a GEMM + fold
     launch_trunc_limb_table(st, p.Rtab, p.L, p.TL8);
     launch_trunc_bit_transpose(st, p.b1, p.Epad, p.B1T);
@@ -1372,7 +1434,7 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
                             ST_TIMEOUT))
         return fail(ctx, MPC_ERR_CUDA, "verify_matmul: tensor map of the limb table");
     }
-    // S = sum_{e_hi} T_hi S_hi: the blocks h >= 1 times r^(2 L h) (matrix h - 1) in place, then the
+    // S = sum_{e_hi} T_hi S_hi: the blocks h >= 1 times rho^(L h) (matrix h - 1) in place, then the
     // sum over the blocks
     if (p.nhi > 1) {
       bool done = false;
@@ -1408,11 +1470,11 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
   int zi = 0;
   for (int k = 1; k <= p.kd; ++k) {   // rounds folding the 64 bits of each output
     u64* sums = cur_sums(s);
-    launch_trunc_round_sums(st, p.V, p.W, p.S, k, sums);
+    launch_weighted_sums(st, p.V, p.W, p.S, 64, k, 1, sums);
     round_tail(ctx, verify_id, batch, k, z, zbuf[zi], s, sums, 64, tr);
     z = zbuf[zi];
     zi ^= 1;
-    launch_trunc_update_vw(st, p.V, p.W, k, s.coef);
+    launch_update_vw(st, p.V, p.W, 64, k, s.coef);
   }
   delete phase;
   phase = new Phase(ctx, MPC_PROF_TRUNC_MATERIALIZE);
@@ -1520,6 +1582,55 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
   rc = run_dense(ctx, verify_id, batch, p.dt, p.Dt, s.zinit, p.kd + 1, p.R1, s, p.ivt, tr);
   delete phase;
   return rc;
+}
+
+// One chunk of batch 1 of Pi_BIVerify (Fig. PBDP): the 2 E inner products of the truncation pairs
+// of outputs e0 .. e0 + E - 1 (E = p.E) of a layer of E_all outputs, with the challenge and round
+// streams of batch `batch`.  pq_all: the layer's 12 rows of <p>, <q> (stride E_all).
+int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, const u64* pq_all,
+                       long long E_all, long long e0, int trunc_bits, u64 verify_id, u32 batch,
+                       u64 matmul_call_id, u64* tr, const u64* row_keys, long long N) {
+  cudaStream_t st = ctx->st;
+  Phase* phase = new Phase(ctx, MPC_PROF_TRUNC_SETUP);
+  const u64 mobj = make_obj(matmul_call_id, 0, 0);
+  const long long E = p.E;
+  int rc;
+  if (p.pqc)   // this chunk's outputs of the 12 rows of <p>, <q>, gathered to a stride of E
+    CK(cudaMemcpy2DAsync(p.pqc, (size_t)E * 8, pq_all + e0, (size_t)E_all * 8, (size_t)E * 8, 12,
+                         cudaMemcpyDeviceToDevice, st));
+  const u64* pq = p.pqc ? p.pqc : pq_all;
+  if ((rc = sums_begin(ctx, s))) return rc;
+  reveal(ctx, P_VER_R, make_obj(verify_id, batch, 0), s, s.r);
+  launch_trunc_u(st, s.r, trunc_bits, p.V);                         // V_j = u_j
+  if (row_keys) {
+    launch_prf_words_keyed(st, E, ctx->k01, make_tag(P_TRUNC_BITS, C_TB1), row_keys, N, p.b1, e0);
+    launch_prf_words_keyed(st, E, ctx->k02, make_tag(P_TRUNC_BITS, C_TB2), row_keys, N, p.b2, e0);
+  } else {
+    launch_prf_words(st, E, ctx->k01, make_tag(P_TRUNC_BITS, C_TB1), mobj, p.b1, e0);
+    launch_prf_words(st, E, ctx->k02, make_tag(P_TRUNC_BITS, C_TB2), mobj, p.b2, e0);
+  }
+  launch_gr_mul1(st, s.r, s.r, s.aux + 64);                          // r^2
+  if ((rc = bit_tables(ctx, p, s, s.aux + 64))) return rc;
+  CK(cudaMemsetAsync(p.Zpq, 0, 12 * 64 * 8, st));
+  // sum_e r^(2e) p_c[e], sum_e r^(2e) q_c[e]: (12 x E) . (E x 64)
+  if (p.compact) {
+    // Zhi[c nhi + h] = sum_{e_lo} pq_c[h L + e_lo] r^(2 e_lo) (E = nhi L: one strided view)
+    GemmTerm T;
+    T.A = op(pq, p.L);
+    T.B = op(p.Rtab, 64);
+    if ((rc = dense_gemm(ctx, 12 * p.nhi, 64, p.L, T, epi_store(p.Zhi, 64), tcs))) return rc;
+    launch_gather_rows_affine(st, 12 * p.nhi, p.Thi, 1, 1, p.nhi, p.Zrep);   // T_hi[h]
+    launch_gr_mul_rows(st, 12 * p.nhi, p.Zhi, p.Zrep, p.Zprod);
+    launch_block_rowsum(st, 12, p.nhi, p.Zprod, p.Zpq);
+  } else {
+    launch_scalar_gr_sum(st, E, pq, E, 12, p.Rtab, p.Zpq);
+  }
+  u64* z0 = p.zt + 384;
+  for (int c = 0; c < 6; ++c)   // z_c = sum r^(2e) p_c + r sum r^(2e) q_c
+    launch_gr_lincomb(st, ctx->cst + CST_ONE, p.Zpq + c * 64, s.r, p.Zpq + (6 + c) * 64,
+                      z0 + c * 64);
+  delete phase;
+  return bit_batch(ctx, p, s, z0, verify_id, batch, tr);
 }
 
 // workspace of a standalone truncation (mpc_trunc)
@@ -1767,7 +1878,8 @@ int64_t mpc_trace_words(const mpc_ctx* ctx, int op, int64_t a, int64_t b, int64_
 }
 
 namespace {
-void nl_plan_take(Arena& a, int nst, const long long np[2]);   // workspace of a non-linear layer
+// workspace of a non-linear layer
+void nl_plan_take(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuning& tu);
 }
 
 int64_t mpc_workspace_size(const mpc_ctx* ctx, int op, int64_t a, int64_t b, int64_t c,
@@ -1808,14 +1920,16 @@ int64_t mpc_workspace_size(const mpc_ctx* ctx, int op, int64_t a, int64_t b, int
     case MPC_OP_RELU: {
       if (a <= 0) return -1;
       const long long np[2] = {64 * ((a + 63) / 64), 0};
-      nl_plan_take(ar, 1, np);
+      nl_plan_take(ar, 1, np, ctx && ctx->gemm_path == MPC_GEMM_LIMB_TC,
+                   ctx ? ctx->tune : default_tuning());
       break;
     }
     case MPC_OP_MAXPOOL2: {
       if (a <= 0 || b <= 0 || c <= 0 || (b & 1) || (c & 1)) return -1;
       const long long nw = a * (b / 2) * (c / 2);
       const long long np[2] = {64 * ((2 * nw + 63) / 64), 64 * ((nw + 63) / 64)};
-      nl_plan_take(ar, 2, np);
+      nl_plan_take(ar, 2, np, ctx && ctx->gemm_path == MPC_GEMM_LIMB_TC,
+                   ctx ? ctx->tune : default_tuning());
       break;
     }
     case MPC_OP_RECONSTRUCT:
@@ -2044,25 +2158,18 @@ namespace {
 int verify_mult_body(mpc_ctx* ctx, uint64_t verify_id, const u64* xs, const u64* ys,
                      const u64* zs, long long n, VMultPlan& p, u64* trace) {
   Phase phase(ctx, MPC_PROF_VERIFY_MULT);
-  cudaStream_t st = ctx->st;
   const Small& s = p.s;
   // Pi_Tran (Fig. MTP): reveal r; x'_i = r^i x_i; y lifted; z = sum r^i z_i
   int rc;
   if ((rc = sums_begin(ctx, s))) return rc;
   reveal(ctx, P_VER_R, make_obj(verify_id, 0, 0), s, s.r);
-  if ((rc = power_table(ctx, s.r, p.pp, p.pw, s.aux))) return rc;
-  Vec& x = p.dv.x[0];
-  Vec ylift;   // y stays in ring words until the first round folds it
+  if ((rc = blk_tables(ctx, p.b, s.r, s.aux))) return rc;
+  Vec x, y;
   for (int c = 0; c < 6; ++c) {
-    launch_gr_scale_rows(st, p.pw, xs + c * n, n, x.c[c]);
-    ylift.c[c] = const_cast<u64*>(ys + c * n);
+    x.c[c] = const_cast<u64*>(xs + c * n);
+    y.c[c] = const_cast<u64*>(ys + c * n);
   }
-  CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
-  {  // z_c = sum_i z_c[i] r^i for the 6 components at once: (6 x n) . (n x 64)
-    launch_scalar_gr_sum(st, n, zs, n, 6, p.pw, s.zinit);
-  }
-  p.dv.cur = 0;
-  return run_dense(ctx, verify_id, 0, p.dv, n, s.zinit, 1, p.R, s, p.iv, trace, &ylift);
+  return run_blk(ctx, verify_id, 0, p.b, x, y, zs, s, trace);
 }
 }  // namespace
 
@@ -2880,28 +2987,20 @@ struct NLPlan {
   long long ne, D1;
   int R1;
   Small s1;
-  u64* pw1;
-  PowPlan pp1;
-  Dense d1;
-  IVBuf iv1;
-  u64* Ye;                       // 6 x D1 ring words: the y side before its first fold
-  u64* S6;                       // 6 x ne: the first round's per-element party-sum words
-  u64* A1;                       // ne x 64: r^g f, the first round's x fold
-  u64** ydev;                    // 6 device pointers (kernel argument)
+  BlkPlan b1;
+  u64* Ye;                       // 6 x D1 ring words: the y side
+  u64* Xe;                       // D1 ring words: the bits m (components 2 and 4 of x)
   // batch 2: AND gates
   GfPlan gf;
   // batch 3: edaBit bit products (nb = 64 sum np), x only [r]_1 and y only [r]_2 (reading N9)
   long long nb;
   int Rb;
   Small sb;
-  PowPlan ppb;
-  u64* pwb;
-  Dense db;
-  IVBuf ivb;
-  u64* Yb;                       // 2 x nb ring words: components 1 and 5 of the b2 bits
+  TruncPlan tb;                  // bit words of 64 products each
+  u64* Zr;                       // 6 x 64 elements: the claim's sums over the bit words
 };
 
-NLPlan plan_nl(Arena& a, int nst, const long long np[2]) {
+NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuning& tu) {
   NLPlan p;
   p.nst = nst;
   p.nm = 0;
@@ -2921,27 +3020,17 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2]) {
   p.D1 = 64 * p.ne;
   p.R1 = default_R(p.D1);
   p.s1 = plan_small(a);
-  p.pw1 = a.take<u64>(p.ne * 64);
-  p.pp1 = plan_pow(a, p.ne);
   const bool xc[6] = {false, false, true, false, true, false};
   const bool yc[6] = {true, true, true, true, true, true};
-  p.d1 = plan_dense(a, p.D1, xc, yc, p.R1, true);
-  p.iv1 = plan_iv(a, dim_after(p.D1, p.R1));
+  p.b1 = plan_blk(a, p.D1, p.R1, 6, false, xc, yc);
   p.Ye = a.take<u64>(6 * p.D1);
-  p.S6 = a.take<u64>(6 * p.ne);
-  p.A1 = a.take<u64>(p.ne * 64);
-  p.ydev = a.take<u64*>(6);
+  p.Xe = a.take<u64>(p.D1);
   p.gf = plan_gf(a, andw, -1);
   p.nb = 64 * p.ne;
   p.Rb = default_R(p.nb);
   p.sb = plan_small(a);
-  p.pwb = a.take<u64>(p.nb * 64);
-  p.ppb = plan_pow(a, p.nb);
-  const bool bx[6] = {true, false, false, true, false, false};
-  const bool by[6] = {false, true, false, false, false, true};
-  p.db = plan_dense(a, p.nb, bx, by, p.Rb);
-  p.ivb = plan_iv(a, dim_after(p.nb, p.Rb));
-  p.Yb = a.take<u64>(2 * p.nb);
+  p.tb = plan_trunc(a, p.ne, p.Rb, tc, false, tu, true);
+  p.Zr = a.take<u64>(384 * 64);
   return p;
 }
 
@@ -2976,17 +3065,13 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     const long long n = p.nm;
     if ((rc = sums_begin(ctx, s))) return rc;
     reveal(ctx, P_VER_R, make_obj(vid, 0, 0), s, s.r);
-    if ((rc = power_table(ctx, s.r, v.pp, v.pw, s.aux))) return rc;
-    Vec& x = v.dv.x[0];
-    Vec ylift;
+    if ((rc = blk_tables(ctx, v.b, s.r, s.aux))) return rc;
+    Vec x, y;
     for (int c = 0; c < 6; ++c) {
-      launch_gr_scale_rows(st, v.pw, p.MX + c * n, n, x.c[c]);
-      ylift.c[c] = p.MY + c * n;
+      x.c[c] = p.MX + c * n;
+      y.c[c] = p.MY + c * n;
     }
-    CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
-    launch_scalar_gr_sum(st, n, p.MZ, n, 6, v.pw, s.zinit);
-    v.dv.cur = 0;
-    if ((rc = run_dense(ctx, vid, 0, v.dv, n, s.zinit, 1, v.R, s, v.iv, trace, &ylift))) return rc;
+    if ((rc = run_blk(ctx, vid, 0, v.b, x, y, p.MZ, s, trace))) return rc;
   }
   u64* tr1 = trace ? trace + (long long)(p.vm.R + 1) * TRACE_ROUND : nullptr;
   // ---- batch 1: the edaBit inner products, weight r^e on row e (e over all stages)
@@ -2994,49 +3079,22 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     const Small& s = p.s1;
     if ((rc = sums_begin(ctx, s))) return rc;
     reveal(ctx, P_VER_R, make_obj(vid, 1, 0), s, s.r);
-    if ((rc = power_table(ctx, s.r, p.pp1, p.pw1, s.aux))) return rc;
-    Vec ylift;
-    for (int c = 0; c < 6; ++c) ylift.c[c] = p.Ye + c * p.D1;
-    CK(cudaMemcpyAsync(p.ydev, ylift.c, 6 * sizeof(u64*), cudaMemcpyHostToDevice, st));
+    BlkPlan& b = p.b1;
+    launch_ones(st, b.B, b.T);   // weights r^e on the 64 entries of element e
+    if ((rc = power_table(ctx, s.r, b.pp, b.Rw, s.aux))) return rc;
     CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
     long long e0 = 0;
-    for (int q = 0; q < p.nst; ++q) {   // the y words and the claim (x is never materialised)
+    for (int q = 0; q < p.nst; ++q) {   // the words and the claim
       CSPlan& c = p.cs[q];
-      launch_eda_tran(st, c.mbw, c.rp, c.np, p.pw1, e0, nullptr, nullptr, p.ydev);
-      launch_scalar_gr_sum(st, c.np, c.ez, c.np, 6, p.pw1 + e0 * 64, s.zinit);
+      launch_eda_words(st, c.mbw, c.rp, c.np, e0, p.D1, p.Xe, p.Ye);
+      launch_scalar_gr_sum(st, c.np, c.ez, c.np, 6, b.Rw + e0 * 64, s.zinit);
       g_launches += 1;
       e0 += c.np;
     }
-    // Round 1 from the bits: x = r^g <m_i> pairs the bits 2k, 2k + 1 of one element, so the
-    // party sums are sum_g r^g s(g) over per-element words (rows P1, P2 of each block; P0's are
-    // zero) and the folded x is a selection among 0, r^g - r^g f, r^g f and r^g.
-    u64* U = cur_sums(s);
-    e0 = 0;
-    for (int q = 0; q < p.nst; ++q) {
-      CSPlan& c = p.cs[q];
-      launch_eda_r1_sums(st, c.mbw, c.rp, c.np, e0, p.ne, p.S6);
-      g_launches += 1;
-      e0 += c.np;
-    }
-    launch_scalar_gr_sum(st, p.ne, p.S6, p.ne, 2, p.pw1, U + 64);                   // S00
-    launch_scalar_gr_sum(st, p.ne, p.S6 + 2 * p.ne, p.ne, 2, p.pw1, U + 192 + 64);  // S01 + S10
-    launch_scalar_gr_sum(st, p.ne, p.S6 + 4 * p.ne, p.ne, 2, p.pw1, U + 576 + 64);  // S11
-    round_tail(ctx, vid, 1, 1, s.zinit, s.z[1], s, U, 64, tr1);
-    Vec& xo = p.d1.x[1];
-    Vec& yo = p.d1.y[1];
-    if ((rc = gr_matmul(ctx, p.ne, p.pw1, nullptr, 1, 64, s.MM, nullptr, 0, p.A1, 64))) return rc;
-    e0 = 0;
-    for (int q = 0; q < p.nst; ++q) {
-      CSPlan& c = p.cs[q];
-      launch_eda_x_fold(st, c.mbw, c.np, e0, p.pw1, p.A1, xo.c[2], xo.c[4]);
-      g_launches += 1;
-      e0 += c.np;
-    }
-    const long long Dh = p.D1 / 2;
-    for (int c = 0; c < 6; ++c) launch_fold_lifted(st, ylift.c[c], Dh, p.D1, s.coef, yo.c[c]);
-    if ((rc = cuda_check(ctx, "edaBit first round"))) return rc;
-    p.d1.cur = 1;
-    if ((rc = run_dense(ctx, vid, 1, p.d1, Dh, s.z[1], 2, p.R1, s, p.iv1, tr1))) return rc;
+    Vec x{}, y;
+    x.c[2] = x.c[4] = p.Xe;
+    for (int c = 0; c < 6; ++c) y.c[c] = p.Ye + c * p.D1;
+    if ((rc = run_blk(ctx, vid, 1, b, x, y, nullptr, s, tr1))) return rc;
   }
   u64* tr2 = tr1 ? tr1 + (long long)(p.R1 + 1) * TRACE_ROUND : nullptr;
   // ---- batch 2: every AND gate over GF(2^64), stage by stage, level by level
@@ -3064,27 +3122,28 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     const Small& s = p.sb;
     if ((rc = sums_begin(ctx, s))) return rc;
     reveal(ctx, P_VER_R, make_obj(vid, 3, 0), s, s.r);
-    if ((rc = power_table(ctx, s.r, p.ppb, p.pwb, s.aux))) return rc;
-    Vec& x = p.db.x[0];
-    Vec ylift{};   // components 1 and 5 of the b2 bits, as ring words
-    ylift.c[1] = p.Yb;
-    ylift.c[5] = p.Yb + p.nb;
-    CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
-    long long e0 = 0;
+    // 64 consecutive products are the bits of one word of the b1 and b2 planes
+    TruncPlan& t = p.tb;
+    long long w0 = 0;
     for (int q = 0; q < p.nst; ++q) {
       CSPlan& c = p.cs[q];
-      const long long N = 64 * c.np;
-      for (int comp : {0, 3})
-        launch_gr_scale_rows(st, p.pwb + e0 * 64, c.B1 + comp * N, N, x.c[comp] + e0 * 64);
-      for (int comp : {1, 5})
-        CK(cudaMemcpyAsync(ylift.c[comp] + e0, c.B2 + comp * N, (size_t)N * 8,
-                           cudaMemcpyDeviceToDevice, st));
-      launch_scalar_gr_sum(st, N, c.eprod, N, 6, p.pwb + e0 * 64, s.zinit);
-      e0 += N;
+      CK(cudaMemcpyAsync(t.b1 + w0, c.b1w, (size_t)c.np * 8, cudaMemcpyDeviceToDevice, st));
+      CK(cudaMemcpyAsync(t.b2 + w0, c.b2w, (size_t)c.np * 8, cudaMemcpyDeviceToDevice, st));
+      w0 += c.np;
     }
-    p.db.cur = 0;
-    if ((rc = run_dense(ctx, vid, 3, p.db, p.nb, s.zinit, 1, p.Rb, s, p.ivb, tr3, &ylift)))
-      return rc;
+    launch_gr_powers(st, s.r, 64, t.V);                                   // V_j = r^j
+    launch_gr_mul1(st, t.V + 63 * 64, s.r, s.aux + 64);                   // rho = r^64
+    if ((rc = bit_tables(ctx, t, s, s.aux + 64))) return rc;
+    CK(cudaMemsetAsync(p.Zr, 0, 384 * 512, st));
+    CK(cudaMemsetAsync(t.zt + 384, 0, 384 * 8, st));
+    w0 = 0;
+    for (int q = 0; q < p.nst; ++q) {
+      CSPlan& c = p.cs[q];
+      launch_words_sums(st, c.eprod, 64 * c.np, c.np, t.Rtab + w0 * 64, p.Zr);
+      w0 += c.np;
+    }
+    launch_blk_claim(st, t.V, p.Zr, 64, t.zt + 384);
+    if ((rc = bit_batch(ctx, t, s, t.zt + 384, vid, 3, tr3))) return rc;
   }
   return MPC_OK;
 }
@@ -3106,7 +3165,9 @@ int nl_finish(mpc_ctx* ctx) {
 
 long long npad64(long long n) { return 64 * ((n + 63) / 64); }
 
-void nl_plan_take(Arena& a, int nst, const long long np[2]) { plan_nl(a, nst, np); }
+void nl_plan_take(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuning& tu) {
+  plan_nl(a, nst, np, tc, tu);
+}
 
 }  // namespace
 
@@ -3118,7 +3179,7 @@ int mpc_relu(mpc_ctx* ctx, uint64_t call_id, uint64_t verify_id, const uint64_t*
   if (!xs || !out || !id_ok(call_id) || !id_ok(verify_id)) return fail(ctx, MPC_ERR_ARG, "relu: bad argument");
   Arena ar{(char*)workspace, workspace_bytes, 0, false};
   const long long np[2] = {npad64(n), 0};
-  NLPlan p = plan_nl(ar, 1, np);
+  NLPlan p = plan_nl(ar, 1, np, ctx->gemm_path == MPC_GEMM_LIMB_TC, ctx->tune);
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "relu: workspace too small");
   Phase phase(ctx, MPC_PROF_NONLINEAR);
   cudaStream_t st = ctx->st;
@@ -3144,7 +3205,7 @@ int mpc_maxpool2(mpc_ctx* ctx, uint64_t call_id, uint64_t verify_id, const uint6
   const long long nw = B * C * (H / 2) * (W / 2);
   Arena ar{(char*)workspace, workspace_bytes, 0, false};
   const long long np[2] = {npad64(2 * nw), npad64(nw)};
-  NLPlan p = plan_nl(ar, 2, np);
+  NLPlan p = plan_nl(ar, 2, np, ctx->gemm_path == MPC_GEMM_LIMB_TC, ctx->tune);
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "maxpool2: workspace too small");
   Phase phase(ctx, MPC_PROF_NONLINEAR);
   cudaStream_t st = ctx->st;

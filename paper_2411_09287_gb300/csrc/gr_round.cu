@@ -290,31 +290,33 @@ k_rec_hash(const u64* __restrict__ log, u32* status, u32 flag) {
     atomicOr(status, flag);
 }
 
-// One round of the first rounds of the truncation batch (index i = 64 e + j, so that round k
-// folds bit k - 1 of j): with V_j, W_j the accumulated public weights of the x- and y-side bit j
-// and S_{j,j'} = sum_e r^(2e) b1_{e,j} b2_{e,j'}, the sums over the pairs (j, j') of one 2^k-block
-//   out[2 a + b] += sum_{bit k-1 of j = a, of j' = b} V_j W_j' S_{j,j'},  64 words at 192 (2 a + b)
-// (P0's S00, S01, S10, S11 of the round; out must be zero on entry).  Block (j, c) takes the c-th
-// eight j' of j's 2^k-block: the eight products share one reduction, so a block runs three
+// One of the first rounds of a batch evaluated from a matrix S_{j,j'}, j, j' < n (the truncation
+// batch's and the edaBits' bit pairs, n = 64: S_{j,j'} = sum_e R_e b1_{e,j} b2_{e,j'}; blocks of
+// ring words, n <= 8, one matrix per party): with V_j, W_j the accumulated weights of the x and y
+// side, the sums over the pairs (j, j') of one 2^k-block
+//   out[2 a + b] += sum_{bit k-1 of j = a, of j' = b} V_j W_j' S_{j,j'},  192 words apart, party p
+// at 64 p (the round's S00, S01, S10, S11; out must be zero on entry).  Block (j, c, p) takes the
+// c-th eight j' of j's 2^k-block: the eight products share one reduction, so a block runs three
 // dependent products' latency.  One thread group per j ran 2^k + 5 products one after another:
-// 201 us for k = 6, 461 us for the six rounds.
+// 201 us for k = 6, 461 us for the six rounds of a bit batch.
 __global__ void __launch_bounds__(256)
-k_trunc_round_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64* __restrict__ S,
-                   int k, u64* __restrict__ out) {
+k_weighted_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64* __restrict__ S,
+                int n, int k, u64* __restrict__ out) {
   __shared__ u64 w[8][64], s[8][64], T[2][64], v[64], scr[4 * 128];
   const int tid = threadIdx.x, t = tid & 63, part = tid >> 6;
   const int j = blockIdx.x, sh = k - 1, bs = 1 << k;
-  const int n = bs < 8 ? bs : 8;
+  const int m = bs < 8 ? bs : 8;
   const int j0 = (j & ~(bs - 1)) + blockIdx.y * 8;
-  for (int i = tid; i < n * 64; i += 256) {
+  S += (long long)blockIdx.z * n * n * 64;
+  for (int i = tid; i < m * 64; i += 256) {
     w[i >> 6][i & 63] = W[(j0 + (i >> 6)) * 64 + (i & 63)];
-    s[i >> 6][i & 63] = S[((long long)j * 64 + j0 + (i >> 6)) * 64 + (i & 63)];
+    s[i >> 6][i & 63] = S[((long long)j * n + j0 + (i >> 6)) * 64 + (i & 63)];
   }
   if (tid < 64) v[t] = V[j * 64 + t];
   __syncthreads();
   // halves of the block: with eight j' of a larger block they all lie in one half
   u64 lo[2] = {0, 0}, hi[2] = {0, 0};
-  for (int q = 0; q < n; ++q) {
+  for (int q = 0; q < m; ++q) {
     u64 l = 0, h = 0;
     gr_mac_part<16>(w[q], s[q], t, part * 16, l, h);
     if (((j0 + q) >> sh) & 1) { lo[1] += l; hi[1] += h; }
@@ -322,13 +324,13 @@ k_trunc_round_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u
   }
   const int aj = (j >> sh) & 1;
   for (int b = 0; b < 2; ++b) {
-    if (n == 8 && bs > 8 && (((j0 >> sh) & 1) != b)) continue;   // uniform over the block
+    if (m == 8 && bs > 8 && (((j0 >> sh) & 1) != b)) continue;   // uniform over the block
     const u64 r = gr_finish<4>(lo[b], hi[b], scr, tid);
     if (tid < 64) T[b][t] = r;
     __syncthreads();
     const u64 y = gr_mul_par<4>(v, T[b], scr, tid);
     if (tid < 64)
-      atomicAdd(reinterpret_cast<unsigned long long*>(out + 192 * (2 * aj + b) + t),
+      atomicAdd(reinterpret_cast<unsigned long long*>(out + 192 * (2 * aj + b) + 64 * blockIdx.z + t),
                 (unsigned long long)y);
   }
 }
@@ -336,10 +338,10 @@ k_trunc_round_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u
 // After round k: V_j <- w(j) V_j and W_j <- w(j) W_j with w = 1 - f or f by bit k-1 of j
 // (coef: f at 0, 1 - f at 384).
 __global__ void __launch_bounds__(256)
-k_trunc_update_vw(u64* __restrict__ V, u64* __restrict__ W, int k, const u64* __restrict__ coef) {
+k_update_vw(u64* __restrict__ V, u64* __restrict__ W, int n, int k, const u64* __restrict__ coef) {
   __shared__ u64 a[64], b[64], scr[4 * 128];
-  const int j = blockIdx.x & 63;
-  u64* X = (blockIdx.x < 64) ? V : W;
+  const int j = blockIdx.x < n ? blockIdx.x : blockIdx.x - n;
+  u64* X = (blockIdx.x < n) ? V : W;
   const int t = threadIdx.x;
   if (t < 64) a[t] = ((j >> (k - 1)) & 1) ? coef[t] : coef[384 + t];
   else if (t < 128) b[t - 64] = X[j * 64 + t - 64];
@@ -368,14 +370,14 @@ void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 fl
   k_rec_hash<<<n, 64, 0, st>>>(log, status, flag);
 }
 
-void launch_trunc_round_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int k,
-                             u64* out) {
+void launch_weighted_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int n, int k,
+                          int np, u64* out) {
   const int bs = 1 << k;
-  k_trunc_round_sums<<<dim3(64, bs < 8 ? 1 : bs / 8), 256, 0, st>>>(V, W, S, k, out);
+  k_weighted_sums<<<dim3(n, bs < 8 ? 1 : bs / 8, np), 256, 0, st>>>(V, W, S, n, k, out);
 }
 
-void launch_trunc_update_vw(cudaStream_t st, u64* V, u64* W, int k, const u64* coef) {
-  k_trunc_update_vw<<<128, 256, 0, st>>>(V, W, k, coef);
+void launch_update_vw(cudaStream_t st, u64* V, u64* W, int n, int k, const u64* coef) {
+  k_update_vw<<<2 * n, 256, 0, st>>>(V, W, n, k, coef);
 }
 
 }  // namespace mpc3

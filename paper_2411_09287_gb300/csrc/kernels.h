@@ -164,10 +164,12 @@ void launch_delta(cudaStream_t st, const u64* S, Key k01, Key k02, u64 obj, u64 
                   u64* rec, u64* out, u64* trace, u32* status, u32 flag);
 // The hash comparisons of n records: `flag` in *status on a mismatch.
 void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 flag);
-// Round k's sums S00, S01, S10, S11 (192 words apart, added into out) of the bit rounds.
-void launch_trunc_round_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int k,
-                             u64* out);
-void launch_trunc_update_vw(cudaStream_t st, u64* V, u64* W, int k, const u64* coef);
+// Round k's sums S00, S01, S10, S11 of np parties (party p at 64 p, the four 192 words apart; added
+// into out) of rounds over a matrix S[p][j][j'] of n x n GR elements with weights V_j, W_j.
+void launch_weighted_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int n, int k,
+                          int np, u64* out);
+// V_j, W_j (j < n) times 1 - f or f (coef) by bit k - 1 of j.
+void launch_update_vw(cudaStream_t st, u64* V, u64* W, int n, int k, const u64* coef);
 
 // ---- elementwise protocol kernels (prf_kernels.cu) ------------------------------------------
 void launch_share_input(cudaStream_t st, const u64* x, long long n, Key k01, Key k02, u64 obj,
@@ -223,16 +225,6 @@ void launch_gr_lincomb(cudaStream_t st, const u64* ca, const u64* a, const u64* 
 void launch_gr_mulmat2(cudaStream_t st, const u64* a, const u64* b, u64* M);
 void launch_gr_inverses(cudaStream_t st, u64* out);
 void launch_gr_fold_reduce(cudaStream_t st, const u64* P, int n, u64* out);
-void launch_gr_scale_rows(cudaStream_t st, const u64* pw, const u64* s, long long n, u64* out);
-void launch_gr_lift(cudaStream_t st, const u64* s, long long n, u64* out);
-// First-round party sums and folds of a claim whose y vectors are lifted ring words (one word per
-// element, components null when absent): S (12 x 64 words, accumulated) receives the party sums
-// of the even pairs at S[0..2], of the cross terms at S[3..5] and of the odd pairs at S[9..11];
-// out_i = lift(Y_{2i}) + f (Y_{2i+1} - Y_{2i}).  Words at or past D read as 0.
-void launch_gram_lifted(cudaStream_t st, const u64* const x[6], const u64* const y[6], long long Dh,
-                        long long D, u64* S);
-void launch_fold_lifted(cudaStream_t st, const u64* Y, long long Dh, long long D, const u64* f,
-                        u64* out);
 void launch_neg_copy(cudaStream_t st, const u64* a, long long n, u64* out);
 void launch_trunc_u(cudaStream_t st, const u64* r, int t, u64* u);
 // out[c] += sum_{e < n} A[c * lda + e] * R[e] (R: n GR elements), c < nrows <= 16, atomically
@@ -264,6 +256,38 @@ void launch_prf_words(cudaStream_t st, long long n, Key key, u32 tag, u64 obj, u
 // the same for a row-keyed truncation-bit stream: word e = word e mod N of object row_keys[e / N]
 void launch_prf_words_keyed(cudaStream_t st, long long n, Key key, u32 tag, const u64* row_keys,
                             long long N, u64* out, long long off);
+
+// ---- first rounds of a batch of weighted ring words (gr_block.cu) ----------------------------
+struct BlkIn {            // share components of x, y (words) and of the claim z (ldz words apart)
+  const u64* x[6];
+  const u64* y[6];
+  const u64* z;
+  long long ldz;
+  long long D;            // words of a component; words past D read as 0
+};
+struct BlkVec {
+  const u64* c[6];
+};
+struct BlkOut {
+  u64* c[6];
+};
+// Rows of launch_blk_sums: the parties' B x B sums, then (full) the claim's 6 x B.
+int blk_rows(int B, bool full);
+// out (blk_rows x 64 words, accumulated): S^p_{j,j'} and Z_{c,j} over the blocks b < nb of B words,
+// weight R[b >> sh].  full: every component and the claim; else x has components 2 and 4 only and
+// the rows are those of parties 1 and 2.
+void launch_blk_sums(cudaStream_t st, const BlkIn& in, int B, bool full, long long nb, int sh,
+                     const u64* R, u64* out);
+// out[c][j] (6 x 64 elements, accumulated) = sum over w < nw of R[w] z[c ldz + 64 w + j].
+void launch_words_sums(cudaStream_t st, const u64* z, long long ldz, long long nw, const u64* R,
+                       u64* out);
+// z_c += sum over j < n of T_j Zr[c n + j] (6 components).
+void launch_blk_claim(cudaStream_t st, const u64* T, const u64* Zr, int n, u64* z);
+// out_c[b] = sum over j < B of in_c[B b + j] G[row], row = (b >> sh) B + j (rows) or j, b < nb.
+void launch_blk_combine(cudaStream_t st, const BlkVec& in, const BlkOut& out, int B, bool rows,
+                        long long D, long long nb, int sh, const u64* G);
+// n rows holding the element 1
+void launch_ones(cudaStream_t st, int n, u64* out);
 
 // ---- trunc-batch S matrix on the tensor cores (trunc_s.cu) ----------------------------------
 void launch_trunc_limb_table(cudaStream_t st, const u64* Tlo, long long L, unsigned char* TL8);
@@ -303,14 +327,10 @@ void launch_b2a_apply(cudaStream_t st, const u64* dbits, const u64* ra, long lon
 void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int sub, u64* out);
 void launch_open_xor(cudaStream_t st, const u64* m, const u64* r1, const u64* r2_in, long long n,
                      u64* out);
-// First round of the edaBit inner-product batch from the bits (see nonlinear.cu): per-element
-// party-sum words (6 rows of ld words) and the x fold (A: r^g f per element g).
-void launch_eda_r1_sums(cudaStream_t st, const u64* mbits, const u64* rp, long long np, long long e0,
-                        long long ld, u64* out);
-void launch_eda_x_fold(cudaStream_t st, const u64* mbits, long long np, long long e0, const u64* pw,
-                       const u64* A, u64* x2, u64* x4);
-void launch_eda_tran(cudaStream_t st, const u64* mbits, const u64* rp, long long np, const u64* pw,
-                     long long e0, u64* x2, u64* x4, u64* const* y_dev);
+// The edaBit inner-product batch's ring words (see nonlinear.cu): bits m into xm, 2^(i+1) r' into y
+// (component c at c ldy), entry (e0 + e) 64 + i.
+void launch_eda_words(cudaStream_t st, const u64* mbits, const u64* rp, long long np, long long e0,
+                      long long ldy, u64* xm, u64* y);
 void launch_gf_powers(cudaStream_t st, const u64* r, long long n, u64* out);
 void launch_gf_tran(cudaStream_t st, const u64* X, const u64* Y, const u64* Z, long long nw,
                     const u64* pw, long long ld, u64* xo, u64* yo, u64* zsum);
