@@ -40,7 +40,8 @@ inline void counted(int k, F f, A... a) {
 #define launch_trunc_p0(...) counted(1, mpc3::launch_trunc_p0, __VA_ARGS__)
 #define launch_trunc_finish(...) counted(1, mpc3::launch_trunc_finish, __VA_ARGS__)
 #define launch_xor_one(...) counted(1, mpc3::launch_xor_one, __VA_ARGS__)
-#define launch_open_p1(...) counted(1, mpc3::launch_open_p1, __VA_ARGS__)
+#define launch_rec_messages(...) counted(1, mpc3::launch_rec_messages, __VA_ARGS__)
+#define launch_hash_jobs(...) counted(2, mpc3::launch_hash_jobs, __VA_ARGS__)
 #define launch_hash_u64(...) counted(2, mpc3::launch_hash_u64, __VA_ARGS__)
 #define launch_digest_check(...) counted(1, mpc3::launch_digest_check, __VA_ARGS__)
 #define launch_gr_random_shared(...) counted(1, mpc3::launch_gr_random_shared, __VA_ARGS__)
@@ -935,6 +936,38 @@ RecPlan plan_rec(Arena& a, long long n, bool need_out) {
   p.dg = a.take<u32>(48);
   p.out_dev = need_out ? a.take<u64>(n) : nullptr;
   return p;
+}
+
+// The armed REC_MSG fault of a Pi_Rec of n words, disarmed: its word index (-1: none) and mask.
+long long take_rec_fault(mpc_ctx* ctx, long long n, u64* mask) {
+  Fault& f = ctx->fault[MPC_SITE_REC_MSG];
+  if (!f.armed) return -1;
+  f.armed = false;
+  *mask = f.mask;
+  return (long long)(f.index % (u64)n);
+}
+
+// Pi_Rec of n words up to the hash comparison (into the status word): P0 sends [r]_1 to P2 and
+// [r]_2 to P1 (fault site REC_MSG, arithmetic sharings), P1 sends m to P0; P1 sends H([r]_1) to P2,
+// P2 H(m) to P0 and H([r]_2) to P1, and every receiver hashes what it received.  out = P1's opening.
+void rec_core(mpc_ctx* ctx, const u64* xs, long long n, const RecPlan& p, u64* out, bool boolean) {
+  cudaStream_t st = ctx->st;
+  const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_REC;
+  u64 xmask = 0;
+  const long long xidx = boolean ? -1 : take_rec_fault(ctx, n, &xmask);
+  count_msgs(ctx, ph, pr, 3, (u64)n * 8);
+  launch_rec_messages(st, xs, n, xidx, xmask, boolean, p.in_p2_r1, p.in_p1_r2, p.in_p0_m, out);
+  HashJobs j;
+  const u64* data[6] = {xs + 3 * n, xs + 4 * n, xs + 5 * n, p.in_p2_r1, p.in_p0_m, p.in_p1_r2};
+  for (int q = 0; q < 6; ++q) {
+    j.data[q] = data[q];
+    j.scratch[q] = p.hs[q];
+    j.digest[q] = p.dg + 8 * q;
+  }
+  launch_hash_jobs(st, j, 6, n);
+  count_msgs(ctx, ph, pr, 3, 32);
+  u32* d = p.dg;
+  launch_digest_check(st, d, d + 24, d + 8, d + 32, d + 16, d + 40, ctx->status, ST_ABORT);
 }
 
 // A table of powers r^i, i < n (rows of 64 words): rows below L by repeated multiplication, row
@@ -2319,21 +2352,8 @@ int mpc_reconstruct(mpc_ctx* ctx, const uint64_t* xs, int64_t n, uint64_t* out, 
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "reconstruct: workspace too small");
   Phase* phase = new Phase(ctx, MPC_PROF_REC);
   cudaStream_t st = ctx->st;
-  const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_REC;
-  if ((rc = deliver(ctx, ph, pr, xs, p.in_p2_r1, n, -1))) return rc;             // P0 -> P2 [r]_1
-  if ((rc = deliver(ctx, ph, pr, xs + n, p.in_p1_r2, n, MPC_SITE_REC_MSG))) return rc;  // P0 -> P1
-  if ((rc = deliver(ctx, ph, pr, xs + 2 * n, p.in_p0_m, n, -1))) return rc;      // P1 -> P0 m
-  u32* d = p.dg;
-  launch_hash_u64(st, xs + 3 * n, n, p.hs[0], d + 0);     // P1: H([r]_1) -> P2
-  launch_hash_u64(st, xs + 4 * n, n, p.hs[1], d + 8);     // P2: H(m) -> P0
-  launch_hash_u64(st, xs + 5 * n, n, p.hs[2], d + 16);    // P2: H([r]_2) -> P1
-  count_msgs(ctx, ph, pr, 3, 32);
-  launch_hash_u64(st, p.in_p2_r1, n, p.hs[3], d + 24);    // P2 hashes received [r]_1
-  launch_hash_u64(st, p.in_p0_m, n, p.hs[4], d + 32);     // P0 hashes received m
-  launch_hash_u64(st, p.in_p1_r2, n, p.hs[5], d + 40);    // P1 hashes received [r]_2
-  launch_digest_check(st, d + 0, d + 24, d + 8, d + 32, d + 16, d + 40, ctx->status, ST_ABORT);
   u64* o = out_on_host ? p.out_dev : (u64*)out;
-  launch_open_p1(st, xs + 2 * n, xs + 3 * n, p.in_p1_r2, n, o);
+  rec_core(ctx, xs, n, p, o, false);
   if (out_on_host) CK(cudaMemcpyAsync(out, o, (size_t)n * 8, cudaMemcpyDeviceToHost, st));
   delete phase;
   if ((rc = cuda_check(ctx, "reconstruct"))) return rc;
@@ -2519,11 +2539,16 @@ int mpc_trunc(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, int64_t n, int
     const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_TRUNC;
     if ((rc = deliver(ctx, ph, pr, p.d1, p.d1_at_p2, n, MPC_SITE_TRUNC_D1))) return rc;   // P1->P2
     if ((rc = deliver(ctx, ph, pr, p.d2, p.d2_at_p1, n, -1))) return rc;                 // P2->P1
-    launch_hash_u64(st, p.d1p0, n, p.hs[0], p.dg);            // P0: H(d1) -> P2
-    launch_hash_u64(st, p.d2p0, n, p.hs[1], p.dg + 8);        // P0: H(d2) -> P1
+    // P0 sends H(d1) to P2 and H(d2) to P1, who hash the d1, d2 they received
+    const u64* data[4] = {p.d1p0, p.d2p0, p.d1_at_p2, p.d2_at_p1};
+    HashJobs hj{};
+    for (int q = 0; q < 4; ++q) {
+      hj.data[q] = data[q];
+      hj.scratch[q] = p.hs[q];
+      hj.digest[q] = p.dg + 8 * q;
+    }
+    launch_hash_jobs(st, hj, 4, n);
     count_msgs(ctx, ph, pr, 2, 32);
-    launch_hash_u64(st, p.d1_at_p2, n, p.hs[2], p.dg + 16);   // P2 hashes the d1 it received
-    launch_hash_u64(st, p.d2_at_p1, n, p.hs[3], p.dg + 24);   // P1 hashes the d2 it received
     launch_digest_check(st, p.dg, p.dg + 16, p.dg + 8, p.dg + 24, p.dg, p.dg + 16, ctx->status,
                         ST_ABORT);
     launch_trunc_online(st, xs, n, p.d1, p.d2_at_p1, p.d1_at_p2, p.d2, t, out);
@@ -2577,9 +2602,8 @@ namespace mpc3 {
 namespace internal {
 int ctx_guard(mpc_ctx* c) { return guard(c); }
 int ctx_fail(mpc_ctx* c, int code, const char* msg) { return fail(c, code, msg); }
-int ctx_deliver(mpc_ctx* c, int phase, int proto, const u64* src, u64* dst, long long n, int site) {
-  return deliver(c, phase, proto, src, dst, n, site);
-}
+// The armed REC_MSG fault of a Pi_Rec of n words, disarmed: its word index (-1: none) and mask.
+long long ctx_take_rec_fault(mpc_ctx* c, long long n, u64* mask) { return take_rec_fault(c, n, mask); }
 void ctx_count(mpc_ctx* c, int phase, int proto, int count, u64 bytes_each) {
   count_msgs(c, phase, proto, count, bytes_each);
 }
@@ -2652,33 +2676,6 @@ int and_p(mpc_ctx* ctx, const u64* xs, const u64* ys, long long nw, u32 purpose,
   if ((rc = deliver_bits(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, m.p2o, m.p1i, nw, -1))) return rc;
   launch_xor_finish(ctx->st, nw, m.p1o, m.p1i, m.p2o, m.p2i, zs);
   g_launches += 1;
-  return MPC_OK;
-}
-
-// Pi_Rec of n words inside a layer (messages, hashes, consistency check into the status word);
-// P1's opening into out: m - [r]_1 - [r]_2, or m XOR [r]_1 XOR [r]_2 for a Boolean sharing.
-int rec_open(mpc_ctx* ctx, const u64* xs, long long n, const RecPlan& p, u64* out, bool boolean) {
-  int rc;
-  cudaStream_t st = ctx->st;
-  const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_REC;
-  if ((rc = deliver(ctx, ph, pr, xs, p.in_p2_r1, n, -1))) return rc;
-  if ((rc = deliver(ctx, ph, pr, xs + n, p.in_p1_r2, n, boolean ? -1 : MPC_SITE_REC_MSG))) return rc;
-  if ((rc = deliver(ctx, ph, pr, xs + 2 * n, p.in_p0_m, n, -1))) return rc;
-  u32* d = p.dg;
-  launch_hash_u64(st, xs + 3 * n, n, p.hs[0], d + 0);
-  launch_hash_u64(st, xs + 4 * n, n, p.hs[1], d + 8);
-  launch_hash_u64(st, xs + 5 * n, n, p.hs[2], d + 16);
-  count_msgs(ctx, ph, pr, 3, 32);
-  launch_hash_u64(st, p.in_p2_r1, n, p.hs[3], d + 24);
-  launch_hash_u64(st, p.in_p0_m, n, p.hs[4], d + 32);
-  launch_hash_u64(st, p.in_p1_r2, n, p.hs[5], d + 40);
-  launch_digest_check(st, d + 0, d + 24, d + 8, d + 32, d + 16, d + 40, ctx->status, ST_ABORT);
-  if (boolean) {
-    launch_open_xor(st, xs + 2 * n, xs + 3 * n, p.in_p1_r2, n, out);
-    g_launches += 1;
-  } else {
-    launch_open_p1(st, xs + 2 * n, xs + 3 * n, p.in_p1_r2, n, out);
-  }
   return MPC_OK;
 }
 
@@ -2776,7 +2773,7 @@ int compare_select(mpc_ctx* ctx, u64 call_id, int stage, const u64* a, const u64
   // msb(d): open Delta = d - r, carry circuit over the bits of Delta + r
   launch_addsub(st, 6 * np, p.d, p.ra, 1, p.dd);
   g_launches += 1;
-  if ((rc = rec_open(ctx, p.dd, np, p.reca, p.delta, false))) return rc;
+  rec_core(ctx, p.dd, np, p.reca, p.delta, false);
   launch_trunc_bit_transpose(st, p.delta, np, p.dpl);
   launch_msb_leaves(st, p.rbits, p.dpl, W, p.G, p.P);
   g_launches += 2;
@@ -2812,7 +2809,7 @@ int compare_select(mpc_ctx* ctx, u64 call_id, int stage, const u64* a, const u64
   launch_lin_apb_m2c(st, 6 * np, p.rpd, p.A3, p.u, p.rad);
   launch_bxor(st, 6 * W, p.ge, p.rb, p.e);
   g_launches += 2;
-  if ((rc = rec_open(ctx, p.e, W, p.recb, p.dbits, true))) return rc;
+  rec_core(ctx, p.e, W, p.recb, p.dbits, true);
   launch_b2a_apply(st, p.dbits, p.rad, np, p.gea);
   g_launches += 1;
   // out = b + (a - b) [a >= b]

@@ -198,31 +198,31 @@ __device__ inline void sha256_init(u32 h[8]) {
   h[4] = 0x510e527fu; h[5] = 0x9b05688cu; h[6] = 0x1f83d9abu; h[7] = 0x5be0cd19u;
 }
 
-// Compress one 64-byte block given as 16 big-endian words.
+// Compress one 64-byte block given as 16 big-endian words.  Four passes over a body of 16 rounds
+// (about 6 KB of code): all 64 rounds unrolled are 25 KB per inlined copy, and a warp that runs
+// alone then waits for instructions (78 cycles a round against 36).
 __device__ inline void sha256_compress(u32 h[8], const u32 wblk[16]) {
   u32 w[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) w[i] = wblk[i];
   u32 a = h[0], b = h[1], c = h[2], d = h[3], e = h[4], f = h[5], g = h[6], hh = h[7];
+#pragma unroll 1
+  for (int r = 0; r < 64; r += 16) {
 #pragma unroll
-  for (int t = 0; t < 64; ++t) {
-    u32 wt;
-    if (t < 16) {
-      wt = w[t];
-    } else {
-      const u32 w15 = w[(t - 15) & 15], w2 = w[(t - 2) & 15];
-      const u32 s0 = rotr32(w15, 7) ^ rotr32(w15, 18) ^ (w15 >> 3);
-      const u32 s1 = rotr32(w2, 17) ^ rotr32(w2, 19) ^ (w2 >> 10);
-      wt = w[t & 15] + s0 + w[(t - 7) & 15] + s1;
-      w[t & 15] = wt;
+    for (int t = 0; t < 16; ++t) {
+      const u32 S1 = rotr32(e, 6) ^ rotr32(e, 11) ^ rotr32(e, 25);
+      const u32 ch = (e & f) ^ (~e & g);
+      const u32 t1 = (hh + SHA_K[r + t] + w[t]) + S1 + ch;
+      const u32 S0 = rotr32(a, 2) ^ rotr32(a, 13) ^ rotr32(a, 22);
+      const u32 mj = (a & b) ^ (a & c) ^ (b & c);
+      const u32 t2 = S0 + mj;
+      hh = g; g = f; f = e; e = d + t1; d = c; c = b; b = a; a = t1 + t2;
+      // w[t] becomes the word of round r + 16 + t, from those of the rounds r + t + 1, + 9, + 14
+      // (at indices that have wrapped, already the next pass's)
+      const u32 w15 = w[(t + 1) & 15], w2 = w[(t + 14) & 15];
+      w[t] += (rotr32(w15, 7) ^ rotr32(w15, 18) ^ (w15 >> 3)) + w[(t + 9) & 15] +
+              (rotr32(w2, 17) ^ rotr32(w2, 19) ^ (w2 >> 10));
     }
-    const u32 S1 = rotr32(e, 6) ^ rotr32(e, 11) ^ rotr32(e, 25);
-    const u32 ch = (e & f) ^ (~e & g);
-    const u32 t1 = hh + S1 + ch + SHA_K[t] + wt;
-    const u32 S0 = rotr32(a, 2) ^ rotr32(a, 13) ^ rotr32(a, 22);
-    const u32 mj = (a & b) ^ (a & c) ^ (b & c);
-    const u32 t2 = S0 + mj;
-    hh = g; g = f; f = e; e = d + t1; d = c; c = b; b = a; a = t1 + t2;
   }
   h[0] += a; h[1] += b; h[2] += c; h[3] += d; h[4] += e; h[5] += f; h[6] += g; h[7] += hh;
 }

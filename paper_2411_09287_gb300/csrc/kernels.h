@@ -195,8 +195,11 @@ void launch_trunc_finish(cudaStream_t st, long long E, Key k01, Key k02, u64 obj
                          const u64* p1_mp1, const u64* p1_mq1, u64* zpre, u64* zout, u64* pq,
                          const u64* row_keys, long long N);
 void launch_xor_one(cudaStream_t st, u64* p, u64 mask);
-void launch_open_p1(cudaStream_t st, const u64* p1_m, const u64* p1_r1, const u64* p1_in_r2,
-                    long long n, u64* out);
+// The messages of Pi_Rec of a sharing xs and P1's opening: in_p2_r1 = P0.[r]_1, in_p1_r2 = P0.[r]_2
+// (word xidx XORed with xmask when xidx >= 0), in_p0_m = P1.m, out = P1.m - P1.[r]_1 - in_p1_r2 (XOR
+// for a Boolean sharing).
+void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask,
+                         bool boolean, u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out);
 
 // ---- SHA-256 Merkle hash (sha_kernels.cu) ---------------------------------------------------
 // Merkle hash of Pi_Rec: 1024-byte leaves, subtree roots of 64 aligned leaves per CTA.
@@ -209,6 +212,14 @@ constexpr long long hash_scratch_words_for(long long n) {
                HASH_CTA_LEAVES - 1) /
          HASH_CTA_LEAVES;
 }
+// The digests of njobs arrays of n words each: one launch over all leaves, one for the trees (a
+// Pi_Rec hashes six arrays, which as launches of their own ran one after another).
+struct HashJobs {
+  const u64* data[6];
+  u32* scratch[6];   // hash_scratch_words(n) 32-bit words each
+  u32* digest[6];    // 8 words each
+};
+void launch_hash_jobs(cudaStream_t st, const HashJobs& jobs, int njobs, long long n);
 // digest (8 words) of the n-word array; scratch needs hash_scratch_words(n) 32-bit words.
 void launch_hash_u64(cudaStream_t st, const u64* data, long long n, u32* scratch, u32* digest);
 void launch_digest_check(cudaStream_t st, const u32* a0, const u32* b0, const u32* a1,
@@ -325,8 +336,6 @@ void launch_msb_out(cudaStream_t st, const u64* rbits, const u64* Groot, const u
 void launch_bxor(cudaStream_t st, long long n6, const u64* a, const u64* b, u64* out);
 void launch_b2a_apply(cudaStream_t st, const u64* dbits, const u64* ra, long long n, u64* out);
 void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int sub, u64* out);
-void launch_open_xor(cudaStream_t st, const u64* m, const u64* r1, const u64* r2_in, long long n,
-                     u64* out);
 // The edaBit inner-product batch's ring words (see nonlinear.cu): bits m into xm, 2^(i+1) r' into y
 // (component c at c ldy), entry (e0 + e) 64 + i.
 void launch_eda_words(cudaStream_t st, const u64* mbits, const u64* rp, long long np, long long e0,

@@ -26,9 +26,9 @@ namespace mpc3 {
 namespace internal {
 int ctx_guard(mpc_ctx* c);
 int ctx_fail(mpc_ctx* c, int code, const char* msg);
-int ctx_deliver(mpc_ctx* c, int phase, int proto, const u64* src, u64* dst, long long n, int site);
 void ctx_count(mpc_ctx* c, int phase, int proto, int count, u64 bytes_each);
 int ctx_read_status(mpc_ctx* c, u32* out);
+long long ctx_take_rec_fault(mpc_ctx* c, long long n, u64* mask);
 bool ctx_has_pending(const mpc_ctx* c);
 cudaStream_t ctx_stream(const mpc_ctx* c);
 u32* ctx_status_word(const mpc_ctx* c);
@@ -93,19 +93,21 @@ extern "C" int mpc_reconstruct_noalloc(mpc_ctx* ctx, const uint64_t* xs, int64_t
   if ((rc = scratch_for_current_device(ctx, &s))) return rc;
   cudaStream_t st = ctx_stream(ctx);
   const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_REC;
-  if ((rc = ctx_deliver(ctx, ph, pr, xs, s->in_p2_r1, n, -1))) return rc;                // P0 -> P2
-  if ((rc = ctx_deliver(ctx, ph, pr, xs + n, s->in_p1_r2, n, MPC_SITE_REC_MSG))) return rc;  // P0 -> P1
-  if ((rc = ctx_deliver(ctx, ph, pr, xs + 2 * n, s->in_p0_m, n, -1))) return rc;         // P1 -> P0
-  u32* d = s->dg;
-  launch_hash_u64(st, xs + 3 * n, n, s->hs[0], d + 0);     // P1: H([r]_1) -> P2
-  launch_hash_u64(st, xs + 4 * n, n, s->hs[1], d + 8);     // P2: H(m) -> P0
-  launch_hash_u64(st, xs + 5 * n, n, s->hs[2], d + 16);    // P2: H([r]_2) -> P1
+  u64 xmask = 0;
+  const long long xidx = ctx_take_rec_fault(ctx, n, &xmask);
+  ctx_count(ctx, ph, pr, 3, (u64)n * 8);
+  launch_rec_messages(st, xs, n, xidx, xmask, false, s->in_p2_r1, s->in_p1_r2, s->in_p0_m, out);
+  HashJobs j;   // sent by P1, P2, P2; of what P2, P0, P1 received
+  const u64* data[6] = {xs + 3 * n, xs + 4 * n, xs + 5 * n, s->in_p2_r1, s->in_p0_m, s->in_p1_r2};
+  for (int q = 0; q < 6; ++q) {
+    j.data[q] = data[q];
+    j.scratch[q] = s->hs[q];
+    j.digest[q] = s->dg + 8 * q;
+  }
+  launch_hash_jobs(st, j, 6, n);
   ctx_count(ctx, ph, pr, 3, 32);
-  launch_hash_u64(st, s->in_p2_r1, n, s->hs[3], d + 24);   // P2 hashes the [r]_1 it received
-  launch_hash_u64(st, s->in_p0_m, n, s->hs[4], d + 32);    // P0 hashes the m it received
-  launch_hash_u64(st, s->in_p1_r2, n, s->hs[5], d + 40);   // P1 hashes the [r]_2 it received
-  launch_digest_check(st, d + 0, d + 24, d + 8, d + 32, d + 16, d + 40, ctx_status_word(ctx), 1u);
-  launch_open_p1(st, xs + 2 * n, xs + 3 * n, s->in_p1_r2, n, out);
+  u32* d = s->dg;
+  launch_digest_check(st, d, d + 24, d + 8, d + 32, d + 16, d + 40, ctx_status_word(ctx), 1u);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return ctx_fail(ctx, MPC_ERR_CUDA, cudaGetErrorString(e));
   u32 stv = 0;

@@ -510,12 +510,6 @@ __global__ void k_addsub(long long n, const u64* __restrict__ a, const u64* __re
   GRID_STRIDE(i, n) { out[i] = sub ? a[i] - b[i] : a[i] + b[i]; }
 }
 
-// P1's opening of a Boolean sharing: m XOR [r]_1 XOR [r]_2 (received)
-__global__ void k_open_xor(const u64* __restrict__ m, const u64* __restrict__ r1,
-                           const u64* __restrict__ r2_in, long long n, u64* __restrict__ out) {
-  GRID_STRIDE(i, n) { out[i] = m[i] ^ r1[i] ^ r2_in[i]; }
-}
-
 // Pi_Tran of the edaBit inner products (rows e of dimension 64, weight r^(e0 + e) on row e) as ring
 // words: entry (e0 + e) 64 + i of xm is the bit m_i of element e (components 2 and 4 of <m_i>,
 // which has no mask), of component c of y 2^(i+1) <r'_i>.  The sources are plane-major: a 64 x 32
@@ -696,11 +690,6 @@ void launch_gf_check_zero(cudaStream_t st, const u64* d, u32* status, u32 flag) 
 void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int sub, u64* out) {
   if (n <= 0) return;
   k_addsub<<<grid_for(n), TPB, 0, st>>>(n, a, b, sub, out);
-}
-void launch_open_xor(cudaStream_t st, const u64* m, const u64* r1, const u64* r2_in, long long n,
-                     u64* out) {
-  if (n <= 0) return;
-  k_open_xor<<<grid_for(n), TPB, 0, st>>>(m, r1, r2_in, n, out);
 }
 void launch_eda_words(cudaStream_t st, const u64* mbits, const u64* rp, long long np, long long e0,
                       long long ldy, u64* xm, u64* y) {

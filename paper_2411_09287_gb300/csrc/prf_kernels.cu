@@ -389,12 +389,19 @@ __global__ void k_prf_words(long long n, long long off, Key key, u32 tag, u64 ob
   }
 }
 
-// x = m - [r]_1 - [r]_2 from P1's view (own m, own [r]_1, received [r]_2).
-__global__ void k_open_p1(const u64* __restrict__ m, const u64* __restrict__ r1,
-                          const u64* __restrict__ r2, long long n, u64* __restrict__ out) {
+// The three messages of Pi_Rec and P1's opening in one pass (the hashes read the copies).
+__global__ void k_rec_messages(const u64* __restrict__ xs, long long n, long long xidx, u64 xmask,
+                               int boolean, u64* __restrict__ in_p2_r1, u64* __restrict__ in_p1_r2,
+                               u64* __restrict__ in_p0_m, u64* __restrict__ out) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    out[i] = m[i] - r1[i] - r2[i];
+       i += (long long)gridDim.x * blockDim.x) {
+    in_p2_r1[i] = xs[i];
+    const u64 r2 = xs[n + i] ^ (i == xidx ? xmask : 0ull);
+    in_p1_r2[i] = r2;
+    const u64 m = xs[2 * n + i], r1 = xs[3 * n + i];
+    in_p0_m[i] = m;
+    out[i] = boolean ? m ^ r1 ^ r2 : m - r1 - r2;
+  }
 }
 
 }  // namespace
@@ -485,10 +492,11 @@ void launch_prf_words(cudaStream_t st, long long n, Key key, u32 tag, u64 obj, u
   k_prf_words<<<grid_for((off + n + 7) / 8 - off / 8), TPB, 0, st>>>(n, off, key, tag, obj, out);
 }
 
-void launch_open_p1(cudaStream_t st, const u64* m, const u64* r1, const u64* r2, long long n,
-                    u64* out) {
+void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask,
+                         bool boolean, u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out) {
   if (n <= 0) return;
-  k_open_p1<<<grid_for(n), TPB, 0, st>>>(m, r1, r2, n, out);
+  k_rec_messages<<<grid_for(n), TPB, 0, st>>>(xs, n, xidx, xmask, boolean ? 1 : 0, in_p2_r1,
+                                              in_p1_r2, in_p0_m, out);
 }
 
 }  // namespace mpc3

@@ -31,9 +31,11 @@ __device__ __forceinline__ void node_hash(const u32* l, const u32* r, u32 h[8]) 
   sha256_compress(h, blk);
 }
 
+// blockIdx.y picks the array; with one CTA per array its root is the digest itself.
 __global__ void __launch_bounds__(HB)
-k_hash_leaves(const u64* __restrict__ data, long long n, long long nleaves,
-              u32* __restrict__ out) {
+k_hash_leaves(const HashJobs jobs, long long n, long long nleaves) {
+  const u64* __restrict__ data = jobs.data[blockIdx.y];
+  u32* __restrict__ out = gridDim.x == 1 ? jobs.digest[blockIdx.y] : jobs.scratch[blockIdx.y];
   __shared__ u32 dg[HB][8];
   const long long leaf = blockIdx.x * (long long)HB + threadIdx.x;
   if (leaf < nleaves) {
@@ -114,10 +116,12 @@ k_hash_leaves(const u64* __restrict__ data, long long n, long long nleaves,
   if (threadIdx.x < 8) out[blockIdx.x * 8 + threadIdx.x] = dg[0][threadIdx.x];
 }
 
-// One CTA: levels of the Merkle tree over `cnt` digests in buf (ping-pong with buf2).
-__global__ void k_hash_tree(u32* buf, u32* buf2, long long cnt, u32* digest) {
-  u32* cur = buf;
-  u32* nxt = buf2;
+// One CTA an array: levels of the Merkle tree over its `cnt` subtree roots (ping-pong between the
+// halves of its scratch).
+__global__ void k_hash_tree(const HashJobs jobs, long long cnt) {
+  u32* cur = jobs.scratch[blockIdx.x];
+  u32* nxt = cur + 8 * cnt;
+  u32* digest = jobs.digest[blockIdx.x];
   while (cnt > 1) {
     const long long half = cnt / 2;
     for (long long p = threadIdx.x; p < half; p += blockDim.x) {
@@ -153,12 +157,20 @@ __global__ void k_digest_check(const u32* a0, const u32* b0, const u32* a1, cons
 
 size_t hash_scratch_words(long long n) { return (size_t)hash_scratch_words_for(n); }
 
-void launch_hash_u64(cudaStream_t st, const u64* data, long long n, u32* scratch, u32* digest) {
+void launch_hash_jobs(cudaStream_t st, const HashJobs& jobs, int njobs, long long n) {
   long long leaves = (8 * n + LEAF_BYTES - 1) / LEAF_BYTES;
   if (leaves < 1) leaves = 1;
   const long long nb = (leaves + HB - 1) / HB;   // subtree roots, one per CTA
-  k_hash_leaves<<<(unsigned)nb, HB, 0, st>>>(data, n, leaves, scratch);
-  k_hash_tree<<<1, 256, 0, st>>>(scratch, scratch + 8 * nb, nb, digest);
+  k_hash_leaves<<<dim3((unsigned)nb, (unsigned)njobs), HB, 0, st>>>(jobs, n, leaves);
+  if (nb > 1) k_hash_tree<<<njobs, 256, 0, st>>>(jobs, nb);
+}
+
+void launch_hash_u64(cudaStream_t st, const u64* data, long long n, u32* scratch, u32* digest) {
+  HashJobs j{};
+  j.data[0] = data;
+  j.scratch[0] = scratch;
+  j.digest[0] = digest;
+  launch_hash_jobs(st, j, 1, n);
 }
 
 void launch_digest_check(cudaStream_t st, const u32* a0, const u32* b0, const u32* a1,
