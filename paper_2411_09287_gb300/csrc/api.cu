@@ -1283,7 +1283,7 @@ TruncPlan plan_trunc(Arena& a, long long E, int R1, bool tc, bool chunked, const
   p.b1 = a.take<u64>(p.Epad);
   p.b2 = a.take<u64>(p.Epad);
   p.Rtab = a.take<u64>((p.compact ? p.L : p.Epad) * 64);
-  p.TL8 = a.take<unsigned char>(1024 * p.L);
+  p.TL8 = a.take<unsigned char>(64ll * TRUNC_LIMBS * p.L);
   p.B1T = a.take<u64>(p.Epad);
   p.B2T = a.take<u64>(p.Epad);
   p.S_hi = a.take<u64>(p.nhi * 4096 * 64);

@@ -301,6 +301,7 @@ void launch_blk_combine(cudaStream_t st, const BlkVec& in, const BlkOut& out, in
 void launch_ones(cudaStream_t st, int n, u64* out);
 
 // ---- trunc-batch S matrix on the tensor cores (trunc_s.cu) ----------------------------------
+constexpr int TRUNC_LIMBS = 13;   // e4m3 limbs of a u64
 void launch_trunc_limb_table(cudaStream_t st, const u64* Tlo, long long L, unsigned char* TL8);
 // BT[j][w] = bit j of words[64 w + i] at bit i, for w < Epad / 64
 void launch_trunc_bit_transpose(cudaStream_t st, const u64* words, long long Epad, u64* BT);

@@ -7,22 +7,29 @@
 // S is computed once per layer.  Writing r^(2e) = T_hi[e_hi] T_lo[e_lo] with e = e_hi L + e_lo:
 //   S_hi[e_hi][(j,j')] = sum_{e_lo} T_lo[e_lo] b1_{e,j} b2_{e,j'}     (this file, tensor cores)
 //   S[(j,j')]          = sum_{e_hi} T_hi[e_hi] (x) S_hi[e_hi][(j,j')]  (a u64 GEMM + fold)
-// Exactness: each u64 coefficient of T_lo is split into 16 unsigned 4-bit limbs; every limb value
-// 0..15 and every bit 0/1 is exact in e4m3, and an accumulator sums at most L <= 2^16 terms of at
-// most 15, so every f32 partial sum is an exact integer below 2^20; the limbs are recombined
-// mod 2^64 when the e_lo loop ends.
+// Exactness: each u64 coefficient v of T_lo is written as v = sum_l d_l 32^l mod 2^64 with 13 limbs,
+// -16 <= d_l <= 15 (d_12 the top four bits); e4m3 has four significant bits, so every integer from
+// -16 to 16 is exact in it, as are the bits, and an accumulator sums at most L <= 2^16 terms, so
+// every f32 partial sum is an exact integer of at most 2^20; the limbs are recombined mod 2^64 when
+// the e_lo loop ends.  13 limbs are the fewest that e4m3
+// allows, and the MMAs and the table grow with their number.
 //
 // Operands, both K-major (K = e):
 //   A (M = 128 pairs per accumulator): byte (p, e) = e4m3(b1_{e,j} AND b2_{e,j'}), generated in
 //     shared memory by four warps from bit-transposed words BT[j][e / 64] (bit e % 64);
-//   B (N = 256 limb columns): TL8[c][e_lo] = e4m3(limb c % 16 of coefficient c / 16 of T_lo[e_lo]),
+//   B (N = 208 limb columns): TL8[c][e_lo] = e4m3(limb c % 13 of coefficient c / 13 of T_lo[e_lo]),
 //     loaded by TMA (128-byte swizzle).
-// CTA = 256 pairs (j = 4 blockIdx.x .. +3, all j') x 256 limb columns (16 coefficients) x one e_hi
-// block; two accumulators (pairs 0..127 and 128..255 of the tile) fill the 512 TMEM columns.
+// CTA = 256 pairs (j = 4 blockIdx.x .. +3, all j') x 208 limb columns (16 coefficients) x one e_hi
+// block; two accumulators (pairs 0..127 and 128..255 of the tile) take 208 of 256 TMEM columns each.
 // Warps 0-3 generate A and drain TMEM at the end, warp 4 issues the TMA loads, warp 5 the MMAs;
-// a 3-stage ring of 64 KB (two A tiles + one B tile per stage) keeps the three roles apart.
+// a 3-stage ring of 58 KB (two A tiles + one B tile per stage) keeps the three roles apart.
 // Every mbarrier wait is bounded; a failure sets err_flag in *err and the CTA lets its copies and
 // MMAs finish (bounded), frees its tensor memory and returns without writing.
+#include <cstring>
+
+#include <cuda_fp16.h>
+#include <cuda_fp8.h>
+
 #include "kernels.h"
 #include "tcgen05.cuh"
 
@@ -32,17 +39,19 @@ namespace {
 
 using namespace tc;
 
+constexpr int S_LIMBS = TRUNC_LIMBS;
 constexpr int S_KC = 128;                  // e per chunk (one 128-byte swizzled row)
 constexpr int S_TPAIRS = 256;              // pairs per CTA (two accumulators of 128)
-constexpr int S_TCOLS = 256;               // limb columns per CTA (16 coefficients x 16 limbs)
+constexpr int S_TCOLS = 16 * S_LIMBS;      // limb columns per CTA (16 coefficients)
 constexpr int S_ATILE = 128 * S_KC;        // 16 KB
-constexpr int S_BTILE = S_TCOLS * S_KC;    // 32 KB
+constexpr int S_BTILE = S_TCOLS * S_KC;    // 26 KB
+static_assert(S_BTILE % 1024 == 0 && S_TCOLS % 16 == 0 && S_TCOLS <= 256, "swizzle atoms, MMA N");
 constexpr int S_STAGE = 2 * S_ATILE + S_BTILE;
 constexpr int S_NST = 3;
 constexpr int S_THREADS = 6 * 32;
 constexpr size_t S_SMEM = (size_t)S_NST * S_STAGE + 1024;
 
-// kind::f8f6f4: f32 accumulator, e4m3 A and B (format 0), both K-major, M = 128, N = 256
+// kind::f8f6f4: f32 accumulator, e4m3 A and B (format 0), both K-major, M = 128, N = 208
 constexpr unsigned S_IDESC = (1u << 4) | ((unsigned)(S_TCOLS >> 3) << 17) | ((unsigned)(128 >> 4) << 24);
 
 template <int ACC>
@@ -58,45 +67,83 @@ __device__ __forceinline__ unsigned nibble_bytes(unsigned nib) {
   return ((nib * 0x00204081u) & 0x01010101u) * 0x38u;
 }
 
-// e4m3 encodings of the integers 0..15
-__device__ __constant__ unsigned char E4M3_INT[16] = {0x00, 0x38, 0x40, 0x44, 0x48, 0x4A, 0x4C, 0x4E,
-                                                      0x50, 0x51, 0x52, 0x53, 0x54, 0x55, 0x56, 0x57};
-
-// TL8[c * L + e] = e4m3(limb c % 16 of coefficient c / 16 of T_lo[e]), c < 1024, e < L.
-// Each thread produces 16 consecutive e of one column (one 16-byte store).
-__global__ void k_limb_table(const u64* __restrict__ Tlo, long long L, unsigned char* __restrict__ TL8) {
-  const long long chunks = L / 16;
-  const long long total = 1024 * chunks;
-  for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < total;
-       w += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(w / chunks);
-    const long long e0 = (w % chunks) * 16;
-    const int coeff = c >> 4, limb = c & 15;
-    unsigned v[4] = {0, 0, 0, 0};
+// TL8[c * L + e] = e4m3(limb c % 13 of coefficient c / 13 of T_lo[e]), e < L.  A block takes 64 e:
+// their words go through shared memory, thread (coefficient, 16 e) then writes 16 bytes of each of
+// its coefficient's 13 rows.  Adding sum_{l < 12} 16 * 32^l makes the limbs plain 5-bit fields less
+// 16; a field n becomes the f16 1024 + n by its bits, and two of them an e4m3 pair by one conversion.
+// Bound by the writes.  (Each thread gathering its 16 words with a stride of 512 bytes and a table in
+// constant memory, indexed per thread: 231 us for L = 2^16, now 33-43 us.)
+__global__ void __launch_bounds__(256)
+k_limb_table(const u64* __restrict__ Tlo, long long L, unsigned char* __restrict__ TL8) {
+  __shared__ u64 tile[64][65];
+  const long long e0 = (long long)blockIdx.x * 64;   // L is a multiple of 64
+  for (int i = threadIdx.x; i < 4096; i += 256) tile[i >> 6][i & 63] = Tlo[e0 * 64 + i];
+  __syncthreads();
+  const int coeff = threadIdx.x & 63, eq = (threadIdx.x >> 6) * 16;
+  u64 bias = 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const unsigned nib = (unsigned)((Tlo[(e0 + i) * 64 + coeff] >> (4 * limb)) & 15ull);
-      v[i >> 2] |= (unsigned)E4M3_INT[nib] << (8 * (i & 3));
+  for (int l = 0; l < S_LIMBS - 1; ++l) bias += 16ull << (5 * l);
+  u64 v[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = tile[eq + i][coeff] + bias;
+  unsigned char* out = TL8 + (long long)coeff * S_LIMBS * L + e0 + eq;
+#pragma unroll
+  for (int l = 0; l < S_LIMBS; ++l) {
+    const __half2 off = __float2half2_rn(l < S_LIMBS - 1 ? 1040.0f : 1024.0f);
+    unsigned o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const unsigned n = ((unsigned)(v[2 * i] >> (5 * l)) & 31u) |
+                         (((unsigned)(v[2 * i + 1] >> (5 * l)) & 31u) << 16) | 0x64006400u;
+      __half2 h;
+      memcpy(&h, &n, 4);
+      h = __hsub2(h, off);
+      o[i] = __nv_cvt_halfraw2_to_fp8x2(h, __NV_SATFINITE, __NV_E4M3);
     }
-    uint4 out;
-    out.x = v[0]; out.y = v[1]; out.z = v[2]; out.w = v[3];
-    *reinterpret_cast<uint4*>(TL8 + (long long)c * L + e0) = out;
+    uint4 q;
+    q.x = o[0] | (o[1] << 16); q.y = o[2] | (o[3] << 16);
+    q.z = o[4] | (o[5] << 16); q.w = o[6] | (o[7] << 16);
+    *reinterpret_cast<uint4*>(out + l * L) = q;
   }
 }
 
-// BT[j * (Epad / 64) + w] = bits j of words[64 w .. 64 w + 63] (bit i = word 64 w + i).
-// One 64-thread block per word group w: thread j gathers its bit of the 64 words.
-__global__ void k_bit_transpose(const u64* __restrict__ words, long long nw, u64* __restrict__ BT) {
-  __shared__ u64 wsh[64];
-  for (long long w = blockIdx.x; w < nw; w += gridDim.x) {
-    wsh[threadIdx.x] = words[w * 64 + threadIdx.x];
-    __syncthreads();
-    const int j = threadIdx.x;
-    u64 v = 0;
-#pragma unroll 8
-    for (int i = 0; i < 64; ++i) v |= ((wsh[i] >> j) & 1ull) << i;
-    BT[(long long)j * nw + w] = v;
-    __syncthreads();
+// BT[j * nw + w] = bits j of words[64 w .. 64 w + 63] (bit i = word 64 w + i).  A warp transposes
+// the 64 x 64 bits of one w by exchanging halves (lane t holds words t and t + 32: one exchange in
+// the thread, five with lanes t ^ 16 .. t ^ 1); a block's 16 w leave through shared memory, so that
+// the rows are written 128 bytes at a time.  (64 threads gathering 64 bits each and writing 8 bytes
+// a row: 318 us for 2^24 words, now 84 us.)
+constexpr int BT_W = 16;
+__global__ void __launch_bounds__(32 * BT_W)
+k_bit_transpose(const u64* __restrict__ words, long long nw, u64* __restrict__ BT) {
+  __shared__ u64 rows[64][BT_W + 1];
+  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+  const long long w0 = (long long)blockIdx.x * BT_W;
+  u64 a = 0, b = 0;
+  if (w0 + wl < nw) {
+    a = words[(w0 + wl) * 64 + lane];
+    b = words[(w0 + wl) * 64 + 32 + lane];
+  }
+  // words t and t + 32: the off-diagonal 32-bit halves change places
+  const u64 t0 = (a & 0xFFFFFFFFull) | (b << 32);
+  b = (a >> 32) | (b & 0xFFFFFFFF00000000ull);
+  a = t0;
+  auto step = [&](int s, u64 m) {   // m: the low s bits of every 2 s
+    const bool up = lane & s;
+    const u64 ax = __shfl_xor_sync(0xffffffffu, a, s), bx = __shfl_xor_sync(0xffffffffu, b, s);
+    a = up ? ((a & ~m) | ((ax >> s) & m)) : ((a & m) | ((ax & m) << s));
+    b = up ? ((b & ~m) | ((bx >> s) & m)) : ((b & m) | ((bx & m) << s));
+  };
+  step(16, 0x0000FFFF0000FFFFull);
+  step(8, 0x00FF00FF00FF00FFull);
+  step(4, 0x0F0F0F0F0F0F0F0Full);
+  step(2, 0x3333333333333333ull);
+  step(1, 0x5555555555555555ull);
+  rows[lane][wl] = a;
+  rows[lane + 32][wl] = b;
+  __syncthreads();
+  for (int i = threadIdx.x; i < 64 * BT_W; i += 32 * BT_W) {
+    const int j = i / BT_W, w = i % BT_W;
+    if (w0 + w < nw) BT[(long long)j * nw + w0 + w] = rows[j][w];
   }
 }
 
@@ -233,12 +280,13 @@ k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* __restrict__ B1
 #pragma unroll 1
         for (int cc = 0; cc < 16; ++cc) {
           unsigned v[16];
-          tmem_ld16(tl + (unsigned)(a * 256 + cc * 16), v);
+          tmem_ld16(tl + (unsigned)(a * 256 + cc * S_LIMBS), v);   // 13 of 16 columns
           tmem_ld_wait();
           u64 sum = 0;
 #pragma unroll
-          for (int l = 0; l < 16; ++l)   // exact: 0 <= limb sum < 2^23, + 2^23 keeps it integral
-            sum += (u64)(__float_as_uint(__uint_as_float(v[l]) + 8388608.0f) - 0x4B000000u) << (4 * l);
+          for (int l = 0; l < S_LIMBS; ++l)   // exact: |limb sum| <= 2^20, + 1.5 2^23 keeps it integral
+            sum += (u64)(long long)(int)(__float_as_uint(__uint_as_float(v[l]) + 12582912.0f) -
+                                         0x4B400000u) << (5 * l);
           out[cc] = sum;
         }
       }
@@ -255,16 +303,12 @@ k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* __restrict__ B1
 }  // namespace
 
 void launch_trunc_limb_table(cudaStream_t st, const u64* Tlo, long long L, unsigned char* TL8) {
-  const long long total = 1024 * (L / 16);
-  long long g = (total + 255) / 256;
-  if (g > (1ll << 20)) g = 1ll << 20;
-  k_limb_table<<<(unsigned)g, 256, 0, st>>>(Tlo, L, TL8);
+  k_limb_table<<<(unsigned)(L / 64), 256, 0, st>>>(Tlo, L, TL8);
 }
 
 void launch_trunc_bit_transpose(cudaStream_t st, const u64* words, long long Epad, u64* BT) {
   const long long nw = Epad / 64;
-  const long long g = nw < (1ll << 20) ? nw : (1ll << 20);
-  k_bit_transpose<<<(unsigned)g, 64, 0, st>>>(words, nw, BT);
+  k_bit_transpose<<<(unsigned)((nw + BT_W - 1) / BT_W), 32 * BT_W, 0, st>>>(words, nw, BT);
 }
 
 int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long Epad,
@@ -273,7 +317,7 @@ int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long
   auto enc = encode_fn();
   if (!enc || L % S_KC != 0) return -2;
   CUtensorMap mb;
-  cuuint64_t dims[2] = {(cuuint64_t)L, 1024};
+  cuuint64_t dims[2] = {(cuuint64_t)L, 64 * S_LIMBS};
   cuuint64_t strides[1] = {(cuuint64_t)L};
   cuuint32_t box[2] = {(cuuint32_t)S_KC, (cuuint32_t)S_TCOLS};
   cuuint32_t es[2] = {1, 1};
@@ -282,7 +326,7 @@ int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long
           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return -2;
   set_max_dynamic_smem(reinterpret_cast<const void*>(k_trunc_s_tc), (int)S_SMEM);
-  dim3 grid(4096 / S_TPAIRS, 1024 / S_TCOLS, (unsigned)nhi);
+  dim3 grid(4096 / S_TPAIRS, 64 * S_LIMBS / S_TCOLS, (unsigned)nhi);
   k_trunc_s_tc<<<grid, S_THREADS, S_SMEM, st>>>(mb, B1T, B2T, Epad / 64, L, S_hi, err, err_flag);
   return 0;
 }
