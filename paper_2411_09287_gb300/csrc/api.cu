@@ -31,7 +31,6 @@ inline void counted(int k, F f, A... a) {
 }
 }  // namespace
 #define gemm_u64(...) counted(1, mpc3::gemm_u64, __VA_ARGS__)
-#define gemm_u64_small(...) counted(1, mpc3::gemm_u64_small, __VA_ARGS__)
 #define launch_share_input(...) counted(1, mpc3::launch_share_input, __VA_ARGS__)
 #define launch_fill_masks(...) counted(1, mpc3::launch_fill_masks, __VA_ARGS__)
 #define launch_mult_offline(...) counted(1, mpc3::launch_mult_offline, __VA_ARGS__)
@@ -44,17 +43,15 @@ inline void counted(int k, F f, A... a) {
 #define launch_hash_jobs(...) counted(2, mpc3::launch_hash_jobs, __VA_ARGS__)
 #define launch_hash_u64(...) counted(2, mpc3::launch_hash_u64, __VA_ARGS__)
 #define launch_digest_check(...) counted(1, mpc3::launch_digest_check, __VA_ARGS__)
-#define launch_gr_random_shared(...) counted(1, mpc3::launch_gr_random_shared, __VA_ARGS__)
 #define launch_gr_powers(...) counted(1, mpc3::launch_gr_powers, __VA_ARGS__)
 #define launch_gr_mul1(...) counted(1, mpc3::launch_gr_mul1, __VA_ARGS__)
-#define launch_gr_lincomb(...) counted(1, mpc3::launch_gr_lincomb, __VA_ARGS__)
-#define launch_gr_mulmat2(...) counted(1, mpc3::launch_gr_mulmat2, __VA_ARGS__)
+#define launch_gr_axpy(...) counted(1, mpc3::launch_gr_axpy, __VA_ARGS__)
 #define launch_gr_inverses(...) counted(1, mpc3::launch_gr_inverses, __VA_ARGS__)
 #define launch_gr_fold_reduce(...) counted(1, mpc3::launch_gr_fold_reduce, __VA_ARGS__)
 #define launch_neg_copy(...) counted(1, mpc3::launch_neg_copy, __VA_ARGS__)
 #define launch_round_tail(...) counted(1, mpc3::launch_round_tail, __VA_ARGS__)
+#define launch_inner_verify(...) counted(1, mpc3::launch_inner_verify, __VA_ARGS__)
 #define launch_reveal(...) counted(1, mpc3::launch_reveal, __VA_ARGS__)
-#define launch_delta(...) counted(1, mpc3::launch_delta, __VA_ARGS__)
 #define launch_rec_hash(...) counted(1, mpc3::launch_rec_hash, __VA_ARGS__)
 #define launch_weighted_sums(...) counted(1, mpc3::launch_weighted_sums, __VA_ARGS__)
 #define launch_update_vw(...) counted(1, mpc3::launch_update_vw, __VA_ARGS__)
@@ -85,9 +82,7 @@ constexpr u32 ST_TIMEOUT = 4u;  // a bounded device wait expired
 
 // device constants block (words)
 constexpr int CST_INV = 0;      // 192: x^-1, (1-x)^-1, (x(x-1))^-1
-constexpr int CST_ONE = 192;    // 64: the element 1
-constexpr int CST_MONE = 256;   // 64: the element -1
-constexpr int CST_WORDS = 320;
+constexpr int CST_WORDS = 192;
 
 constexpr int TRACE_ROUND = 832;  // words per round in a verification trace
 
@@ -120,12 +115,6 @@ __global__ void k_derive_keys(Key master, u32* out) {
   u32 o[16];
   chacha_block(master, 0u, 0x0059454Bu, (u32)pair, 0u, o);
   for (int i = 0; i < 8; ++i) out[(pair - 1) * 8 + i] = o[i];
-}
-
-__global__ void k_init_consts(int mode, u64* cst) {
-  const int t = threadIdx.x;
-  cst[CST_ONE + t] = (t == 0) ? 1ull : 0ull;
-  cst[CST_MONE + t] = (t == 0) ? ~0ull : 0ull;
 }
 
 inline long long ceil_log2(long long v) {
@@ -430,17 +419,14 @@ struct Small {   // per-verification small scratch (all device, from the workspa
   u64* Pmat;     // 4 x 3 x 4096
   u64* S;        // 4 x 192: S00, S01, S10, S11 (reduced; u64 path)
   u64* U;        // 2 x 12 x 128: a round's party sums ee, S01, S10, oo (3 parties each), the other
-                 // half cleared for the next round (sums_begin, next_sums)
+                 // half cleared for the next round (sums_begin, next_sums); then Pi_InnerVerify's
   u64* rec;      // REC_SLOTS records of opened single elements, hashed by flush_recs
   u64* z[2];     // 384 each
   u64* coef;     // 448: the fold element f at 0, 1 - f at 384
   u64* zp;       // 64
   u64* r;        // 64
   u64* MM;       // 128 x 64
-  u64* MA;       // 5 x 4096 (multiplication matrices of alpha components)
-  u64* alpha;    // 384
   u64* aux;      // 4 x 64
-  u64* Sfull;    // 192
   u64* zinit;    // 384: the claim entering the first round (never round scratch)
   mutable int nrec = 0, uc = 0;   // records not hashed yet; half of U in use
 };
@@ -451,7 +437,7 @@ Small plan_small(Arena& a) {
   Small s;
   s.Pmat = a.take<u64>(4 * 3 * 4096);
   s.S = a.take<u64>(4 * 192);
-  s.U = a.take<u64>(2 * SUMS_WORDS);
+  s.U = a.take<u64>(2 * SUMS_WORDS + IV_ACC_WORDS);
   s.rec = a.take<u64>(REC_SLOTS * REC_WORDS);
   s.z[0] = a.take<u64>(384);
   s.z[1] = a.take<u64>(384);
@@ -459,10 +445,7 @@ Small plan_small(Arena& a) {
   s.zp = a.take<u64>(64);
   s.r = a.take<u64>(64);
   s.MM = a.take<u64>(128 * 64);
-  s.MA = a.take<u64>(5 * 4096);
-  s.alpha = a.take<u64>(384);
   s.aux = a.take<u64>(4 * 64);
-  s.Sfull = a.take<u64>(192);
   s.zinit = a.take<u64>(384);
   return s;
 }
@@ -477,36 +460,6 @@ struct Dense {
   long long cap[2];
   int cur = 0;
 };
-
-// Inner-verify buffers for a final dimension D.
-struct IVBuf {
-  u64* xp;    // 6 x (D+1) x 64
-  u64* yy;    // 6 x (D+1) x 64
-  u64* g2o;   // (D+1) x 64
-  u64* g2i;
-  u64* p1o;
-  u64* p2o;
-  u64* p1i;
-  u64* p2i;
-  u64* zero;  // D x 64 zeros
-  u64* delta; // 64
-};
-
-IVBuf plan_iv(Arena& a, long long D) {
-  IVBuf b;
-  const long long w = (D + 1) * 64;
-  b.xp = a.take<u64>(6 * w);
-  b.yy = a.take<u64>(6 * w);
-  b.g2o = a.take<u64>(w);
-  b.g2i = a.take<u64>(w);
-  b.p1o = a.take<u64>(w);
-  b.p2o = a.take<u64>(w);
-  b.p1i = a.take<u64>(w);
-  b.p2i = a.take<u64>(w);
-  b.zero = a.take<u64>(w);
-  b.delta = a.take<u64>(64);
-  return b;
-}
 
 // The hash comparisons of the Pi_Rec calls recorded since the last flush; each batch flushes
 // before its Delta is read.
@@ -544,11 +497,11 @@ void reveal(mpc_ctx* ctx, u32 purpose, u64 obj, const Small& s, u64* out) {
   launch_reveal(ctx->st, ctx->k01, ctx->k02, ctx->k12, purpose, obj, r.mask, r.idx, out, r.rec);
 }
 
-// Clears both halves of the round sums; a round adds into cur_sums, and its tail clears the other
+// Clears both halves of the round sums and Pi_InnerVerify's; a round adds into cur_sums, and its tail clears the other
 // half for the next round.
 int sums_begin(mpc_ctx* ctx, const Small& s) {
   s.uc = 0;
-  CK(cudaMemsetAsync(s.U, 0, 2 * SUMS_WORDS * 8, ctx->st));
+  CK(cudaMemsetAsync(s.U, 0, (2 * SUMS_WORDS + IV_ACC_WORDS) * 8, ctx->st));
   return MPC_OK;
 }
 u64* cur_sums(const Small& s) { return s.U + s.uc * SUMS_WORDS; }
@@ -646,8 +599,9 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       launch_gr_fold_reduce(st, s.Pmat, 3, s.aux);            // aux: G00, G11, Gsum (64 each)
       CK(cudaMemcpyAsync(S00, s.aux, 512, cudaMemcpyDeviceToDevice, st));
       CK(cudaMemcpyAsync(S11, s.aux + 64, 512, cudaMemcpyDeviceToDevice, st));
-      launch_gr_lincomb(st, ctx->cst + CST_ONE, s.aux + 128, ctx->cst + CST_MONE, s.aux, s.aux + 192);
-      launch_gr_lincomb(st, ctx->cst + CST_ONE, s.aux + 192, ctx->cst + CST_MONE, s.aux + 64, S01);
+      launch_addsub(st, 64, s.aux + 128, s.aux, 1, s.aux + 192);
+      launch_addsub(st, 64, s.aux + 192, s.aux + 64, 1, S01);
+      g_launches += 2;
     }
   } else {
     bool done = false;
@@ -751,97 +705,36 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
 
 // Pi_InnerVerify (Fig. DPV) on a dense claim of dimension D.
 int inner_verify_dense(mpc_ctx* ctx, u64 vid, u32 batch, const Vec& x, const Vec& y, long long D,
-                       const u64* z, const Small& s, const IVBuf& b, u64* trace, int R) {
-  cudaStream_t st = ctx->st;
-  const u64 obj = make_obj(vid, batch, 0);
-  const long long w = (D + 1) * 64;
-  const u64 M1 = ~0ull;
-  // alpha random, not revealed
-  launch_gr_random_shared(st, 1, ctx->k01, ctx->k02, ctx->k12, P_VER_ALPHA, obj, s.alpha);
-  const u64* a = s.alpha;
-  // multiplication matrices: r_a = a0 + a1 (P0), a3 (P1's [r]_1), a2 (P1's m),
-  // a4 - a5 (P2's m - [r]_2), a4 (P2's m)
-  u64* ra = s.aux;
-  u64* d45 = s.aux + 64;
-  launch_gr_lincomb(st, ctx->cst + CST_ONE, a, ctx->cst + CST_ONE, a + 64, ra);
-  launch_gr_lincomb(st, ctx->cst + CST_ONE, a + 256, ctx->cst + CST_MONE, a + 320, d45);
-  launch_gr_mulmat2(st, ra, a + 192, s.MA);            // MA[0] = M(r_a), MA[1] = M(a3)
-  launch_gr_mulmat2(st, a + 128, d45, s.MA + 8192);    // MA[2] = M(a2), MA[3] = M(a4 - a5)
-  launch_gr_mulmat2(st, a + 256, nullptr, s.MA + 16384);  // MA[4] = M(a4)
-  CK(cudaMemsetAsync(b.zero, 0, (size_t)w * 8, st));
-  auto comp = [&](int c) -> const u64* { return x.c[c] ? x.c[c] : b.zero; };
-  // masks of x' = x alpha (words i*64 + c of the (P_VER_XA, R1/R2) streams)
-  launch_fill_masks(st, w, ctx->k01, ctx->k02, P_VER_XA, obj, b.xp);
-  {  // P0: Gamma_i = r_{x_i} r_a + [r_{x'_i}]_1 + [r_{x'_i}]_2, message [Gamma]_2 = Gamma - [Gamma]_1
-    GemmTerm T;
-    T.A = op(comp(0), 64, 0, x.c[1], 1);
-    T.B = op(s.MA, 64);
-    Epi e = epi_store(b.g2o, 64);
-    e.add0 = b.xp;
-    e.add1 = b.xp + w;
-    e.prf_sign = M1;
-    e.key = ctx->k01;
-    e.tag = make_tag(P_VER_XA, C_G1);
-    e.obj = obj;
-    gemm_u64_small(st, D, 64, 64, 1, &T, e);
-  }
-  int rc;
-  if ((rc = deliver(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, b.g2o, b.g2i, D * 64, -1))) return rc;
-  {  // P1: [m]_1 = -(m_x [r_a]_1 + m_a [r_x]_1) + [Gamma]_1
-    GemmTerm T[2];
-    T[0].A = op(comp(2), 64);
-    T[0].B = op(s.MA + 4096, 64);
-    T[1].A = op(comp(3), 64);
-    T[1].B = op(s.MA + 8192, 64);
-    Epi e = epi_store(b.p1o, 64);
-    e.acc_sign = M1;
-    e.prf_sign = 1;
-    e.key = ctx->k01;
-    e.tag = make_tag(P_VER_XA, C_G1);
-    e.obj = obj;
-    gemm_u64_small(st, D, 64, 64, 2, T, e);
-  }
-  {  // P2: [m]_2 = m_x (m_a - [r_a]_2) - [r_x]_2 m_a + [Gamma]_2
-    GemmTerm T[2];
-    T[0].A = op(comp(4), 64);
-    T[0].B = op(s.MA + 12288, 64);
-    T[1].A = op(comp(5), 64, 0, nullptr, 1, M1);
-    T[1].B = op(s.MA + 16384, 64);
-    Epi e = epi_store(b.p2o, 64);
-    e.add0 = b.g2i;
-    gemm_u64_small(st, D, 64, 64, 2, T, e);
-  }
-  if ((rc = deliver(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, b.p1o, b.p2i, D * 64, -1))) return rc;
-  if ((rc = deliver(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, b.p2o, b.p1i, D * 64, -1))) return rc;
-  launch_exchange_finish(st, w, b.p1o, b.p1i, b.p2o, b.p2i, b.xp, -1, nullptr);
-  // x'' = [x'_0 .. x'_{D-1}, alpha]; y'' = [y_0 .. y_{D-1}, -z]
+                       const u64* z, const Small& s, u64* trace, int R) {
+  InnerVerify a;
   for (int c = 0; c < 6; ++c) {
-    CK(cudaMemcpyAsync(b.xp + c * w + D * 64, a + c * 64, 512, cudaMemcpyDeviceToDevice, st));
-    if (y.c[c])
-      CK(cudaMemcpyAsync(b.yy + c * w, y.c[c], (size_t)D * 512, cudaMemcpyDeviceToDevice, st));
-    else
-      CK(cudaMemsetAsync(b.yy + c * w, 0, (size_t)D * 512, st));
-    launch_neg_copy(st, z + c * 64, 64, b.yy + c * w + D * 64);
+    a.x[c] = x.c[c];
+    a.y[c] = y.c[c];
   }
-  View u, v;
-  for (int c = 0; c < 6; ++c) {
-    u.c[c] = b.xp + c * w;
-    v.c[c] = b.yy + c * w;
-  }
-  u.ld = 64;
-  v.ld = 64;
-  if ((rc = party_sums(ctx, u, v, D + 1, s.Pmat, s.Sfull))) return rc;
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);
+  a.z = z;
+  a.D = D;
+  a.k01 = ctx->k01;
+  a.k02 = ctx->k02;
+  a.k12 = ctx->k12;
+  a.obj = make_obj(vid, batch, 0);
+  a.acc = s.U + 2 * SUMS_WORDS;
+  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, (u64)D * 512);   // x alpha
+  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);            // the inner product
   const Rec1 r = begin_rec(ctx, s);
-  launch_delta(st, s.Sfull, ctx->k01, ctx->k02, obj, r.mask, r.idx, r.rec, b.delta,
-               trace ? trace + (long long)R * TRACE_ROUND : nullptr, ctx->status, ST_VERIFY);
+  a.rec = r.rec;
+  a.xmask = r.mask;
+  a.xidx = r.idx;
+  a.trace = trace ? trace + (long long)R * TRACE_ROUND : nullptr;
+  a.status = ctx->status;
+  a.flag = ST_VERIFY;
+  launch_inner_verify(ctx->st, a);
   flush_recs(ctx, s);
   return cuda_check(ctx, "inner_verify");
 }
 
 // Dense rounds k = k0..R followed by Pi_InnerVerify.
 int run_dense(mpc_ctx* ctx, u64 vid, u32 batch, Dense& dv, long long D, const u64* z0, int k0,
-              int R, const Small& s, const IVBuf& ivb, u64* trace) {
+              int R, const Small& s, u64* trace) {
   int rc;
   const u64* z = z0;
   int zi = 0;
@@ -857,7 +750,7 @@ int run_dense(mpc_ctx* ctx, u64 vid, u32 batch, Dense& dv, long long D, const u6
     dv.cur ^= 1;
     D = (D + 1) / 2;
   }
-  return inner_verify_dense(ctx, vid, batch, dv.x[dv.cur], dv.y[dv.cur], D, z, s, ivb, trace, R);
+  return inner_verify_dense(ctx, vid, batch, dv.x[dv.cur], dv.y[dv.cur], D, z, s, trace, R);
 }
 
 long long dim_after(long long D, int R) {
@@ -1030,7 +923,6 @@ struct BlkPlan {
   PowPlan pp;
   u64 *T, *Rw, *S, *V, *W, *Vm, *G;
   Dense dv;
-  IVBuf iv;
 };
 
 // wlog: log2 of the words per weight step (0: weights r^i; 6: r^(i / 64), T_j = 1)
@@ -1055,7 +947,6 @@ BlkPlan plan_blk(Arena& a, long long D, int R, int wlog, bool full, const bool x
   p.Vm = a.take<u64>(p.B * 4096);
   p.G = a.take<u64>(p.nwp * p.B * 64);
   p.dv = plan_dense(a, p.nb, xc, yc);
-  p.iv = plan_iv(a, dim_after(p.nb, R - p.kap));
   return p;
 }
 
@@ -1133,7 +1024,7 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
   if (z != s.zinit) CK(cudaMemcpyAsync(s.zinit, z, 384 * 8, cudaMemcpyDeviceToDevice, st));
   p.dv.cur = 0;
   if ((rc = cuda_check(ctx, "block rounds"))) return rc;
-  return run_dense(ctx, vid, batch, p.dv, p.nb, s.zinit, p.kap + 1, p.R, s, p.iv, trace);
+  return run_dense(ctx, vid, batch, p.dv, p.nb, s.zinit, p.kap + 1, p.R, s, trace);
 }
 
 struct VMultPlan {
@@ -1188,7 +1079,6 @@ struct TruncPlan {
   u64 *Zhi = nullptr, *Zrep = nullptr, *Zprod = nullptr, *Prow = nullptr;
   u64* pqc = nullptr;        // the chunk's 12 rows of <p>, <q> gathered (chunked batches only)
   Dense dt;
-  IVBuf ivt;
 };
 
 // A truncation batch of E outputs: nchunks chunks of C outputs (the last one ragged).
@@ -1202,7 +1092,6 @@ struct VMatPlan {
   u64 *Q, *P, *T, *Pz;
   PowPlan powQ, powP;
   Dense dv;
-  IVBuf iv;
   int R0;
   bool trunc = false;
   TruncBatch tb;
@@ -1313,7 +1202,6 @@ TruncPlan plan_trunc(Arena& a, long long E, int R1, bool tc, bool chunked, const
   const bool xc[6] = {true, false, false, true, false, false};
   const bool yc[6] = {false, true, false, false, false, true};
   p.dt = plan_dense(a, p.Dt, xc, yc);
-  p.ivt = plan_iv(a, dim_after(p.Dt, p.R1 - p.kd));
   return p;
 }
 
@@ -1377,7 +1265,6 @@ bool plan_vmat(Arena& a, long long M, long long N, long long K, int t, int R0, i
   p.Pz = a.take<u64>(6 * 4096);
   const bool all[6] = {true, true, true, true, true, true};
   p.dv = plan_dense(a, K, all, all);
-  p.iv = plan_iv(a, dim_after(K, p.R0));
   if (p.trunc) plan_trunc_batch(a, E, R1, tc, tu, p.tb);
   return true;
 }
@@ -1612,7 +1499,7 @@ int bit_batch(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* z0, u64 ver
   // the claim entering the dense rounds must not alias their round scratch
   CK(cudaMemcpyAsync(s.zinit, z, 384 * 8, cudaMemcpyDeviceToDevice, st));
   p.dt.cur = 0;
-  rc = run_dense(ctx, verify_id, batch, p.dt, p.Dt, s.zinit, p.kd + 1, p.R1, s, p.ivt, tr);
+  rc = run_dense(ctx, verify_id, batch, p.dt, p.Dt, s.zinit, p.kd + 1, p.R1, s, tr);
   delete phase;
   return rc;
 }
@@ -1659,9 +1546,7 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
     launch_scalar_gr_sum(st, E, pq, E, 12, p.Rtab, p.Zpq);
   }
   u64* z0 = p.zt + 384;
-  for (int c = 0; c < 6; ++c)   // z_c = sum r^(2e) p_c + r sum r^(2e) q_c
-    launch_gr_lincomb(st, ctx->cst + CST_ONE, p.Zpq + c * 64, s.r, p.Zpq + (6 + c) * 64,
-                      z0 + c * 64);
+  launch_gr_axpy(st, 6, s.r, p.Zpq, p.Zpq + 384, z0);   // z_c = sum r^(2e) p_c + r sum r^(2e) q_c
   delete phase;
   return bit_batch(ctx, p, s, z0, verify_id, batch, tr);
 }
@@ -1743,7 +1628,6 @@ int mpc_create(const mpc_config* cfg, mpc_ctx** out) {
   std::memcpy(master.k, cfg->seed, 32);
   k_derive_keys<<<1, 32, 0, ctx->st>>>(master, keys_dev);
   launch_gr_inverses(ctx->st, ctx->cst + CST_INV);
-  k_init_consts<<<1, 64, 0, ctx->st>>>(ctx->reduce_mode, ctx->cst);
   e = cudaMemsetAsync(ctx->status, 0, sizeof(u32), ctx->st);
   if (e != cudaSuccess) return bail("cudaMemset", e);
   u32 kh[24];
@@ -2327,7 +2211,7 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
     launch_gr_fold_reduce(st, p.Pz, 6, s.zinit);
   }
   p.dv.cur = 0;
-  rc = run_dense(ctx, verify_id, 0, p.dv, K, s.zinit, 1, p.R0, s, p.iv, trace);
+  rc = run_dense(ctx, verify_id, 0, p.dv, K, s.zinit, 1, p.R0, s, trace);
   delete phase;
   if (rc) return rc;
   // ---- batch 1: the truncation pairs, chunk by chunk ----

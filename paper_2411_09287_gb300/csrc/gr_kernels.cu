@@ -20,31 +20,6 @@ inline unsigned grid_for(long long n) {
   return (unsigned)g;
 }
 
-// ---- random sharing ---------------------------------------------------------------------------
-__global__ void k_gr_random_shared(long long nwords, Key k01, Key k02, Key k12, u32 t1, u32 t2,
-                                   u32 tm, u64 obj, u64* __restrict__ s) {
-  const long long nb = (nwords + 7) / 8;
-  for (long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x; b < nb;
-       b += (long long)gridDim.x * blockDim.x) {
-    u64 r1[8], r2[8], m[8];
-    prf_block8(k01, t1, obj, (u64)b, r1);
-    prf_block8(k02, t2, obj, (u64)b, r2);
-    prf_block8(k12, tm, obj, (u64)b, m);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const long long i = b * 8 + j;
-      if (i < nwords) {
-        s[i] = r1[j];
-        s[nwords + i] = r2[j];
-        s[2 * nwords + i] = m[j];
-        s[3 * nwords + i] = r1[j];
-        s[4 * nwords + i] = m[j];
-        s[5 * nwords + i] = r2[j];
-      }
-    }
-  }
-}
-
 // ---- powers ---------------------------------------------------------------------------------
 // Block b writes table[16 b .. 16 b + 15]: the squares a^(2^k) by one half of the block while the
 // other multiplies the ones of 16 b's bits into a^(16 b), then four doublings of the row count
@@ -99,27 +74,17 @@ __global__ void k_gr_mul1(const u64* a, const u64* b, u64* out) {
   out[threadIdx.x] = sa[threadIdx.x];
 }
 
-// out = ca * a + cb * b  (single elements; b / cb may be null)
-__global__ void k_gr_lincomb(const u64* ca, const u64* a, const u64* cb, const u64* b,
-                             u64* out) {
-  __shared__ u64 x[64], y[64], s1[64], s2[64], scr[128];
-  const int t = threadIdx.x;
-  x[t] = a[t];
-  s1[t] = ca[t];
-  if (b) { y[t] = b[t]; s2[t] = cb[t]; }
+// out_c = a_c + r b_c, one block per c
+__global__ void __launch_bounds__(256)
+k_gr_axpy(const u64* __restrict__ r, const u64* __restrict__ a, const u64* __restrict__ b,
+          u64* __restrict__ out) {
+  __shared__ u64 x[64], y[64], scr[4 * 128];
+  const int t = threadIdx.x, c = blockIdx.x;
+  if (t < 64) x[t] = r[t];
+  else if (t < 128) y[t - 64] = b[c * 64 + t - 64];
   __syncthreads();
-  gr_mul_block(s1, x, x, scr);
-  if (b) gr_mul_block(s2, y, y, scr);
-  out[t] = x[t] + (b ? y[t] : 0ull);
-}
-
-// [M_a; M_b]: rows 0..63 the multiplication matrix of a, rows 64..127 that of b.
-__global__ void __launch_bounds__(256) k_gr_mulmat2(const u64* a, const u64* b, u64* M) {
-  __shared__ u64 e[64];
-  if (threadIdx.x < 64) e[threadIdx.x] = (blockIdx.x == 0 ? a : b)[threadIdx.x];
-  __syncthreads();
-  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x)
-    M[blockIdx.x * 4096 + i] = gr_mulmat_at(e, i >> 6, i & 63);
+  const u64 p = gr_mul_par<4>(x, y, scr, t);
+  if (t < 64) out[c * 64 + t] = a[c * 64 + t] + p;
 }
 
 // M[i] = multiplication matrix of the GR element src + i * stride, for i < n (one block each).
@@ -461,14 +426,6 @@ k_scalar_gr_sum(long long n, const u64* __restrict__ A, long long lda, int nrows
 }  // namespace
 
 // ---- launchers --------------------------------------------------------------------------------
-void launch_gr_random_shared(cudaStream_t st, long long n, Key k01, Key k02, Key k12,
-                             u32 purpose, u64 obj, u64* s6) {
-  const long long nw = n * 64;
-  k_gr_random_shared<<<grid_for((nw + 7) / 8), TPB, 0, st>>>(
-      nw, k01, k02, k12, make_tag(purpose, C_R1), make_tag(purpose, C_R2),
-      make_tag(purpose, C_M12), obj, s6);
-}
-
 void launch_gr_powers(cudaStream_t st, const u64* a, long long n, u64* table) {
   if (n <= 0) return;
   k_gr_powers<<<(unsigned)((n + POW_ROWS - 1) / POW_ROWS), 256, 0, st>>>(a, n, table);
@@ -478,13 +435,8 @@ void launch_gr_mul1(cudaStream_t st, const u64* a, const u64* b, u64* out) {
   k_gr_mul1<<<1, 64, 0, st>>>(a, b, out);
 }
 
-void launch_gr_lincomb(cudaStream_t st, const u64* ca, const u64* a, const u64* cb, const u64* b,
-                       u64* out) {
-  k_gr_lincomb<<<1, 64, 0, st>>>(ca, a, cb, b, out);
-}
-
-void launch_gr_mulmat2(cudaStream_t st, const u64* a, const u64* b, u64* M) {
-  k_gr_mulmat2<<<b ? 2 : 1, 256, 0, st>>>(a, b, M);
+void launch_gr_axpy(cudaStream_t st, int n, const u64* r, const u64* a, const u64* b, u64* out) {
+  if (n > 0) k_gr_axpy<<<n, 256, 0, st>>>(r, a, b, out);
 }
 
 void launch_gr_mulmat_batch(cudaStream_t st, long long n, const u64* src, long long stride,

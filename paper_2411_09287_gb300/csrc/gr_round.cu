@@ -184,36 +184,122 @@ k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u
   out[t] = m - r1 - r2in;
 }
 
-// Delta of Pi_InnerVerify from its party sums S (3 x 64, reduced): the secure inner product's
-// finish, Pi_Rec of the result (messages to rec), and `flag` in *status unless it is zero.
-__global__ void __launch_bounds__(64)
-k_delta(const u64* __restrict__ S, Key k01, Key k02, u64 obj, u64 xmask, int xidx,
-        u64* __restrict__ rec, u64* __restrict__ out, u64* __restrict__ trace, u32* status,
-        u32 flag) {
-  __shared__ u64 st[3][64];
-  const int t = threadIdx.x;
-  if (t < 24) {
-    const int s = t >> 3;
-    stream64(s == 1 ? k02 : k01, make_tag(P_VER_DELTA, s == 0 ? C_R1 : s == 1 ? C_R2 : C_G1), obj,
-             t & 7, st[s]);
+// Pi_InnerVerify (Fig. DPV) on a claim of D elements, in one launch.  Row i < D: x'_i = alpha x_i
+// (alpha random, shared, never opened) by Pi_Mult over GR, whose messages are Gamma_i - [Gamma_i]_1
+// (P0 -> P2) and the two halves of m (P1 <-> P2); row D: alpha against -z.  Every block takes some
+// rows and adds their party sums of sum_i x'_i y_i - alpha z,
+//   S0 = sum r_u r_v, S1 = -sum (m_u [r_v]_1 + m_v [r_u]_1), S2 = sum m_u (m_v - [r_v]_2) - m_v [r_u]_2,
+// to acc; the last one finishes the inner product, opens Delta (messages to rec) and sets `flag` in
+// *status unless it is zero.  A row is ten GR products: the five of x'_i are added before they are
+// reduced, so it is two dependent products and one ChaCha20 block of latency, about 8 us with the
+// opening.  As separate launches (streams, multiplication matrices, three small GEMMs, messages,
+// copies of x' and y, Gram sums, reductions: 40 launches) it took 150-200 us a batch.
+__global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
+  __shared__ u64 al[6][64];           // r1, r2, m of alpha; r_a, m - r2
+  __shared__ u64 u[6][64], v[6][64], st[3][64], scr[4 * 128];
+  __shared__ int last;
+  const int tid = threadIdx.x, t = tid & 63, i0 = (tid >> 6) * 16;
+  if (tid < 24) {
+    const int q = tid >> 3;
+    stream64(q == 0 ? a.k01 : q == 1 ? a.k02 : a.k12,
+             make_tag(P_VER_ALPHA, q == 0 ? C_R1 : q == 1 ? C_R2 : C_M12), a.obj, tid & 7, al[q]);
   }
   __syncthreads();
+  if (tid < 64) {
+    al[3][t] = al[0][t] + al[1][t];
+    al[4][t] = al[2][t] - al[1][t];
+  }
+  u64 lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+  for (long long i = blockIdx.x; i <= a.D; i += gridDim.x) {
+    __syncthreads();
+    for (int e = tid; e < 6 * 64; e += 256) {
+      const int c = e >> 6, w = e & 63;
+      if (i < a.D) {
+        u[c][w] = a.x[c] ? a.x[c][i * 64 + w] : 0ull;
+        v[c][w] = a.y[c] ? a.y[c][i * 64 + w] : 0ull;
+      } else {
+        u[c][w] = al[c == 0 || c == 3 ? 0 : c == 1 || c == 5 ? 1 : 2][w];
+        v[c][w] = 0ull - a.z[e];
+      }
+    }
+    if (i < a.D) {   // u = x_i becomes x'_i; uniform over the block
+      if (tid >= 232) {   // masks and [Gamma]_1, words 64 i .. 64 i + 63 of their streams
+        const int q = (tid - 232) >> 3, l = tid & 7;
+        u64 o[8];
+        prf_block8(q == 1 ? a.k02 : a.k01, make_tag(P_VER_XA, q == 0 ? C_R1 : q == 1 ? C_R2 : C_G1),
+                   a.obj, (u64)i * 8 + l, o);
+#pragma unroll
+        for (int w = 0; w < 8; ++w) st[q][l * 8 + w] = o[w];
+      }
+      __syncthreads();
+      if (tid < 64) u[0][t] += u[1][t];   // r_x = [r]_1 + [r]_2 at P0
+      __syncthreads();
+      u64 gl = 0, gh = 0, nl = 0, nh = 0;
+      gr_mac_part<16>(u[0], al[3], t, i0, gl, gh);   // P0: r_x r_a
+      gr_mac_part<16>(u[4], al[4], t, i0, gl, gh);   // P2: m_x (m_a - [r_a]_2)
+      gr_mac_part<16>(u[2], al[0], t, i0, nl, nh);   // P1: -(m_x [r_a]_1 + m_a [r_x]_1)
+      gr_mac_part<16>(u[3], al[2], t, i0, nl, nh);
+      gr_mac_part<16>(u[5], al[2], t, i0, nl, nh);   // P2: -[r_x]_2 m_a
+      const u64 r = gr_finish<4>(gl - nl, gh - nh, scr, tid);
+      if (tid < 64) {
+        // Gamma = r_x r_a + r1 + r2; [m]_1 + [m]_2 takes [Gamma]_1 + (Gamma - [Gamma]_1)
+        const u64 r1 = st[0][t], r2 = st[1][t], g1 = st[2][t], g2 = r1 + r2 - g1;
+        const u64 m = r + g1 + g2;
+        u[0][t] = r1; u[1][t] = r2; u[2][t] = m;
+        u[3][t] = r1; u[4][t] = m; u[5][t] = r2;
+      }
+    }
+    __syncthreads();
+    if (tid < 64) {
+      u[0][t] += u[1][t];
+      v[0][t] += v[1][t];
+      v[1][t] = v[4][t] - v[5][t];
+    }
+    __syncthreads();
+    u64 nl = 0, nh = 0;
+    gr_mac_part<16>(u[0], v[0], t, i0, lo[0], hi[0]);
+    gr_mac_part<16>(u[2], v[3], t, i0, nl, nh);
+    gr_mac_part<16>(v[2], u[3], t, i0, nl, nh);
+    lo[1] -= nl; hi[1] -= nh;
+    nl = nh = 0;
+    gr_mac_part<16>(u[4], v[1], t, i0, lo[2], hi[2]);
+    gr_mac_part<16>(v[4], u[5], t, i0, nl, nh);
+    lo[2] -= nl; hi[2] -= nh;
+  }
+  __syncthreads();
+  for (int q = 0; q < 3; ++q) {
+    const u64 r = gr_finish<4>(lo[q], hi[q], scr, tid);
+    if (tid < 64)
+      atomicAdd(reinterpret_cast<unsigned long long*>(a.acc + q * 64 + t), (unsigned long long)r);
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0)
+    last = atomicAdd(reinterpret_cast<unsigned long long*>(a.acc + 192), 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (tid < 24) {
+    const int q = tid >> 3;
+    stream64(q == 1 ? a.k02 : a.k01, make_tag(P_VER_DELTA, q == 0 ? C_R1 : q == 1 ? C_R2 : C_G1),
+             a.obj, tid & 7, st[q]);
+  }
+  __syncthreads();
+  if (tid >= 64) return;
   const u64 r1 = st[0][t], r2 = st[1][t], g1 = st[2][t];
-  const u64 g2 = S[t] + r1 + r2 - g1;                       // P0 -> P2
-  const u64 m1 = (S[64 + t] + g1) + (S[128 + t] + g2);      // P1: own + received
-  const u64 m2 = m1;                                        // P2: received + own
-  const u64 r2in = r2 ^ (t == xidx ? xmask : 0ull);
-  rec[t] = r1;
-  rec[64 + t] = r2;
-  rec[128 + t] = m1;
-  rec[192 + t] = r1;
-  rec[256 + t] = r2;
-  rec[320 + t] = m2;
-  rec[384 + t] = r2in;
-  const u64 d = m1 - r1 - r2in;
-  out[t] = d;
-  if (trace) trace[t] = d;
-  if (d != 0ull) atomicOr(status, flag);
+  const u64 g2 = __ldcg(a.acc + t) + r1 + r2 - g1;                          // P0 -> P2
+  const u64 m = (__ldcg(a.acc + 64 + t) + g1) + (__ldcg(a.acc + 128 + t) + g2);   // P1 <-> P2
+  const u64 r2in = r2 ^ (t == a.xidx ? a.xmask : 0ull);
+  a.rec[t] = r1;
+  a.rec[64 + t] = r2;
+  a.rec[128 + t] = m;
+  a.rec[192 + t] = r1;
+  a.rec[256 + t] = r2;
+  a.rec[320 + t] = m;
+  a.rec[384 + t] = r2in;
+  const u64 d = m - r1 - r2in;
+  if (a.trace) a.trace[t] = d;
+  if (d != 0ull) atomicOr(a.status, a.flag);
 }
 
 // The hash comparisons of n Pi_Rec calls of single GR elements (one block each): P1 sends H([r]_1)
@@ -359,9 +445,9 @@ void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 
   k_reveal<<<1, 64, 0, st>>>(k01, k02, k12, purpose, obj, xmask, xidx, out, rec);
 }
 
-void launch_delta(cudaStream_t st, const u64* S, Key k01, Key k02, u64 obj, u64 xmask, int xidx,
-                  u64* rec, u64* out, u64* trace, u32* status, u32 flag) {
-  k_delta<<<1, 64, 0, st>>>(S, k01, k02, obj, xmask, xidx, rec, out, trace, status, flag);
+void launch_inner_verify(cudaStream_t st, const InnerVerify& a) {
+  const long long n = a.D + 1;   // four blocks an SM at most: rows beyond that are looped over
+  k_inner_verify<<<(unsigned)(n < 608 ? n : 608), 256, 0, st>>>(a);
 }
 
 void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 flag) {

@@ -49,10 +49,6 @@ void gemm_u64_gram_batch(cudaStream_t st, long long K, int n, const GemmTerm* te
 // K across grid.z and requires epi.atomic = 1.
 void gemm_u64(cudaStream_t st, long long M, long long N, long long K, int nterms,
               const GemmTerm* terms, const Epi& epi, int nsplit);
-// The same product in 16 x 16 output tiles, one output per thread and no split: for small
-// products (a few thousand outputs, short K) that one 64 x 64 tile would leave on one SM.
-void gemm_u64_small(cudaStream_t st, long long M, long long N, long long K, int nterms,
-                    const GemmTerm* terms, const Epi& epi);
 
 // ---- exact u64 GEMM on the tcgen05 tensor cores (limb_gemm_tc.cu) ---------------------------
 // Same contract as gemm_u64 without split-K (epi.atomic must be 0; returns -1 otherwise, -2 if
@@ -158,10 +154,25 @@ void launch_round_tail(cudaStream_t st, const RoundTail& a);
 // A random GR element of the streams of (purpose, obj), opened into out; record in rec.
 void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
                    int xidx, u64* out, u64* rec);
-// Delta from the party sums S (3 x 64, reduced), opened into out (and trace when not null); `flag`
-// in *status unless it is zero.
-void launch_delta(cudaStream_t st, const u64* S, Key k01, Key k02, u64 obj, u64 xmask, int xidx,
-                  u64* rec, u64* out, u64* trace, u32* status, u32 flag);
+// Pi_InnerVerify of a claim of D elements: x, y component pointers (null = zero), z the claim (6 x
+// 64), acc 193 words that are zero on entry (party sums and a count of finished blocks).  Delta is
+// opened into trace (when not null); `flag` in *status unless it is zero.
+struct InnerVerify {
+  const u64 *x[6], *y[6];
+  const u64* z;
+  long long D;
+  Key k01, k02, k12;
+  u64 obj;
+  u64* acc;
+  u64* rec;             // this Pi_Rec's record (REC_WORDS)
+  u64 xmask;            // fault: word xidx of the P0 -> P1 message is XORed with xmask
+  int xidx;
+  u64* trace;
+  u32* status;
+  u32 flag;
+};
+constexpr int IV_ACC_WORDS = 193;
+void launch_inner_verify(cudaStream_t st, const InnerVerify& a);
 // The hash comparisons of n records: `flag` in *status on a mismatch.
 void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 flag);
 // Round k's sums S00, S01, S10, S11 of np parties (party p at 64 p, the four 192 words apart; added
@@ -227,13 +238,10 @@ void launch_digest_check(cudaStream_t st, const u32* a0, const u32* b0, const u3
 size_t hash_scratch_words(long long n);
 
 // ---- GR(2^64, 64) kernels (gr_kernels.cu) ---------------------------------------------------
-void launch_gr_random_shared(cudaStream_t st, long long n, Key k01, Key k02, Key k12,
-                             u32 purpose, u64 obj, u64* s6);
 void launch_gr_powers(cudaStream_t st, const u64* a, long long n, u64* table);
 void launch_gr_mul1(cudaStream_t st, const u64* a, const u64* b, u64* out);
-void launch_gr_lincomb(cudaStream_t st, const u64* ca, const u64* a, const u64* cb, const u64* b,
-                       u64* out);
-void launch_gr_mulmat2(cudaStream_t st, const u64* a, const u64* b, u64* M);
+// out_c = a_c + r b_c for n GR elements (rows of 64 words)
+void launch_gr_axpy(cudaStream_t st, int n, const u64* r, const u64* a, const u64* b, u64* out);
 void launch_gr_inverses(cudaStream_t st, u64* out);
 void launch_gr_fold_reduce(cudaStream_t st, const u64* P, int n, u64* out);
 void launch_neg_copy(cudaStream_t st, const u64* a, long long n, u64* out);
