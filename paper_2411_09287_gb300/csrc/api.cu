@@ -2708,151 +2708,58 @@ struct GfPlan {   // GF(2^64) Pi_MultVerify of D AND gates
   long long D;
   int R;
   u64 *XA, *YA, *ZA;        // concatenated triples, 6 x nw words each
-  u64 *pw;                  // D
-  u64 *x[2], *y[2];         // ping-pong GF vectors, 6 x (D + 1) and 6 x ((D + 1) / 2 + 1)
-  u64 *small;               // 64 words: z, h0, h2, S, coef, r, zeta', tmp6, alpha, delta
-  u64 *lhs, *rhs;           // 6 x (Dfinal + 1)
+  u64 *pw, *st;
+  GfWork* w;
+  u64 *x[2], *y[2];
 };
 
-GfPlan plan_gf(Arena& a, long long nw, int R) {
+GfPlan plan_gf(Arena& a, long long nw) {
   GfPlan g;
   g.D = 64 * nw;
-  g.R = R < 0 ? default_R(g.D) : R;
+  g.R = default_R(g.D);
   g.XA = a.take<u64>(6 * nw); g.YA = a.take<u64>(6 * nw); g.ZA = a.take<u64>(6 * nw);
-  g.pw = a.take<u64>(g.D);
-  g.x[0] = a.take<u64>(6 * (g.D + 1)); g.y[0] = a.take<u64>(6 * (g.D + 1));
-  g.x[1] = a.take<u64>(6 * ((g.D + 1) / 2 + 1)); g.y[1] = a.take<u64>(6 * ((g.D + 1) / 2 + 1));
-  g.small = a.take<u64>(128);
-  const long long Df = dim_after(g.D, g.R);
-  g.lhs = a.take<u64>(6 * (Df + 1)); g.rhs = a.take<u64>(6 * (Df + 1));
+  g.pw = a.take<u64>(8 * nw);
+  g.st = a.take<u64>(9 * (g.R + 1));
+  g.w = a.take<GfWork>(1);
+  for (int i = 0; i < 2; ++i) {
+    g.x[i] = a.take<u64>(i ? 24 * nw : 48 * nw);
+    g.y[i] = a.take<u64>(i ? 24 * nw : 48 * nw);
+  }
   return g;
-}
-
-// random shared GF element revealed with Pi_Rec (3 one-word messages, 3 hashes)
-void gf_reveal(mpc_ctx* ctx, u32 purpose, u64 obj, u64* tmp6, u64* out) {
-  launch_gf_random_shared(ctx->st, ctx->k01, ctx->k02, ctx->k12, purpose, obj, tmp6);
-  launch_gf_rec1(ctx->st, tmp6, 0ull, out, ctx->status, ST_ABORT);
-  g_launches += 2;
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 8);
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 32);
-}
-
-// secure GF inner product of (u, v) from their party sums (S must be zeroed by the caller, then
-// filled by launch_gf_party_sums): finish + 3 one-word messages
-void gf_inner_finish(mpc_ctx* ctx, const u64* S, u32 purpose, u64 obj, u64* h6) {
-  launch_gf_inner_finish(ctx->st, S, ctx->k01, ctx->k02, purpose, obj, h6);
-  g_launches += 1;
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 8);
 }
 
 // Pi_MultVerify (Fig. PPEV) over GF(2^64) of the AND triples in g.XA/YA/ZA (batch 2)
 int gf_verify(mpc_ctx* ctx, u64 vid, GfPlan& g, u64* trace) {
-  cudaStream_t st = ctx->st;
-  u64* z = g.small;          // 6
-  u64* h0 = g.small + 8;     // 6
-  u64* h2 = g.small + 16;    // 6
-  u64* S = g.small + 24;     // 3
-  u64* coef = g.small + 32;  // 5
-  u64* r = g.small + 40;     // 1
-  u64* zp = g.small + 41;    // 1
-  u64* tmp6 = g.small + 48;  // 6
-  u64* alpha = g.small + 56; // 6
-  u64* dl = g.small + 64;    // 1
-  u64* zn = g.small + 72;    // 6
-  const long long nw = g.D / 64;
-  CK(cudaMemsetAsync(g.small, 0, 128 * 8, st));
-  gf_reveal(ctx, P_VER_R, make_obj(vid, 2, 0), tmp6, r);
-  launch_gf_powers(st, r, g.D, g.pw);
-  launch_gf_tran(st, g.XA, g.YA, g.ZA, nw, g.pw, g.D + 1, g.x[0], g.y[0], z);
-  g_launches += 2;
-  long long D = g.D;
-  int cur = 0;
-  const u64 X1 = 3ull, XX = 2ull;   // 1 + x and x: the fold weights at the third point x
-  for (int k = 1; k <= g.R; ++k) {
-    const long long cap = cur == 0 ? g.D + 1 : (g.D + 1) / 2 + 1;
-    u64* xv = g.x[cur];
-    u64* yv = g.y[cur];
-    if (D & 1)
-      for (int c = 0; c < 6; ++c) {
-        CK(cudaMemsetAsync(xv + c * cap + D, 0, 8, st));
-        CK(cudaMemsetAsync(yv + c * cap + D, 0, 8, st));
-      }
-    const long long Dh = (D + 1) / 2;
-    const u64 obj = make_obj(vid, 2, (u32)k);
-    const u64* uc[6];
-    const u64* vc[6];
-    for (int c = 0; c < 6; ++c) {
-      uc[c] = xv + c * cap;
-      vc[c] = yv + c * cap;
-    }
-    CK(cudaMemsetAsync(S, 0, 3 * 8, st));
-    launch_gf_party_sums(st, uc, vc, Dh, 2, 0, 0, 0, 0, S);           // even entries
-    g_launches += 1;
-    gf_inner_finish(ctx, S, P_VER_H0, obj, h0);
-    CK(cudaMemsetAsync(S, 0, 3 * 8, st));
-    launch_gf_party_sums(st, uc, vc, Dh, 1, 0, 1, X1, XX, S);         // f(x) = (1+x) f(0) + x f(1)
-    g_launches += 1;
-    gf_inner_finish(ctx, S, P_VER_H2, obj, h2);
-    gf_reveal(ctx, P_VER_ZETA, obj, tmp6, zp);
-    launch_gf_lagrange(st, zp, coef);
-    launch_gf_combine_z(st, coef, h0, h2, z, zn);
-    g_launches += 2;
-    CK(cudaMemcpyAsync(z, zn, 6 * 8, cudaMemcpyDeviceToDevice, st));
-    const long long ocap = (g.D + 1) / 2 + 1;
-    u64* xo = g.x[1];
-    u64* yo = g.y[1];
-    if (cur == 1) {   // fold in place is not allowed: fold into slot 0's storage
-      xo = g.x[0];
-      yo = g.y[0];
-    }
-    const long long ocap2 = cur == 1 ? g.D + 1 : ocap;
-    launch_gf_fold6x2(st, xv, yv, cap, D, coef, xo, yo, ocap2);
-    g_launches += 1;
-    if (trace) {
-      u64* t = trace + (long long)(k - 1) * MPC_TRACE_GF_ROUND;
-      CK(cudaMemcpyAsync(t, zp, 8, cudaMemcpyDeviceToDevice, st));
-      CK(cudaMemcpyAsync(t + 1, h0, 48, cudaMemcpyDeviceToDevice, st));
-      CK(cudaMemcpyAsync(t + 7, h2, 48, cudaMemcpyDeviceToDevice, st));
-    }
-    cur ^= 1;
-    D = Dh;
+  GfVerify v;
+  v.X = g.XA;
+  v.Y = g.YA;
+  v.Z = g.ZA;
+  v.nw = g.D / 64;
+  v.R = g.R;
+  v.k01 = ctx->k01;
+  v.k02 = ctx->k02;
+  v.k12 = ctx->k12;
+  v.obj = make_obj(vid, 2, 0);
+  v.pw = g.pw;
+  v.st = g.st;
+  v.w = g.w;
+  for (int i = 0; i < 2; ++i) {
+    v.x[i] = g.x[i];
+    v.y[i] = g.y[i];
   }
-  // Pi_InnerVerify (Fig. DPV): alpha random (kept shared), x' = x alpha, Delta = <[x'; alpha],
-  // [y; -z]> opened, accept iff 0
-  const long long cap = cur == 0 ? g.D + 1 : (g.D + 1) / 2 + 1;
-  u64* xv = g.x[cur];
-  u64* yv = g.y[cur];
-  const u64 obj = make_obj(vid, 2, 0);
-  launch_gf_random_shared(st, ctx->k01, ctx->k02, ctx->k12, P_VER_ALPHA, obj, alpha);
-  g_launches += 1;
-  const u64* xc[6];
-  for (int c = 0; c < 6; ++c) xc[c] = xv + c * cap;
-  const long long Df = D;
-  launch_gf_mult_alpha(st, xc, alpha, Df, Df + 1, ctx->k01, ctx->k02, obj, g.lhs);
-  g_launches += 1;
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, (u64)8 * Df);
-  // lhs = [x alpha ; alpha], rhs = [y ; -z] (-z = z in characteristic 2), Df + 1 entries each
-  for (int c = 0; c < 6; ++c) {
-    CK(cudaMemcpyAsync(g.lhs + c * (Df + 1) + Df, alpha + c, 8, cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpyAsync(g.rhs + c * (Df + 1), yv + c * cap, (size_t)Df * 8, cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpyAsync(g.rhs + c * (Df + 1) + Df, z + c, 8, cudaMemcpyDeviceToDevice, st));
-  }
-  const u64* uc[6];
-  const u64* vc[6];
-  for (int c = 0; c < 6; ++c) {
-    uc[c] = g.lhs + c * (Df + 1);
-    vc[c] = g.rhs + c * (Df + 1);
-  }
-  CK(cudaMemsetAsync(S, 0, 3 * 8, st));
-  launch_gf_party_sums(st, uc, vc, Df + 1, 1, 0, 0, 0, 0, S);
-  g_launches += 1;
-  gf_inner_finish(ctx, S, P_VER_DELTA, obj, tmp6);
-  launch_gf_rec1(st, tmp6, 0ull, dl, ctx->status, ST_ABORT);
-  launch_gf_check_zero(st, dl, ctx->status, ST_VERIFY);
-  g_launches += 2;
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 8);
-  count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 32);
-  if (trace) CK(cudaMemcpyAsync(trace + (long long)g.R * MPC_TRACE_GF_ROUND, dl, 8, cudaMemcpyDeviceToDevice, st));
+  v.trace = trace;
+  v.trace_ld = MPC_TRACE_GF_ROUND;
+  v.status = ctx->status;
+  v.flag_verify = ST_VERIFY;
+  v.flag_abort = ST_ABORT;
+  g_launches += launch_gf_verify(ctx->st, v);
+  // Pi_Rec of r, the zetas and Delta (3 words and 3 hashes each); two secure inner products a round,
+  // x alpha and the last inner product
+  const int ph = MPC_PHASE_VERIFY, pr = MPC_PROTO_VERIFY;
+  count_msgs(ctx, ph, pr, 3 * (g.R + 2), 8);
+  count_msgs(ctx, ph, pr, 3 * (g.R + 2), 32);
+  count_msgs(ctx, ph, pr, 3 * (2 * g.R + 1), 8);
+  count_msgs(ctx, ph, pr, 3, (u64)8 * dim_after(g.D, g.R));
   return cuda_check(ctx, "gf_verify");
 }
 
@@ -2906,7 +2813,7 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuni
   p.b1 = plan_blk(a, p.D1, p.R1, 6, false, xc, yc);
   p.Ye = a.take<u64>(6 * p.D1);
   p.Xe = a.take<u64>(p.D1);
-  p.gf = plan_gf(a, andw, -1);
+  p.gf = plan_gf(a, andw);
   p.nb = 64 * p.ne;
   p.Rb = default_R(p.nb);
   p.sb = plan_small(a);

@@ -349,29 +349,34 @@ void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int
 // (component c at c ldy), entry (e0 + e) 64 + i.
 void launch_eda_words(cudaStream_t st, const u64* mbits, const u64* rp, long long np, long long e0,
                       long long ldy, u64* xm, u64* y);
-void launch_gf_powers(cudaStream_t st, const u64* r, long long n, u64* out);
-void launch_gf_tran(cudaStream_t st, const u64* X, const u64* Y, const u64* Z, long long nw,
-                    const u64* pw, long long ld, u64* xo, u64* yo, u64* zsum);
-void launch_gf_party_sums(cudaStream_t st, const u64* const u[6], const u64* const v[6], long long D,
-                          long long stride, long long off, int fold, u64 fa, u64 fb, u64* S);
-// The GF fold of the six components of x and of y (component c at c * cap in, c * ocap out).
-void launch_gf_fold6x2(cudaStream_t st, const u64* xv, const u64* yv, long long cap, long long D,
-                       const u64* zeta, u64* xo, u64* yo, long long ocap);
-void launch_gf_inner_finish(cudaStream_t st, const u64* S, Key k01, Key k02, u32 purpose, u64 obj,
-                            u64* h6);
-void launch_gf_random_shared(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj,
-                             u64* s6);
-void launch_gf_rec1(cudaStream_t st, const u64* s6, u64 xor_mask, u64* out, u32* status, u32 flag);
-void launch_gf_lagrange(cudaStream_t st, const u64* zeta, u64* coef);
-void launch_gf_combine_z(cudaStream_t st, const u64* coef, const u64* h0, const u64* h2, const u64* z,
-                         u64* zo);
-void launch_gf_mult_alpha(cudaStream_t st, const u64* const x[6], const u64* a6, long long D,
-                          long long ld, Key k01, Key k02, u64 obj, u64* xa);
 void launch_gather(cudaStream_t st, const u64* xs, long long n_in, const long long* idx,
                    long long n_out, u64* out);
 void launch_window_gather(cudaStream_t st, const u64* x, long long BC, long long H, long long W,
                           long long np, u64* left, u64* right);
-void launch_gf_check_zero(cudaStream_t st, const u64* d, u32* status, u32 flag);
+// ---- Pi_MultVerify of AND gates over GF(2^64) (gf_verify.cu) ----------------------------------
+constexpr int GF_MAX_ROUNDS = 60;
+struct GfWork {          // cleared by launch_gf_verify
+  u64 S[240], V[8], W[8], z[6], zeta, r;
+  u64 sums[6 * (GF_MAX_ROUNDS + 1)];
+  u32 count[GF_MAX_ROUNDS + 1];
+};
+struct GfVerify {
+  const u64 *X, *Y, *Z;  // the triples: 6 x nw words each, bit i of the 64 nw gates = bit i % 64
+  long long nw;          // at least 125
+  int R;                 // rounds, at least 4, to at most 64 elements
+  Key k01, k02, k12;
+  u64 obj;               // the batch's stream object (round k: + k)
+  u64* pw;               // 8 nw words
+  u64* st;               // 9 (R + 1) words
+  GfWork* w;
+  u64 *x[2], *y[2];      // 48 nw and 24 nw words each
+  u64* trace;            // zeta | h(0) | h(x) of round k at (k - 1) trace_ld, Delta at R trace_ld; or null
+  long long trace_ld;
+  u32* status;
+  u32 flag_verify, flag_abort;   // Delta != 0; a hash mismatch
+};
+// Returns the number of launches.
+int launch_gf_verify(cudaStream_t st, const GfVerify& a);
 // arithmetic Pi_Mult with the streams of `purpose` (prf_kernels.cu)
 void launch_mult_offline_p(cudaStream_t st, const u64* xs, const u64* ys, long long n, Key k01,
                            Key k02, u32 purpose, u64 obj, u64* zs, u64* p0_out_g2);
