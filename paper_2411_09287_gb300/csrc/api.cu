@@ -2502,204 +2502,95 @@ void ctx_set_aborted(mpc_ctx* c) { c->aborted = true; }
 // ---- non-linear layers (Sec. 4.3) -------------------------------------------------------------
 namespace {
 
-// messages of one Pi_Mult / AND batch of up to n words
-struct MsgBuf {
-  u64 *g2o, *g2i, *p1o, *p2o, *p1i, *p2i;
-};
-MsgBuf plan_msg(Arena& a, long long n) {
-  MsgBuf m;
-  m.g2o = a.take<u64>(n); m.g2i = a.take<u64>(n);
-  m.p1o = a.take<u64>(n); m.p2o = a.take<u64>(n);
-  m.p1i = a.take<u64>(n); m.p2i = a.take<u64>(n);
-  return m;
-}
-
-// A Boolean message of nw words; the AND_GAMMA2 site flips bit `index` of it (when mask & 1), the
-// Boolean counterpart of an element fault; HIGH_BIT at l = 1 is the same bit flip.
-int deliver_bits(mpc_ctx* ctx, int phase, int proto, const u64* src, u64* dst, long long nw, int site) {
-  if (nw > 0) CK(cudaMemcpyAsync(dst, src, (size_t)nw * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  ctx->ledger[phase][proto] += (u64)nw * 8;
-  ctx->nmsg += 1;
-  if (site >= 0 && nw > 0) {
-    Fault& f = ctx->fault[site];
-    if (f.armed) {
-      const u64 bit = f.index % (u64)(64 * nw);
-      if (f.mask & 1ull) launch_xor_one(ctx->st, dst + bit / 64, 1ull << (bit % 64));
-      f.armed = false;
-    }
+// The fault armed at `site` for a message of n words, disarmed.
+MsgFault take_fault(mpc_ctx* ctx, int site, long long n) {
+  if (site == MPC_SITE_GAMMA2 && ctx->fault[MPC_SITE_HIGH_BIT].armed) {
+    ctx->fault[MPC_SITE_HIGH_BIT].armed = false;
+    ctx->fault[MPC_SITE_GAMMA2] = {true, ctx->fault[MPC_SITE_HIGH_BIT].index, 1ull << 63};
   }
-  return MPC_OK;
+  Fault& f = ctx->fault[site];
+  if (!f.armed) return {-1, 0};
+  f.armed = false;
+  return {(long long)(f.index % (u64)n), f.mask};
 }
 
-// arithmetic Pi_Mult (Fig. MultP) with the streams of (purpose, obj)
-int mult_p(mpc_ctx* ctx, const u64* xs, const u64* ys, long long n, u32 purpose, u64 obj, u64* zs,
-           const MsgBuf& m) {
-  int rc;
-  launch_mult_offline_p(ctx->st, xs, ys, n, ctx->k01, ctx->k02, purpose, obj, zs, m.g2o);
-  g_launches += 1;
-  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_MULT, m.g2o, m.g2i, n, MPC_SITE_GAMMA2))) return rc;
-  launch_mult_online_p(ctx->st, xs, ys, n, ctx->k01, purpose, obj, m.g2i, m.p1o, m.p2o);
-  g_launches += 1;
-  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, m.p1o, m.p2i, n, MPC_SITE_MZ1))) return rc;
-  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, m.p2o, m.p1i, n, MPC_SITE_MZ2))) return rc;
-  launch_exchange_finish(ctx->st, n, m.p1o, m.p1i, m.p2o, m.p2i, zs, -1, nullptr);
-  return MPC_OK;
+// The same for a Boolean message of nw words: the AND_GAMMA2 site flips bit `index` of it (when mask
+// & 1), the Boolean counterpart of an element fault; HIGH_BIT at l = 1 is the same bit flip.
+MsgFault take_bit_fault(mpc_ctx* ctx, int site, long long nw) {
+  const MsgFault f = take_fault(ctx, site, 64 * nw);
+  if (f.idx < 0 || !(f.mask & 1ull)) return {-1, 0};
+  return {f.idx / 64, 1ull << (f.idx % 64)};
 }
 
-// Boolean AND gates (Fig. MultP over Z_2) on nw bit-sliced words
-int and_p(mpc_ctx* ctx, const u64* xs, const u64* ys, long long nw, u32 purpose, u64 obj, u64* zs,
-          const MsgBuf& m) {
-  int rc;
-  launch_and_offline(ctx->st, xs, ys, nw, ctx->k01, ctx->k02, purpose, obj, zs, m.g2o);
-  g_launches += 1;
-  if ((rc = deliver_bits(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_MULT, m.g2o, m.g2i, nw, MPC_SITE_AND_GAMMA2)))
-    return rc;
-  launch_and_online(ctx->st, xs, ys, nw, ctx->k01, purpose, obj, m.g2i, m.p1o, m.p2o);
-  g_launches += 1;
-  if ((rc = deliver_bits(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, m.p1o, m.p2i, nw, -1))) return rc;
-  if ((rc = deliver_bits(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, m.p2o, m.p1i, nw, -1))) return rc;
-  launch_xor_finish(ctx->st, nw, m.p1o, m.p1i, m.p2o, m.p2i, zs);
-  g_launches += 1;
-  return MPC_OK;
+// The messages of a Pi_Mult (three of n words; offline [Gamma]_2, online the halves of m)
+void count_mult(mpc_ctx* ctx, long long n) {
+  count_msgs(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_MULT, 1, (u64)n * 8);
+  count_msgs(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, 2, (u64)n * 8);
 }
 
 constexpr int NL_LEVELS = 6;
 inline int level_planes(int l) { return l == NL_LEVELS ? 1 : 2 * (32 >> (l - 1)); }   // 64,32,..,4,1
 
-// Buffers of one compare-select stage of np (padded) elements, W = np / 64 words per plane.
+// Buffers of one compare-select stage of np (padded) elements, W = np / 64 words per plane; the bit
+// planes eda[0], eda[1], the triples and the outputs are the layer's (plan_nl).
 struct CSPlan {
-  long long np, W;
-  MsgBuf ma, mb;                 // arithmetic (64 np) and Boolean (64 W) message buffers
-  u64 *b1w, *b2w, *mbw, *rbits;  // edaBit bit planes (64 W each), Boolean sharing (6 x 64 W)
-  u64 *B1, *B2, *eprod, *rp;     // 6 x 64 np each
-  u64 *ez, *ra, *dd;             // 6 x np: edaBit inner products, <r>, <x - r>
-  u64 *delta, *dpl;              // np public words, 64 W bit planes
-  u64 *G, *P, *G2, *P2;          // 6 x 64 W each
-  u64 *X[NL_LEVELS + 1], *Y[NL_LEVELS + 1], *Z[NL_LEVELS + 1];   // AND triples per level
-  u64 *ge, *r1w, *r2w, *r3w, *rb, *e, *dbits;                    // Boolean, W-sized
-  u64 *A1, *A2, *A3, *t, *rpd, *u, *rad, *gea, *d, *prod;        // 6 x np
+  CompareSelect k;
+  u64 *delta, *dpl, *dbits;      // np public words, their 64 W bit planes, W words
   RecPlan reca, recb;
-  long long and_words;           // words of all AND triples (per component)
 };
 
 CSPlan plan_cs(Arena& a, long long np) {
   CSPlan p;
-  p.np = np;
-  p.W = np / 64;
-  const long long W = p.W, N = 64 * np;
-  p.ma = plan_msg(a, N);
-  p.mb = plan_msg(a, 64 * W);
-  p.b1w = a.take<u64>(64 * W); p.b2w = a.take<u64>(64 * W); p.mbw = a.take<u64>(64 * W);
-  p.rbits = a.take<u64>(6 * 64 * W);
-  p.B1 = a.take<u64>(6 * N); p.B2 = a.take<u64>(6 * N);
-  p.eprod = a.take<u64>(6 * N); p.rp = a.take<u64>(6 * N);
-  p.ez = a.take<u64>(6 * np); p.ra = a.take<u64>(6 * np); p.dd = a.take<u64>(6 * np);
-  p.delta = a.take<u64>(np); p.dpl = a.take<u64>(64 * W);
-  p.G = a.take<u64>(6 * 64 * W); p.P = a.take<u64>(6 * 64 * W);
-  p.G2 = a.take<u64>(6 * 64 * W); p.P2 = a.take<u64>(6 * 64 * W);
-  p.and_words = 0;
-  for (int l = 1; l <= NL_LEVELS; ++l) {
-    const long long nw = (long long)level_planes(l) * W;
-    p.X[l] = a.take<u64>(6 * nw); p.Y[l] = a.take<u64>(6 * nw); p.Z[l] = a.take<u64>(6 * nw);
-    p.and_words += nw;
-  }
-  p.ge = a.take<u64>(6 * W);
-  p.r1w = a.take<u64>(W); p.r2w = a.take<u64>(W); p.r3w = a.take<u64>(W);
-  p.rb = a.take<u64>(6 * W); p.e = a.take<u64>(6 * W); p.dbits = a.take<u64>(W);
-  p.A1 = a.take<u64>(6 * np); p.A2 = a.take<u64>(6 * np); p.A3 = a.take<u64>(6 * np);
-  p.t = a.take<u64>(6 * np); p.rpd = a.take<u64>(6 * np); p.u = a.take<u64>(6 * np);
-  p.rad = a.take<u64>(6 * np); p.gea = a.take<u64>(6 * np); p.d = a.take<u64>(6 * np);
-  p.prod = a.take<u64>(6 * np);
+  CompareSelect& k = p.k;
+  const long long W = np / 64;
+  k.np = np;
+  k.eda[2] = a.take<u64>(np);
+  for (int q = 0; q < 3; ++q) k.da[q] = a.take<u64>(W);
+  k.eprod = a.take<u64>(6 * 64 * np);
+  k.ez = a.take<u64>(6 * np);
+  k.dd = a.take<u64>(6 * np);
+  k.rad = a.take<u64>(6 * np);
+  k.e = a.take<u64>(6 * W);
+  p.delta = a.take<u64>(np);
+  p.dpl = a.take<u64>(np);
+  p.dbits = a.take<u64>(W);
+  k.dpl = p.dpl;
+  k.dbits = p.dbits;
   p.reca = plan_rec(a, np, false);
   p.recb = plan_rec(a, W, false);
   return p;
 }
 
-// Boolean sharing (6 x nw words) whose components are the pair-known bit planes (r1, r2, m):
-// P0 (r1, r2), P1 (m, r1), P2 (m, r2)
-int bool_from_planes(mpc_ctx* ctx, const u64* r1, const u64* r2, const u64* m, long long nw, u64* s) {
-  const u64* src[6] = {r1, r2, m, r1, m, r2};
-  for (int c = 0; c < 6; ++c)
-    CK(cudaMemcpyAsync(s + c * nw, src[c], (size_t)nw * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  return MPC_OK;
-}
+constexpr int AND_PLANES = 125;   // AND gates of the carry tree, per element: 64 + 32 + 16 + 8 + 4 + 1
 
-// <max(a, b)> into out (6 np each; out may alias neither a nor b): Sec. 4.3 compare-select
-int compare_select(mpc_ctx* ctx, u64 call_id, int stage, const u64* a, const u64* b, CSPlan& p,
-                   u64* out) {
-  int rc;
+// <max(a, b)> of a stage (p.k.a, p.k.b into p.k.out): Sec. 4.3 compare-select
+int compare_select(mpc_ctx* ctx, u64 call_id, int stage, CSPlan& p) {
   cudaStream_t st = ctx->st;
-  const long long np = p.np, W = p.W, N = 64 * np;
-  const u64 obj = make_obj(call_id, (u32)stage, 0);
-  launch_addsub(st, 6 * np, a, b, 1, p.d);                                  // d = a - b
-  g_launches += 1;
-  // edaBits (Fig. edabits)
-  launch_prf_words(st, 64 * W, ctx->k01, make_tag(P_EDABIT, C_R1), obj, p.b1w, 0ll);
-  launch_prf_words(st, 64 * W, ctx->k02, make_tag(P_EDABIT, C_R2), obj, p.b2w, 0ll);
-  launch_prf_words(st, 64 * W, ctx->k12, make_tag(P_EDABIT, C_M12), obj, p.mbw, 0ll);
-  if ((rc = bool_from_planes(ctx, p.b1w, p.b2w, p.mbw, 64 * W, p.rbits))) return rc;
-  launch_bits_to_arith(st, p.b1w, N, 0, p.B1);
-  launch_bits_to_arith(st, p.b2w, N, 1, p.B2);
-  g_launches += 2;
-  if ((rc = mult_p(ctx, p.B1, p.B2, N, P_EDA_MULT, obj, p.eprod, p.ma))) return rc;
-  launch_lin_apb_m2c(st, 6 * N, p.B1, p.B2, p.eprod, p.rp);                 // r' = b1 + b2 - 2 b1 b2
-  launch_eda_inner_offline(st, np, ctx->k01, ctx->k02, obj, p.ez, p.ma.g2o);
-  g_launches += 2;
-  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_INNER, p.ma.g2o, p.ma.g2i, np, MPC_SITE_GAMMA2)))
-    return rc;
-  launch_eda_inner_online(st, p.mbw, p.rp, np, ctx->k01, obj, p.ma.g2i, p.ma.p1o, p.ma.p2o);
-  g_launches += 1;
-  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_INNER, p.ma.p1o, p.ma.p2i, np, MPC_SITE_MZ1))) return rc;
-  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_INNER, p.ma.p2o, p.ma.p1i, np, MPC_SITE_MZ2))) return rc;
-  launch_exchange_finish(st, np, p.ma.p1o, p.ma.p1i, p.ma.p2o, p.ma.p2i, p.ez, -1, nullptr);
-  launch_eda_compose(st, p.mbw, p.rp, p.ez, np, p.ra);
-  g_launches += 2;
-  // msb(d): open Delta = d - r, carry circuit over the bits of Delta + r
-  launch_addsub(st, 6 * np, p.d, p.ra, 1, p.dd);
-  g_launches += 1;
-  rec_core(ctx, p.dd, np, p.reca, p.delta, false);
+  CompareSelect& k = p.k;
+  const long long np = k.np, W = np / 64, N = 64 * np;
+  k.k01 = ctx->k01;
+  k.k02 = ctx->k02;
+  k.k12 = ctx->k12;
+  k.obj = make_obj(call_id, (u32)stage, 0);
+  k.fault[0] = take_fault(ctx, MPC_SITE_GAMMA2, N);
+  k.fault[1] = take_fault(ctx, MPC_SITE_MZ1, N);
+  k.fault[2] = take_fault(ctx, MPC_SITE_MZ2, N);
+  k.fault[3] = take_bit_fault(ctx, MPC_SITE_AND_GAMMA2, 64 * W);
+  // edaBits (Fig. edabits) and Delta = d - r, d = a - b
+  g_launches += launch_cs_open_delta(st, k);
+  count_mult(ctx, N);                                                    // the bit products
+  count_msgs(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_INNER, 3, (u64)np * 8);   // the inner products
+  rec_core(ctx, k.dd, np, p.reca, p.delta, false);
+  // msb(d) by the carry circuit over the bits of Delta + r; daBits; e = [d >= 0] XOR bit
   launch_trunc_bit_transpose(st, p.delta, np, p.dpl);
-  launch_msb_leaves(st, p.rbits, p.dpl, W, p.G, p.P);
-  g_launches += 2;
-  u64 *G = p.G, *P = p.P, *G2 = p.G2, *P2 = p.P2;
-  for (int l = 1; l <= NL_LEVELS; ++l) {
-    const int C = 32 >> (l - 1);
-    const int root = l == NL_LEVELS;
-    const long long nw = (long long)level_planes(l) * W;
-    launch_msb_gather(st, G, P, C, root, W, p.X[l], p.Y[l]);
-    g_launches += 1;
-    if ((rc = and_p(ctx, p.X[l], p.Y[l], nw, P_AND, make_obj(call_id, (u32)stage, (u32)l), p.Z[l], p.mb)))
-      return rc;
-    launch_msb_combine(st, G, p.Z[l], C, root, W, G2, P2);
-    g_launches += 1;
-    std::swap(G, G2);
-    std::swap(P, P2);
-  }
-  launch_msb_out(st, p.rbits, G, p.dpl + 63 * W, W, 1, p.ge);               // [d >= 0] = NOT msb
-  g_launches += 1;
-  // daBit and B2A
-  launch_prf_words(st, W, ctx->k01, make_tag(P_DABIT, C_R1), obj, p.r1w, 0ll);
-  launch_prf_words(st, W, ctx->k02, make_tag(P_DABIT, C_R2), obj, p.r2w, 0ll);
-  launch_prf_words(st, W, ctx->k12, make_tag(P_DABIT, C_M12), obj, p.r3w, 0ll);
-  if ((rc = bool_from_planes(ctx, p.r1w, p.r2w, p.r3w, W, p.rb))) return rc;
-  launch_bits_to_arith(st, p.r1w, np, 0, p.A1);
-  launch_bits_to_arith(st, p.r2w, np, 1, p.A2);
-  launch_bits_to_arith(st, p.r3w, np, 2, p.A3);
-  g_launches += 3;
-  if ((rc = mult_p(ctx, p.A1, p.A2, np, P_DA_MULT1, obj, p.t, p.ma))) return rc;
-  launch_lin_apb_m2c(st, 6 * np, p.A1, p.A2, p.t, p.rpd);
-  g_launches += 1;
-  if ((rc = mult_p(ctx, p.rpd, p.A3, np, P_DA_MULT2, obj, p.u, p.ma))) return rc;
-  launch_lin_apb_m2c(st, 6 * np, p.rpd, p.A3, p.u, p.rad);
-  launch_bxor(st, 6 * W, p.ge, p.rb, p.e);
-  g_launches += 2;
-  rec_core(ctx, p.e, W, p.recb, p.dbits, true);
-  launch_b2a_apply(st, p.dbits, p.rad, np, p.gea);
-  g_launches += 1;
+  g_launches += launch_cs_open_bit(st, k);
+  for (int l = 1; l <= NL_LEVELS; ++l) count_mult(ctx, level_planes(l) * W);
+  count_mult(ctx, np);   // the daBits' two products
+  count_mult(ctx, np);
+  rec_core(ctx, k.e, W, p.recb, p.dbits, true);
   // out = b + (a - b) [a >= b]
-  if ((rc = mult_p(ctx, p.d, p.gea, np, P_NL_MULT, obj, p.prod, p.ma))) return rc;
-  launch_addsub(st, 6 * np, b, p.prod, 0, out);
-  g_launches += 1;
+  g_launches += launch_cs_select(st, k);
+  count_mult(ctx, np);
   return cuda_check(ctx, "compare_select");
 }
 
@@ -2766,7 +2657,7 @@ int gf_verify(mpc_ctx* ctx, u64 vid, GfPlan& g, u64* trace) {
 struct NLPlan {
   int nst;
   CSPlan cs[2];
-  u64 *a[2], *b[2], *o[2];       // stage operands (6 x np each)
+  u64 *a, *b, *o;                // max-pool's first stage: operands and result (6 x np each)
   // batch 0: arithmetic products
   long long nm;
   u64 *MX, *MY, *MZ;
@@ -2793,16 +2684,16 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuni
   p.nst = nst;
   p.nm = 0;
   p.ne = 0;
-  long long andw = 0;
   for (int s = 0; s < nst; ++s) {
-    p.a[s] = a.take<u64>(6 * np[s]);
-    p.b[s] = a.take<u64>(6 * np[s]);
-    p.o[s] = a.take<u64>(6 * np[s]);
     p.cs[s] = plan_cs(a, np[s]);
     p.nm += 3 * np[s];
     p.ne += np[s];
-    andw += p.cs[s].and_words;
   }
+  const long long n0 = nst > 1 ? 6 * np[0] : 0;
+  p.a = a.take<u64>(n0);
+  p.b = a.take<u64>(n0);
+  p.o = a.take<u64>(n0);
+  const long long andw = AND_PLANES * (p.ne / 64);
   p.MX = a.take<u64>(6 * p.nm); p.MY = a.take<u64>(6 * p.nm); p.MZ = a.take<u64>(6 * p.nm);
   p.vm = plan_vmult(a, p.nm, -1);
   p.D1 = 64 * p.ne;
@@ -2819,15 +2710,27 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuni
   p.sb = plan_small(a);
   p.tb = plan_trunc(a, p.ne, p.Rb, tc, false, tu, true);
   p.Zr = a.take<u64>(384 * 64);
+  // each stage's part of the batches: its triples and its edaBits' bit words
+  long long e0 = 0;
+  for (int s = 0; s < nst; ++s) {
+    CompareSelect& k = p.cs[s].k;
+    k.nm = p.nm;
+    for (int q = 0; q < 3; ++q) {
+      const long long o = 3 * e0 + q * np[s];
+      k.mx[q] = p.MX + o;
+      k.my[q] = p.MY + o;
+      k.mz[q] = p.MZ + o;
+    }
+    k.eda[0] = p.tb.b1 + e0;
+    k.eda[1] = p.tb.b2 + e0;
+    k.ax = p.gf.XA;
+    k.ay = p.gf.YA;
+    k.az = p.gf.ZA;
+    k.and_words = andw;
+    k.and_off = AND_PLANES * (e0 / 64);
+    e0 += np[s];
+  }
   return p;
-}
-
-// copy component c of an n-element sharing into a concatenated sharing of total length tot at
-// offset off
-int append_sharing(mpc_ctx* ctx, const u64* src, long long n, u64* dst, long long tot, long long off) {
-  for (int c = 0; c < 6; ++c)
-    CK(cudaMemcpyAsync(dst + c * tot + off, src + c * n, (size_t)n * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  return MPC_OK;
 }
 
 int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
@@ -2835,18 +2738,6 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
   cudaStream_t st = ctx->st;
   // ---- batch 0: the daBit products (two) and the final product, stage by stage (the edaBit
   // bit products are batch 3)
-  long long off = 0;
-  for (int s = 0; s < p.nst; ++s) {
-    CSPlan& c = p.cs[s];
-    const u64* trip[3][3] = {{c.A1, c.A2, c.t}, {c.rpd, c.A3, c.u}, {c.d, c.gea, c.prod}};
-    const long long len[3] = {c.np, c.np, c.np};
-    for (int q = 0; q < 3; ++q) {
-      if ((rc = append_sharing(ctx, trip[q][0], len[q], p.MX, p.nm, off))) return rc;
-      if ((rc = append_sharing(ctx, trip[q][1], len[q], p.MY, p.nm, off))) return rc;
-      if ((rc = append_sharing(ctx, trip[q][2], len[q], p.MZ, p.nm, off))) return rc;
-      off += len[q];
-    }
-  }
   {
     VMultPlan& v = p.vm;
     const Small& s = v.s;
@@ -2873,8 +2764,8 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
     long long e0 = 0;
     for (int q = 0; q < p.nst; ++q) {   // the words and the claim
-      CSPlan& c = p.cs[q];
-      launch_eda_words(st, c.mbw, c.rp, c.np, e0, p.D1, p.Xe, p.Ye);
+      const CompareSelect& c = p.cs[q].k;
+      launch_eda_words(st, c.eda, c.eprod, c.np, e0, p.D1, p.Xe, p.Ye);
       launch_scalar_gr_sum(st, c.np, c.ez, c.np, 6, b.Rw + e0 * 64, s.zinit);
       g_launches += 1;
       e0 += c.np;
@@ -2886,22 +2777,7 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
   }
   u64* tr2 = tr1 ? tr1 + (long long)(p.R1 + 1) * TRACE_ROUND : nullptr;
   // ---- batch 2: every AND gate over GF(2^64), stage by stage, level by level
-  {
-    GfPlan& g = p.gf;
-    const long long nw = g.D / 64;
-    long long woff = 0;
-    for (int s = 0; s < p.nst; ++s) {
-      CSPlan& c = p.cs[s];
-      for (int l = 1; l <= NL_LEVELS; ++l) {
-        const long long lw = (long long)level_planes(l) * c.W;
-        if ((rc = append_sharing(ctx, c.X[l], lw, g.XA, nw, woff))) return rc;
-        if ((rc = append_sharing(ctx, c.Y[l], lw, g.YA, nw, woff))) return rc;
-        if ((rc = append_sharing(ctx, c.Z[l], lw, g.ZA, nw, woff))) return rc;
-        woff += lw;
-      }
-    }
-    if ((rc = gf_verify(ctx, vid, g, tr2))) return rc;
-  }
+  if ((rc = gf_verify(ctx, vid, p.gf, tr2))) return rc;
   u64* tr3 = tr2 ? tr2 + (long long)(p.gf.R + 1) * MPC_TRACE_GF_ROUND : nullptr;
   // ---- batch 3: the edaBit bit products b_{i,1} b_{i,2}, stage by stage (plane-major); x has
   // only the [r]_1 components and y only the [r]_2 ones, so the dense rounds take the
@@ -2912,21 +2788,14 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     reveal(ctx, P_VER_R, make_obj(vid, 3, 0), s, s.r);
     // 64 consecutive products are the bits of one word of the b1 and b2 planes
     TruncPlan& t = p.tb;
-    long long w0 = 0;
-    for (int q = 0; q < p.nst; ++q) {
-      CSPlan& c = p.cs[q];
-      CK(cudaMemcpyAsync(t.b1 + w0, c.b1w, (size_t)c.np * 8, cudaMemcpyDeviceToDevice, st));
-      CK(cudaMemcpyAsync(t.b2 + w0, c.b2w, (size_t)c.np * 8, cudaMemcpyDeviceToDevice, st));
-      w0 += c.np;
-    }
     launch_gr_powers(st, s.r, 64, t.V);                                   // V_j = r^j
     launch_gr_mul1(st, t.V + 63 * 64, s.r, s.aux + 64);                   // rho = r^64
     if ((rc = bit_tables(ctx, t, s, s.aux + 64))) return rc;
     CK(cudaMemsetAsync(p.Zr, 0, 384 * 512, st));
     CK(cudaMemsetAsync(t.zt + 384, 0, 384 * 8, st));
-    w0 = 0;
+    long long w0 = 0;
     for (int q = 0; q < p.nst; ++q) {
-      CSPlan& c = p.cs[q];
+      const CompareSelect& c = p.cs[q].k;
       launch_words_sums(st, c.eprod, 64 * c.np, c.np, t.Rtab + w0 * 64, p.Zr);
       w0 += c.np;
     }
@@ -2970,14 +2839,13 @@ int mpc_relu(mpc_ctx* ctx, uint64_t call_id, uint64_t verify_id, const uint64_t*
   NLPlan p = plan_nl(ar, 1, np, ctx->gemm_path == MPC_GEMM_LIMB_TC, ctx->tune);
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "relu: workspace too small");
   Phase phase(ctx, MPC_PROF_NONLINEAR);
-  cudaStream_t st = ctx->st;
-  CK(cudaMemsetAsync(p.a[0], 0, (size_t)6 * np[0] * 8, st));
-  CK(cudaMemsetAsync(p.b[0], 0, (size_t)6 * np[0] * 8, st));
-  if ((rc = append_sharing(ctx, xs, n, p.a[0], np[0], 0))) return rc;      // zero-padded x, b = 0
-  if ((rc = compare_select(ctx, call_id, 0, p.a[0], p.b[0], p.cs[0], p.o[0]))) return rc;
+  CompareSelect& k = p.cs[0].k;
+  k.a = {xs, n, n};
+  k.b = {nullptr, 0, 0};
+  k.out = out;
+  k.out_ld = k.out_n = n;
+  if ((rc = compare_select(ctx, call_id, 0, p.cs[0]))) return rc;
   if ((rc = verify_nl(ctx, verify_id, p, trace))) return rc;
-  for (int c = 0; c < 6; ++c)
-    CK(cudaMemcpyAsync(out + c * n, p.o[0] + c * np[0], (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
   if ((rc = cuda_check(ctx, "relu"))) return rc;
   return nl_finish(ctx);
 }
@@ -2997,22 +2865,23 @@ int mpc_maxpool2(mpc_ctx* ctx, uint64_t call_id, uint64_t verify_id, const uint6
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "maxpool2: workspace too small");
   Phase phase(ctx, MPC_PROF_NONLINEAR);
   cudaStream_t st = ctx->st;
-  for (int s = 0; s < 2; ++s) {
-    CK(cudaMemsetAsync(p.a[s], 0, (size_t)6 * np[s] * 8, st));
-    CK(cudaMemsetAsync(p.b[s], 0, (size_t)6 * np[s] * 8, st));
-  }
-  // stage 0 operands: left = [a ; c], right = [b ; d] of every window
-  launch_window_gather(st, xs, B * C, H, W, np[0], p.a[0], p.b[0]);
+  // stage 0 operands: left = [a ; c], right = [b ; d] of every window; stage 1: the two halves of its
+  // result
+  launch_window_gather(st, xs, B * C, H, W, np[0], p.a, p.b);
   g_launches += 1;
-  if ((rc = compare_select(ctx, call_id, 0, p.a[0], p.b[0], p.cs[0], p.o[0]))) return rc;
-  for (int c = 0; c < 6; ++c) {
-    CK(cudaMemcpyAsync(p.a[1] + c * np[1], p.o[0] + c * np[0], (size_t)nw * 8, cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpyAsync(p.b[1] + c * np[1], p.o[0] + c * np[0] + nw, (size_t)nw * 8, cudaMemcpyDeviceToDevice, st));
-  }
-  if ((rc = compare_select(ctx, call_id, 1, p.a[1], p.b[1], p.cs[1], p.o[1]))) return rc;
+  CompareSelect &k0 = p.cs[0].k, &k1 = p.cs[1].k;
+  k0.a = {p.a, np[0], 2 * nw};
+  k0.b = {p.b, np[0], 2 * nw};
+  k0.out = p.o;
+  k0.out_ld = np[0];
+  k0.out_n = 2 * nw;
+  k1.a = {p.o, np[0], nw};
+  k1.b = {p.o + nw, np[0], nw};
+  k1.out = out;
+  k1.out_ld = k1.out_n = nw;
+  for (int s = 0; s < 2; ++s)
+    if ((rc = compare_select(ctx, call_id, s, p.cs[s]))) return rc;
   if ((rc = verify_nl(ctx, verify_id, p, trace))) return rc;
-  for (int c = 0; c < 6; ++c)
-    CK(cudaMemcpyAsync(out + c * nw, p.o[1] + c * np[1], (size_t)nw * 8, cudaMemcpyDeviceToDevice, st));
   if ((rc = cuda_check(ctx, "maxpool2"))) return rc;
   return nl_finish(ctx);
 }

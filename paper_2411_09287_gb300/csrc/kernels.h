@@ -319,36 +319,47 @@ int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long
                       const unsigned char* TL8, long long L, long long nhi, u64* S_hi,
                       unsigned* err, unsigned err_flag);
 
-// ---- non-linear layers: Boolean sharings, AND gates, GF(2^64) (nonlinear.cu) ------------------
-void launch_and_offline(cudaStream_t st, const u64* xs, const u64* ys, long long nw, Key k01, Key k02,
-                        u32 purpose, u64 obj, u64* zs, u64* g2_out);
-void launch_and_online(cudaStream_t st, const u64* xs, const u64* ys, long long nw, Key k01,
-                       u32 purpose, u64 obj, const u64* g2_in, u64* p1_out, u64* p2_out);
-void launch_xor_finish(cudaStream_t st, long long nw, const u64* p1_own, const u64* p1_in,
-                       const u64* p2_own, const u64* p2_in, u64* zs);
-void launch_bits_to_arith(cudaStream_t st, const u64* bits, long long n, int kind, u64* out);
-void launch_lin_apb_m2c(cudaStream_t st, long long n, const u64* a, const u64* b, const u64* c, u64* out);
-void launch_eda_inner_offline(cudaStream_t st, long long np, Key k01, Key k02, u64 obj, u64* zs,
-                              u64* g2_out);
-void launch_eda_inner_online(cudaStream_t st, const u64* mbits, const u64* rp, long long np, Key k01,
-                             u64 obj, const u64* g2_in, u64* p1_out, u64* p2_out);
-void launch_eda_compose(cudaStream_t st, const u64* mbits, const u64* rp, const u64* z, long long np,
-                        u64* ra);
-void launch_msb_leaves(cudaStream_t st, const u64* rbits, const u64* dplanes, long long W, u64* G,
-                       u64* P);
-void launch_msb_gather(cudaStream_t st, const u64* G, const u64* P, int C, int root, long long W,
-                       u64* X, u64* Y);
-void launch_msb_combine(cudaStream_t st, const u64* G, const u64* Z, int C, int root, long long W,
-                        u64* Gout, u64* Pout);
-void launch_msb_out(cudaStream_t st, const u64* rbits, const u64* Groot, const u64* d63, long long W,
-                    int negate, u64* out);
-void launch_bxor(cudaStream_t st, long long n6, const u64* a, const u64* b, u64* out);
-void launch_b2a_apply(cudaStream_t st, const u64* dbits, const u64* ra, long long n, u64* out);
+// ---- compare-select of the non-linear layers (compare.cu) --------------------------------------
+struct CsView {          // component c of element e at p[c stride + e], 0 for e >= valid or p = null
+  const u64* p;
+  long long stride, valid;
+};
+struct MsgFault {        // word idx of a message XORed with mask (idx < 0: none)
+  long long idx;
+  u64 mask;
+};
+// One stage of np elements (a multiple of 64): out = max(a, b).
+struct CompareSelect {
+  CsView a, b;
+  u64* out;              // component c of element e < out_n at c out_ld + e
+  long long out_ld, out_n;
+  long long np;
+  Key k01, k02, k12;
+  u64 obj;               // the stage's stream object (AND level l: + l)
+  MsgFault fault[4];     // edaBit products' GAMMA2, MZ1, MZ2; the first AND level's [Gamma]_2
+  u64 *eda[3], *da[3];   // bit planes of the public-seed bits: np words each, np / 64 words each
+  u64 *eprod, *ez;       // edaBit products (6 x 64 np) and inner products (6 np)
+  u64* dd;               // 6 np: Delta's sharing to open
+  u64 *mx[3], *my[3], *mz[3];   // the daBit products' and the selection's triples, components nm apart
+  long long nm;
+  u64* rad;              // 6 np: the daBits' arithmetic sharing
+  const u64* dpl;        // the opened Delta's bit planes
+  u64 *ax, *ay, *az;     // AND triples, components and_words apart, this stage's from and_off
+  long long and_off, and_words;
+  u64* e;                // 6 np / 64: Boolean sharing to open
+  const u64* dbits;      // e opened
+};
+// The three parts around the openings of dd and e; each returns its number of launches.
+int launch_cs_open_delta(cudaStream_t st, const CompareSelect& a);
+int launch_cs_open_bit(cudaStream_t st, const CompareSelect& a);
+int launch_cs_select(cudaStream_t st, const CompareSelect& a);
+
+// ---- non-linear layers (nonlinear.cu) -----------------------------------------------------------
 void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int sub, u64* out);
 // The edaBit inner-product batch's ring words (see nonlinear.cu): bits m into xm, 2^(i+1) r' into y
 // (component c at c ldy), entry (e0 + e) 64 + i.
-void launch_eda_words(cudaStream_t st, const u64* mbits, const u64* rp, long long np, long long e0,
-                      long long ldy, u64* xm, u64* y);
+void launch_eda_words(cudaStream_t st, const u64* const bits[3], const u64* eprod, long long np,
+                      long long e0, long long ldy, u64* xm, u64* y);
 void launch_gather(cudaStream_t st, const u64* xs, long long n_in, const long long* idx,
                    long long n_out, u64* out);
 void launch_window_gather(cudaStream_t st, const u64* x, long long BC, long long H, long long W,
@@ -377,12 +388,6 @@ struct GfVerify {
 };
 // Returns the number of launches.
 int launch_gf_verify(cudaStream_t st, const GfVerify& a);
-// arithmetic Pi_Mult with the streams of `purpose` (prf_kernels.cu)
-void launch_mult_offline_p(cudaStream_t st, const u64* xs, const u64* ys, long long n, Key k01,
-                           Key k02, u32 purpose, u64 obj, u64* zs, u64* p0_out_g2);
-void launch_mult_online_p(cudaStream_t st, const u64* xs, const u64* ys, long long n, Key k01,
-                          u32 purpose, u64 obj, const u64* p2_in_g2, u64* p1_out, u64* p2_out);
-
 // ---- layer-level calls (layer_kernels.cu) ----------------------------------------------------
 // Geometry of a convolution: NCHW input (B, C, H, W), kh x kw kernel, stride, zero padding; the
 // output is Ho x Wo per image.
