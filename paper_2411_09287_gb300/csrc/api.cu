@@ -352,7 +352,7 @@ int gr_matmul(mpc_ctx* ctx, long long R, const u64* p0, const u64* p1, u64 s1, l
 // C = A B (+ epilogue) for a one-term product that the limb path runs on the tensor cores
 // (scratch: limb_tc_scratch_bytes(M, N, K, 1) bytes) and the u64 path on the CUDA cores.
 int dense_gemm(mpc_ctx* ctx, long long M, long long N, long long K, const GemmTerm& T,
-               const Epi& e, void* scratch) {
+               const Epi& e, void* scratch, const GemmGroups& groups = GemmGroups{}) {
   if (scratch && !e.atomic) {
     g_launches += 4;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -362,7 +362,7 @@ int dense_gemm(mpc_ctx* ctx, long long M, long long N, long long K, const GemmTe
       ctx->recs.push_back({MPC_PROF_K_LIMB_GEMM, e0, e1, (double)M * N * K});
     }
     if (limb_gemm_tc(ctx->st, M, N, K, 1, &T, e, scratch, ctx->status, ST_TIMEOUT, e0, e1,
-                     ctx->tune.gemm_split_min))
+                     ctx->tune.gemm_split_min, groups))
       return fail(ctx, MPC_ERR_CUDA, "tensor-core GEMM setup failed");
     return MPC_OK;
   }
@@ -1096,7 +1096,12 @@ struct VMatPlan {
   bool trunc = false;
   TruncBatch tb;
   void* tcs = nullptr;            // tensor-core digit planes (limb path only)
+  bool grouped = false;           // X^T P and W Q of all six components as one product each
 };
+// Words of a grouped operand at most (256 MB of digit planes).  Below, a product of one component is
+// a few CTAs and its four launches take longer than its work (17 products of a layer: 1.67 ms a
+// verified product of 64 x 64 x 128, 1.32 ms with seven); above, each fills the GPU.
+constexpr long long GROUPED_MAX = 1ll << 24;
 
 // Layout decisions of a truncation chunk of E outputs (no allocation).
 struct TruncShape {
@@ -1253,8 +1258,11 @@ bool plan_vmat(Arena& a, long long M, long long N, long long K, int t, int R0, i
   if (p.trunc && (trunc_tcs = trunc_batch_tcs(E, R1, tc, tu)) < 0) return false;
   // digit planes of the batch-0 products (X^T P, W Q, Z Q) and of the truncation chunks'
   // tensor-core products, on the tensor-core path
+  const long long G = 6 * (K + 1);
+  p.grouped = tc && G * std::max(M, N) <= GROUPED_MAX;
   p.tcs = tc ? (void*)a.take<unsigned char>((long long)std::max(
-                   {limb_tc_scratch_bytes(K, 64, M, 1), limb_tc_scratch_bytes(K, 64, N, 1),
+                   {limb_tc_scratch_bytes(p.grouped ? G : K, 64, M, 1),
+                    limb_tc_scratch_bytes(p.grouped ? G : K, 64, N, 1),
                     limb_tc_scratch_bytes(6 * M, 64, N, 1), (size_t)trunc_tcs}))
              : nullptr;
   p.Q = a.take<u64>(N * 64);
@@ -2187,7 +2195,16 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
   if ((rc = power_table(ctx, s.aux, p.powP, p.P, s.aux + 64))) return rc; // rho^a
   Vec& x = p.dv.x[0];
   Vec& y = p.dv.y[0];
-  for (int c = 0; c < 6; ++c) {
+  if (p.grouped) {   // all six components of a side in one product: rows c (K + 1) + k, row K zero
+    GemmTerm T;
+    T.A = op(xs, K, 1);
+    T.B = op(p.P, 64);
+    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, M, T, epi_store(x.c[0], 64), p.tcs, {K + 1, MK}))) return rc;
+    T.A = op(ws_, N);
+    T.B = op(p.Q, 64);
+    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, N, T, epi_store(y.c[0], 64), p.tcs, {K + 1, KN}))) return rc;
+  }
+  for (int c = 0; c < 6 && !p.grouped; ++c) {
     GemmTerm T;
     T.A = op(xs + c * MK, K, 1);        // Xt_k = sum_a rho^a X_ak  (K x M) . (M x 64)
     T.B = op(p.P, 64);

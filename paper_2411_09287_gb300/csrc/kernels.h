@@ -51,15 +51,21 @@ void gemm_u64(cudaStream_t st, long long M, long long N, long long K, int nterms
               const GemmTerm* terms, const Epi& epi, int nsplit);
 
 // ---- exact u64 GEMM on the tcgen05 tensor cores (limb_gemm_tc.cu) ---------------------------
-// Same contract as gemm_u64 without split-K (epi.atomic must be 0; returns -1 otherwise, -2 if
+// Same contract as gemm_u64 without split-K (epi.atomic must be 0; returns -1 otherwise and
+// for terms of different layouts, -2 if
 // the tensor maps cannot be encoded).  scratch: limb_tc_scratch_bytes(M, N, K, nterms) bytes,
 // 256-byte aligned (the bf16 digit planes of both operands).  A bounded wait that expires
 // sets err_flag in *err and leaves the output undefined.
 size_t limb_tc_scratch_bytes(long long M, long long N, long long K, int nterms);
 // ev0 / ev1 (may be null) are recorded on st around the tensor-core kernel alone.
+// Groups of A's rows: row r is row r % rows of group r / rows, the groups `stride` words apart and the
+// last row of each zeros (rows = 0: no groups).
+struct GemmGroups {
+  long long rows = 0, stride = 0;
+};
 int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nterms,
                  const GemmTerm* terms, const Epi& epi, void* scratch, unsigned* err,
-                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min = 0);
+                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min = 0, const GemmGroups& groups = GemmGroups{});
 
 // Row map of a GR matrix product: logical row rho sits at word offset (rho % q) s1 + (rho / q) s2
 // (q = 0: rho s1).  q must be a multiple of 128.

@@ -332,10 +332,7 @@ k_limb_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }
 
 // ---- digit split ------------------------------------------------------------------------------
-__device__ __forceinline__ u64 load_opnd(const Opnd& o, long long r, long long c, long long R,
-                                         long long Cn) {
-  if (r >= R || c >= Cn) return 0;
-  const long long off = o.trans ? (c * o.ld + r) : (r * o.ld + c);
+__device__ __forceinline__ u64 load_opnd(const Opnd& o, long long off) {
   u64 v = o.p0[off];
   if (o.p1) {
     const u64 w = o.p1[off];
@@ -343,6 +340,14 @@ __device__ __forceinline__ u64 load_opnd(const Opnd& o, long long r, long long c
   }
   if (o.scale != 1ull) v = (o.scale == ~0ull) ? (0ull - v) : o.scale * v;
   return v;
+}
+// Word offset of an operand's row r (without the K index); false: a row of zeros.
+__device__ __forceinline__ bool row_base(const GemmGroups& g, long long r, long long R, long long pitch,
+                                         long long* off) {
+  if (r >= R) return false;
+  const long long c = g.rows ? r / g.rows : 0, q = r - c * g.rows;
+  *off = c * g.stride + q * pitch;
+  return !g.rows || q < g.rows - 1;
 }
 
 // 8 consecutive u64 values -> 8 digit planes of 8 f16 each (one 16-byte unit per plane).
@@ -403,51 +408,52 @@ __device__ __forceinline__ uint4 bits_plane0(unsigned bits) {
 }
 
 // planes[i][row][k'] (f16), row-major with pitch Kp; element (row, k') of the concatenated
-// operand: term t = k' / K, column k' mod K; values beyond nterms*K are zero.
-__global__ void k_split_digits(GemmTerm t0, GemmTerm t1, int nterms, int which /*0 A, 1 B*/,
-                               long long R, long long K, long long Kp,
-                               unsigned short* __restrict__ planes) {
+// operand: term t = k' / K, column k' mod K; values beyond nterms*K are zero.  For operands whose
+// words run along K (A with trans = 0, B with trans = 1): consecutive threads take consecutive k.
+__global__ void k_split_digits(Opnd o0, Opnd o1, int nterms, GemmGroups g, long long R, long long K,
+                               long long Kp, unsigned short* __restrict__ planes) {
   const long long chunks = Kp / 8;
   const long long total = R * chunks;
   for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < total;
        w += (long long)gridDim.x * blockDim.x) {
-    // consecutive threads take consecutive rows for B (coalesced column reads of a row-major
-    // K x N operand) and consecutive k chunks for A
-    long long row, kc;
-    if (which) { row = w % R; kc = w / R; } else { row = w / chunks; kc = w % chunks; }
+    const long long row = w / chunks, kc = w % chunks;
     u64 v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const long long kk = kc * 8 + q;
       v[q] = 0;
       if (kk < (long long)nterms * K) {
-        const GemmTerm& T = (kk < K) ? t0 : t1;
-        const long long k = kk < K ? kk : kk - K;
-        v[q] = which ? load_opnd(T.B, k, row, K, R) : load_opnd(T.A, row, k, R, K);
+        const Opnd& o = kk < K ? o0 : o1;
+        long long off;
+        if (row_base(g, row, R, o.ld, &off)) v[q] = load_opnd(o, off + (kk < K ? kk : kk - K));
       }
     }
     split8_store(v, reinterpret_cast<unsigned char*>(planes + row * Kp + kc * 8), R * Kp * 2, 0);
   }
 }
 
-// The B split for a row-major K x R source (trans = 0): a 64 k x 32 r block goes through shared
-// memory, so that the reads run along r and every plane row gets 128 contiguous bytes per 8
-// threads (the direct split writes one 16-byte unit per row and thread).
+// The split for operands whose words run along the rows (A with trans = 1, B with trans = 0): a 64 k x
+// 32 row block goes through shared memory, so that the reads run along the rows and every plane row
+// gets 128 contiguous bytes per 8 threads (the direct split reads 8 bytes of each sector it touches
+// and, over rows, writes one 16-byte unit per row and thread).
 __global__ void __launch_bounds__(256)
-k_split_digits_bt(GemmTerm t0, GemmTerm t1, int nterms, long long R, long long K, long long Kp,
-                  unsigned short* __restrict__ planes) {
+k_split_digits_t(Opnd o0, Opnd o1, int nterms, GemmGroups g, long long R, long long K, long long Kp,
+                 unsigned short* __restrict__ planes) {
   __shared__ u64 tile[32][65];
-  const long long r0 = (long long)blockIdx.x * 32;
-  const long long k0 = (long long)blockIdx.y * 64;
+  const unsigned nr = (unsigned)((R + 31) / 32);   // row blocks run fastest
+  const long long r0 = (long long)(blockIdx.x % nr) * 32;
+  const long long k0 = (long long)(blockIdx.x / nr) * 64;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  long long base;
+  const bool ok = row_base(g, r0 + lane, R, 1, &base);
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int kl = w * 8 + j;
     const long long kk = k0 + kl;
     u64 v = 0;
-    if (kk < (long long)nterms * K && r0 + lane < R) {
-      const GemmTerm& T = (kk < K) ? t0 : t1;
-      v = load_opnd(T.B, kk < K ? kk : kk - K, r0 + lane, K, R);
+    if (ok && kk < (long long)nterms * K) {
+      const Opnd& o = kk < K ? o0 : o1;
+      v = load_opnd(o, base + (kk < K ? kk : kk - K) * o.ld);
     }
     tile[lane][kl] = v;
   }
@@ -459,6 +465,19 @@ k_split_digits_bt(GemmTerm t0, GemmTerm t1, int nterms, long long R, long long K
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = tile[rl][kc * 8 + q];
     split8_store(v, reinterpret_cast<unsigned char*>(planes + r * Kp + kk0), R * Kp * 2, 0);
+  }
+}
+
+// Splits one operand of R rows; along_k: its words run along K.
+void split_operand(cudaStream_t st, const Opnd& o0, const Opnd& o1, int nterms, bool along_k,
+                   const GemmGroups& g, long long R, long long K, long long Kp, unsigned short* planes) {
+  if (along_k) {
+    long long n = (R * (Kp / 8) + 255) / 256;
+    if (n > (1 << 20)) n = 1 << 20;
+    k_split_digits<<<(unsigned)n, 256, 0, st>>>(o0, o1, nterms, g, R, K, Kp, planes);
+  } else {
+    const long long n = ((R + 31) / 32) * ((Kp + 63) / 64);
+    k_split_digits_t<<<(unsigned)n, 256, 0, st>>>(o0, o1, nterms, g, R, K, Kp, planes);
   }
 }
 
@@ -1726,25 +1745,18 @@ size_t limb_tc_scratch_bytes(long long M, long long N, long long K, int nterms) 
 
 int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nterms,
                  const GemmTerm* terms, const Epi& epi, void* scratch, unsigned* err,
-                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min) {
+                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min,
+                 const GemmGroups& groups) {
   if (M <= 0 || N <= 0) return 0;
-  if (epi.atomic) return -1;
+  const GemmTerm& t1 = nterms > 1 ? terms[1] : terms[0];
+  if (epi.atomic || t1.A.trans != terms[0].A.trans || t1.B.trans != terms[0].B.trans) return -1;
   const long long Kp = ((nterms * K + TC_BK - 1) / TC_BK) * TC_BK;
   unsigned short* Ap = reinterpret_cast<unsigned short*>(scratch);
   const long long abytes = (8 * M * Kp * 2 + 255) & ~255ll;
   unsigned short* Bp = reinterpret_cast<unsigned short*>(reinterpret_cast<char*>(scratch) + abytes);
-  GemmTerm t1 = nterms > 1 ? terms[1] : terms[0];
-  const int tpb = 256;
-  long long ga = (M * (Kp / 8) + tpb - 1) / tpb, gb = (N * (Kp / 8) + tpb - 1) / tpb;
-  if (ga > (1 << 20)) ga = 1 << 20;
-  if (gb > (1 << 20)) gb = 1 << 20;
-  k_split_digits<<<(unsigned)ga, tpb, 0, st>>>(terms[0], t1, nterms, 0, M, K, Kp, Ap);
-  if (terms[0].B.trans == 0 && t1.B.trans == 0 && (Kp + 63) / 64 <= 65535) {
-    dim3 g2((unsigned)((N + 31) / 32), (unsigned)((Kp + 63) / 64));
-    k_split_digits_bt<<<g2, 256, 0, st>>>(terms[0], t1, nterms, N, K, Kp, Bp);
-  } else {
-    k_split_digits<<<(unsigned)gb, tpb, 0, st>>>(terms[0], t1, nterms, 1, N, K, Kp, Bp);
-  }
+  // the terms of a product have one layout per side
+  split_operand(st, terms[0].A, t1.A, nterms, !terms[0].A.trans, groups, M, K, Kp, Ap);
+  split_operand(st, terms[0].B, t1.B, nterms, terms[0].B.trans, GemmGroups{}, N, K, Kp, Bp);
   CUtensorMap ma, mb;
   if (!make_map(&ma, Ap, M, Kp, TC_BM) || !make_map(&mb, Bp, N, Kp, TC_BN)) return -2;
   const size_t smem = (size_t)NSTAGE * STAGE + (size_t)NDRAIN * 32 * 48 + 1024;
