@@ -915,6 +915,8 @@ int power_table(mpc_ctx* ctx, const u64* r, const PowPlan& p, u64* table, u64* a
 // A batch of weighted ring words (gr_block.cu): x_i = R_{b >> sh} T_j X_i, y_i = lift(Y_i), i =
 // B b + j < D, whose first kap = log2(B) rounds need no GR vectors.
 constexpr int BLK_ROUNDS = 3;
+// Blocks from which the sums go to the tensor cores (@BLKMIN@).
+constexpr long long BLK_TC_MIN = 8192;
 struct BlkPlan {
   long long D, nb;        // words, blocks
   long long nw, nwp;      // weight rows R, rounded up to whole tiles
@@ -975,7 +977,21 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
   in.D = p.D;
   // parties 1 and 2 only: their matrices sit where those of a full batch's first two would
   const int np = p.full ? 3 : 2, p0 = p.full ? 0 : 1;
-  if (p.full || p.kap > 0) launch_blk_sums(st, in, B, p.full, p.nb, p.sh, p.Rw, p.S);
+  // long batches on the tensor cores; the digit planes (4864 bytes a block at most) lie in the
+  // vectors' storage (4096 or 6144 bytes a block), which is written after the rounds
+  bool sums = !(p.full || p.kap > 0);
+  if (!sums && ctx->gemm_path == MPC_GEMM_LIMB_TC && B == 8 && p.nb >= BLK_TC_MIN &&
+      p.sh == (p.full ? 0 : 3)) {
+    g_launches += 3;
+    u64* planes = p.dv.x[0].c[p.full ? 0 : 2];
+    sums = blk_sums_tc(st, in, p.full, p.nw, p.Rw, p.S, planes, ctx->status, ST_TIMEOUT,
+                       ctx->tune.gemm_split_min) == 0;
+    if (!sums) {
+      g_launches -= 3;
+      CK(cudaMemsetAsync(p.S, 0, (size_t)blk_rows(B, p.full) * 512, st));
+    }
+  }
+  if (!sums) launch_blk_sums(st, in, B, p.full, p.nb, p.sh, p.Rw, p.S);
   if (p.full) {
     CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
     launch_blk_claim(st, p.T, p.S + 3ll * B * B * 64, B, s.zinit);
@@ -2199,10 +2215,10 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
     GemmTerm T;
     T.A = op(xs, K, 1);
     T.B = op(p.P, 64);
-    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, M, T, epi_store(x.c[0], 64), p.tcs, {K + 1, MK}))) return rc;
+    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, M, T, epi_store(x.c[0], 64), p.tcs, {K + 1, K, MK}))) return rc;
     T.A = op(ws_, N);
     T.B = op(p.Q, 64);
-    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, N, T, epi_store(y.c[0], 64), p.tcs, {K + 1, KN}))) return rc;
+    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, N, T, epi_store(y.c[0], 64), p.tcs, {K + 1, K, KN}))) return rc;
   }
   for (int c = 0; c < 6 && !p.grouped; ++c) {
     GemmTerm T;
@@ -2694,7 +2710,11 @@ struct NLPlan {
   Small sb;
   TruncPlan tb;                  // bit words of 64 products each
   u64* Zr;                       // 6 x 64 elements: the claim's sums over the bit words
+  void* wsum = nullptr;          // digit planes for them (long batches on the limb path)
 };
+
+// Elements of a stage from which the sums over its bit words go to the tensor cores (@WMIN@).
+constexpr long long WORDS_TC_MIN = 4096;
 
 NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuning& tu) {
   NLPlan p;
@@ -2727,6 +2747,8 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuni
   p.sb = plan_small(a);
   p.tb = plan_trunc(a, p.ne, p.Rb, tc, false, tu, true);
   p.Zr = a.take<u64>(384 * 64);
+  if (tc && np[0] >= WORDS_TC_MIN)
+    p.wsum = a.take<unsigned char>((long long)limb_tc_scratch_bytes(384, 64, np[0], 1));
   // each stage's part of the batches: its triples and its edaBits' bit words
   long long e0 = 0;
   for (int s = 0; s < nst; ++s) {
@@ -2808,15 +2830,24 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     launch_gr_powers(st, s.r, 64, t.V);                                   // V_j = r^j
     launch_gr_mul1(st, t.V + 63 * 64, s.r, s.aux + 64);                   // rho = r^64
     if ((rc = bit_tables(ctx, t, s, s.aux + 64))) return rc;
-    CK(cudaMemsetAsync(p.Zr, 0, 384 * 512, st));
     CK(cudaMemsetAsync(t.zt + 384, 0, 384 * 8, st));
     long long w0 = 0;
     for (int q = 0; q < p.nst; ++q) {
       const CompareSelect& c = p.cs[q].k;
-      launch_words_sums(st, c.eprod, 64 * c.np, c.np, t.Rtab + w0 * 64, p.Zr);
+      // sum over w of rho^w z_c[64 w + j] for the 384 rows (c, j)
+      if (p.wsum) {
+        GemmTerm T;
+        T.A = op(c.eprod, 64, 1);
+        T.B = op(t.Rtab + w0 * 64, 64);
+        if ((rc = dense_gemm(ctx, 384, 64, c.np, T, epi_store(p.Zr, 64), p.wsum, {64, 64, 64 * c.np})))
+          return rc;
+      } else {
+        CK(cudaMemsetAsync(p.Zr, 0, 384 * 512, st));
+        launch_words_sums(st, c.eprod, 64 * c.np, c.np, t.Rtab + w0 * 64, p.Zr);
+      }
+      launch_blk_claim(st, t.V, p.Zr, 64, t.zt + 384);
       w0 += c.np;
     }
-    launch_blk_claim(st, t.V, p.Zr, 64, t.zt + 384);
     if ((rc = bit_batch(ctx, t, s, t.zt + 384, vid, 3, tr3))) return rc;
   }
   return MPC_OK;

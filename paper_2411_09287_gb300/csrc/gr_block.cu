@@ -164,36 +164,53 @@ k_blk_claim(const u64* __restrict__ T, const u64* __restrict__ Zr, int n, u64* _
 }
 
 // out_c[b] = sum_{j < B} in_c[B b + j] G_j, G_j row (b >> sh) B + j of Gt (ROWS) or row j for every
-// b, for the present components (words at or past D read as 0).  64 threads an element; bound by
-// the rows written (and read).
-template <int B, bool ROWS>
+// b, for the present components (words at or past D read as 0).  A warp takes an element, two
+// coefficients a lane; VEC: 16-byte loads of the words (16-byte aligned components, B even).  Bound by
+// the rows written; with 64 threads an element and a load a word it was bound by those loads (a load
+// for each multiply-add): 264 us for 131072 edaBit blocks, now 182 us.
+template <int B, bool ROWS, bool VEC>
 __global__ void __launch_bounds__(256)
 k_blk_combine(const BlkVec in, const BlkOut out, long long D, long long nb, int sh,
               const u64* __restrict__ Gt) {
-  const int t = threadIdx.x & 63;
-  const long long stride = (long long)gridDim.x * 4;
-  u64 G[B];
-  if (!ROWS) {
+  const int t = threadIdx.x & 31;
+  const long long stride = (long long)gridDim.x * 8;
+  u64 G[B][2];
+  auto load_g = [&](const u64* g) {
 #pragma unroll
-    for (int j = 0; j < B; ++j) G[j] = Gt[j * 64 + t];
-  }
-  for (long long b = (long long)blockIdx.x * 4 + (threadIdx.x >> 6); b < nb; b += stride) {
-    if (ROWS) {
-#pragma unroll
-      for (int j = 0; j < B; ++j) G[j] = Gt[((b >> sh) * B + j) * 64 + t];
+    for (int j = 0; j < B; ++j) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(g + j * 64 + 2 * t);
+      G[j][0] = v.x;
+      G[j][1] = v.y;
     }
+  };
+  if (!ROWS) load_g(Gt);
+  for (long long b = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); b < nb; b += stride) {
+    if (ROWS) load_g(Gt + (b >> sh) * B * 64);
     const bool whole = (b + 1) * B <= D;
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       const u64* w = in.c[c];
       if (!w) continue;
-      u64 v = 0;
+      w += b * B;
+      u64 s[B];
+      if (VEC && whole) {
+#pragma unroll
+        for (int j = 0; j < B; j += 2) {
+          const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(w + j));
+          s[j] = v.x;
+          s[j + 1 < B ? j + 1 : j] = v.y;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < B; ++j) s[j] = (whole || b * B + j < D) ? __ldg(w + j) : 0ull;
+      }
+      u64 v0 = 0, v1 = 0;
 #pragma unroll
       for (int j = 0; j < B; ++j) {
-        const u64 s = (whole || b * B + j < D) ? __ldg(w + b * B + j) : 0ull;
-        v += s * G[j];
+        v0 += s[j] * G[j][0];
+        v1 += s[j] * G[j][1];
       }
-      out.c[c][b * 64 + t] = v;
+      *reinterpret_cast<ulonglong2*>(out.c[c] + b * 64 + 2 * t) = make_ulonglong2(v0, v1);
     }
   }
 }
@@ -241,19 +258,23 @@ void launch_blk_claim(cudaStream_t st, const u64* T, const u64* Zr, int n, u64* 
 
 void launch_blk_combine(cudaStream_t st, const BlkVec& in, const BlkOut& out, int B, bool rows,
                         long long D, long long nb, int sh, const u64* G) {
-  long long g = (nb + 3) / 4;
+  long long g = (nb + 7) / 8;
   if (g > 152 * 8) g = 152 * 8;
+  bool vec = B == 8;   // 16-byte loads of all components, or of none
+  for (int c = 0; c < 6; ++c) vec = vec && (reinterpret_cast<uintptr_t>(in.c[c]) & 15) == 0;
   auto go = [&](auto kern) { kern<<<(unsigned)g, 256, 0, st>>>(in, out, D, nb, sh, G); };
   if (rows) {
-    if (B == 1) go(k_blk_combine<1, true>);
-    else if (B == 2) go(k_blk_combine<2, true>);
-    else if (B == 4) go(k_blk_combine<4, true>);
-    else go(k_blk_combine<8, true>);
+    if (B == 1) go(k_blk_combine<1, true, false>);
+    else if (B == 2) go(k_blk_combine<2, true, false>);
+    else if (B == 4) go(k_blk_combine<4, true, false>);
+    else if (vec) go(k_blk_combine<8, true, true>);
+    else go(k_blk_combine<8, true, false>);
   } else {
-    if (B == 1) go(k_blk_combine<1, false>);
-    else if (B == 2) go(k_blk_combine<2, false>);
-    else if (B == 4) go(k_blk_combine<4, false>);
-    else go(k_blk_combine<8, false>);
+    if (B == 1) go(k_blk_combine<1, false, false>);
+    else if (B == 2) go(k_blk_combine<2, false, false>);
+    else if (B == 4) go(k_blk_combine<4, false, false>);
+    else if (vec) go(k_blk_combine<8, false, true>);
+    else go(k_blk_combine<8, false, false>);
   }
 }
 

@@ -59,9 +59,9 @@ void gemm_u64(cudaStream_t st, long long M, long long N, long long K, int nterms
 size_t limb_tc_scratch_bytes(long long M, long long N, long long K, int nterms);
 // ev0 / ev1 (may be null) are recorded on st around the tensor-core kernel alone.
 // Groups of A's rows: row r is row r % rows of group r / rows, the groups `stride` words apart and the
-// last row of each zeros (rows = 0: no groups).
+// rows from `valid` on zeros (rows = 0: no groups).
 struct GemmGroups {
-  long long rows = 0, stride = 0;
+  long long rows = 0, valid = 0, stride = 0;
 };
 int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nterms,
                  const GemmTerm* terms, const Epi& epi, void* scratch, unsigned* err,
@@ -303,6 +303,12 @@ int blk_rows(int B, bool full);
 // the rows are those of parties 1 and 2.
 void launch_blk_sums(cudaStream_t st, const BlkIn& in, int B, bool full, long long nb, int sh,
                      const u64* R, u64* out);
+// The same sums for full batches (B = 8, sh = 0) and the edaBits' (B = 8, sh = 3) on the tensor cores:
+// a product of the blocks' words (nw columns, those of a weight added) and R.  scratch:
+// blk_sums_tc_bytes(full, nw), 256-byte aligned; 0, or not 0 when the tensor maps cannot be encoded.
+size_t blk_sums_tc_bytes(bool full, long long nw);
+int blk_sums_tc(cudaStream_t st, const BlkIn& in, bool full, long long nw, const u64* R, u64* out,
+                void* scratch, unsigned* err, unsigned err_flag, int split_min);
 // out[c][j] (6 x 64 elements, accumulated) = sum over w < nw of R[w] z[c ldz + 64 w + j].
 void launch_words_sums(cudaStream_t st, const u64* z, long long ldz, long long nw, const u64* R,
                        u64* out);

@@ -347,7 +347,7 @@ __device__ __forceinline__ bool row_base(const GemmGroups& g, long long r, long 
   if (r >= R) return false;
   const long long c = g.rows ? r / g.rows : 0, q = r - c * g.rows;
   *off = c * g.stride + q * pitch;
-  return !g.rows || q < g.rows - 1;
+  return !g.rows || q < g.valid;
 }
 
 // 8 consecutive u64 values -> 8 digit planes of 8 f16 each (one 16-byte unit per plane).
@@ -479,6 +479,78 @@ void split_operand(cudaStream_t st, const Opnd& o0, const Opnd& o1, int nterms, 
     const long long n = ((R + 31) / 32) * ((Kp + 63) / 64);
     k_split_digits_t<<<(unsigned)n, 256, 0, st>>>(o0, o1, nterms, g, R, K, Kp, planes);
   }
+}
+
+// Digit planes of the block words of a full batch (gr_block.cu): row (p, j, j') < 192 the party's word
+// word^p_{b,j,j'}, row 192 + 8 c + j the claim's Z_c[8 b + j], column b < Kp (zero past the batch).  A
+// block takes 32 b: their words, with the parties' sums of shares, in shared memory (padded so that
+// the four groups of eight b that a half-warp reads lie in different banks), then eight columns of a
+// row a thread.  Bound by the writes (3840 bytes a block of eight triples).
+__global__ void __launch_bounds__(256)
+k_blk_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) {
+  constexpr int LD = 4 * 68;
+  __shared__ u64 a[16][LD];   // X0+X1, Y0+Y1, X2, Y3, X3, Y2, X4, Y4-Y5, X5, Y4, Z0 .. Z5
+  const long long b0 = (long long)blockIdx.x * 32;
+  const int tid = threadIdx.x;
+  {
+    const long long i = b0 * 8 + tid;
+    const bool ok = i < in.D;
+    u64 x[6], y[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      x[c] = ok ? in.x[c][i] : 0ull;
+      y[c] = ok ? in.y[c][i] : 0ull;
+    }
+    const int o = tid + 4 * (tid >> 6);
+    a[0][o] = x[0] + x[1]; a[1][o] = y[0] + y[1];
+    a[2][o] = x[2]; a[3][o] = y[3]; a[4][o] = x[3]; a[5][o] = y[2];
+    a[6][o] = x[4]; a[7][o] = y[4] - y[5]; a[8][o] = x[5]; a[9][o] = y[4];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) a[10 + c][o] = ok ? in.z[c * in.ldz + i] : 0ull;
+  }
+  __syncthreads();
+  for (int u = tid; u < 240 * 4; u += 256) {
+    const int g = u & 3, row = u >> 2, p = row >> 6, j = g * 68 + ((row >> 3) & 7), k = g * 68 + (row & 7);
+    u64 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (p == 0) v[q] = a[0][j + 8 * q] * a[1][k + 8 * q];
+      else if (p == 1) v[q] = 0ull - (a[2][j + 8 * q] * a[3][k + 8 * q] + a[4][j + 8 * q] * a[5][k + 8 * q]);
+      else if (p == 2) v[q] = a[6][j + 8 * q] * a[7][k + 8 * q] - a[8][j + 8 * q] * a[9][k + 8 * q];
+      else v[q] = a[10 + ((row - 192) >> 3)][k + 8 * q];
+    }
+    split8_store(v, reinterpret_cast<unsigned char*>(planes + row * Kp + b0 + g * 8), 240 * Kp * 2, 0);
+  }
+}
+
+// The same for the edaBits' inner products (x has components 2 and 4 only): rows (p, j, j') of the
+// parties 1 and 2, column e the sum over the eight blocks of element e, which share a weight.
+__global__ void __launch_bounds__(256)
+k_eda_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) {
+  __shared__ u64 a[4][16 * 64];   // X2, Y3, X4, Y4 - Y5 of 16 elements
+  const long long e0 = (long long)blockIdx.x * 16;
+  const int tid = threadIdx.x;
+  for (int o = tid; o < 1024; o += 256) {
+    const long long i = e0 * 64 + o;
+    const bool ok = i < in.D;
+    a[0][o] = ok ? in.x[2][i] : 0ull;
+    a[1][o] = ok ? in.y[3][i] : 0ull;
+    a[2][o] = ok ? in.x[4][i] : 0ull;
+    a[3][o] = ok ? in.y[4][i] - in.y[5][i] : 0ull;
+  }
+  __syncthreads();
+  const int g = tid & 1, row = tid >> 1, p = row >> 6, j = (row >> 3) & 7, k = row & 7;
+  const u64* x = a[2 * p] + g * 512 + j;
+  const u64* y = a[2 * p + 1] + g * 512 + k;
+  u64 v[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    u64 t = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) t += x[e * 64 + 8 * q] * y[e * 64 + 8 * q];
+    v[e] = p == 0 ? 0ull - t : t;
+  }
+  split8_store(v, reinterpret_cast<unsigned char*>(planes + row * Kp + e0 + g * 8), 128 * Kp * 2, 0);
 }
 
 // out[i] = acc_sign*out[i] + add0 + add1 + prf_sign*PRF(i) (the protocol epilogue of gemm_u64).
@@ -1743,20 +1815,10 @@ size_t limb_tc_scratch_bytes(long long M, long long N, long long K, int nterms) 
   return (size_t)(((a + 255) & ~255ll) + ((b + 255) & ~255ll) + 256);
 }
 
-int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nterms,
-                 const GemmTerm* terms, const Epi& epi, void* scratch, unsigned* err,
-                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min,
-                 const GemmGroups& groups) {
-  if (M <= 0 || N <= 0) return 0;
-  const GemmTerm& t1 = nterms > 1 ? terms[1] : terms[0];
-  if (epi.atomic || t1.A.trans != terms[0].A.trans || t1.B.trans != terms[0].B.trans) return -1;
-  const long long Kp = ((nterms * K + TC_BK - 1) / TC_BK) * TC_BK;
-  unsigned short* Ap = reinterpret_cast<unsigned short*>(scratch);
-  const long long abytes = (8 * M * Kp * 2 + 255) & ~255ll;
-  unsigned short* Bp = reinterpret_cast<unsigned short*>(reinterpret_cast<char*>(scratch) + abytes);
-  // the terms of a product have one layout per side
-  split_operand(st, terms[0].A, t1.A, nterms, !terms[0].A.trans, groups, M, K, Kp, Ap);
-  split_operand(st, terms[0].B, t1.B, nterms, terms[0].B.trans, GemmGroups{}, N, K, Kp, Bp);
+// C = A B from digit planes (and the epilogue, when it has any terms)
+int limb_gemm_planes(cudaStream_t st, long long M, long long N, long long Kp, unsigned short* Ap,
+                     unsigned short* Bp, const Epi& epi, unsigned* err, unsigned err_flag,
+                     cudaEvent_t ev0, cudaEvent_t ev1, int split_min) {
   CUtensorMap ma, mb;
   if (!make_map(&ma, Ap, M, Kp, TC_BM) || !make_map(&mb, Bp, N, Kp, TC_BN)) return -2;
   const size_t smem = (size_t)NSTAGE * STAGE + (size_t)NDRAIN * 32 * 48 + 1024;
@@ -1780,11 +1842,56 @@ int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nte
   if (ev0) cudaEventRecord(ev0, st);
   k_limb_gemm_tc<<<grid, TC_THREADS, smem, st>>>(ma, mb, M, N, Kp, epi.out, epi.ldc, err, err_flag);
   if (ev1) cudaEventRecord(ev1, st);
+  if (epi.acc_sign == 1 && !epi.add0 && !epi.add1 && !epi.prf_sign) return 0;
   long long ge = ((M * N + 7) / 8 + 255) / 256;
   if (ge > (1 << 20)) ge = 1 << 20;
   if (ge < 1) ge = 1;
   k_apply_epilogue<<<(unsigned)ge, 256, 0, st>>>(M, N, epi);
   return 0;
+}
+
+int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nterms,
+                 const GemmTerm* terms, const Epi& epi, void* scratch, unsigned* err,
+                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min,
+                 const GemmGroups& groups) {
+  if (M <= 0 || N <= 0) return 0;
+  const GemmTerm& t1 = nterms > 1 ? terms[1] : terms[0];
+  // the terms of a product have one layout per side
+  if (epi.atomic || t1.A.trans != terms[0].A.trans || t1.B.trans != terms[0].B.trans) return -1;
+  const long long Kp = ((nterms * K + TC_BK - 1) / TC_BK) * TC_BK;
+  unsigned short* Ap = reinterpret_cast<unsigned short*>(scratch);
+  const long long abytes = (8 * M * Kp * 2 + 255) & ~255ll;
+  unsigned short* Bp = reinterpret_cast<unsigned short*>(reinterpret_cast<char*>(scratch) + abytes);
+  split_operand(st, terms[0].A, t1.A, nterms, !terms[0].A.trans, groups, M, K, Kp, Ap);
+  split_operand(st, terms[0].B, t1.B, nterms, terms[0].B.trans, GemmGroups{}, N, K, Kp, Bp);
+  return limb_gemm_planes(st, M, N, Kp, Ap, Bp, epi, err, err_flag, ev0, ev1, split_min);
+}
+
+size_t blk_sums_tc_bytes(bool full, long long nw) {
+  return limb_tc_scratch_bytes(full ? 240 : 128, 64, nw, 1);
+}
+
+int blk_sums_tc(cudaStream_t st, const BlkIn& in, bool full, long long nw, const u64* R, u64* out,
+                void* scratch, unsigned* err, unsigned err_flag, int split_min) {
+  const long long M = full ? 240 : 128, Kp = (nw + TC_BK - 1) / TC_BK * TC_BK;
+  unsigned short* Ap = reinterpret_cast<unsigned short*>(scratch);
+  unsigned short* Bp = reinterpret_cast<unsigned short*>(reinterpret_cast<char*>(scratch) +
+                                                         ((8 * M * Kp * 2 + 255) & ~255ll));
+  if (full) k_blk_planes<<<(unsigned)(Kp / 32), 256, 0, st>>>(in, Kp, Ap);
+  else k_eda_planes<<<(unsigned)(Kp / 16), 256, 0, st>>>(in, Kp, Ap);
+  Opnd b;
+  b.p0 = R;
+  b.p1 = nullptr;
+  b.ld = 64;
+  b.s1 = b.scale = 1;
+  b.trans = 0;
+  split_operand(st, b, b, 1, false, GemmGroups{}, 64, nw, Kp, Bp);
+  Epi e;
+  memset(&e, 0, sizeof(e));
+  e.acc_sign = 1;
+  e.out = out;
+  e.ldc = 64;
+  return limb_gemm_planes(st, M, 64, Kp, Ap, Bp, e, err, err_flag, nullptr, nullptr, split_min);
 }
 
 // Tensor map of the A rows of a GR-matrix product for the TMA producers: element (k, y, z) is
