@@ -54,7 +54,6 @@ inline void counted(int k, F f, A... a) {
 #define launch_reveal(...) counted(1, mpc3::launch_reveal, __VA_ARGS__)
 #define launch_rec_hash(...) counted(1, mpc3::launch_rec_hash, __VA_ARGS__)
 #define launch_weighted_sums(...) counted(1, mpc3::launch_weighted_sums, __VA_ARGS__)
-#define launch_update_vw(...) counted(1, mpc3::launch_update_vw, __VA_ARGS__)
 #define launch_blk_sums(...) counted(1, mpc3::launch_blk_sums, __VA_ARGS__)
 #define launch_words_sums(...) counted(1, mpc3::launch_words_sums, __VA_ARGS__)
 #define launch_blk_claim(...) counted(1, mpc3::launch_blk_claim, __VA_ARGS__)
@@ -511,8 +510,13 @@ u64* cur_sums(const Small& s) { return s.U + s.uc * SUMS_WORDS; }
 // inner products, zeta revealed, the next claim zo, and M_zeta (s.MM) for the folds; the fold
 // element is s.coef[0..63].
 void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, const Small& s,
-                const u64* sums, int ld, u64* trace) {
+                const u64* sums, int ld, u64* trace, u64* V = nullptr, u64* W = nullptr,
+                int nvw = 0) {
   RoundTail a;
+  a.V = V;   // the weights of a round over a matrix S: folded along bit k - 1
+  a.W = W;
+  a.nvw = nvw;
+  a.vwbit = k - 1;
   a.sums = sums;
   a.ld = ld;
   a.mode = ctx->reduce_mode;
@@ -944,7 +948,7 @@ BlkPlan plan_blk(Arena& a, long long D, int R, int wlog, bool full, const bool x
   p.T = a.take<u64>((p.B + 1) * 64);
   p.Rw = a.take<u64>(p.nwp * 64);
   p.S = a.take<u64>(blk_rows(p.B, full) * 64);
-  p.V = a.take<u64>(p.B * 64);
+  p.V = p.T;   // the claim is taken from T before the rounds fold it
   p.W = a.take<u64>(p.B * 64);
   p.Vm = a.take<u64>(p.B * 4096);
   p.G = a.take<u64>(p.nwp * p.B * 64);
@@ -996,16 +1000,14 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
     CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
     launch_blk_claim(st, p.T, p.S + 3ll * B * B * 64, B, s.zinit);
   }
-  CK(cudaMemcpyAsync(p.V, p.T, (size_t)B * 512, cudaMemcpyDeviceToDevice, st));
   launch_ones(st, B, p.W);
   const u64* z = s.zinit;
   for (int k = 1; k <= p.kap; ++k) {
     u64* sums = cur_sums(s);
     launch_weighted_sums(st, p.V, p.W, p.S, B, k, np, sums + 64 * p0);
     u64* zo = s.z[k & 1];
-    round_tail(ctx, vid, batch, k, z, zo, s, sums, 64, trace);
+    round_tail(ctx, vid, batch, k, z, zo, s, sums, 64, trace, p.V, p.W, B);
     z = zo;
-    launch_update_vw(st, p.V, p.W, B, k, s.coef);
   }
   // G row b B + j = R_b V_j
   bool done = false;
@@ -1415,10 +1417,9 @@ int bit_batch(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* z0, u64 ver
   for (int k = 1; k <= p.kd; ++k) {   // rounds folding the 64 bits of each output
     u64* sums = cur_sums(s);
     launch_weighted_sums(st, p.V, p.W, p.S, 64, k, 1, sums);
-    round_tail(ctx, verify_id, batch, k, z, zbuf[zi], s, sums, 64, tr);
+    round_tail(ctx, verify_id, batch, k, z, zbuf[zi], s, sums, 64, tr, p.V, p.W, 64);
     z = zbuf[zi];
     zi ^= 1;
-    launch_update_vw(st, p.V, p.W, 64, k, s.coef);
   }
   delete phase;
   phase = new Phase(ctx, MPC_PROF_TRUNC_MATERIALIZE);

@@ -33,8 +33,9 @@ constexpr int REC_ROWS = 7;
 // One Pi_Reduce round after its party sums (Fig. Reduce): h(0) and h(p2) by secure GR inner
 // products, zeta' drawn and opened, the next claim z' = L0 h(0) + L1 (z - h(0)) + L2 h(p2), the
 // fold element f and its multiplication matrix.  Block c < 6 computes component c of h(0), h(p2)
-// and z'; block 6 the matrix, the Pi_Rec messages and the next round's cleared sums.  Every block
-// derives zeta' from its streams, so that no block waits for another.
+// and z'; block 6 the matrix, the Pi_Rec messages and the next round's cleared sums; in a round over
+// a matrix S (nvw > 0) the blocks from 7 on take the weights V_j, W_j, two each: times 1 - f or f by
+// bit vwbit of j.  Every block derives zeta' from its streams, so that no block waits for another.
 //
 // L0 + L1 + L2 = 1 in both readings of the third point, hence z' = h(0) + L1 (z - 2 h(0)) +
 // L2 (h(p2) - h(0)), with (points 0, 1, x) L2 = (z^2 - z) / (x (x - 1)), L1 = z - (z^2 - z) / x -
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
   __shared__ u64 scr[2][4 * 128];
   const int tid = threadIdx.x, blk = blockIdx.x;
   const int t = tid & 63;
-  if (tid < 72) {
+  if (tid < 72 && (blk < 7 || tid >= 48)) {
     const int s = tid >> 3, q = s % 3, g = s / 3;
     const u32 purpose = g == 0 ? P_VER_H0 : g == 1 ? P_VER_H2 : P_VER_ZETA;
     const Key& key = q == 0 ? a.k01 : q == 1 ? a.k02 : (g == 2 ? a.k12 : a.k01);
@@ -99,6 +100,20 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
     return;
   }
   const int sub = tid & 255, grp = tid >> 8;
+  if (blk > 6) {
+    __shared__ u64 w[2][64], e[2][64];
+    const int i = 2 * (blk - 7) + grp, j = i < a.nvw ? i : i - a.nvw;
+    u64* X = (i < a.nvw ? a.V : a.W) + j * 64;
+    if (sub < 64) {
+      const u64 f = a.mode == 1 ? 2 * zt[t] : zt[t];
+      w[grp][t] = ((j >> a.vwbit) & 1) ? f : (t == 0 ? 1ull : 0ull) - f;
+      e[grp][t] = X[t];
+    }
+    __syncthreads();
+    const u64 v = gr_mul_par<4>(w[grp], e[grp], scr[grp], sub);
+    if (sub < 64) X[t] = v;
+    return;
+  }
   // z^2 (the second group idles), then L2
   u64 r = gr_mul_par<4>(zt, zt, scr[grp], sub);
   if (tid < 64) sq[t] = a.mode == 1 ? r : r - zt[t];   // z^2, or z^2 - z
@@ -421,24 +436,11 @@ k_weighted_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64*
   }
 }
 
-// After round k: V_j <- w(j) V_j and W_j <- w(j) W_j with w = 1 - f or f by bit k-1 of j
-// (coef: f at 0, 1 - f at 384).
-__global__ void __launch_bounds__(256)
-k_update_vw(u64* __restrict__ V, u64* __restrict__ W, int n, int k, const u64* __restrict__ coef) {
-  __shared__ u64 a[64], b[64], scr[4 * 128];
-  const int j = blockIdx.x < n ? blockIdx.x : blockIdx.x - n;
-  u64* X = (blockIdx.x < n) ? V : W;
-  const int t = threadIdx.x;
-  if (t < 64) a[t] = ((j >> (k - 1)) & 1) ? coef[t] : coef[384 + t];
-  else if (t < 128) b[t - 64] = X[j * 64 + t - 64];
-  __syncthreads();
-  const u64 r = gr_mul_par<4>(a, b, scr, t);
-  if (t < 64) X[j * 64 + t] = r;
-}
-
 }  // namespace
 
-void launch_round_tail(cudaStream_t st, const RoundTail& a) { k_round_tail<<<7, 512, 0, st>>>(a); }
+void launch_round_tail(cudaStream_t st, const RoundTail& a) {
+  k_round_tail<<<7 + a.nvw, 512, 0, st>>>(a);
+}
 
 void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
                    int xidx, u64* out, u64* rec) {
@@ -460,10 +462,6 @@ void launch_weighted_sums(cudaStream_t st, const u64* V, const u64* W, const u64
                           int np, u64* out) {
   const int bs = 1 << k;
   k_weighted_sums<<<dim3(n, bs < 8 ? 1 : bs / 8, np), 256, 0, st>>>(V, W, S, n, k, out);
-}
-
-void launch_update_vw(cudaStream_t st, u64* V, u64* W, int n, int k, const u64* coef) {
-  k_update_vw<<<2 * n, 256, 0, st>>>(V, W, n, k, coef);
 }
 
 }  // namespace mpc3

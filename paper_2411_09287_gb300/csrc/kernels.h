@@ -155,6 +155,8 @@ struct RoundTail {
   u64* zero;            // nzero words cleared for the next round
   long long nzero;
   u64* trace;           // zeta' | h(0) | h(p2) of the round, or null
+  u64 *V, *W;           // nvw elements each (nvw = 0: none), times f or 1 - f by bit vwbit of j
+  int nvw, vwbit;
 };
 void launch_round_tail(cudaStream_t st, const RoundTail& a);
 // A random GR element of the streams of (purpose, obj), opened into out; record in rec.
@@ -185,8 +187,6 @@ void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 fl
 // into out) of rounds over a matrix S[p][j][j'] of n x n GR elements with weights V_j, W_j.
 void launch_weighted_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int n, int k,
                           int np, u64* out);
-// V_j, W_j (j < n) times 1 - f or f (coef) by bit k - 1 of j.
-void launch_update_vw(cudaStream_t st, u64* V, u64* W, int n, int k, const u64* coef);
 
 // ---- elementwise protocol kernels (prf_kernels.cu) ------------------------------------------
 void launch_share_input(cudaStream_t st, const u64* x, long long n, Key k01, Key k02, u64 obj,
