@@ -23,12 +23,12 @@ inline unsigned grid_for(long long n) {
 // ---- powers ---------------------------------------------------------------------------------
 // Block b writes table[16 b .. 16 b + 15]: the squares a^(2^k) by one half of the block while the
 // other multiplies the ones of 16 b's bits into a^(16 b), then four doublings of the row count
-// (row 2^k + i = row i a^(2^k)).  A block is a chain of about log2(n) + 5 products, so its time is
-// their latency: 64 rows a block, one product after another on 64 threads, took 186 to 305 us.
+// (row 2^k + i = row i a^(2^k)), the block's threads spread over the products of each.  A block is a
+// chain of about log2(n) + 4 products, so its time is their latency: @POW@.
 constexpr int POW_ROWS = 16, POW_LG = 4;
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(512)
 k_gr_powers(const u64* __restrict__ a, long long n, u64* __restrict__ table) {
-  __shared__ u64 rows[POW_ROWS][64], P[64], Pk[POW_LG][64], scr[4 * 128];
+  __shared__ u64 rows[POW_ROWS][64], P[64], Pk[POW_LG][64], scr[8 * 128];
   const int tid = threadIdx.x, t = tid & 63;
   const long long start = (long long)blockIdx.x * POW_ROWS;
   if (tid < 64) {
@@ -36,42 +36,40 @@ k_gr_powers(const u64* __restrict__ a, long long n, u64* __restrict__ table) {
     rows[0][t] = t == 0 ? 1ull : 0ull;
   }
   __syncthreads();
-  const int half = tid >> 7, sub = tid & 127;
+  const int half = tid >> 8, quarter = tid >> 7, g = tid >> 6;
   for (int k = 0; k < POW_LG || (start >> k); ++k) {   // P = a^(2^k)
     const bool bit = (start >> k) & 1;
     if (k < POW_LG && tid < 64) Pk[k][t] = P[t];
-    const u64 r = gr_mul_par<2>(half ? rows[0] : P, P, scr + half * 256, sub);
-    if (sub < 64) {
+    const u64 r = gr_mul_par<4>(half ? rows[0] : P, P, scr + half * 512, tid & 255);
+    if ((tid & 255) < 64) {
       if (!half) P[t] = r;
       else if (bit) rows[0][t] = r;
     }
     __syncthreads();
   }
-  u64 r = gr_mul_par<4>(rows[0], Pk[0], scr, tid);
+  u64 r = gr_mul_par<8>(rows[0], Pk[0], scr, tid);
   if (tid < 64) rows[1][t] = r;
   __syncthreads();
-  r = gr_mul_par<2>(rows[half], Pk[1], scr + half * 256, sub);
-  if (sub < 64) rows[2 + half][t] = r;
+  r = gr_mul_par<4>(rows[half], Pk[1], scr + half * 512, tid & 255);
+  if ((tid & 255) < 64) rows[2 + half][t] = r;
   __syncthreads();
-  const int g = tid >> 6;
-  r = gr_mul_par<1>(rows[g], Pk[2], scr + g * 128, t);
-  rows[4 + g][t] = r;
+  r = gr_mul_par<2>(rows[quarter], Pk[2], scr + quarter * 256, tid & 127);
+  if ((tid & 127) < 64) rows[4 + quarter][t] = r;
   __syncthreads();
-  for (int q = 0; q < 8; q += 4) {
-    r = gr_mul_par<1>(rows[q + g], Pk[3], scr + g * 128, t);
-    rows[8 + q + g][t] = r;
-  }
+  r = gr_mul_par<1>(rows[g], Pk[3], scr + g * 128, t);
+  rows[8 + g][t] = r;
   __syncthreads();
-  for (int i = g; i < POW_ROWS && start + i < n; i += 4) table[(start + i) * 64 + t] = rows[i][t];
+  for (int i = g; i < POW_ROWS && start + i < n; i += 8) table[(start + i) * 64 + t] = rows[i][t];
 }
 
-__global__ void k_gr_mul1(const u64* a, const u64* b, u64* out) {
-  __shared__ u64 sa[64], sb[64], scr[128];
-  sa[threadIdx.x] = a[threadIdx.x];
-  sb[threadIdx.x] = b[threadIdx.x];
+__global__ void __launch_bounds__(256) k_gr_mul1(const u64* a, const u64* b, u64* out) {
+  __shared__ u64 sa[64], sb[64], scr[4 * 128];
+  const int t = threadIdx.x;
+  if (t < 64) sa[t] = a[t];
+  else if (t < 128) sb[t - 64] = b[t - 64];
   __syncthreads();
-  gr_mul_block(sa, sb, sa, scr);
-  out[threadIdx.x] = sa[threadIdx.x];
+  const u64 r = gr_mul_par<4>(sa, sb, scr, t);
+  if (t < 64) out[t] = r;
 }
 
 // out_c = a_c + r b_c, one block per c
@@ -428,11 +426,11 @@ k_scalar_gr_sum(long long n, const u64* __restrict__ A, long long lda, int nrows
 // ---- launchers --------------------------------------------------------------------------------
 void launch_gr_powers(cudaStream_t st, const u64* a, long long n, u64* table) {
   if (n <= 0) return;
-  k_gr_powers<<<(unsigned)((n + POW_ROWS - 1) / POW_ROWS), 256, 0, st>>>(a, n, table);
+  k_gr_powers<<<(unsigned)((n + POW_ROWS - 1) / POW_ROWS), 512, 0, st>>>(a, n, table);
 }
 
 void launch_gr_mul1(cudaStream_t st, const u64* a, const u64* b, u64* out) {
-  k_gr_mul1<<<1, 64, 0, st>>>(a, b, out);
+  k_gr_mul1<<<1, 256, 0, st>>>(a, b, out);
 }
 
 void launch_gr_axpy(cudaStream_t st, int n, const u64* r, const u64* a, const u64* b, u64* out) {

@@ -7,34 +7,39 @@
 namespace mpc3 {
 
 // Coefficient c of the reduction mod f of a 127-coefficient product (lo: coefficients 0..63, hi:
-// 64..126, hi[63] ignored).
+// 64..126, hi[63] ignored): lo - H g + g H2 with x^64 = -g = -(x^4 + x^3 + x + 1), H2 the three
+// coefficients that H g carries past 63.
 __device__ __forceinline__ u64 gr_reduce_at(const u64* lo, const u64* hi, int c) {
-  u64 v = lo[c] - gr_hg(hi, c);
-  if (c < 7) {
-    u64 h2[3];
-#pragma unroll
-    for (int m = 0; m < 3; ++m) h2[m] = gr_hg(hi, 64 + m);
-    u64 g = 0;
-    if (c < 3) g += h2[c];
-    if (c - 1 >= 0 && c - 1 < 3) g += h2[c - 1];
-    if (c - 3 >= 0 && c - 3 < 3) g += h2[c - 3];
-    if (c - 4 >= 0 && c - 4 < 3) g += h2[c - 4];
-    v += g;
+  u64 v = lo[c];
+  if (c < 63) v -= hi[c];
+  if (c >= 1) v -= hi[c - 1];
+  if (c >= 3) v -= hi[c - 3];
+  if (c >= 4) v -= hi[c - 4];
+  if (c < 7) {   // H2 = (h_60 + h_61, h_61 + h_62, h_62), at the shifts 0, 1, 3, 4 of g
+    const u64 h0 = hi[60], h1 = hi[61], h2 = hi[62];
+    if ((0x1B >> c) & 1) v += h0 + h1;
+    if ((0x36 >> c) & 1) v += h1 + h2;
+    if ((0x6C >> c) & 1) v += h2;
   }
   return v;
 }
 
 // lo += product terms of coefficient t, hi += those of coefficient 64 + t, over the factors
-// a_i, i0 <= i < i0 + N.
+// a_i, i0 <= i < i0 + N.  The terms with i <= t belong to lo: one running sum, its value after
+// i = t kept, so that the additions stay inside the multiply-adds.
 template <int N>
 __device__ __forceinline__ void gr_mac_part(const u64* a, const u64* b, int t, int i0, u64& lo,
                                             u64& hi) {
+  u64 s = 0, l = 0;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
     const int i = i0 + k;
-    const u64 pr = a[i] * b[(t - i) & 63];
-    if (i <= t) lo += pr; else hi += pr;
+    s += a[i] * b[(t - i) & 63];
+    if (i == t) l = s;
   }
+  if (t >= i0 + N) l = s;
+  lo += l;
+  hi += s - l;
 }
 
 // The sum of the P parts' (lo, hi) and its reduction: every thread of the block calls it (sub =
