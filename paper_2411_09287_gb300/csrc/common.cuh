@@ -14,6 +14,36 @@ namespace mpc3 {
 typedef uint64_t u64;
 typedef uint32_t u32;
 
+// ---------------------------------------------------------------------------------------------
+// Launches.  A protocol call is a chain of 50 to 400 kernels of 2 to 20 us, each of which needs its
+// predecessor's results, so what passes between two kernels counts as much as a kernel: launch_dep
+// lets a kernel's blocks be set up while its predecessor runs, and grid_dep, the first statement of
+// every kernel launched this way, waits for the predecessor's end (its writes visible, and through
+// its own grid_dep those of everything before it) and allows the successor's set-up in turn.
+// A kernel that takes tensor memory calls grid_dep before it allocates: a block that held it while it
+// waited could keep a block of its predecessor, on the same SM, from getting any.
+// Verified product of 64 x 64 x 128: 1.26 ms without, 1.05 ms with it; ReLU of 128: 1.30, 1.09 ms.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void grid_dep() {
+  asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+template <class... P, class... A>
+inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int GR_D = 64;                 // extension degree d (Sec. 5: d = 64)
 
 // ---------------------------------------------------------------------------------------------

@@ -39,6 +39,7 @@ __device__ __forceinline__ u64 bit_of(const u64* __restrict__ w, long long i) {
 
 // The public-seed bits: blockIdx.y = 0..2 the edaBits' planes (np words), 3..5 the daBits' (W words).
 __global__ void __launch_bounds__(TPB) k_cs_bits(const CompareSelect a) {
+  grid_dep();
   const int q = blockIdx.y % 3, da = blockIdx.y / 3;
   const long long n = da ? a.np / 64 : a.np;
   u64* out = da ? a.da[q] : a.eda[q];
@@ -55,6 +56,7 @@ __global__ void __launch_bounds__(TPB) k_cs_bits(const CompareSelect a) {
 
 // The edaBit bit products b1 b2 of all 64 np bits, eight consecutive ones a thread.
 __global__ void __launch_bounds__(TPB) k_cs_products(const CompareSelect a) {
+  grid_dep();
   const long long N = 64 * a.np, nb = N / 8;
   for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b < nb; b += (long long)gridDim.x * TPB) {
     u64 r1[8], r2[8], g1[8];
@@ -93,6 +95,7 @@ __device__ __forceinline__ u64 rprime(int c, u64 n1, u64 n2, u64 z) {
 // Delta's sharing d - r with d = a - b (stored: the selection's first operand).  A block takes 32
 // elements, eight threads an element for eight bits each; its threads 0..95 draw the streams.
 __global__ void __launch_bounds__(TPB) k_cs_inner(const CompareSelect a) {
+  grid_dep();
   __shared__ u64 red[8][8][33], str[3][32];
   const long long np = a.np, N = 64 * np, e0 = (long long)blockIdx.x * 32;
   const int l = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -150,6 +153,7 @@ __global__ void __launch_bounds__(TPB) k_cs_inner(const CompareSelect a) {
 
 // The daBits: t = b1 b2, r' = b1 + b2 - 2 t, u = r' b3, r = r' + b3 - 2 u, and the first two triples.
 __global__ void __launch_bounds__(TPB) k_cs_dabits(const CompareSelect a) {
+  grid_dep();
   const long long np = a.np, nm = a.nm;
   for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < np; b += (long long)gridDim.x * TPB) {
     const long long e0 = b * 8;
@@ -199,6 +203,7 @@ __global__ void __launch_bounds__(TPB) k_cs_dabits(const CompareSelect a) {
 // joins neighbours: X = [P_hi ; P_hi], Y = [G_lo ; P_lo] over 2 C planes (C at the root), Z = X AND Y
 // (Fig. MultP over Z_2), G' = G_hi XOR Z, P' = Z of the second half.
 __global__ void __launch_bounds__(TPB) k_cs_msb(const CompareSelect a) {
+  grid_dep();
   __shared__ u64 G[6][64][4], P[6][64][4];
   const long long W = a.np / 64;
   const int wl = threadIdx.x & 3, p = threadIdx.x >> 2;
@@ -273,6 +278,7 @@ __global__ void __launch_bounds__(TPB) k_cs_msb(const CompareSelect a) {
 
 // B2A of e (opened: dbits) and the selection out = b + d [a >= b], with the third triple.
 __global__ void __launch_bounds__(TPB) k_cs_select(const CompareSelect a) {
+  grid_dep();
   const long long np = a.np, nm = a.nm;
   for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < np; b += (long long)gridDim.x * TPB) {
     const long long e0 = b * 8;
@@ -312,20 +318,20 @@ inline unsigned grid_for(long long threads) {
 }  // namespace
 
 int launch_cs_open_delta(cudaStream_t st, const CompareSelect& a) {
-  k_cs_bits<<<dim3(grid_for((a.np + 7) / 8), 6), TPB, 0, st>>>(a);
-  k_cs_products<<<grid_for(8 * a.np), TPB, 0, st>>>(a);
-  k_cs_inner<<<(unsigned)(a.np / 32), TPB, 0, st>>>(a);
+  launch_dep(k_cs_bits, dim3(grid_for((a.np + 7) / 8), 6), TPB, 0, st, a);
+  launch_dep(k_cs_products, grid_for(8 * a.np), TPB, 0, st, a);
+  launch_dep(k_cs_inner, (unsigned)(a.np / 32), TPB, 0, st, a);
   return 3;
 }
 
 int launch_cs_open_bit(cudaStream_t st, const CompareSelect& a) {
-  k_cs_dabits<<<grid_for(a.np / 8), TPB, 0, st>>>(a);
-  k_cs_msb<<<(unsigned)((a.np / 64 + 3) / 4), TPB, 0, st>>>(a);
+  launch_dep(k_cs_dabits, grid_for(a.np / 8), TPB, 0, st, a);
+  launch_dep(k_cs_msb, (unsigned)((a.np / 64 + 3) / 4), TPB, 0, st, a);
   return 2;
 }
 
 int launch_cs_select(cudaStream_t st, const CompareSelect& a) {
-  k_cs_select<<<grid_for(a.np / 8), TPB, 0, st>>>(a);
+  launch_dep(k_cs_select, grid_for(a.np / 8), TPB, 0, st, a);
   return 1;
 }
 

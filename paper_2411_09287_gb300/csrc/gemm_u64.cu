@@ -175,6 +175,7 @@ template <int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 gemm_u64_kernel(long long M, long long N, long long K, int nterms, GemmTerm t0, GemmTerm t1,
                 Epi epi, long long k_per_split) {
+  grid_dep();
   gemm_u64_body<BM, BN, BK, TM, TN>(M, N, K, nterms, t0, t1, epi, k_per_split, blockIdx.x,
                                     blockIdx.y, blockIdx.z);
 }
@@ -187,6 +188,7 @@ struct GramBatchArgs {
 };
 __global__ void __launch_bounds__(256)
 gemm_u64_gram_batch_kernel(long long K, GramBatchArgs b, long long k_per_split) {
+  grid_dep();
   const int t = blockIdx.y;
   gemm_u64_body<64, 64, 8, 4, 4>(64, 64, K, 1, b.T[t], b.T[t], b.e[t], k_per_split, 0, 0,
                                  blockIdx.z);
@@ -205,7 +207,7 @@ void gemm_u64_gram_batch(cudaStream_t st, long long K, int n, const GemmTerm* te
   }
   const long long kps = (K + nsplit - 1) / nsplit;
   dim3 grid(1, (unsigned)(n < GRAM_BATCH_MAX ? n : GRAM_BATCH_MAX), (unsigned)nsplit);
-  gemm_u64_gram_batch_kernel<<<grid, 256, 0, st>>>(K, b, kps);
+  launch_dep(gemm_u64_gram_batch_kernel, grid, 256, 0, st, K, b, kps);
 }
 
 void gemm_u64(cudaStream_t st, long long M, long long N, long long K, int nterms,
@@ -217,18 +219,15 @@ void gemm_u64(cudaStream_t st, long long M, long long N, long long K, int nterms
   if (M <= 64 && N <= 64) {   // Gram sums (64 x 64 outputs, long K)
     constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4;
     dim3 grid(1, 1, (unsigned)nsplit);
-    gemm_u64_kernel<BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(
-        M, N, K, nterms, terms[0], t1, epi, kps);
+    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, nterms, terms[0], t1, epi, kps);
   } else if (N <= 64) {
     constexpr int BM = 128, BN = 64, BK = 8, TM = 8, TN = 4;
     dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)nsplit);
-    gemm_u64_kernel<BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(
-        M, N, K, nterms, terms[0], t1, epi, kps);
+    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, nterms, terms[0], t1, epi, kps);
   } else {
     constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
     dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)nsplit);
-    gemm_u64_kernel<BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(
-        M, N, K, nterms, terms[0], t1, epi, kps);
+    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, nterms, terms[0], t1, epi, kps);
   }
 }
 

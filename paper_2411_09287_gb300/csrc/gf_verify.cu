@@ -109,6 +109,7 @@ __device__ __forceinline__ void pair_sums(const u64 (&x0)[6], const u64 (&x1)[6]
 // r and its powers R_b = r^(8 b), b < nb (8 a thread, from the squares); block 0 also draws every
 // stream word of the rounds.
 __global__ void __launch_bounds__(256) k_gf_setup(const GfVerify a, long long nb) {
+  grid_dep();
   __shared__ u64 sq[40], st[3];
   const int tid = threadIdx.x;
   if (tid < 3) st[tid] = round_stream(a, 0, tid);
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(256) k_gf_setup(const GfVerify a, long long nb
 // bits of a word are one AND/XOR of the shifted words, each of them masks one R_b.  Bound by the
 // masked XORs (about 6 instructions for each).
 __global__ void __launch_bounds__(256) k_gf_sums(const GfVerify a, const Coef cf) {
+  grid_dep();
   constexpr int NB = 16;
   __shared__ u64 raw[18][NB], pw[NB * 8];
   const int tid = threadIdx.x, p = tid >> 6, j = (tid >> 3) & 7, k = tid & 7;
@@ -227,6 +229,7 @@ __global__ void __launch_bounds__(256) k_gf_sums(const GfVerify a, const Coef cf
 
 // The vectors after three rounds (element b = 8 w + q from byte q of word w) and round 4.
 __global__ void __launch_bounds__(256) k_gf_vectors(const GfVerify a, const Coef cf, u64* x, u64* y) {
+  grid_dep();
   __shared__ u64 tv[256], tw[256], V[8], W[8];
   const int tid = threadIdx.x;
   if (tid < 8) {
@@ -279,6 +282,7 @@ __global__ void __launch_bounds__(128)
 k_gf_round(const GfVerify a, const Coef cf, int k, long long D, const u64* __restrict__ x,
            const u64* __restrict__ y, long long ld, u64* __restrict__ xo, u64* __restrict__ yo,
            long long ldo) {
+  grid_dep();
   const long long Dh = (D + 1) / 2, np = (Dh + 1) / 2;
   const u64 zeta = a.w->zeta;
   u64 s[6] = {0, 0, 0, 0, 0, 0};
@@ -330,6 +334,7 @@ __device__ void sha256_word(u64 w, u32 h[8]) {
 __global__ void __launch_bounds__(512)
 k_gf_last(const GfVerify a, const Coef cf, int k, long long D0, const u64* x, const u64* y,
           long long ld) {
+  grid_dep();
   __shared__ u64 buf[12][GF_TAIL];
   __shared__ u64 s6[6], z[6], zeta, sd[3], dl;
   __shared__ u32 bad;
@@ -457,25 +462,25 @@ int launch_gf_verify(cudaStream_t st, const GfVerify& a) {
   const long long nb = 8 * a.nw;
   int n = 3;
   cudaMemsetAsync(a.w, 0, sizeof(GfWork), st);
-  k_gf_setup<<<(unsigned)((nb + 2047) / 2048), 256, 0, st>>>(a, nb);
+  launch_dep(k_gf_setup, (unsigned)((nb + 2047) / 2048), 256, 0, st, a, nb);
   long long g = (a.nw + 15) / 16;
-  k_gf_sums<<<(unsigned)(g < 608 ? g : 608), 256, 0, st>>>(a, cf);
+  launch_dep(k_gf_sums, (unsigned)(g < 608 ? g : 608), 256, 0, st, a, cf);
   g = (nb / 2 + 255) / 256;
   u64 *x = a.x[0], *y = a.y[0], *xo = a.x[1], *yo = a.y[1];
-  k_gf_vectors<<<(unsigned)(g < 1216 ? g : 1216), 256, 0, st>>>(a, cf, x, y);
+  launch_dep(k_gf_vectors, (unsigned)(g < 1216 ? g : 1216), 256, 0, st, a, cf, x, y);
   long long D = nb, ld = nb;
   int k = 4;
   for (; (D + 1) / 2 > GF_TAIL; ++k) {
     const long long Dh = (D + 1) / 2, ldo = Dh;
     g = ((Dh + 1) / 2 + 127) / 128;
-    k_gf_round<<<(unsigned)(g < 2432 ? g : 2432), 128, 0, st>>>(a, cf, k + 1, D, x, y, ld, xo, yo, ldo);
+    launch_dep(k_gf_round, (unsigned)(g < 2432 ? g : 2432), 128, 0, st, a, cf, k + 1, D, x, y, ld, xo, yo, ldo);
     ++n;
     u64* t = x; x = xo; xo = t;
     t = y; y = yo; yo = t;
     D = Dh;
     ld = ldo;
   }
-  k_gf_last<<<1, 512, 0, st>>>(a, cf, k, D, x, y, ld);
+  launch_dep(k_gf_last, 1, 512, 0, st, a, cf, k, D, x, y, ld);
   return n + 1;
 }
 

@@ -39,6 +39,7 @@ struct BlkRows {
 template <int B, bool FULL>
 __global__ void __launch_bounds__(512)
 k_blk_sums(const BlkIn in, long long nb, int sh, const u64* __restrict__ R, u64* __restrict__ out) {
+  grid_dep();
   using Rows = BlkRows<B, FULL>;
   constexpr int NB = 8;
   constexpr int G = Rows::PAD / 8;             // rows of a group, even
@@ -112,6 +113,7 @@ k_blk_sums(const BlkIn in, long long nb, int sh, const u64* __restrict__ R, u64*
 __global__ void __launch_bounds__(512)
 k_words_sums(const u64* __restrict__ z, long long ldz, long long nw, const u64* __restrict__ R,
              u64* __restrict__ out) {
+  grid_dep();
   constexpr int NB = 8, G = 48;
   __shared__ __align__(16) u64 wd[NB][384];
   const int tid = threadIdx.x, t = tid & 63, g = tid >> 6;
@@ -148,6 +150,7 @@ k_words_sums(const u64* __restrict__ z, long long ldz, long long nw, const u64* 
 // z_c += sum_j T_j Zr[c n + j] over the eight j of block (c, y): the claim from its row sums.
 __global__ void __launch_bounds__(256)
 k_blk_claim(const u64* __restrict__ T, const u64* __restrict__ Zr, int n, u64* __restrict__ z) {
+  grid_dep();
   __shared__ u64 a[8][64], b[8][64], scr[4 * 128];
   const int tid = threadIdx.x, c = blockIdx.x, j0 = blockIdx.y * 8;
   const int cnt = n - j0 < 8 ? n - j0 : 8;
@@ -172,6 +175,7 @@ template <int B, bool ROWS, bool VEC>
 __global__ void __launch_bounds__(256)
 k_blk_combine(const BlkVec in, const BlkOut out, long long D, long long nb, int sh,
               const u64* __restrict__ Gt) {
+  grid_dep();
   const int t = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * 8;
   u64 G[B][2];
@@ -217,6 +221,7 @@ k_blk_combine(const BlkVec in, const BlkOut out, long long D, long long nb, int 
 
 // rows i < n of 64 words: the element 1
 __global__ void k_ones(int n, u64* __restrict__ out) {
+  grid_dep();
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i < n * 64) out[i] = (i & 63) == 0 ? 1ull : 0ull;
 }
@@ -233,7 +238,7 @@ int blk_rows(int B, bool full) { return (full ? 3 : 2) * B * B + (full ? 6 * B :
 void launch_blk_sums(cudaStream_t st, const BlkIn& in, int B, bool full, long long nb, int sh,
                      const u64* R, u64* out) {
   const unsigned g = blk_grid(nb);
-  auto go = [&](auto kern) { kern<<<g, 512, 0, st>>>(in, nb, sh, R, out); };
+  auto go = [&](auto kern) { launch_dep(kern, g, 512, 0, st, in, nb, sh, R, out); };
   if (full) {
     if (B == 1) go(k_blk_sums<1, true>);
     else if (B == 2) go(k_blk_sums<2, true>);
@@ -249,11 +254,11 @@ void launch_blk_sums(cudaStream_t st, const BlkIn& in, int B, bool full, long lo
 
 void launch_words_sums(cudaStream_t st, const u64* z, long long ldz, long long nw, const u64* R,
                        u64* out) {
-  k_words_sums<<<blk_grid(nw), 512, 0, st>>>(z, ldz, nw, R, out);
+  launch_dep(k_words_sums, blk_grid(nw), 512, 0, st, z, ldz, nw, R, out);
 }
 
 void launch_blk_claim(cudaStream_t st, const u64* T, const u64* Zr, int n, u64* z) {
-  k_blk_claim<<<dim3(6, (unsigned)((n + 7) / 8)), 256, 0, st>>>(T, Zr, n, z);
+  launch_dep(k_blk_claim, dim3(6, (unsigned)((n + 7) / 8)), 256, 0, st, T, Zr, n, z);
 }
 
 void launch_blk_combine(cudaStream_t st, const BlkVec& in, const BlkOut& out, int B, bool rows,
@@ -262,7 +267,7 @@ void launch_blk_combine(cudaStream_t st, const BlkVec& in, const BlkOut& out, in
   if (g > 152 * 8) g = 152 * 8;
   bool vec = B == 8;   // 16-byte loads of all components, or of none
   for (int c = 0; c < 6; ++c) vec = vec && (reinterpret_cast<uintptr_t>(in.c[c]) & 15) == 0;
-  auto go = [&](auto kern) { kern<<<(unsigned)g, 256, 0, st>>>(in, out, D, nb, sh, G); };
+  auto go = [&](auto kern) { launch_dep(kern, (unsigned)g, 256, 0, st, in, out, D, nb, sh, G); };
   if (rows) {
     if (B == 1) go(k_blk_combine<1, true, false>);
     else if (B == 2) go(k_blk_combine<2, true, false>);
@@ -278,6 +283,6 @@ void launch_blk_combine(cudaStream_t st, const BlkVec& in, const BlkOut& out, in
   }
 }
 
-void launch_ones(cudaStream_t st, int n, u64* out) { k_ones<<<(n * 64 + 255) / 256, 256, 0, st>>>(n, out); }
+void launch_ones(cudaStream_t st, int n, u64* out) { launch_dep(k_ones, (n * 64 + 255) / 256, 256, 0, st, n, out); }
 
 }  // namespace mpc3

@@ -24,10 +24,12 @@ inline unsigned grid_for(long long n) {
 // Block b writes table[16 b .. 16 b + 15]: the squares a^(2^k) by one half of the block while the
 // other multiplies the ones of 16 b's bits into a^(16 b), then four doublings of the row count
 // (row 2^k + i = row i a^(2^k)), the block's threads spread over the products of each.  A block is a
-// chain of about log2(n) + 4 products, so its time is their latency: @POW@.
+// chain of about log2(n) + 4 products, so its time is their latency: 13.7 us for 1024
+// rows (16.3 with 256 threads).
 constexpr int POW_ROWS = 16, POW_LG = 4;
 __global__ void __launch_bounds__(512)
 k_gr_powers(const u64* __restrict__ a, long long n, u64* __restrict__ table) {
+  grid_dep();
   __shared__ u64 rows[POW_ROWS][64], P[64], Pk[POW_LG][64], scr[8 * 128];
   const int tid = threadIdx.x, t = tid & 63;
   const long long start = (long long)blockIdx.x * POW_ROWS;
@@ -63,6 +65,7 @@ k_gr_powers(const u64* __restrict__ a, long long n, u64* __restrict__ table) {
 }
 
 __global__ void __launch_bounds__(256) k_gr_mul1(const u64* a, const u64* b, u64* out) {
+  grid_dep();
   __shared__ u64 sa[64], sb[64], scr[4 * 128];
   const int t = threadIdx.x;
   if (t < 64) sa[t] = a[t];
@@ -76,6 +79,7 @@ __global__ void __launch_bounds__(256) k_gr_mul1(const u64* a, const u64* b, u64
 __global__ void __launch_bounds__(256)
 k_gr_axpy(const u64* __restrict__ r, const u64* __restrict__ a, const u64* __restrict__ b,
           u64* __restrict__ out) {
+  grid_dep();
   __shared__ u64 x[64], y[64], scr[4 * 128];
   const int t = threadIdx.x, c = blockIdx.x;
   if (t < 64) x[t] = r[t];
@@ -88,6 +92,7 @@ k_gr_axpy(const u64* __restrict__ r, const u64* __restrict__ a, const u64* __res
 // M[i] = multiplication matrix of the GR element src + i * stride, for i < n (one block each).
 __global__ void __launch_bounds__(256)
 k_gr_mulmat_batch(const u64* src, long long stride, u64* M) {
+  grid_dep();
   __shared__ u64 e[64];
   if (threadIdx.x < 64) e[threadIdx.x] = src[blockIdx.x * stride + threadIdx.x];
   __syncthreads();
@@ -99,6 +104,7 @@ k_gr_mulmat_batch(const u64* src, long long stride, u64* M) {
 // read as 0 (32 x 32 tiles through shared memory).
 __global__ void k_word_transpose(long long rows, long long cols, long long n, const u64* in,
                                  u64* out) {
+  grid_dep();
   __shared__ u64 tile[32][33];
   const long long r0 = (long long)blockIdx.y * 32, c0 = (long long)blockIdx.x * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 256 threads: 8 rows per pass
@@ -117,6 +123,7 @@ __global__ void k_word_transpose(long long rows, long long cols, long long n, co
 // out[i] = src[idx(i)] for rows of 64 words, idx(i) = ((i mul) / div) mod m (m = 0: no mod).
 __global__ void k_gather_rows_affine(long long n, const u64* __restrict__ src, long long mul,
                                      long long div, long long m, u64* __restrict__ out) {
+  grid_dep();
   for (long long i = blockIdx.x; i < n; i += gridDim.x) {
     long long idx = (i * mul) / div;
     if (m) idx %= m;
@@ -128,6 +135,7 @@ __global__ void k_gather_rows_affine(long long n, const u64* __restrict__ src, l
 __global__ void __launch_bounds__(256)
 k_sum_blocks(long long m, long long n, long long ld, const u64* __restrict__ in,
              u64* __restrict__ out) {
+  grid_dep();
   const long long i = blockIdx.x * 256ll + threadIdx.x;
   if (i >= m) return;
   u64 v = 0;
@@ -138,6 +146,7 @@ k_sum_blocks(long long m, long long n, long long ld, const u64* __restrict__ in,
 
 // out[c] = sum_{h < nper} in[c nper + h] for c < ncomp (rows of 64 words).
 __global__ void k_block_rowsum(long long nper, const u64* __restrict__ in, u64* __restrict__ out) {
+  grid_dep();
   const long long c = blockIdx.x;
   u64 v = 0;
 #pragma unroll 8
@@ -197,6 +206,7 @@ __global__ void k_gr_inverses(u64* out) {
 // ---- fold of Gram sums ------------------------------------------------------------------------
 // P: n matrices of 64x64 (P[a][b] = sum u_a v_b); out: n reduced GR elements.
 __global__ void k_gr_fold_reduce(const u64* __restrict__ P, u64* __restrict__ out) {
+  grid_dep();
   __shared__ u64 prod[128];
   const u64* M = P + (long long)blockIdx.x * 4096;
   const int s = threadIdx.x;   // 128 threads
@@ -226,6 +236,7 @@ __global__ void k_gr_fold_reduce(const u64* __restrict__ P, u64* __restrict__ ou
 }
 
 __global__ void k_neg_copy(const u64* __restrict__ a, long long n, u64* __restrict__ out) {
+  grid_dep();
   for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < n;
        w += (long long)gridDim.x * blockDim.x)
     out[w] = 0ull - a[w];
@@ -234,6 +245,7 @@ __global__ void k_neg_copy(const u64* __restrict__ a, long long n, u64* __restri
 // ---- truncation-pair batch --------------------------------------------------------------------
 // u_j = c_j + r c'_j with c_j = -2^(j+1), c'_j = -2 w_j (w_j the weight of bit j in >>_arith t).
 __global__ void k_trunc_u(const u64* __restrict__ r, int t, u64* __restrict__ u) {
+  grid_dep();
   const int j = blockIdx.x;
   const int c = threadIdx.x;
   u64 cj = 0ull - (2ull << j);                         // -2^(j+1) mod 2^64 (0 for j = 63)
@@ -257,6 +269,7 @@ __global__ void k_trunc_u(const u64* __restrict__ r, int t, u64* __restrict__ u)
 __global__ void __launch_bounds__(256)
 k_trunc_materialize(long long E, const u64* __restrict__ words, const u64* __restrict__ VW,
                     const u64* __restrict__ R, int kd, u64* __restrict__ out) {
+  grid_dep();
   __shared__ u64 vw[64 * 64];
   __shared__ u64 xs[4][64], rr[4][64], hp[4][64];
   const int tid = threadIdx.x;
@@ -318,6 +331,7 @@ __device__ __forceinline__ int padj(int j) { return j + (j >> 3); }
 
 __global__ void __launch_bounds__(256)
 k_gr_mul_rows(long long n, const u64* __restrict__ a, const u64* __restrict__ b, u64* out) {
+  grid_dep();
   __shared__ u64 sa[8][64], sbp[8][216], sc[8][128];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   for (int i = l; i < 216; i += 32) sbp[w][i] = 0;
@@ -383,6 +397,7 @@ template <int NR>
 __global__ void __launch_bounds__(256)
 k_scalar_gr_sum(long long n, const u64* __restrict__ A, long long lda, int nrows,
                 const u64* __restrict__ R, u64* __restrict__ out) {
+  grid_dep();
   __shared__ __align__(16) u64 as[256][NR];
   const int t = threadIdx.x & 63, grp = threadIdx.x >> 6;
   const long long per = (n + gridDim.x - 1) / gridDim.x;
@@ -426,61 +441,61 @@ k_scalar_gr_sum(long long n, const u64* __restrict__ A, long long lda, int nrows
 // ---- launchers --------------------------------------------------------------------------------
 void launch_gr_powers(cudaStream_t st, const u64* a, long long n, u64* table) {
   if (n <= 0) return;
-  k_gr_powers<<<(unsigned)((n + POW_ROWS - 1) / POW_ROWS), 512, 0, st>>>(a, n, table);
+  launch_dep(k_gr_powers, (unsigned)((n + POW_ROWS - 1) / POW_ROWS), 512, 0, st, a, n, table);
 }
 
 void launch_gr_mul1(cudaStream_t st, const u64* a, const u64* b, u64* out) {
-  k_gr_mul1<<<1, 256, 0, st>>>(a, b, out);
+  launch_dep(k_gr_mul1, 1, 256, 0, st, a, b, out);
 }
 
 void launch_gr_axpy(cudaStream_t st, int n, const u64* r, const u64* a, const u64* b, u64* out) {
-  if (n > 0) k_gr_axpy<<<n, 256, 0, st>>>(r, a, b, out);
+  if (n > 0) launch_dep(k_gr_axpy, n, 256, 0, st, r, a, b, out);
 }
 
 void launch_gr_mulmat_batch(cudaStream_t st, long long n, const u64* src, long long stride,
                             u64* M) {
   if (n <= 0) return;
-  k_gr_mulmat_batch<<<(unsigned)n, 256, 0, st>>>(src, stride, M);
+  launch_dep(k_gr_mulmat_batch, (unsigned)n, 256, 0, st, src, stride, M);
 }
 
 void launch_word_transpose(cudaStream_t st, long long rows, long long cols, long long n,
                            const u64* in, u64* out) {
   if (rows <= 0 || cols <= 0) return;
   dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-  k_word_transpose<<<grid, 256, 0, st>>>(rows, cols, n, in, out);
+  launch_dep(k_word_transpose, grid, 256, 0, st, rows, cols, n, in, out);
 }
 
 void launch_gather_rows_affine(cudaStream_t st, long long n, const u64* src, long long mul,
                                long long div, long long m, u64* out) {
   if (n <= 0) return;
-  k_gather_rows_affine<<<(unsigned)(n < 65536 ? n : 65536), 64, 0, st>>>(n, src, mul, div, m, out);
+  launch_dep(k_gather_rows_affine, (unsigned)(n < 65536 ? n : 65536), 64, 0, st, n, src, mul, div, m, out);
 }
 
 void launch_block_rowsum(cudaStream_t st, int ncomp, long long nper, const u64* in, u64* out) {
   if (ncomp <= 0) return;
-  k_block_rowsum<<<(unsigned)ncomp, 64, 0, st>>>(nper, in, out);
+  launch_dep(k_block_rowsum, (unsigned)ncomp, 64, 0, st, nper, in, out);
 }
 
 void launch_sum_blocks(cudaStream_t st, long long m, long long n, long long ld, const u64* in,
                        u64* out) {
   if (m <= 0) return;
-  k_sum_blocks<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(m, n, ld, in, out);
+  launch_dep(k_sum_blocks, (unsigned)((m + 255) / 256), 256, 0, st, m, n, ld, in, out);
 }
 
 void launch_gr_inverses(cudaStream_t st, u64* out) { k_gr_inverses<<<1, 64, 0, st>>>(out); }
 
 void launch_gr_fold_reduce(cudaStream_t st, const u64* P, int n, u64* out) {
   if (n <= 0) return;
-  k_gr_fold_reduce<<<n, 128, 0, st>>>(P, out);
+  launch_dep(k_gr_fold_reduce, n, 128, 0, st, P, out);
 }
 
 void launch_neg_copy(cudaStream_t st, const u64* a, long long n, u64* out) {
   if (n <= 0) return;
-  k_neg_copy<<<grid_for(n), TPB, 0, st>>>(a, n, out);
+  launch_dep(k_neg_copy, grid_for(n), TPB, 0, st, a, n, out);
 }
 
 void launch_trunc_u(cudaStream_t st, const u64* r, int t, u64* u) {
-  k_trunc_u<<<64, 64, 0, st>>>(r, t, u);
+  launch_dep(k_trunc_u, 64, 64, 0, st, r, t, u);
 }
 
 void launch_trunc_materialize(cudaStream_t st, long long E, const u64* words, const u64* VW,
@@ -489,14 +504,14 @@ void launch_trunc_materialize(cudaStream_t st, long long E, const u64* words, co
   long long nout = E * (64 >> kd);
   long long g = (nout + 3) / 4;
   if (g > 152 * 16) g = 152 * 16;
-  k_trunc_materialize<<<(unsigned)g, 256, 0, st>>>(E, words, VW, R, kd, out);
+  launch_dep(k_trunc_materialize, (unsigned)g, 256, 0, st, E, words, VW, R, kd, out);
 }
 
 void launch_gr_mul_rows(cudaStream_t st, long long n, const u64* a, const u64* b, u64* out) {
   if (n <= 0) return;
   long long g = (n + 7) / 8;
   if (g > 152 * 8) g = 152 * 8;
-  k_gr_mul_rows<<<(unsigned)g, 256, 0, st>>>(n, a, b, out);
+  launch_dep(k_gr_mul_rows, (unsigned)g, 256, 0, st, n, a, b, out);
 }
 
 void launch_scalar_gr_sum(cudaStream_t st, long long n, const u64* A, long long lda, int nrows,
@@ -505,7 +520,7 @@ void launch_scalar_gr_sum(cudaStream_t st, long long n, const u64* A, long long 
   // 64 e a block while the batch is small, then eight blocks an SM
   long long g = (n + 63) / 64;
   if (g > 152 * 8) g = 152 * 8;
-  auto go = [&](auto kern) { kern<<<(unsigned)g, 256, 0, st>>>(n, A, lda, nrows, R, out); };
+  auto go = [&](auto kern) { launch_dep(kern, (unsigned)g, 256, 0, st, n, A, lda, nrows, R, out); };
   if (nrows <= 2) go(k_scalar_gr_sum<2>);
   else if (nrows <= 6) go(k_scalar_gr_sum<6>);
   else if (nrows <= 12) go(k_scalar_gr_sum<12>);

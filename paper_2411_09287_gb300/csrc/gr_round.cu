@@ -41,6 +41,7 @@ constexpr int REC_ROWS = 7;
 // L2 (h(p2) - h(0)), with (points 0, 1, x) L2 = (z^2 - z) / (x (x - 1)), L1 = z - (z^2 - z) / x -
 // L2, z = zeta'; (points 0, 1, 2) L2 = 2 z^2 - z, L1 = 4 z - 4 z^2, zeta = 2 zeta'.
 __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
+  grid_dep();
   __shared__ u64 st[9][64];       // streams: H0 (r1, r2, g1), H2 (r1, r2, g1), zeta (r1, r2, m)
   __shared__ u64 zt[64], sq[64], L1[64], L2[64], inv[64], va[64], vb[64];
   __shared__ u64 S[9][64];        // reduced party sums: ee (3 parties), cross, oo
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
 __global__ void __launch_bounds__(64)
 k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u64* __restrict__ out,
          u64* __restrict__ rec) {
+  grid_dep();
   __shared__ u64 st[3][64];
   const int t = threadIdx.x;
   if (t < 24) {
@@ -210,6 +212,7 @@ k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u
 // opening.  As separate launches (streams, multiplication matrices, three small GEMMs, messages,
 // copies of x' and y, Gram sums, reductions: 40 launches) it took 150-200 us a batch.
 __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
+  grid_dep();
   __shared__ u64 al[6][64];           // r1, r2, m of alpha; r_a, m - r2
   __shared__ u64 u[6][64], v[6][64], st[3][64], scr[4 * 128];
   __shared__ int last;
@@ -324,6 +327,7 @@ __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
 // dependent chain is what the launch takes.
 __global__ void __launch_bounds__(64)
 k_rec_hash(const u64* __restrict__ log, u32* status, u32 flag) {
+  grid_dep();
   constexpr int LD = 55;             // words of one schedule step, 54 used
   __shared__ u32 wk[64 * LD];
   __shared__ u32 dig[6][8];
@@ -403,6 +407,7 @@ k_rec_hash(const u64* __restrict__ log, u32* status, u32 flag) {
 __global__ void __launch_bounds__(256)
 k_weighted_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64* __restrict__ S,
                 int n, int k, u64* __restrict__ out) {
+  grid_dep();
   __shared__ u64 w[8][64], s[8][64], T[2][64], v[64], scr[4 * 128];
   const int tid = threadIdx.x, t = tid & 63, part = tid >> 6;
   const int j = blockIdx.x, sh = k - 1, bs = 1 << k;
@@ -439,29 +444,29 @@ k_weighted_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64*
 }  // namespace
 
 void launch_round_tail(cudaStream_t st, const RoundTail& a) {
-  k_round_tail<<<7 + a.nvw, 512, 0, st>>>(a);
+  launch_dep(k_round_tail, 7 + a.nvw, 512, 0, st, a);
 }
 
 void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
                    int xidx, u64* out, u64* rec) {
-  k_reveal<<<1, 64, 0, st>>>(k01, k02, k12, purpose, obj, xmask, xidx, out, rec);
+  launch_dep(k_reveal, 1, 64, 0, st, k01, k02, k12, purpose, obj, xmask, xidx, out, rec);
 }
 
 void launch_inner_verify(cudaStream_t st, const InnerVerify& a) {
   const long long n = a.D + 1;   // four blocks an SM at most: rows beyond that are looped over
-  k_inner_verify<<<(unsigned)(n < 608 ? n : 608), 256, 0, st>>>(a);
+  launch_dep(k_inner_verify, (unsigned)(n < 608 ? n : 608), 256, 0, st, a);
 }
 
 void launch_rec_hash(cudaStream_t st, const u64* log, int n, u32* status, u32 flag) {
   if (n <= 0) return;
   static_assert(REC_ROWS * 64 == REC_WORDS, "record size");
-  k_rec_hash<<<n, 64, 0, st>>>(log, status, flag);
+  launch_dep(k_rec_hash, n, 64, 0, st, log, status, flag);
 }
 
 void launch_weighted_sums(cudaStream_t st, const u64* V, const u64* W, const u64* S, int n, int k,
                           int np, u64* out) {
   const int bs = 1 << k;
-  k_weighted_sums<<<dim3(n, bs < 8 ? 1 : bs / 8, np), 256, 0, st>>>(V, W, S, n, k, out);
+  launch_dep(k_weighted_sums, dim3(n, bs < 8 ? 1 : bs / 8, np), 256, 0, st, V, W, S, n, k, out);
 }
 
 }  // namespace mpc3

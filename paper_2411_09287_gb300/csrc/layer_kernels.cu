@@ -25,6 +25,7 @@ inline unsigned lgrid(long long n) {
 // is floor; the conversion is exact inside the range.
 __global__ void k_encode_fixed(const double* __restrict__ x, long long n, int k,
                                u64* __restrict__ out) {
+  grid_dep();
   const double lo = -9223372036854775808.0, hi = 9223372036854775808.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
@@ -41,6 +42,7 @@ __global__ void k_encode_fixed(const double* __restrict__ x, long long n, int k,
 // the signed value of a word divided by 2^k
 __global__ void k_decode_fixed(const u64* __restrict__ v, long long n, int k,
                                double* __restrict__ out) {
+  grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     out[i] = ldexp((double)(long long)v[i], -k);
@@ -49,6 +51,7 @@ __global__ void k_decode_fixed(const u64* __restrict__ v, long long n, int k,
 // cols[c][row][col] = x[c][b][ch][i s + di - p][j s + dj - p] (0 outside the image) for every
 // share component c, row = (b Ho + i) Wo + j, col = (ch kh + di) kw + dj.
 __global__ void k_im2col(const u64* __restrict__ x, ConvGeom g, u64* __restrict__ cols) {
+  grid_dep();
   const long long Mr = (long long)g.B * g.Ho * g.Wo, Kc = (long long)g.C * g.kh * g.kw;
   const long long n_in = (long long)g.B * g.C * g.H * g.W, per = Mr * Kc, total = 6 * per;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
@@ -70,6 +73,7 @@ __global__ void k_im2col(const u64* __restrict__ x, ConvGeom g, u64* __restrict_
 __global__ void k_trunc_remask(const u64* __restrict__ xs, const u64* __restrict__ rx, long long n,
                                u64* __restrict__ d1_p1, u64* __restrict__ d2_p2,
                                u64* __restrict__ d1_p0, u64* __restrict__ d2_p0) {
+  grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     d1_p1[i] = rx[3 * n + i] - xs[3 * n + i];
@@ -84,6 +88,7 @@ __global__ void k_trunc_remask(const u64* __restrict__ xs, const u64* __restrict
 __global__ void k_trunc_online(const u64* __restrict__ xs, long long n, const u64* __restrict__ d1,
                                const u64* __restrict__ d2_at_p1, const u64* __restrict__ d1_at_p2,
                                const u64* __restrict__ d2, int t, u64* __restrict__ out) {
+  grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const u64 m1 = xs[2 * n + i] + d1[i] + d2_at_p1[i];
@@ -97,31 +102,31 @@ __global__ void k_trunc_online(const u64* __restrict__ xs, long long n, const u6
 
 void launch_encode_fixed(cudaStream_t st, const double* x, long long n, int k, u64* out) {
   if (n <= 0) return;
-  k_encode_fixed<<<lgrid(n), LTPB, 0, st>>>(x, n, k, out);
+  launch_dep(k_encode_fixed, lgrid(n), LTPB, 0, st, x, n, k, out);
 }
 
 void launch_decode_fixed(cudaStream_t st, const u64* v, long long n, int k, double* out) {
   if (n <= 0) return;
-  k_decode_fixed<<<lgrid(n), LTPB, 0, st>>>(v, n, k, out);
+  launch_dep(k_decode_fixed, lgrid(n), LTPB, 0, st, v, n, k, out);
 }
 
 void launch_im2col(cudaStream_t st, const u64* x, const ConvGeom& g, u64* cols) {
   const long long total = 6ll * g.B * g.Ho * g.Wo * g.C * g.kh * g.kw;
   if (total <= 0) return;
-  k_im2col<<<lgrid(total), LTPB, 0, st>>>(x, g, cols);
+  launch_dep(k_im2col, lgrid(total), LTPB, 0, st, x, g, cols);
 }
 
 void launch_trunc_remask(cudaStream_t st, const u64* xs, const u64* rx, long long n, u64* d1_p1,
                          u64* d2_p2, u64* d1_p0, u64* d2_p0) {
   if (n <= 0) return;
-  k_trunc_remask<<<lgrid(n), LTPB, 0, st>>>(xs, rx, n, d1_p1, d2_p2, d1_p0, d2_p0);
+  launch_dep(k_trunc_remask, lgrid(n), LTPB, 0, st, xs, rx, n, d1_p1, d2_p2, d1_p0, d2_p0);
 }
 
 void launch_trunc_online(cudaStream_t st, const u64* xs, long long n, const u64* d1,
                          const u64* d2_at_p1, const u64* d1_at_p2, const u64* d2, int t,
                          u64* out) {
   if (n <= 0) return;
-  k_trunc_online<<<lgrid(n), LTPB, 0, st>>>(xs, n, d1, d2_at_p1, d1_at_p2, d2, t, out);
+  launch_dep(k_trunc_online, lgrid(n), LTPB, 0, st, xs, n, d1, d2_at_p1, d1_at_p2, d2, t, out);
 }
 
 }  // namespace mpc3

@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 k_limb_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                long long M, long long N, long long Kp, u64* __restrict__ C, long long ldc,
                unsigned* __restrict__ err, unsigned err_flag) {
+  grid_dep();
   // split K over gridDim.z: this CTA takes chunks [cbeg, cbeg + nchunks); with more than one
   // split the partial tiles are added atomically into C (zeroed by the host)
   extern __shared__ unsigned char dsm[];
@@ -412,6 +413,7 @@ __device__ __forceinline__ uint4 bits_plane0(unsigned bits) {
 // words run along K (A with trans = 0, B with trans = 1): consecutive threads take consecutive k.
 __global__ void k_split_digits(Opnd o0, Opnd o1, int nterms, GemmGroups g, long long R, long long K,
                                long long Kp, unsigned short* __restrict__ planes) {
+  grid_dep();
   const long long chunks = Kp / 8;
   const long long total = R * chunks;
   for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < total;
@@ -439,6 +441,7 @@ __global__ void k_split_digits(Opnd o0, Opnd o1, int nterms, GemmGroups g, long 
 __global__ void __launch_bounds__(256)
 k_split_digits_t(Opnd o0, Opnd o1, int nterms, GemmGroups g, long long R, long long K, long long Kp,
                  unsigned short* __restrict__ planes) {
+  grid_dep();
   __shared__ u64 tile[32][65];
   const unsigned nr = (unsigned)((R + 31) / 32);   // row blocks run fastest
   const long long r0 = (long long)(blockIdx.x % nr) * 32;
@@ -474,10 +477,10 @@ void split_operand(cudaStream_t st, const Opnd& o0, const Opnd& o1, int nterms, 
   if (along_k) {
     long long n = (R * (Kp / 8) + 255) / 256;
     if (n > (1 << 20)) n = 1 << 20;
-    k_split_digits<<<(unsigned)n, 256, 0, st>>>(o0, o1, nterms, g, R, K, Kp, planes);
+    launch_dep(k_split_digits, (unsigned)n, 256, 0, st, o0, o1, nterms, g, R, K, Kp, planes);
   } else {
     const long long n = ((R + 31) / 32) * ((Kp + 63) / 64);
-    k_split_digits_t<<<(unsigned)n, 256, 0, st>>>(o0, o1, nterms, g, R, K, Kp, planes);
+    launch_dep(k_split_digits_t, (unsigned)n, 256, 0, st, o0, o1, nterms, g, R, K, Kp, planes);
   }
 }
 
@@ -488,6 +491,7 @@ void split_operand(cudaStream_t st, const Opnd& o0, const Opnd& o1, int nterms, 
 // row a thread.  Bound by the writes (3840 bytes a block of eight triples).
 __global__ void __launch_bounds__(256)
 k_blk_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) {
+  grid_dep();
   constexpr int LD = 4 * 68;
   __shared__ u64 a[16][LD];   // X0+X1, Y0+Y1, X2, Y3, X3, Y2, X4, Y4-Y5, X5, Y4, Z0 .. Z5
   const long long b0 = (long long)blockIdx.x * 32;
@@ -527,6 +531,7 @@ k_blk_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) 
 // parties 1 and 2, column e the sum over the eight blocks of element e, which share a weight.
 __global__ void __launch_bounds__(256)
 k_eda_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) {
+  grid_dep();
   __shared__ u64 a[4][16 * 64];   // X2, Y3, X4, Y4 - Y5 of 16 elements
   const long long e0 = (long long)blockIdx.x * 16;
   const int tid = threadIdx.x;
@@ -555,6 +560,7 @@ k_eda_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) 
 
 // out[i] = acc_sign*out[i] + add0 + add1 + prf_sign*PRF(i) (the protocol epilogue of gemm_u64).
 __global__ void k_apply_epilogue(long long M, long long N, Epi epi) {
+  grid_dep();
   const long long total = M * N;
   for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < (total + 7) / 8;
        w += (long long)gridDim.x * blockDim.x) {
@@ -654,6 +660,7 @@ template <int MODE, bool TMA, int ND>
 __global__ void __launch_bounds__((ND + GM_PROD + 1) * 32, 1)
 k_gr_matmul_tc(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
                const GrMMArgs a, unsigned* __restrict__ err, unsigned err_flag) {
+  grid_dep();
   static_assert(!TMA || MODE != 2, "bit operands take the register path");
   constexpr int DC = 256 / ND;                              // columns per drain warp
   static_assert(ND == 8 || ND == 16, "drain warps");
@@ -1322,6 +1329,7 @@ template <int MODE>
 __global__ void __launch_bounds__(TM_THREADS, 1)
 k_gr_matmul_tm(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
                const GrMMArgs a, unsigned* __restrict__ err, unsigned err_flag) {
+  grid_dep();
   static_assert(MODE == 0 || MODE == 1, "plain and fold modes");
   constexpr int NRAW = MODE == 1 ? 1 : 2;                    // raw tile buffers
   constexpr int RAW_TILE = (MODE == 1 ? 2 : 1) * TM_RAW_ARR;
@@ -1581,6 +1589,7 @@ constexpr size_t GR_SMEM = (size_t)NSTAGE * STAGE + 1024;   // 2 x (64 KB A + 32
 template <bool GEN>
 __global__ void __launch_bounds__(GM_THREADS, 1)
 k_gram_tc(long long Dh, const GramJobs jobs, unsigned* __restrict__ err, unsigned err_flag) {
+  grid_dep();
   extern __shared__ unsigned char dsm[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(dsm) + 1023) & ~uintptr_t(1023));
@@ -1840,13 +1849,13 @@ int limb_gemm_planes(cudaStream_t st, long long M, long long N, long long Kp, un
   dim3 grid((unsigned)((M + TC_BM - 1) / TC_BM), (unsigned)((N + TC_BN - 1) / TC_BN),
             (unsigned)nsplit);
   if (ev0) cudaEventRecord(ev0, st);
-  k_limb_gemm_tc<<<grid, TC_THREADS, smem, st>>>(ma, mb, M, N, Kp, epi.out, epi.ldc, err, err_flag);
+  launch_dep(k_limb_gemm_tc, grid, TC_THREADS, smem, st, ma, mb, M, N, Kp, epi.out, epi.ldc, err, err_flag);
   if (ev1) cudaEventRecord(ev1, st);
   if (epi.acc_sign == 1 && !epi.add0 && !epi.add1 && !epi.prf_sign) return 0;
   long long ge = ((M * N + 7) / 8 + 255) / 256;
   if (ge > (1 << 20)) ge = 1 << 20;
   if (ge < 1) ge = 1;
-  k_apply_epilogue<<<(unsigned)ge, 256, 0, st>>>(M, N, epi);
+  launch_dep(k_apply_epilogue, (unsigned)ge, 256, 0, st, M, N, epi);
   return 0;
 }
 
@@ -1877,8 +1886,8 @@ int blk_sums_tc(cudaStream_t st, const BlkIn& in, bool full, long long nw, const
   unsigned short* Ap = reinterpret_cast<unsigned short*>(scratch);
   unsigned short* Bp = reinterpret_cast<unsigned short*>(reinterpret_cast<char*>(scratch) +
                                                          ((8 * M * Kp * 2 + 255) & ~255ll));
-  if (full) k_blk_planes<<<(unsigned)(Kp / 32), 256, 0, st>>>(in, Kp, Ap);
-  else k_eda_planes<<<(unsigned)(Kp / 16), 256, 0, st>>>(in, Kp, Ap);
+  if (full) launch_dep(k_blk_planes, (unsigned)(Kp / 32), 256, 0, st, in, Kp, Ap);
+  else launch_dep(k_eda_planes, (unsigned)(Kp / 16), 256, 0, st, in, Kp, Ap);
   Opnd b;
   b.p0 = R;
   b.p1 = nullptr;
@@ -1968,7 +1977,7 @@ int gr_matmul_tc_ex(cudaStream_t st, const GrMMArgs& args, unsigned* err, unsign
     const size_t smem = tm_smem(mode);
     auto launch_tm = [&](auto kern) {
       set_max_dynamic_smem(reinterpret_cast<const void*>(kern), (int)smem);
-      kern<<<grid, TM_THREADS, smem, st>>>(m0, m1, a, err, err_flag);
+      launch_dep(kern, grid, TM_THREADS, smem, st, m0, m1, a, err, err_flag);
     };
     if (mode == 1) launch_tm(k_gr_matmul_tm<1>);
     else launch_tm(k_gr_matmul_tm<0>);
@@ -1979,7 +1988,7 @@ int gr_matmul_tc_ex(cudaStream_t st, const GrMMArgs& args, unsigned* err, unsign
                       (size_t)nd * GM_OSTAGE + 1024;
   auto launch = [&](auto kern) {
     set_max_dynamic_smem(reinterpret_cast<const void*>(kern), (int)smem);
-    kern<<<grid, (nd + GM_PROD + 1) * 32, smem, st>>>(m0, m1, a, err, err_flag);
+    launch_dep(kern, grid, (nd + GM_PROD + 1) * 32, smem, st, m0, m1, a, err, err_flag);
   };
   if (nd == 16) {
     if (mode == 2) launch(k_gr_matmul_tc<2, false, 16>);
@@ -2033,11 +2042,11 @@ int gram_jobs_tc(cudaStream_t st, long long Dh, const GramJobs& jobs, unsigned* 
   };
   if (one.n) {
     set_max_dynamic_smem(reinterpret_cast<const void*>(k_gram_tc<false>), (int)GR_SMEM);
-    k_gram_tc<false><<<grid_of(one.n), GM_THREADS, GR_SMEM, st>>>(Dh, one, err, err_flag);
+    launch_dep(k_gram_tc<false>, grid_of(one.n), GM_THREADS, GR_SMEM, st, Dh, one, err, err_flag);
   }
   if (two.n) {
     set_max_dynamic_smem(reinterpret_cast<const void*>(k_gram_tc<true>), (int)GR_SMEM);
-    k_gram_tc<true><<<grid_of(two.n), GM_THREADS, GR_SMEM, st>>>(Dh, two, err, err_flag);
+    launch_dep(k_gram_tc<true>, grid_of(two.n), GM_THREADS, GR_SMEM, st, Dh, two, err, err_flag);
   }
   return 0;
 }

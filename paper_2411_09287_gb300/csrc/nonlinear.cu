@@ -18,6 +18,7 @@ inline unsigned grid_for(long long n) {
 // out = a - b (sub = 1) or a + b (sub = 0) over n words
 __global__ void k_addsub(long long n, const u64* __restrict__ a, const u64* __restrict__ b, int sub,
                          u64* __restrict__ out) {
+  grid_dep();
   GRID_STRIDE(i, n) { out[i] = sub ? a[i] - b[i] : a[i] + b[i]; }
 }
 
@@ -30,6 +31,7 @@ __global__ void __launch_bounds__(TPB)
 k_eda_words(const u64* __restrict__ b1, const u64* __restrict__ b2, const u64* __restrict__ mbits,
             const u64* __restrict__ eprod, long long np, long long e0, long long ldy,
             u64* __restrict__ xm, u64* __restrict__ y) {
+  grid_dep();
   __shared__ u64 tile[64][33];
   const long long N = 64 * np, eb = (long long)blockIdx.x * 32;
   const int q = blockIdx.y, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -51,6 +53,7 @@ k_eda_words(const u64* __restrict__ b1, const u64* __restrict__ b2, const u64* _
 // b = [2i][2j+1], c = [2i+1][2j], d = [2i+1][2j+1]; nw windows, stage width np.
 __global__ void k_window_gather(const u64* __restrict__ x, long long BC, long long H, long long W,
                                 long long np, u64* __restrict__ left, u64* __restrict__ right) {
+  grid_dep();
   const long long H2 = H / 2, W2 = W / 2, nw = BC * H2 * W2, n = BC * H * W;
   GRID_STRIDE(t, 6 * nw) {
     const int c = (int)(t / nw);
@@ -67,6 +70,7 @@ __global__ void k_window_gather(const u64* __restrict__ x, long long BC, long lo
 // out[c][k] = idx[k] >= 0 ? xs[c][idx[k]] : 0 for the six components (a local linear map)
 __global__ void k_gather(const u64* __restrict__ xs, long long n_in, const long long* __restrict__ idx,
                          long long n_out, u64* __restrict__ out) {
+  grid_dep();
   GRID_STRIDE(t, 6 * n_out) {
     const int c = (int)(t / n_out);
     const long long k = t % n_out;
@@ -80,23 +84,23 @@ __global__ void k_gather(const u64* __restrict__ xs, long long n_in, const long 
 // ---- launchers ------------------------------------------------------------------------------
 void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int sub, u64* out) {
   if (n <= 0) return;
-  k_addsub<<<grid_for(n), TPB, 0, st>>>(n, a, b, sub, out);
+  launch_dep(k_addsub, grid_for(n), TPB, 0, st, n, a, b, sub, out);
 }
 void launch_eda_words(cudaStream_t st, const u64* const bits[3], const u64* eprod, long long np,
                       long long e0, long long ldy, u64* xm, u64* y) {
-  k_eda_words<<<dim3((unsigned)(np / 32), 7), TPB, 0, st>>>(bits[0], bits[1], bits[2], eprod, np, e0,
+  launch_dep(k_eda_words, dim3((unsigned)(np / 32), 7), TPB, 0, st, bits[0], bits[1], bits[2], eprod, np, e0,
                                                             ldy, xm, y);
 }
 
 void launch_window_gather(cudaStream_t st, const u64* x, long long BC, long long H, long long W,
                           long long np, u64* left, u64* right) {
-  k_window_gather<<<grid_for(6 * BC * (H / 2) * (W / 2)), TPB, 0, st>>>(x, BC, H, W, np, left, right);
+  launch_dep(k_window_gather, grid_for(6 * BC * (H / 2) * (W / 2)), TPB, 0, st, x, BC, H, W, np, left, right);
 }
 
 void launch_gather(cudaStream_t st, const u64* xs, long long n_in, const long long* idx,
                    long long n_out, u64* out) {
   if (n_out <= 0) return;
-  k_gather<<<grid_for(6 * n_out), TPB, 0, st>>>(xs, n_in, idx, n_out, out);
+  launch_dep(k_gather, grid_for(6 * n_out), TPB, 0, st, xs, n_in, idx, n_out, out);
 }
 
 }  // namespace mpc3

@@ -91,6 +91,7 @@ __device__ __forceinline__ void load8w(const u64* __restrict__ in, long long e0,
 __global__ void __launch_bounds__(TPB)
 k_share_input(const u64* __restrict__ x, long long n, Key k01, Key k02, u32 tag1, u32 tag2,
               u64 obj, u64* __restrict__ s, u64* __restrict__ m_out) {
+  grid_dep();
   __shared__ u64 stage[TPB / 32][32 * 9];
   u64* st = stage[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -116,6 +117,7 @@ k_share_input(const u64* __restrict__ x, long long n, Key k01, Key k02, u32 tag1
 // [r] <- Pi_[.] (random) into the mask components of a sharing (output wires of Pi_Mult / Pi_Inner).
 __global__ void __launch_bounds__(TPB)
 k_fill_masks(long long n, Key k01, Key k02, u32 tag1, u32 tag2, u64 obj, u64* __restrict__ s) {
+  grid_dep();
   __shared__ u64 stage[TPB / 32][32 * 9];
   u64* st = stage[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -139,6 +141,7 @@ k_fill_masks(long long n, Key k01, Key k02, u32 tag1, u32 tag2, u64 obj, u64* __
 __global__ void k_mult_offline(const u64* __restrict__ xs, const u64* __restrict__ ys,
                                long long n, Key k01, Key k02, u32 tr1, u32 tr2, u32 tg1, u64 obj,
                                u64* __restrict__ zs, u64* __restrict__ g2_out) {
+  grid_dep();
   const long long nb = (n + 7) / 8;
   for (long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x; b < nb;
        b += (long long)gridDim.x * blockDim.x) {
@@ -169,6 +172,7 @@ __global__ void k_mult_online(const u64* __restrict__ xs, const u64* __restrict_
                               long long n, Key k01, u32 tg1, u64 obj,
                               const u64* __restrict__ g2_in, u64* __restrict__ p1_out,
                               u64* __restrict__ p2_out) {
+  grid_dep();
   const long long nb = (n + 7) / 8;
   for (long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x; b < nb;
        b += (long long)gridDim.x * blockDim.x) {
@@ -195,6 +199,7 @@ __global__ void k_exchange_finish(long long n, const u64* __restrict__ p1_own,
                                   const u64* __restrict__ p1_in, const u64* __restrict__ p2_own,
                                   const u64* __restrict__ p2_in, u64* __restrict__ zs, int t,
                                   u64* __restrict__ outs) {
+  grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const u64 m1 = p1_own[i] + p1_in[i];
@@ -223,6 +228,7 @@ k_trunc_p0(long long E, Key k01, Key k02, u64 obj, const u64* __restrict__ row_k
            u64* __restrict__ zpre, u64* __restrict__ zout, u64* __restrict__ pq,
            u64* __restrict__ gp2_out, u64* __restrict__ gq2_out,
            u64* __restrict__ mp1_out, u64* __restrict__ mq1_out) {
+  grid_dep();
   __shared__ u64 stage[TPB / 32][32 * 9];
   u64* st = stage[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -299,6 +305,7 @@ k_trunc_finish(long long E, Key k01, Key k02, u64 obj, const u64* __restrict__ r
                const u64* __restrict__ p2_gq2, const u64* __restrict__ p1_mp1,
                const u64* __restrict__ p1_mq1, u64* __restrict__ zpre,
                u64* __restrict__ zout, u64* __restrict__ pq) {
+  grid_dep();
   __shared__ u64 stage[TPB / 32][32 * 9];
   u64* st = stage[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -353,12 +360,14 @@ k_trunc_finish(long long E, Key k01, Key k02, u64 obj, const u64* __restrict__ r
   }
 }
 
-__global__ void k_xor_one(u64* p, u64 mask) { *p ^= mask; }
+__global__ void k_xor_one(u64* p, u64 mask) {
+  grid_dep(); *p ^= mask; }
 
 // words off .. off + n - 1 of a row-keyed truncation-bit stream (see bits_block8) into out
 __global__ void k_prf_words_keyed(long long n, long long off, Key key, u32 tag,
                                   const u64* __restrict__ row_keys, long long N,
                                   u64* __restrict__ out) {
+  grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const long long e = off + i, row = e / N, col = e - row * N;
@@ -375,6 +384,7 @@ __global__ void k_prf_words_keyed(long long n, long long off, Key key, u32 tag,
 // stream words off .. off + n - 1 (block b holds words 8b .. 8b + 7) into out[0 .. n)
 __global__ void k_prf_words(long long n, long long off, Key key, u32 tag, u64 obj,
                             u64* __restrict__ out) {
+  grid_dep();
   const long long b0 = off / 8, nb = (off + n + 7) / 8 - b0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nb;
        i += (long long)gridDim.x * blockDim.x) {
@@ -393,6 +403,7 @@ __global__ void k_prf_words(long long n, long long off, Key key, u32 tag, u64 ob
 __global__ void k_rec_messages(const u64* __restrict__ xs, long long n, long long xidx, u64 xmask,
                                int boolean, u64* __restrict__ in_p2_r1, u64* __restrict__ in_p1_r2,
                                u64* __restrict__ in_p0_m, u64* __restrict__ out) {
+  grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     in_p2_r1[i] = xs[i];
@@ -409,44 +420,42 @@ __global__ void k_rec_messages(const u64* __restrict__ xs, long long n, long lon
 void launch_share_input(cudaStream_t st, const u64* x, long long n, Key k01, Key k02, u64 obj,
                         u64* s6, u64* p0_out_m) {
   if (n <= 0) return;
-  k_share_input<<<grid_for((n + 7) / 8), TPB, 0, st>>>(x, n, k01, k02, make_tag(P_SHARE, C_R1),
+  launch_dep(k_share_input, grid_for((n + 7) / 8), TPB, 0, st, x, n, k01, k02, make_tag(P_SHARE, C_R1),
                                                        make_tag(P_SHARE, C_R2), obj, s6, p0_out_m);
 }
 
 void launch_fill_masks(cudaStream_t st, long long n, Key k01, Key k02, u32 purpose, u64 obj,
                        u64* s6) {
   if (n <= 0) return;
-  k_fill_masks<<<grid_for((n + 7) / 8), TPB, 0, st>>>(n, k01, k02, make_tag(purpose, C_R1),
+  launch_dep(k_fill_masks, grid_for((n + 7) / 8), TPB, 0, st, n, k01, k02, make_tag(purpose, C_R1),
                                                       make_tag(purpose, C_R2), obj, s6);
 }
 
 void launch_mult_offline(cudaStream_t st, const u64* xs, const u64* ys, long long n, Key k01,
                          Key k02, u64 obj, u64* zs, u64* p0_out_g2) {
   if (n <= 0) return;
-  k_mult_offline<<<grid_for((n + 7) / 8), TPB, 0, st>>>(
-      xs, ys, n, k01, k02, make_tag(P_MULT, C_R1), make_tag(P_MULT, C_R2),
+  launch_dep(k_mult_offline, grid_for((n + 7) / 8), TPB, 0, st, xs, ys, n, k01, k02, make_tag(P_MULT, C_R1), make_tag(P_MULT, C_R2),
       make_tag(P_MULT, C_G1), obj, zs, p0_out_g2);
 }
 
 void launch_mult_online(cudaStream_t st, const u64* xs, const u64* ys, long long n, Key k01,
                         u64 obj, const u64* p2_in_g2, u64* p1_out, u64* p2_out) {
   if (n <= 0) return;
-  k_mult_online<<<grid_for((n + 7) / 8), TPB, 0, st>>>(xs, ys, n, k01, make_tag(P_MULT, C_G1),
+  launch_dep(k_mult_online, grid_for((n + 7) / 8), TPB, 0, st, xs, ys, n, k01, make_tag(P_MULT, C_G1),
                                                        obj, p2_in_g2, p1_out, p2_out);
 }
 
 void launch_exchange_finish(cudaStream_t st, long long n, const u64* p1_own, const u64* p1_in,
                             const u64* p2_own, const u64* p2_in, u64* zs, int t, u64* outs) {
   if (n <= 0) return;
-  k_exchange_finish<<<grid_for(n), TPB, 0, st>>>(n, p1_own, p1_in, p2_own, p2_in, zs, t, outs);
+  launch_dep(k_exchange_finish, grid_for(n), TPB, 0, st, n, p1_own, p1_in, p2_own, p2_in, zs, t, outs);
 }
 
 void launch_trunc_p0(cudaStream_t st, long long E, Key k01, Key k02, u64 obj, int t, u64* zpre,
                      u64* zout, u64* pq, u64* p0_out_gp2, u64* p0_out_gq2, u64* p1_out_mp,
                      u64* p1_out_mq, const u64* row_keys, long long N) {
   if (E <= 0) return;
-  k_trunc_p0<<<grid_for((E + 7) / 8), TPB, 0, st>>>(
-      E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2),
+  launch_dep(k_trunc_p0, grid_for((E + 7) / 8), TPB, 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2),
       make_tag(P_TRUNC_P, C_R1), make_tag(P_TRUNC_P, C_R2), make_tag(P_TRUNC_P, C_G1),
       make_tag(P_TRUNC_Q, C_R1), make_tag(P_TRUNC_Q, C_R2), make_tag(P_TRUNC_Q, C_G1), zpre, zout,
       pq, p0_out_gp2, p0_out_gq2, p1_out_mp, p1_out_mq);
@@ -458,29 +467,28 @@ void launch_trunc_finish(cudaStream_t st, long long E, Key k01, Key k02, u64 obj
                          const u64* p1_mp1, const u64* p1_mq1, u64* zpre, u64* zout, u64* pq,
                          const u64* row_keys, long long N) {
   if (E <= 0) return;
-  k_trunc_finish<<<grid_for((E + 7) / 8), TPB, 0, st>>>(
-      E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2), p1_in_mp,
+  launch_dep(k_trunc_finish, grid_for((E + 7) / 8), TPB, 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2), p1_in_mp,
       p1_in_mq, p2_in_mp, p2_in_mq, p2_gp2, p2_gq2, p1_mp1, p1_mq1, zpre, zout, pq);
 }
 
-void launch_xor_one(cudaStream_t st, u64* p, u64 mask) { k_xor_one<<<1, 1, 0, st>>>(p, mask); }
+void launch_xor_one(cudaStream_t st, u64* p, u64 mask) { launch_dep(k_xor_one, 1, 1, 0, st, p, mask); }
 
 void launch_prf_words_keyed(cudaStream_t st, long long n, Key key, u32 tag, const u64* row_keys,
                             long long N, u64* out, long long off) {
   if (n <= 0 || off < 0) return;
-  k_prf_words_keyed<<<grid_for(n), TPB, 0, st>>>(n, off, key, tag, row_keys, N, out);
+  launch_dep(k_prf_words_keyed, grid_for(n), TPB, 0, st, n, off, key, tag, row_keys, N, out);
 }
 
 void launch_prf_words(cudaStream_t st, long long n, Key key, u32 tag, u64 obj, u64* out,
                       long long off) {
   if (n <= 0 || off < 0) return;
-  k_prf_words<<<grid_for((off + n + 7) / 8 - off / 8), TPB, 0, st>>>(n, off, key, tag, obj, out);
+  launch_dep(k_prf_words, grid_for((off + n + 7) / 8 - off / 8), TPB, 0, st, n, off, key, tag, obj, out);
 }
 
 void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask,
                          bool boolean, u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out) {
   if (n <= 0) return;
-  k_rec_messages<<<grid_for(n), TPB, 0, st>>>(xs, n, xidx, xmask, boolean ? 1 : 0, in_p2_r1,
+  launch_dep(k_rec_messages, grid_for(n), TPB, 0, st, xs, n, xidx, xmask, boolean ? 1 : 0, in_p2_r1,
                                               in_p1_r2, in_p0_m, out);
 }
 

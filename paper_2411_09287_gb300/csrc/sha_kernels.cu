@@ -34,6 +34,7 @@ __device__ __forceinline__ void node_hash(const u32* l, const u32* r, u32 h[8]) 
 // blockIdx.y picks the array; with one CTA per array its root is the digest itself.
 __global__ void __launch_bounds__(HB)
 k_hash_leaves(const HashJobs jobs, long long n, long long nleaves) {
+  grid_dep();
   const u64* __restrict__ data = jobs.data[blockIdx.y];
   u32* __restrict__ out = gridDim.x == 1 ? jobs.digest[blockIdx.y] : jobs.scratch[blockIdx.y];
   __shared__ u32 dg[HB][8];
@@ -119,6 +120,7 @@ k_hash_leaves(const HashJobs jobs, long long n, long long nleaves) {
 // One CTA an array: levels of the Merkle tree over its `cnt` subtree roots (ping-pong between the
 // halves of its scratch).
 __global__ void k_hash_tree(const HashJobs jobs, long long cnt) {
+  grid_dep();
   u32* cur = jobs.scratch[blockIdx.x];
   u32* nxt = cur + 8 * cnt;
   u32* digest = jobs.digest[blockIdx.x];
@@ -147,6 +149,7 @@ __global__ void k_hash_tree(const HashJobs jobs, long long cnt) {
 // Compare three (received value's hash, received hash) pairs; any mismatch sets `flag`.
 __global__ void k_digest_check(const u32* a0, const u32* b0, const u32* a1, const u32* b1,
                                const u32* a2, const u32* b2, u32* status, u32 flag) {
+  grid_dep();
   const int t = threadIdx.x;
   bool bad = false;
   if (t < 8) bad = (a0[t] != b0[t]) || (a1[t] != b1[t]) || (a2[t] != b2[t]);
@@ -161,8 +164,8 @@ void launch_hash_jobs(cudaStream_t st, const HashJobs& jobs, int njobs, long lon
   long long leaves = (8 * n + LEAF_BYTES - 1) / LEAF_BYTES;
   if (leaves < 1) leaves = 1;
   const long long nb = (leaves + HB - 1) / HB;   // subtree roots, one per CTA
-  k_hash_leaves<<<dim3((unsigned)nb, (unsigned)njobs), HB, 0, st>>>(jobs, n, leaves);
-  if (nb > 1) k_hash_tree<<<njobs, 256, 0, st>>>(jobs, nb);
+  launch_dep(k_hash_leaves, dim3((unsigned)nb, (unsigned)njobs), HB, 0, st, jobs, n, leaves);
+  if (nb > 1) launch_dep(k_hash_tree, njobs, 256, 0, st, jobs, nb);
 }
 
 void launch_hash_u64(cudaStream_t st, const u64* data, long long n, u32* scratch, u32* digest) {
@@ -175,7 +178,7 @@ void launch_hash_u64(cudaStream_t st, const u64* data, long long n, u32* scratch
 
 void launch_digest_check(cudaStream_t st, const u32* a0, const u32* b0, const u32* a1,
                          const u32* b1, const u32* a2, const u32* b2, u32* status, u32 flag) {
-  k_digest_check<<<1, 32, 0, st>>>(a0, b0, a1, b1, a2, b2, status, flag);
+  launch_dep(k_digest_check, 1, 32, 0, st, a0, b0, a1, b1, a2, b2, status, flag);
 }
 
 }  // namespace mpc3

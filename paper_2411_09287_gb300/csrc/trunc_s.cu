@@ -75,6 +75,7 @@ __device__ __forceinline__ unsigned nibble_bytes(unsigned nib) {
 // constant memory, indexed per thread: 231 us for L = 2^16, now 33-43 us.)
 __global__ void __launch_bounds__(256)
 k_limb_table(const u64* __restrict__ Tlo, long long L, unsigned char* __restrict__ TL8) {
+  grid_dep();
   __shared__ u64 tile[64][65];
   const long long e0 = (long long)blockIdx.x * 64;   // L is a multiple of 64
   for (int i = threadIdx.x; i < 4096; i += 256) tile[i >> 6][i & 63] = Tlo[e0 * 64 + i];
@@ -115,6 +116,7 @@ k_limb_table(const u64* __restrict__ Tlo, long long L, unsigned char* __restrict
 constexpr int BT_W = 16;
 __global__ void __launch_bounds__(32 * BT_W)
 k_bit_transpose(const u64* __restrict__ words, long long nw, u64* __restrict__ BT) {
+  grid_dep();
   __shared__ u64 rows[64][BT_W + 1];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   const long long w0 = (long long)blockIdx.x * BT_W;
@@ -151,6 +153,7 @@ __global__ void __launch_bounds__(S_THREADS, 1)
 k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* __restrict__ B1T,
              const u64* __restrict__ B2T, long long nw, long long L, u64* __restrict__ S_hi,
              unsigned* __restrict__ err, unsigned err_flag) {
+  grid_dep();
   extern __shared__ unsigned char dsm[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(dsm) + 1023) & ~uintptr_t(1023));
@@ -303,12 +306,12 @@ k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* __restrict__ B1
 }  // namespace
 
 void launch_trunc_limb_table(cudaStream_t st, const u64* Tlo, long long L, unsigned char* TL8) {
-  k_limb_table<<<(unsigned)(L / 64), 256, 0, st>>>(Tlo, L, TL8);
+  launch_dep(k_limb_table, (unsigned)(L / 64), 256, 0, st, Tlo, L, TL8);
 }
 
 void launch_trunc_bit_transpose(cudaStream_t st, const u64* words, long long Epad, u64* BT) {
   const long long nw = Epad / 64;
-  k_bit_transpose<<<(unsigned)((nw + BT_W - 1) / BT_W), 32 * BT_W, 0, st>>>(words, nw, BT);
+  launch_dep(k_bit_transpose, (unsigned)((nw + BT_W - 1) / BT_W), 32 * BT_W, 0, st, words, nw, BT);
 }
 
 int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long Epad,
@@ -327,7 +330,7 @@ int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long
     return -2;
   set_max_dynamic_smem(reinterpret_cast<const void*>(k_trunc_s_tc), (int)S_SMEM);
   dim3 grid(4096 / S_TPAIRS, 64 * S_LIMBS / S_TCOLS, (unsigned)nhi);
-  k_trunc_s_tc<<<grid, S_THREADS, S_SMEM, st>>>(mb, B1T, B2T, Epad / 64, L, S_hi, err, err_flag);
+  launch_dep(k_trunc_s_tc, grid, S_THREADS, S_SMEM, st, mb, B1T, B2T, Epad / 64, L, S_hi, err, err_flag);
   return 0;
 }
 
