@@ -141,6 +141,8 @@ mpc_tuning default_tuning() {
 }
 }  // namespace
 
+constexpr int NSIDE = 3;
+
 struct mpc_ctx {
   int device = 0;
   mpc_tuning tune = default_tuning();
@@ -171,6 +173,9 @@ struct mpc_ctx {
   cudaStream_t copy_st = nullptr;
   cudaEvent_t copy_ev[MPC_H2D_SLOTS] = {};
   cudaEvent_t order_ev = nullptr;   // the context stream's work before a download
+  // side streams of independent verification batches (Fork)
+  cudaStream_t side[NSIDE] = {};
+  cudaEvent_t fork_ev = nullptr, join_ev[NSIDE] = {};
 };
 
 namespace {
@@ -221,6 +226,44 @@ struct Phase {
       c->recs.push_back({id, a, b, work});
     }
   }
+};
+
+// Independent verification batches side by side.  A batch is a chain of launches that mostly wait for
+// one another's results on a few SMs, and the batches of a call share nothing but the status word (an
+// atomic OR) and the inputs, so they run on streams of their own: on(i) sends what follows to side
+// stream i (i < 0: the context's own), after everything before the fork; join() (or the end of the
+// scope) makes the context's stream wait for all of them, so that a call leaves nothing running that
+// its stream does not cover.  Recorded by a stream capture like any fork and join.  With phase timers
+// on, everything stays on the one stream.
+struct Fork {
+  mpc_ctx* c;
+  cudaStream_t main;
+  bool used[NSIDE] = {};
+  explicit Fork(mpc_ctx* ctx, bool enable = true) : c(ctx), main(ctx->st) {
+    on_ = enable && !c->prof && cudaEventRecord(c->fork_ev, main) == cudaSuccess;
+  }
+  void on(int i) {
+    c->st = main;
+    if (!on_ || i < 0 || cudaStreamWaitEvent(c->side[i], c->fork_ev, 0) != cudaSuccess) return;
+    c->st = c->side[i];
+    used[i] = true;
+  }
+  void join() {
+    c->st = main;
+    for (int i = 0; i < NSIDE; ++i) {
+      if (!used[i]) continue;
+      used[i] = false;
+      if (cudaEventRecord(c->join_ev[i], c->side[i]) != cudaSuccess ||
+          cudaStreamWaitEvent(main, c->join_ev[i], 0) != cudaSuccess)
+        cudaStreamSynchronize(c->side[i]);
+    }
+  }
+  ~Fork() { join(); }
+  Fork(const Fork&) = delete;
+  Fork& operator=(const Fork&) = delete;
+
+ private:
+  bool on_;
 };
 
 int guard(mpc_ctx* ctx) {
@@ -1106,16 +1149,21 @@ struct TruncBatch {
 };
 
 struct VMatPlan {
-  Small s;
+  Small s, st;                    // batch 0's and the truncation batch's
   u64 *Q, *P, *T, *Pz;
   PowPlan powQ, powP;
   Dense dv;
   int R0;
   bool trunc = false;
   TruncBatch tb;
-  void* tcs = nullptr;            // tensor-core digit planes (limb path only)
+  void *tcs = nullptr, *tcst = nullptr;   // tensor-core digit planes of the two (limb path only)
+  bool fork = false;              // the two side by side (their scratch apart)
   bool grouped = false;           // X^T P and W Q of all six components as one product each
 };
+// Outputs up to which batch 0 and the truncation batch run side by side: above, batch 0 is a few
+// percent of the call and its scratch is better shared (64 x 64 x 128: 1.05 ms one after the other, 0.89
+// side by side).
+constexpr long long FORK_MAX = 1ll << 22;
 // Words of a grouped operand at most (256 MB of digit planes).  Below, a product of one component is
 // a few CTAs and its four launches take longer than its work (17 products of a layer: 1.67 ms a
 // verified product of 64 x 64 x 128, 1.32 ms with seven); above, each fills the GPU.
@@ -1272,6 +1320,8 @@ bool plan_vmat(Arena& a, long long M, long long N, long long K, int t, int R0, i
   p.s = plan_small(a);
   p.trunc = t >= 0;
   const long long E = M * N;
+  p.fork = p.trunc && E <= FORK_MAX;
+  p.st = p.fork ? plan_small(a) : p.s;
   long long trunc_tcs = 0;
   if (p.trunc && (trunc_tcs = trunc_batch_tcs(E, R1, tc, tu)) < 0) return false;
   // digit planes of the batch-0 products (X^T P, W Q, Z Q) and of the truncation chunks'
@@ -1281,8 +1331,9 @@ bool plan_vmat(Arena& a, long long M, long long N, long long K, int t, int R0, i
   p.tcs = tc ? (void*)a.take<unsigned char>((long long)std::max(
                    {limb_tc_scratch_bytes(p.grouped ? G : K, 64, M, 1),
                     limb_tc_scratch_bytes(p.grouped ? G : K, 64, N, 1),
-                    limb_tc_scratch_bytes(6 * M, 64, N, 1), (size_t)trunc_tcs}))
+                    limb_tc_scratch_bytes(6 * M, 64, N, 1), (size_t)(p.fork ? 0 : trunc_tcs)}))
              : nullptr;
+  p.tcst = p.fork && tc && trunc_tcs > 0 ? (void*)a.take<unsigned char>(trunc_tcs) : p.tcs;
   p.Q = a.take<u64>(N * 64);
   p.P = a.take<u64>(M * 64);
   p.powQ = plan_pow(a, N);
@@ -1615,6 +1666,16 @@ int verify_trunc_batch(mpc_ctx* ctx, TruncBatch& b, const Small& s, void* tcs, c
 // =================================================================================================
 // C-ABI
 // =================================================================================================
+namespace {
+void destroy_side(mpc_ctx* ctx) {
+  for (int i = 0; i < NSIDE; ++i) {
+    if (ctx->side[i]) cudaStreamDestroy(ctx->side[i]);
+    if (ctx->join_ev[i]) cudaEventDestroy(ctx->join_ev[i]);
+  }
+  if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
+}
+}  // namespace
+
 extern "C" {
 
 int mpc_create(const mpc_config* cfg, mpc_ctx** out) {
@@ -1632,6 +1693,7 @@ int mpc_create(const mpc_config* cfg, mpc_ctx** out) {
     std::fprintf(stderr, "mpc_create: %s: %s\n", what, cudaGetErrorString(e));
     if (ctx->cst) cudaFree(ctx->cst);
     if (ctx->own_stream && ctx->st) cudaStreamDestroy(ctx->st);
+    destroy_side(ctx);
     delete ctx;
     return MPC_ERR_CUDA;
   };
@@ -1644,6 +1706,12 @@ int mpc_create(const mpc_config* cfg, mpc_ctx** out) {
     if (e != cudaSuccess) return bail("cudaStreamCreate", e);
     ctx->own_stream = true;
   }
+  e = cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming);
+  for (int i = 0; i < NSIDE && e == cudaSuccess; ++i) {
+    e = cudaStreamCreateWithFlags(&ctx->side[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->join_ev[i], cudaEventDisableTiming);
+  }
+  if (e != cudaSuccess) return bail("side streams", e);
   // constants block + status word + key staging
   e = cudaMalloc(&ctx->cst, CST_WORDS * 8 + 256 + 256);
   if (e != cudaSuccess) return bail("cudaMalloc", e);
@@ -1681,6 +1749,7 @@ void mpc_destroy(mpc_ctx* ctx) {
   for (cudaEvent_t e : ctx->pool) cudaEventDestroy(e);
   if (ctx->cst) cudaFree(ctx->cst);
   if (ctx->own_stream && ctx->st) cudaStreamDestroy(ctx->st);
+  destroy_side(ctx);
   delete ctx;
 }
 
@@ -2200,10 +2269,12 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
                  ctx->tune, p))
     return fail(ctx, MPC_ERR_SHAPE, "verify_matmul: more than 15 truncation chunks");
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "verify_matmul: workspace too small");
-  cudaStream_t st = ctx->st;
   const Small& s = p.s;
   const long long MK = M * K, KN = K * N;
+  Fork fork(ctx, p.fork);
+  fork.on(0);
   // ---- batch 0: the M N inner products of Z = X W, rank-1 consolidation ----
+  cudaStream_t st = ctx->st;
   Phase* phase = new Phase(ctx, MPC_PROF_VERIFY_GEMM);
   if ((rc = sums_begin(ctx, s))) return rc;
   reveal(ctx, P_VER_R, make_obj(verify_id, 0, 0), s, s.r);
@@ -2249,11 +2320,13 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
   delete phase;
   if (rc) return rc;
   // ---- batch 1: the truncation pairs, chunk by chunk ----
+  fork.on(-1);
   if (trunc &&
-      (rc = verify_trunc_batch(ctx, p.tb, s, p.tcs, pq, trunc_bits, verify_id, matmul_call_id,
+      (rc = verify_trunc_batch(ctx, p.tb, p.st, p.tcst, pq, trunc_bits, verify_id, matmul_call_id,
                                trace ? trace + (long long)(p.R0 + 1) * TRACE_ROUND : nullptr,
                                (const u64*)row_keys, N)))
     return rc;
+  fork.join();
   return finish_verify(ctx, (matmul_call_id << 1) | 1);
 }
 
@@ -2775,26 +2848,14 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuni
 
 int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
   int rc;
-  cudaStream_t st = ctx->st;
-  // ---- batch 0: the daBit products (two) and the final product, stage by stage (the edaBit
-  // bit products are batch 3)
-  {
-    VMultPlan& v = p.vm;
-    const Small& s = v.s;
-    const long long n = p.nm;
-    if ((rc = sums_begin(ctx, s))) return rc;
-    reveal(ctx, P_VER_R, make_obj(vid, 0, 0), s, s.r);
-    if ((rc = blk_tables(ctx, v.b, s.r, s.aux))) return rc;
-    Vec x, y;
-    for (int c = 0; c < 6; ++c) {
-      x.c[c] = p.MX + c * n;
-      y.c[c] = p.MY + c * n;
-    }
-    if ((rc = run_blk(ctx, vid, 0, v.b, x, y, p.MZ, s, trace))) return rc;
-  }
   u64* tr1 = trace ? trace + (long long)(p.vm.R + 1) * TRACE_ROUND : nullptr;
+  u64* tr2 = tr1 ? tr1 + (long long)(p.R1 + 1) * TRACE_ROUND : nullptr;
+  u64* tr3 = tr2 ? tr2 + (long long)(p.gf.R + 1) * MPC_TRACE_GF_ROUND : nullptr;
+  Fork fork(ctx);   // four independent batches, the longest chains of launches first
   // ---- batch 1: the edaBit inner products, weight r^e on row e (e over all stages)
+  fork.on(0);
   {
+    cudaStream_t st = ctx->st;
     const Small& s = p.s1;
     if ((rc = sums_begin(ctx, s))) return rc;
     reveal(ctx, P_VER_R, make_obj(vid, 1, 0), s, s.r);
@@ -2815,14 +2876,12 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     for (int c = 0; c < 6; ++c) y.c[c] = p.Ye + c * p.D1;
     if ((rc = run_blk(ctx, vid, 1, b, x, y, nullptr, s, tr1))) return rc;
   }
-  u64* tr2 = tr1 ? tr1 + (long long)(p.R1 + 1) * TRACE_ROUND : nullptr;
-  // ---- batch 2: every AND gate over GF(2^64), stage by stage, level by level
-  if ((rc = gf_verify(ctx, vid, p.gf, tr2))) return rc;
-  u64* tr3 = tr2 ? tr2 + (long long)(p.gf.R + 1) * MPC_TRACE_GF_ROUND : nullptr;
   // ---- batch 3: the edaBit bit products b_{i,1} b_{i,2}, stage by stage (plane-major); x has
   // only the [r]_1 components and y only the [r]_2 ones, so the dense rounds take the
   // single-Gram form
+  fork.on(1);
   {
+    cudaStream_t st = ctx->st;
     const Small& s = p.sb;
     if ((rc = sums_begin(ctx, s))) return rc;
     reveal(ctx, P_VER_R, make_obj(vid, 3, 0), s, s.r);
@@ -2851,6 +2910,26 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
     }
     if ((rc = bit_batch(ctx, t, s, t.zt + 384, vid, 3, tr3))) return rc;
   }
+  // ---- batch 0: the daBit products (two) and the final product, stage by stage (the edaBit
+  // bit products are batch 3)
+  fork.on(2);
+  {
+    VMultPlan& v = p.vm;
+    const Small& s = v.s;
+    const long long n = p.nm;
+    if ((rc = sums_begin(ctx, s))) return rc;
+    reveal(ctx, P_VER_R, make_obj(vid, 0, 0), s, s.r);
+    if ((rc = blk_tables(ctx, v.b, s.r, s.aux))) return rc;
+    Vec x, y;
+    for (int c = 0; c < 6; ++c) {
+      x.c[c] = p.MX + c * n;
+      y.c[c] = p.MY + c * n;
+    }
+    if ((rc = run_blk(ctx, vid, 0, v.b, x, y, p.MZ, s, trace))) return rc;
+  }
+  // ---- batch 2: every AND gate over GF(2^64), stage by stage, level by level
+  fork.on(-1);
+  if ((rc = gf_verify(ctx, vid, p.gf, tr2))) return rc;
   return MPC_OK;
 }
 
