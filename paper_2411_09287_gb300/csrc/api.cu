@@ -962,12 +962,15 @@ int power_table(mpc_ctx* ctx, const u64* r, const PowPlan& p, u64* table, u64* a
 // A batch of weighted ring words (gr_block.cu): x_i = R_{b >> sh} T_j X_i, y_i = lift(Y_i), i =
 // B b + j < D, whose first kap = log2(B) rounds need no GR vectors.
 constexpr int BLK_ROUNDS = 3;
-// Blocks from which the sums go to the tensor cores (@BLKMIN@).
-constexpr long long BLK_TC_MIN = 8192;
+// Words from which a batch takes four rounds that way, its sums on the tensor cores (65520
+// words: 58 us of CUDA-core sums for three rounds; 65536: 65 us in three launches for four, and the dense
+// round on 8192 elements, about 70 us, is gone).
+constexpr long long BLK_TC_MIN = 1 << 16;
 struct BlkPlan {
   long long D, nb;        // words, blocks
   long long nw, nwp;      // weight rows R, rounded up to whole tiles
   int R, kap, B, sh;
+  bool tc;                // B = 16, sums on the tensor cores
   bool full;              // all components and the claim's sums; else x has 2 and 4 only
   PowPlan pp;
   u64 *T, *Rw, *S, *V, *W, *Vm, *G;
@@ -976,11 +979,12 @@ struct BlkPlan {
 
 // wlog: log2 of the words per weight step (0: weights r^i; 6: r^(i / 64), T_j = 1)
 BlkPlan plan_blk(Arena& a, long long D, int R, int wlog, bool full, const bool xc[6],
-                 const bool yc[6]) {
+                 const bool yc[6], bool tc) {
   BlkPlan p;
   p.D = D;
   p.R = R;
-  p.kap = std::min(R, BLK_ROUNDS);
+  p.tc = tc && D >= BLK_TC_MIN && R > BLK_ROUNDS;
+  p.kap = p.tc ? BLK_ROUNDS + 1 : std::min(R, BLK_ROUNDS);
   p.B = 1 << p.kap;
   p.nb = (D + p.B - 1) / p.B;
   p.sh = wlog > p.kap ? wlog - p.kap : 0;
@@ -1013,7 +1017,7 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
   cudaStream_t st = ctx->st;
   const int B = p.B;
   int rc;
-  CK(cudaMemsetAsync(p.S, 0, (size_t)blk_rows(B, p.full) * 512, st));
+  if (!p.tc) CK(cudaMemsetAsync(p.S, 0, (size_t)blk_rows(B, p.full) * 512, st));
   BlkIn in;
   for (int c = 0; c < 6; ++c) {
     in.x[c] = xw.c[c];
@@ -1024,21 +1028,16 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
   in.D = p.D;
   // parties 1 and 2 only: their matrices sit where those of a full batch's first two would
   const int np = p.full ? 3 : 2, p0 = p.full ? 0 : 1;
-  // long batches on the tensor cores; the digit planes (4864 bytes a block at most) lie in the
-  // vectors' storage (4096 or 6144 bytes a block), which is written after the rounds
-  bool sums = !(p.full || p.kap > 0);
-  if (!sums && ctx->gemm_path == MPC_GEMM_LIMB_TC && B == 8 && p.nb >= BLK_TC_MIN &&
-      p.sh == (p.full ? 0 : 3)) {
+  if (p.tc) {
+    // the digit planes (14848 bytes a block of a full batch, 2304 of the edaBits') lie where the
+    // products R_b V_j and the vectors come after the rounds (17408 and 8192)
     g_launches += 3;
-    u64* planes = p.dv.x[0].c[p.full ? 0 : 2];
-    sums = blk_sums_tc(st, in, p.full, p.nw, p.Rw, p.S, planes, ctx->status, ST_TIMEOUT,
-                       ctx->tune.gemm_split_min) == 0;
-    if (!sums) {
-      g_launches -= 3;
-      CK(cudaMemsetAsync(p.S, 0, (size_t)blk_rows(B, p.full) * 512, st));
-    }
+    if (blk_sums_tc(st, in, p.full, p.nw, p.Rw, p.S, p.G, ctx->status, ST_TIMEOUT,
+                    ctx->tune.gemm_split_min))
+      return fail(ctx, MPC_ERR_CUDA, "block sums: tensor maps");
+  } else if (p.full || p.kap > 0) {
+    launch_blk_sums(st, in, B, p.full, p.nb, p.sh, p.Rw, p.S);
   }
-  if (!sums) launch_blk_sums(st, in, B, p.full, p.nb, p.sh, p.Rw, p.S);
   if (p.full) {
     CK(cudaMemsetAsync(s.zinit, 0, 384 * 8, st));
     launch_blk_claim(st, p.T, p.S + 3ll * B * B * 64, B, s.zinit);
@@ -1094,12 +1093,12 @@ struct VMultPlan {
   int R;
 };
 
-VMultPlan plan_vmult(Arena& a, long long n, int R) {
+VMultPlan plan_vmult(Arena& a, long long n, int R, bool tc) {
   VMultPlan p;
   p.R = R < 0 ? default_R(n) : R;
   p.s = plan_small(a);
   const bool all[6] = {true, true, true, true, true, true};
-  p.b = plan_blk(a, n, p.R, 0, true, all, all);
+  p.b = plan_blk(a, n, p.R, 0, true, all, all, tc);
   return p;
 }
 
@@ -1109,12 +1108,12 @@ struct VMultCallsPlan {
   VMultPlan v;
 };
 
-VMultCallsPlan plan_vmult_calls(Arena& a, long long n, int R) {
+VMultCallsPlan plan_vmult_calls(Arena& a, long long n, int R, bool tc) {
   VMultCallsPlan p;
   p.x = a.take<u64>(6 * n);
   p.y = a.take<u64>(6 * n);
   p.z = a.take<u64>(6 * n);
-  p.v = plan_vmult(a, n, R);
+  p.v = plan_vmult(a, n, R, tc);
   return p;
 }
 
@@ -1913,11 +1912,11 @@ int64_t mpc_workspace_size(const mpc_ctx* ctx, int op, int64_t a, int64_t b, int
       break;
     case MPC_OP_VERIFY_MULT:
       if (a <= 0) return -1;
-      plan_vmult(ar, a, R_main);
+      plan_vmult(ar, a, R_main, ctx && ctx->gemm_path == MPC_GEMM_LIMB_TC);
       break;
     case MPC_OP_VERIFY_MULT_CALLS:
       if (a <= 0) return -1;
-      plan_vmult_calls(ar, a, R_main);
+      plan_vmult_calls(ar, a, R_main, ctx && ctx->gemm_path == MPC_GEMM_LIMB_TC);
       break;
     case MPC_OP_VERIFY_MATMUL: {
       if (a <= 0 || b <= 0 || c <= 0 || trunc_bits > 63) return -1;
@@ -2192,7 +2191,7 @@ int mpc_verify_mult(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs, const 
   if (n <= 0) return fail(ctx, MPC_ERR_SHAPE, "verify_mult: n <= 0");
   if (!xs || !ys || !zs || !id_ok(verify_id)) return fail(ctx, MPC_ERR_ARG, "verify_mult: bad argument");
   Arena ar{(char*)workspace, workspace_bytes, 0, false};
-  VMultPlan p = plan_vmult(ar, n, R);
+  VMultPlan p = plan_vmult(ar, n, R, ctx->gemm_path == MPC_GEMM_LIMB_TC);
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "verify_mult: workspace too small");
   if ((rc = verify_mult_body(ctx, verify_id, xs, ys, zs, n, p, trace))) return rc;
   return finish_verify(ctx, (mult_call_id << 1) | 0);
@@ -2221,7 +2220,7 @@ int mpc_verify_mult_calls(mpc_ctx* ctx, uint64_t verify_id, int ncalls,
     if (N > (1ll << 40)) return fail(ctx, MPC_ERR_SHAPE, "verify_mult_calls: batch too large");
   }
   Arena ar{(char*)workspace, workspace_bytes, 0, false};
-  VMultCallsPlan p = plan_vmult_calls(ar, N, R);
+  VMultCallsPlan p = plan_vmult_calls(ar, N, R, ctx->gemm_path == MPC_GEMM_LIMB_TC);
   if (!workspace || !ar.ok())
     return fail(ctx, MPC_ERR_WORKSPACE, "verify_mult_calls: workspace too small");
   // the batch: component c of call l at c N + (n[0] + ... + n[l-1]) of each gathered sharing
@@ -2787,7 +2786,8 @@ struct NLPlan {
   void* wsum = nullptr;          // digit planes for them (long batches on the limb path)
 };
 
-// Elements of a stage from which the sums over its bit words go to the tensor cores (@WMIN@).
+// Elements of a stage from which the sums over its bit words go to the tensor cores (61 us on
+// the CUDA cores at 4032, 60 us at 4096 in three launches; 235 and 80 us at 16384).
 constexpr long long WORDS_TC_MIN = 4096;
 
 NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuning& tu) {
@@ -2806,13 +2806,13 @@ NLPlan plan_nl(Arena& a, int nst, const long long np[2], bool tc, const mpc_tuni
   p.o = a.take<u64>(n0);
   const long long andw = AND_PLANES * (p.ne / 64);
   p.MX = a.take<u64>(6 * p.nm); p.MY = a.take<u64>(6 * p.nm); p.MZ = a.take<u64>(6 * p.nm);
-  p.vm = plan_vmult(a, p.nm, -1);
+  p.vm = plan_vmult(a, p.nm, -1, tc);
   p.D1 = 64 * p.ne;
   p.R1 = default_R(p.D1);
   p.s1 = plan_small(a);
   const bool xc[6] = {false, false, true, false, true, false};
   const bool yc[6] = {true, true, true, true, true, true};
-  p.b1 = plan_blk(a, p.D1, p.R1, 6, false, xc, yc);
+  p.b1 = plan_blk(a, p.D1, p.R1, 6, false, xc, yc, tc);
   p.Ye = a.take<u64>(6 * p.D1);
   p.Xe = a.take<u64>(p.D1);
   p.gf = plan_gf(a, andw);

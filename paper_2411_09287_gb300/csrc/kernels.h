@@ -303,7 +303,7 @@ int blk_rows(int B, bool full);
 // the rows are those of parties 1 and 2.
 void launch_blk_sums(cudaStream_t st, const BlkIn& in, int B, bool full, long long nb, int sh,
                      const u64* R, u64* out);
-// The same sums for full batches (B = 8, sh = 0) and the edaBits' (B = 8, sh = 3) on the tensor cores:
+// The same sums for full batches (sh = 0) and the edaBits' (sh = 2) with B = 16, on the tensor cores:
 // a product of the blocks' words (nw columns, those of a weight added) and R.  scratch:
 // blk_sums_tc_bytes(full, nw), 256-byte aligned; 0, or not 0 when the tensor maps cannot be encoded.
 size_t blk_sums_tc_bytes(bool full, long long nw);

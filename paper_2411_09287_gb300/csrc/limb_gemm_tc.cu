@@ -484,20 +484,20 @@ void split_operand(cudaStream_t st, const Opnd& o0, const Opnd& o1, int nterms, 
   }
 }
 
-// Digit planes of the block words of a full batch (gr_block.cu): row (p, j, j') < 192 the party's word
-// word^p_{b,j,j'}, row 192 + 8 c + j the claim's Z_c[8 b + j], column b < Kp (zero past the batch).  A
-// block takes 32 b: their words, with the parties' sums of shares, in shared memory (padded so that
-// the four groups of eight b that a half-warp reads lie in different banks), then eight columns of a
-// row a thread.  Bound by the writes (3840 bytes a block of eight triples).
+// Digit planes of the block words of a full batch (gr_block.cu, B = 16): row (p, j, j') < 768 the
+// party's word word^p_{b,j,j'}, row 768 + 16 c + j the claim's Z_c[16 b + j], column b < Kp (zero past
+// the batch).  A block takes 16 b: their words, with the parties' sums of shares, in shared memory
+// (four words of padding a 64, against bank conflicts), then eight columns of a row a thread.  Bound by
+// the writes (13.8 KB a block of sixteen triples).
 __global__ void __launch_bounds__(256)
 k_blk_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) {
   grid_dep();
-  constexpr int LD = 4 * 68;
-  __shared__ u64 a[16][LD];   // X0+X1, Y0+Y1, X2, Y3, X3, Y2, X4, Y4-Y5, X5, Y4, Z0 .. Z5
-  const long long b0 = (long long)blockIdx.x * 32;
+  constexpr int ROWS = 3 * 256 + 6 * 16;
+  __shared__ u64 a[16][4 * 68];   // X0+X1, Y0+Y1, X2, Y3, X3, Y2, X4, Y4-Y5, X5, Y4, Z0 .. Z5
+  const long long b0 = (long long)blockIdx.x * 16;
   const int tid = threadIdx.x;
   {
-    const long long i = b0 * 8 + tid;
+    const long long i = b0 * 16 + tid;
     const bool ok = i < in.D;
     u64 x[6], y[6];
 #pragma unroll
@@ -513,22 +513,23 @@ k_blk_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) 
     for (int c = 0; c < 6; ++c) a[10 + c][o] = ok ? in.z[c * in.ldz + i] : 0ull;
   }
   __syncthreads();
-  for (int u = tid; u < 240 * 4; u += 256) {
-    const int g = u & 3, row = u >> 2, p = row >> 6, j = g * 68 + ((row >> 3) & 7), k = g * 68 + (row & 7);
+  for (int u = tid; u < ROWS * 2; u += 256) {
+    const int g = u & 1, row = u >> 1, p = row >> 8, j = g * 136 + ((row >> 4) & 15), k = g * 136 + (row & 15);
     u64 v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      if (p == 0) v[q] = a[0][j + 8 * q] * a[1][k + 8 * q];
-      else if (p == 1) v[q] = 0ull - (a[2][j + 8 * q] * a[3][k + 8 * q] + a[4][j + 8 * q] * a[5][k + 8 * q]);
-      else if (p == 2) v[q] = a[6][j + 8 * q] * a[7][k + 8 * q] - a[8][j + 8 * q] * a[9][k + 8 * q];
-      else v[q] = a[10 + ((row - 192) >> 3)][k + 8 * q];
+      const int o = 16 * q + 4 * (q >> 2);
+      if (p == 0) v[q] = a[0][j + o] * a[1][k + o];
+      else if (p == 1) v[q] = 0ull - (a[2][j + o] * a[3][k + o] + a[4][j + o] * a[5][k + o]);
+      else if (p == 2) v[q] = a[6][j + o] * a[7][k + o] - a[8][j + o] * a[9][k + o];
+      else v[q] = a[10 + ((row - 768) >> 4)][k + o];
     }
-    split8_store(v, reinterpret_cast<unsigned char*>(planes + row * Kp + b0 + g * 8), 240 * Kp * 2, 0);
+    split8_store(v, reinterpret_cast<unsigned char*>(planes + row * Kp + b0 + g * 8), ROWS * Kp * 2, 0);
   }
 }
 
 // The same for the edaBits' inner products (x has components 2 and 4 only): rows (p, j, j') of the
-// parties 1 and 2, column e the sum over the eight blocks of element e, which share a weight.
+// parties 1 and 2, column e the sum over the four blocks of element e, which share a weight.
 __global__ void __launch_bounds__(256)
 k_eda_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) {
   grid_dep();
@@ -544,18 +545,20 @@ k_eda_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) 
     a[3][o] = ok ? in.y[4][i] - in.y[5][i] : 0ull;
   }
   __syncthreads();
-  const int g = tid & 1, row = tid >> 1, p = row >> 6, j = (row >> 3) & 7, k = row & 7;
-  const u64* x = a[2 * p] + g * 512 + j;
-  const u64* y = a[2 * p + 1] + g * 512 + k;
-  u64 v[8];
+  for (int u = tid; u < 1024; u += 256) {
+    const int g = u & 1, row = u >> 1, p = row >> 8, j = (row >> 4) & 15, k = row & 15;
+    const u64* x = a[2 * p] + g * 512 + j;
+    const u64* y = a[2 * p + 1] + g * 512 + k;
+    u64 v[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    u64 t = 0;
+    for (int e = 0; e < 8; ++e) {
+      u64 t = 0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) t += x[e * 64 + 8 * q] * y[e * 64 + 8 * q];
-    v[e] = p == 0 ? 0ull - t : t;
+      for (int q = 0; q < 4; ++q) t += x[e * 64 + 16 * q] * y[e * 64 + 16 * q];
+      v[e] = p == 0 ? 0ull - t : t;
+    }
+    split8_store(v, reinterpret_cast<unsigned char*>(planes + row * Kp + e0 + g * 8), 512 * Kp * 2, 0);
   }
-  split8_store(v, reinterpret_cast<unsigned char*>(planes + row * Kp + e0 + g * 8), 128 * Kp * 2, 0);
 }
 
 // out[i] = acc_sign*out[i] + add0 + add1 + prf_sign*PRF(i) (the protocol epilogue of gemm_u64).
@@ -1877,16 +1880,16 @@ int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nte
 }
 
 size_t blk_sums_tc_bytes(bool full, long long nw) {
-  return limb_tc_scratch_bytes(full ? 240 : 128, 64, nw, 1);
+  return limb_tc_scratch_bytes(blk_rows(16, full), 64, nw, 1);
 }
 
 int blk_sums_tc(cudaStream_t st, const BlkIn& in, bool full, long long nw, const u64* R, u64* out,
                 void* scratch, unsigned* err, unsigned err_flag, int split_min) {
-  const long long M = full ? 240 : 128, Kp = (nw + TC_BK - 1) / TC_BK * TC_BK;
+  const long long M = blk_rows(16, full), Kp = (nw + TC_BK - 1) / TC_BK * TC_BK;
   unsigned short* Ap = reinterpret_cast<unsigned short*>(scratch);
   unsigned short* Bp = reinterpret_cast<unsigned short*>(reinterpret_cast<char*>(scratch) +
                                                          ((8 * M * Kp * 2 + 255) & ~255ll));
-  if (full) launch_dep(k_blk_planes, (unsigned)(Kp / 32), 256, 0, st, in, Kp, Ap);
+  if (full) launch_dep(k_blk_planes, (unsigned)(Kp / 16), 256, 0, st, in, Kp, Ap);
   else launch_dep(k_eda_planes, (unsigned)(Kp / 16), 256, 0, st, in, Kp, Ap);
   Opnd b;
   b.p0 = R;
