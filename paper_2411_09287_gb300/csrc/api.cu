@@ -50,6 +50,7 @@ inline void counted(int k, F f, A... a) {
 #define launch_gr_fold_reduce(...) counted(1, mpc3::launch_gr_fold_reduce, __VA_ARGS__)
 #define launch_neg_copy(...) counted(1, mpc3::launch_neg_copy, __VA_ARGS__)
 #define launch_round_tail(...) counted(1, mpc3::launch_round_tail, __VA_ARGS__)
+#define launch_small_round(...) counted(1, mpc3::launch_small_round, __VA_ARGS__)
 #define launch_inner_verify(...) counted(1, mpc3::launch_inner_verify, __VA_ARGS__)
 #define launch_reveal(...) counted(1, mpc3::launch_reveal, __VA_ARGS__)
 #define launch_rec_hash(...) counted(1, mpc3::launch_rec_hash, __VA_ARGS__)
@@ -779,13 +780,20 @@ int inner_verify_dense(mpc_ctx* ctx, u64 vid, u32 batch, const Vec& x, const Vec
   return cuda_check(ctx, "inner_verify");
 }
 
+// Elements of a claim up to which a round's fold and sums are one launch on the CUDA cores (on the
+// limb path): at 512 its 256 blocks still run at once, 20 us against 36; it would double with each
+// doubling, the tensor-core launches hardly grow up to 4096.
+constexpr long long SMALL_MAX = 512;
+
 // Dense rounds k = k0..R followed by Pi_InnerVerify.
 int run_dense(mpc_ctx* ctx, u64 vid, u32 batch, Dense& dv, long long D, const u64* z0, int k0,
               int R, const Small& s, u64* trace) {
   int rc;
   const u64* z = z0;
   int zi = 0;
-  for (int k = k0; k <= R; ++k) {
+  const bool tc = ctx->gemm_path == MPC_GEMM_LIMB_TC;
+  int k = k0;
+  for (; k <= R && !(tc && D <= SMALL_MAX); ++k) {
     Vec& x = dv.x[dv.cur];
     Vec& y = dv.y[dv.cur];
     Vec& xo = dv.x[dv.cur ^ 1];
@@ -796,6 +804,33 @@ int run_dense(mpc_ctx* ctx, u64 vid, u32 batch, Dense& dv, long long D, const u6
     zi ^= 1;
     dv.cur ^= 1;
     D = (D + 1) / 2;
+  }
+  // short claims: each launch folds by the round before's f and takes this round's sums
+  bool fold = false;
+  for (; k <= R + 1; ++k) {
+    if (k > R && !fold) break;
+    SmallRound a;
+    const int o = dv.cur ^ 1;
+    for (int c = 0; c < 6; ++c) {
+      a.in[c] = dv.x[dv.cur].c[c];
+      a.in[6 + c] = dv.y[dv.cur].c[c];
+      a.out[c] = dv.x[o].c[c];
+      a.out[6 + c] = dv.y[o].c[c];
+    }
+    a.f = s.coef;
+    a.D = D;
+    a.fold = fold;
+    a.sums = k <= R ? cur_sums(s) : nullptr;
+    launch_small_round(ctx->st, a);
+    if (fold) {
+      dv.cur = o;
+      D = (D + 1) / 2;
+    }
+    if (k > R) break;
+    round_tail(ctx, vid, batch, k, z, s.z[zi], s, a.sums, 128, trace);
+    z = s.z[zi];
+    zi ^= 1;
+    fold = true;
   }
   return inner_verify_dense(ctx, vid, batch, dv.x[dv.cur], dv.y[dv.cur], D, z, s, trace, R);
 }

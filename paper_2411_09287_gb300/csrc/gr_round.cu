@@ -201,6 +201,103 @@ k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u
   out[t] = m - r1 - r2in;
 }
 
+// The vectors' part of a Pi_Reduce round on a short claim, in one launch: the fold by the last round's
+// f (fold set: a_2e + f (a_2e+1 - a_2e), D elements into ceil(D / 2)), and this round's party sums over
+// the pairs of what it leaves (sums not null): blocks S00, S11 and the cross sum S01 + S10 as (e + o)(e'
+// + o') - S00 - S11, 127 unreduced coefficients each.  A block takes one pair: its 24 products one a
+// 64-thread group, then the fifteen products of the sums a quarter each a group.  Bound by latency; on
+// the tensor cores, whose tiles want 128 rows and whose kernels first split their operands, the two
+// Gram launches and the fold of such a round took 36 us at 512 elements, this 20 us (15 without the fold).
+__global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
+  grid_dep();
+  __shared__ u64 f[64], v[2][12][64], d[4][64], red[9][128];
+  const int tid = threadIdx.x, t = tid & 63, g = tid >> 6;
+  const long long pair = blockIdx.x;
+  if (a.fold) {
+    if (tid < 64) f[t] = a.f[t];
+    for (int i = g; i < 24; i += 4) {   // (element, component): six of each group
+      const int e = i / 12, c = i % 12;
+      const u64* src = a.in[c];
+      const long long s0 = 2 * (2 * pair + e);
+      u64 base = 0, diff = 0;
+      if (src && s0 < a.D) {
+        base = src[s0 * 64 + t];
+        diff = (s0 + 1 < a.D ? src[(s0 + 1) * 64 + t] : 0ull) - base;
+      }
+      d[g][t] = diff;
+      __syncthreads();
+      u64 lo = 0, hi = 0;
+      if (src) gr_mac_part<64>(f, d[g], t, 0, lo, hi);
+      const u64 r = base + gr_finish<1>(lo, hi, red[g], t);
+      v[e][c][t] = r;
+      if (src && s0 < a.D) a.out[c][(2 * pair + e) * 64 + t] = r;
+    }
+  } else {
+    for (int i = g; i < 24; i += 4) {
+      const int e = i / 12, c = i % 12;
+      const long long s0 = 2 * pair + e;
+      v[e][c][t] = a.in[c] && s0 < a.D ? a.in[c][s0 * 64 + t] : 0ull;
+    }
+  }
+  __syncthreads();
+  if (!a.sums) return;
+  // the parties' factors: P0 r_u, r_v; P2 m_v - [r_v]_2 (in places that are not needed any more)
+  if (tid < 128) {
+    const int e = tid >> 6;
+    v[e][0][t] += v[e][1][t];
+    v[e][6][t] += v[e][7][t];
+    v[e][1][t] = v[e][10][t] - v[e][11][t];
+  }
+  __syncthreads();
+  // sums over even, odd and even + odd elements; pairs of components (u, v) of x at c, of y at 6 + c
+  u64 lo[9], hi[9];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) lo[q] = hi[q] = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (k == 2) {
+      __syncthreads();
+      for (int i = g; i < 12; i += 4) v[0][i][t] += v[1][i][t];
+      __syncthreads();
+    }
+    u64(*w)[64] = v[k == 1 ? 1 : 0];
+    u64 nl = 0, nh = 0;
+    if ((a.in[0] || a.in[1]) && (a.in[6] || a.in[7])) gr_mac_part<16>(w[0], w[6], t, g * 16, lo[3 * k], hi[3 * k]);
+    if (a.in[2] && a.in[9]) gr_mac_part<16>(w[2], w[9], t, g * 16, nl, nh);
+    if (a.in[8] && a.in[3]) gr_mac_part<16>(w[8], w[3], t, g * 16, nl, nh);
+    lo[3 * k + 1] = 0ull - nl;
+    hi[3 * k + 1] = 0ull - nh;
+    nl = nh = 0;
+    if (a.in[4] && (a.in[10] || a.in[11])) gr_mac_part<16>(w[4], w[1], t, g * 16, lo[3 * k + 2], hi[3 * k + 2]);
+    if (a.in[10] && a.in[5]) gr_mac_part<16>(w[10], w[5], t, g * 16, nl, nh);
+    lo[3 * k + 2] -= nl;
+    hi[3 * k + 2] -= nh;
+  }
+  for (int p = 0; p < 4; ++p) {   // the groups' quarters
+    if (g == p) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        if (p == 0) {
+          red[q][t] = lo[q];
+          red[q][64 + t] = hi[q];
+        } else {
+          red[q][t] += lo[q];
+          red[q][64 + t] += hi[q];
+        }
+      }
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < 9 * 128; i += 256) {
+    const int q = i >> 7, c = i & 127, k = q / 3, p = q % 3;
+    u64 s = red[q][c];
+    if (k == 2) s -= red[p][c] + red[3 + p][c];
+    // S00 at 0, the cross sum at 3, S11 at 9 (blocks of 128 words)
+    if (s) atomicAdd(reinterpret_cast<unsigned long long*>(a.sums + ((k == 0 ? 0 : k == 1 ? 9 : 3) + p) * 128 + c),
+                     (unsigned long long)s);
+  }
+}
+
 // Pi_InnerVerify (Fig. DPV) on a claim of D elements, in one launch.  Row i < D: x'_i = alpha x_i
 // (alpha random, shared, never opened) by Pi_Mult over GR, whose messages are Gamma_i - [Gamma_i]_1
 // (P0 -> P2) and the two halves of m (P1 <-> P2); row D: alpha against -z.  Every block takes some
@@ -450,6 +547,11 @@ void launch_round_tail(cudaStream_t st, const RoundTail& a) {
 void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
                    int xidx, u64* out, u64* rec) {
   launch_dep(k_reveal, 1, 64, 0, st, k01, k02, k12, purpose, obj, xmask, xidx, out, rec);
+}
+
+void launch_small_round(cudaStream_t st, const SmallRound& a) {
+  const long long n = a.fold ? (a.D + 1) / 2 : a.D;
+  launch_dep(k_small_round, (unsigned)((n + 1) / 2), 256, 0, st, a);
 }
 
 void launch_inner_verify(cudaStream_t st, const InnerVerify& a) {

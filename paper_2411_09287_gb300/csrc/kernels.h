@@ -162,6 +162,16 @@ void launch_round_tail(cudaStream_t st, const RoundTail& a);
 // A random GR element of the streams of (purpose, obj), opened into out; record in rec.
 void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
                    int xidx, u64* out, u64* rec);
+// A round's fold and party sums on a claim of D elements, for short claims.
+struct SmallRound {
+  const u64* in[12];    // x's components, then y's (null = zero)
+  u64* out[12];         // folded (fold set)
+  const u64* f;
+  long long D;
+  bool fold;
+  u64* sums;            // 12 blocks of 128 words, added into (S01 + S10 in S01's place), or null
+};
+void launch_small_round(cudaStream_t st, const SmallRound& a);
 // Pi_InnerVerify of a claim of D elements: x, y component pointers (null = zero), z the claim (6 x
 // 64), acc 193 words that are zero on entry (party sums and a count of finished blocks).  Delta is
 // opened into trace (when not null); `flag` in *status unless it is zero.
