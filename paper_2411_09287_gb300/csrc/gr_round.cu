@@ -40,14 +40,17 @@ constexpr int REC_ROWS = 7;
 // L0 + L1 + L2 = 1 in both readings of the third point, hence z' = h(0) + L1 (z - 2 h(0)) +
 // L2 (h(p2) - h(0)), with (points 0, 1, x) L2 = (z^2 - z) / (x (x - 1)), L1 = z - (z^2 - z) / x -
 // L2, z = zeta'; (points 0, 1, 2) L2 = 2 z^2 - z, L1 = 4 z - 4 z^2, zeta = 2 zeta'.
+//
+// Everything that the keys alone decide (the streams, zeta', the Lagrange weights: a ChaCha20 block
+// and two dependent products, half of the kernel's latency) comes before grid_dep, while the
+// predecessor still runs; no memory that a kernel of the chain writes is touched there.
 __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
-  grid_dep();
   __shared__ u64 st[9][64];       // streams: H0 (r1, r2, g1), H2 (r1, r2, g1), zeta (r1, r2, m)
   __shared__ u64 zt[64], sq[64], L1[64], L2[64], inv[64], va[64], vb[64];
   __shared__ u64 S[9][64];        // reduced party sums: ee (3 parties), cross, oo
   __shared__ u64 scr[2][4 * 128];
   const int tid = threadIdx.x, blk = blockIdx.x;
-  const int t = tid & 63;
+  const int t = tid & 63, sub = tid & 255, grp = tid >> 8;
   if (tid < 72 && (blk < 7 || tid >= 48)) {
     const int s = tid >> 3, q = s % 3, g = s / 3;
     const u32 purpose = g == 0 ? P_VER_H0 : g == 1 ? P_VER_H2 : P_VER_ZETA;
@@ -55,20 +58,7 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
     const u32 comp = q == 0 ? C_R1 : q == 1 ? C_R2 : (g == 2 ? C_M12 : C_G1);
     stream64(key, make_tag(purpose, comp), a.obj, tid & 7, st[s]);
   } else if (tid >= 128 && tid < 192) {
-    inv[t] = a.inv[t];
-  }
-  const bool msg = blk == 2 || blk == 4;   // the components m, which take the party sums
-  if (msg && tid >= 192) {
-    for (int i = tid - 192; i < 9 * 64; i += 320) {
-      const int q = i >> 6, c = i & 63;
-      const u64* s0 = a.sums + (q < 3 ? q : q < 6 ? q : q + 3) * a.ld;   // ee, S01, oo
-      u64 v = a.ld == 128 ? gr_reduce_at(s0, s0 + 64, c) : s0[c];
-      if (q >= 3 && q < 6) {   // cross: S01 + S10
-        const u64* s1 = a.sums + (q + 3) * a.ld;
-        v += a.ld == 128 ? gr_reduce_at(s1, s1 + 64, c) : s1[c];
-      }
-      S[q][c] = v;
-    }
+    inv[t] = a.inv[t];   // a constant of the context
   }
   __syncthreads();
   if (tid < 64) {   // P1's opening: m - [r]_1 - [r]_2 as received
@@ -76,6 +66,29 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
     zt[t] = st[8][t] - st[6][t] - r2;
   }
   __syncthreads();
+  if (blk < 6) {
+    // z^2 (the second group idles), then L2
+    u64 r = gr_mul_par<4>(zt, zt, scr[grp], sub);
+    if (tid < 64) sq[t] = a.mode == 1 ? r : r - zt[t];   // z^2, or z^2 - z
+    __syncthreads();
+    if (a.mode == 1) {
+      if (tid < 64) {
+        L2[t] = 2 * sq[t] - zt[t];
+        L1[t] = 4 * zt[t] - 4 * sq[t];
+      }
+    } else {
+      r = gr_mul_par<4>(inv, sq, scr[grp], sub);
+      if (tid < 64) {
+        // (z^2 - z) / x: the coefficients move down one, the constant term times
+        // x^-1 = -(x^63 + x^3 + x^2 + 1)
+        u64 u = t < 63 ? sq[t + 1] : 0ull;
+        if (t == 0 || t == 2 || t == 3 || t == 63) u -= sq[0];
+        L2[t] = r;
+        L1[t] = zt[t] - u - r;
+      }
+    }
+  }
+  grid_dep();
   if (blk == 6) {
     __shared__ u64 fe[64];
     if (tid < 64) {
@@ -100,7 +113,6 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
     for (long long i = tid; i < a.nzero; i += 512) a.zero[i] = 0ull;
     return;
   }
-  const int sub = tid & 255, grp = tid >> 8;
   if (blk > 6) {
     __shared__ u64 w[2][64], e[2][64];
     const int i = 2 * (blk - 7) + grp, j = i < a.nvw ? i : i - a.nvw;
@@ -115,26 +127,21 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
     if (sub < 64) X[t] = v;
     return;
   }
-  // z^2 (the second group idles), then L2
-  u64 r = gr_mul_par<4>(zt, zt, scr[grp], sub);
-  if (tid < 64) sq[t] = a.mode == 1 ? r : r - zt[t];   // z^2, or z^2 - z
-  __syncthreads();
-  if (a.mode == 1) {
-    if (tid < 64) {
-      L2[t] = 2 * sq[t] - zt[t];
-      L1[t] = 4 * zt[t] - 4 * sq[t];
-    }
-  } else {
-    r = gr_mul_par<4>(inv, sq, scr[grp], sub);
-    if (tid < 64) {
-      // (z^2 - z) / x: the coefficients move down one, the constant term times
-      // x^-1 = -(x^63 + x^3 + x^2 + 1)
-      u64 u = t < 63 ? sq[t + 1] : 0ull;
-      if (t == 0 || t == 2 || t == 3 || t == 63) u -= sq[0];
-      L2[t] = r;
-      L1[t] = zt[t] - u - r;
+  const bool msg = blk == 2 || blk == 4;   // the components m, which take the party sums
+  if (msg) {
+    for (int i = tid; i < 9 * 64; i += 512) {
+      const int q = i >> 6, c = i & 63;
+      const u64* s0 = a.sums + (q < 6 ? q : q + 3) * a.ld;   // ee, S01, oo
+      u64 v = a.ld == 128 ? gr_reduce_at(s0, s0 + 64, c) : s0[c];
+      if (q >= 3 && q < 6) {   // cross: S01 + S10
+        const u64* s1 = a.sums + (q + 3) * a.ld;
+        v += a.ld == 128 ? gr_reduce_at(s1, s1 + 64, c) : s1[c];
+      }
+      S[q][c] = v;
     }
   }
+  __syncthreads();
+  u64 r;
   u64 h0 = 0, z = 0;
   if (tid < 64) {
     u64 h2;
@@ -180,7 +187,6 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
 __global__ void __launch_bounds__(64)
 k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u64* __restrict__ out,
          u64* __restrict__ rec) {
-  grid_dep();
   __shared__ u64 st[3][64];
   const int t = threadIdx.x;
   if (t < 24) {
@@ -189,6 +195,7 @@ k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u
              make_tag(purpose, s == 0 ? C_R1 : s == 1 ? C_R2 : C_M12), obj, t & 7, st[s]);
   }
   __syncthreads();
+  grid_dep();   // the streams come from the keys alone
   const u64 r1 = st[0][t], r2 = st[1][t], m = st[2][t];
   const u64 r2in = r2 ^ (t == xidx ? xmask : 0ull);
   rec[t] = r1;
@@ -309,7 +316,6 @@ __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
 // opening.  As separate launches (streams, multiplication matrices, three small GEMMs, messages,
 // copies of x' and y, Gram sums, reductions: 40 launches) it took 150-200 us a batch.
 __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
-  grid_dep();
   __shared__ u64 al[6][64];           // r1, r2, m of alpha; r_a, m - r2
   __shared__ u64 u[6][64], v[6][64], st[3][64], scr[4 * 128];
   __shared__ int last;
@@ -324,6 +330,7 @@ __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
     al[3][t] = al[0][t] + al[1][t];
     al[4][t] = al[2][t] - al[1][t];
   }
+  grid_dep();   // alpha comes from the keys alone
   u64 lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
   for (long long i = blockIdx.x; i <= a.D; i += gridDim.x) {
     __syncthreads();
