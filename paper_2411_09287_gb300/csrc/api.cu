@@ -781,7 +781,7 @@ int inner_verify_dense(mpc_ctx* ctx, u64 vid, u32 batch, const Vec& x, const Vec
 }
 
 // Elements of a claim up to which a round's fold and sums are one launch on the CUDA cores (on the
-// limb path): at 512 its 256 blocks still run at once, 20 us against 36; it would double with each
+// limb path): at 512 its 256 blocks still run at once, 16 us against 36; it would double with each
 // doubling, the tensor-core launches hardly grow up to 4096.
 constexpr long long SMALL_MAX = 512;
 

@@ -6,22 +6,27 @@
 
 namespace mpc3 {
 
+// What coefficient c of the reduction subtracts from lo[c], from the coefficients hi (64 ..).
+__device__ __forceinline__ u64 gr_carry_at(const u64* hi, int c) {
+  u64 v = 0;
+  if (c < 63) v += hi[c];
+  if (c >= 1) v += hi[c - 1];
+  if (c >= 3) v += hi[c - 3];
+  if (c >= 4) v += hi[c - 4];
+  if (c < 7) {   // H2 = (h_60 + h_61, h_61 + h_62, h_62), at the shifts 0, 1, 3, 4 of g
+    const u64 h0 = hi[60], h1 = hi[61], h2 = hi[62];
+    if ((0x1B >> c) & 1) v -= h0 + h1;
+    if ((0x36 >> c) & 1) v -= h1 + h2;
+    if ((0x6C >> c) & 1) v -= h2;
+  }
+  return v;
+}
+
 // Coefficient c of the reduction mod f of a 127-coefficient product (lo: coefficients 0..63, hi:
 // 64..126, hi[63] ignored): lo - H g + g H2 with x^64 = -g = -(x^4 + x^3 + x + 1), H2 the three
 // coefficients that H g carries past 63.
 __device__ __forceinline__ u64 gr_reduce_at(const u64* lo, const u64* hi, int c) {
-  u64 v = lo[c];
-  if (c < 63) v -= hi[c];
-  if (c >= 1) v -= hi[c - 1];
-  if (c >= 3) v -= hi[c - 3];
-  if (c >= 4) v -= hi[c - 4];
-  if (c < 7) {   // H2 = (h_60 + h_61, h_61 + h_62, h_62), at the shifts 0, 1, 3, 4 of g
-    const u64 h0 = hi[60], h1 = hi[61], h2 = hi[62];
-    if ((0x1B >> c) & 1) v += h0 + h1;
-    if ((0x36 >> c) & 1) v += h1 + h2;
-    if ((0x6C >> c) & 1) v += h2;
-  }
-  return v;
+  return lo[c] - gr_carry_at(hi, c);
 }
 
 // lo += product terms of coefficient t, hi += those of coefficient 64 + t, over the factors
@@ -71,6 +76,47 @@ __device__ __forceinline__ u64 gr_mul_par(const u64* a, const u64* b, u64* scr, 
   u64 lo = 0, hi = 0;
   gr_mac_part<64 / P>(a, b, sub & 63, (sub >> 6) * (64 / P), lo, hi);
   return gr_finish<P>(lo, hi, scr, sub);
+}
+
+// The terms of coefficients 2 l and 2 l + 1 (lo) and of 64 + 2 l, 65 + 2 l (hi) over the factors a_i,
+// i0 <= i < i0 + N (both even): a warp, lane l, takes all coefficients.  a, b 16-byte aligned: with
+// two coefficients a lane a pair of b serves four multiply-adds, half the shared-memory reads of
+// gr_mac_part, which bound blocks of many products.
+struct Gr2 {
+  u64 lo[2] = {0, 0}, hi[2] = {0, 0};
+  __device__ __forceinline__ void sub(const Gr2& o) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      lo[q] -= o.lo[q];
+      hi[q] -= o.hi[q];
+    }
+  }
+};
+template <int N>
+__device__ __forceinline__ void gr_mac2(const u64* a, const u64* b, int l, int i0, Gr2& g) {
+  u64 s0 = 0, s1 = 0, l0 = 0, l1 = 0;
+  ulonglong2 p = *reinterpret_cast<const ulonglong2*>(b + ((2 * l - i0) & 63));
+#pragma unroll
+  for (int k = 0; k < N; k += 2) {
+    const int i = i0 + k;
+    const ulonglong2 f = *reinterpret_cast<const ulonglong2*>(a + i);
+    const ulonglong2 n = *reinterpret_cast<const ulonglong2*>(b + ((2 * l - i - 2) & 63));
+    s0 += f.x * p.x;   // b_(2l - i)
+    s1 += f.x * p.y;   // b_(2l + 1 - i)
+    if (i == 2 * l) l0 = s0;
+    s0 += f.y * n.y;   // b_(2l - i - 1)
+    s1 += f.y * p.x;   // b_(2l - i)
+    if (i == 2 * l) l1 = s1;
+    p = n;
+  }
+  if (2 * l >= i0 + N) {
+    l0 = s0;
+    l1 = s1;
+  }
+  g.lo[0] += l0;
+  g.lo[1] += l1;
+  g.hi[0] += s0 - l0;
+  g.hi[1] += s1 - l1;
 }
 
 // Coefficient t of x v and of x^2 v (x^64 = -(x^4 + x^3 + x + 1)).

@@ -212,32 +212,41 @@ k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u
 // f (fold set: a_2e + f (a_2e+1 - a_2e), D elements into ceil(D / 2)), and this round's party sums over
 // the pairs of what it leaves (sums not null): blocks S00, S11 and the cross sum S01 + S10 as (e + o)(e'
 // + o') - S00 - S11, 127 unreduced coefficients each.  A block takes one pair: its 24 products one a
-// 64-thread group, then the fifteen products of the sums a quarter each a group.  Bound by latency; on
+// warp, then an eighth of each of the fifteen products of the sums a warp.  Bound by latency; on
 // the tensor cores, whose tiles want 128 rows and whose kernels first split their operands, the two
-// Gram launches and the fold of such a round took 36 us at 512 elements, this 20 us (15 without the fold).
+// Gram launches and the fold of such a round took 36 us at 512 elements, this 16 us, 13 without the fold (20 and 15 us
+// with a coefficient a thread and a load an operand and multiply-add).
 __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
   grid_dep();
-  __shared__ u64 f[64], v[2][12][64], d[4][64], red[9][128];
-  const int tid = threadIdx.x, t = tid & 63, g = tid >> 6;
+  __shared__ __align__(16) u64 f[64], v[2][12][64], d[8][64], red[9][128];
+  const int tid = threadIdx.x, t = tid & 63, g = tid >> 6, wp = tid >> 5, l = tid & 31;
   const long long pair = blockIdx.x;
   if (a.fold) {
     if (tid < 64) f[t] = a.f[t];
-    for (int i = g; i < 24; i += 4) {   // (element, component): six of each group
+    __syncthreads();
+    for (int i = wp; i < 24; i += 8) {   // (element, component): three of each warp
       const int e = i / 12, c = i % 12;
       const u64* src = a.in[c];
       const long long s0 = 2 * (2 * pair + e);
-      u64 base = 0, diff = 0;
-      if (src && s0 < a.D) {
-        base = src[s0 * 64 + t];
-        diff = (s0 + 1 < a.D ? src[(s0 + 1) * 64 + t] : 0ull) - base;
+      ulonglong2 base = make_ulonglong2(0, 0), r = base;
+      if (src && s0 < a.D) {   // uniform over the warp
+        base = reinterpret_cast<const ulonglong2*>(src + s0 * 64)[l];
+        if (s0 + 1 < a.D) r = reinterpret_cast<const ulonglong2*>(src + (s0 + 1) * 64)[l];
+        *reinterpret_cast<ulonglong2*>(&d[wp][2 * l]) = make_ulonglong2(r.x - base.x, r.y - base.y);
+        __syncwarp();
+        Gr2 m;
+        gr_mac2<64>(f, d[wp], l, 0, m);
+        __syncwarp();
+        u64* scr = d[wp];   // coefficients 64 .. 126
+        scr[2 * l] = m.hi[0];
+        scr[2 * l + 1] = m.hi[1];
+        __syncwarp();
+        r.x = base.x + m.lo[0] - gr_carry_at(scr, 2 * l);
+        r.y = base.y + m.lo[1] - gr_carry_at(scr, 2 * l + 1);
+        __syncwarp();
+        reinterpret_cast<ulonglong2*>(a.out[c] + (2 * pair + e) * 64)[l] = r;
       }
-      d[g][t] = diff;
-      __syncthreads();
-      u64 lo = 0, hi = 0;
-      if (src) gr_mac_part<64>(f, d[g], t, 0, lo, hi);
-      const u64 r = base + gr_finish<1>(lo, hi, red[g], t);
-      v[e][c][t] = r;
-      if (src && s0 < a.D) a.out[c][(2 * pair + e) * 64 + t] = r;
+      *reinterpret_cast<ulonglong2*>(&v[e][c][2 * l]) = r;
     }
   } else {
     for (int i = g; i < 24; i += 4) {
@@ -256,10 +265,9 @@ __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
     v[e][1][t] = v[e][10][t] - v[e][11][t];
   }
   __syncthreads();
-  // sums over even, odd and even + odd elements; pairs of components (u, v) of x at c, of y at 6 + c
-  u64 lo[9], hi[9];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) lo[q] = hi[q] = 0;
+  // sums over even, odd and even + odd elements; pairs of components (u, v) of x at c, of y at 6 + c;
+  // warp wp takes the factors 8 wp .. 8 wp + 7 of every product
+  Gr2 m[9];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     if (k == 2) {
@@ -268,28 +276,24 @@ __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
       __syncthreads();
     }
     u64(*w)[64] = v[k == 1 ? 1 : 0];
-    u64 nl = 0, nh = 0;
-    if ((a.in[0] || a.in[1]) && (a.in[6] || a.in[7])) gr_mac_part<16>(w[0], w[6], t, g * 16, lo[3 * k], hi[3 * k]);
-    if (a.in[2] && a.in[9]) gr_mac_part<16>(w[2], w[9], t, g * 16, nl, nh);
-    if (a.in[8] && a.in[3]) gr_mac_part<16>(w[8], w[3], t, g * 16, nl, nh);
-    lo[3 * k + 1] = 0ull - nl;
-    hi[3 * k + 1] = 0ull - nh;
-    nl = nh = 0;
-    if (a.in[4] && (a.in[10] || a.in[11])) gr_mac_part<16>(w[4], w[1], t, g * 16, lo[3 * k + 2], hi[3 * k + 2]);
-    if (a.in[10] && a.in[5]) gr_mac_part<16>(w[10], w[5], t, g * 16, nl, nh);
-    lo[3 * k + 2] -= nl;
-    hi[3 * k + 2] -= nh;
+    Gr2 n;
+    if ((a.in[0] || a.in[1]) && (a.in[6] || a.in[7])) gr_mac2<8>(w[0], w[6], l, wp * 8, m[3 * k]);
+    if (a.in[2] && a.in[9]) gr_mac2<8>(w[2], w[9], l, wp * 8, n);
+    if (a.in[8] && a.in[3]) gr_mac2<8>(w[8], w[3], l, wp * 8, n);
+    m[3 * k + 1].sub(n);
+    n = Gr2();
+    if (a.in[4] && (a.in[10] || a.in[11])) gr_mac2<8>(w[4], w[1], l, wp * 8, m[3 * k + 2]);
+    if (a.in[10] && a.in[5]) gr_mac2<8>(w[10], w[5], l, wp * 8, n);
+    m[3 * k + 2].sub(n);
   }
-  for (int p = 0; p < 4; ++p) {   // the groups' quarters
-    if (g == p) {
+  for (int p = 0; p < 8; ++p) {
+    if (wp == p) {
 #pragma unroll
       for (int q = 0; q < 9; ++q) {
-        if (p == 0) {
-          red[q][t] = lo[q];
-          red[q][64 + t] = hi[q];
-        } else {
-          red[q][t] += lo[q];
-          red[q][64 + t] += hi[q];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          red[q][2 * l + h] = m[q].lo[h] + (p ? red[q][2 * l + h] : 0ull);
+          red[q][64 + 2 * l + h] = m[q].hi[h] + (p ? red[q][64 + 2 * l + h] : 0ull);
         }
       }
     }
