@@ -20,6 +20,14 @@ inline unsigned grid_for(long long n8) {
   return (unsigned)g;
 }
 
+// Threads a block of a kernel that gives a warp 256 words and a long chain of streams: two warps while
+// full blocks would leave SMs without one, so that the warps spread out.
+inline unsigned warp_block(long long n8) { return n8 < 152ll * 2 * TPB ? 64 : TPB; }
+inline unsigned warp_grid(long long n8) {
+  const long long g = (n8 + warp_block(n8) - 1) / warp_block(n8);
+  return (unsigned)(g > (1ll << 20) ? 1ll << 20 : g);
+}
+
 __device__ __forceinline__ u64 asr64(u64 v, int t) { return (u64)(((long long)v) >> t); }
 
 // Words 8 blk .. 8 blk + 7 of a truncation-bit stream.  Unkeyed: words of the stream (tag, obj).
@@ -455,7 +463,7 @@ void launch_trunc_p0(cudaStream_t st, long long E, Key k01, Key k02, u64 obj, in
                      u64* zout, u64* pq, u64* p0_out_gp2, u64* p0_out_gq2, u64* p1_out_mp,
                      u64* p1_out_mq, const u64* row_keys, long long N) {
   if (E <= 0) return;
-  launch_dep(k_trunc_p0, grid_for((E + 7) / 8), TPB, 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2),
+  launch_dep(k_trunc_p0, warp_grid((E + 7) / 8), warp_block((E + 7) / 8), 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2),
       make_tag(P_TRUNC_P, C_R1), make_tag(P_TRUNC_P, C_R2), make_tag(P_TRUNC_P, C_G1),
       make_tag(P_TRUNC_Q, C_R1), make_tag(P_TRUNC_Q, C_R2), make_tag(P_TRUNC_Q, C_G1), zpre, zout,
       pq, p0_out_gp2, p0_out_gq2, p1_out_mp, p1_out_mq);
@@ -467,7 +475,7 @@ void launch_trunc_finish(cudaStream_t st, long long E, Key k01, Key k02, u64 obj
                          const u64* p1_mp1, const u64* p1_mq1, u64* zpre, u64* zout, u64* pq,
                          const u64* row_keys, long long N) {
   if (E <= 0) return;
-  launch_dep(k_trunc_finish, grid_for((E + 7) / 8), TPB, 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2), p1_in_mp,
+  launch_dep(k_trunc_finish, warp_grid((E + 7) / 8), warp_block((E + 7) / 8), 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2), p1_in_mp,
       p1_in_mq, p2_in_mp, p2_in_mq, p2_gp2, p2_gq2, p1_mp1, p1_mq1, zpre, zout, pq);
 }
 
