@@ -50,6 +50,7 @@ inline void counted(int k, F f, A... a) {
 #define launch_gr_fold_reduce(...) counted(1, mpc3::launch_gr_fold_reduce, __VA_ARGS__)
 #define launch_neg_copy(...) counted(1, mpc3::launch_neg_copy, __VA_ARGS__)
 #define launch_round_tail(...) counted(1, mpc3::launch_round_tail, __VA_ARGS__)
+#define launch_zero_rows(...) counted(1, mpc3::launch_zero_rows, __VA_ARGS__)
 #define launch_small_round(...) counted(1, mpc3::launch_small_round, __VA_ARGS__)
 #define launch_inner_verify(...) counted(1, mpc3::launch_inner_verify, __VA_ARGS__)
 #define launch_reveal(...) counted(1, mpc3::launch_reveal, __VA_ARGS__)
@@ -555,8 +556,9 @@ u64* cur_sums(const Small& s) { return s.U + s.uc * SUMS_WORDS; }
 // element is s.coef[0..63].
 void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, const Small& s,
                 const u64* sums, int ld, u64* trace, u64* V = nullptr, u64* W = nullptr,
-                int nvw = 0) {
+                int nvw = 0, const ZeroRows* pad = nullptr) {
   RoundTail a;
+  for (int q = 0; q < 12; ++q) a.pad[q] = pad ? pad->p[q] : nullptr;
   a.V = V;   // the weights of a round over a matrix S: folded along bit k - 1
   a.W = W;
   a.nvw = nvw;
@@ -586,6 +588,16 @@ void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, 
   s.uc ^= 1;
 }
 
+// The rows past vectors of D elements, when D is odd.
+ZeroRows pad_rows(const Vec& x, const Vec& y, long long D) {
+  ZeroRows r{};
+  for (int c = 0; c < 6 && (D & 1); ++c) {
+    r.p[c] = x.c[c] ? x.c[c] + D * 64 : nullptr;
+    r.p[6 + c] = y.c[c] ? y.c[c] + D * 64 : nullptr;
+  }
+  return r;
+}
+
 // One Pi_Reduce round on a dense claim (Fig. Reduce).  x, y: current vectors (D elements, with
 // capacity for D+1), z: current claim; writes the folded vectors into xo, yo and z into zo.
 int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, const Vec& y,
@@ -593,12 +605,9 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
                        u64* trace) {
   cudaStream_t st = ctx->st;
   const long long Dh = (D + 1) / 2;
-  if (D & 1) {
-    for (int c = 0; c < 6; ++c) {
-      if (x.c[c]) CK(cudaMemsetAsync(x.c[c] + D * 64, 0, 512, st));
-      if (y.c[c]) CK(cudaMemsetAsync(y.c[c] + D * 64, 0, 512, st));
-    }
-  }
+  // a vector of odd length is followed by a row of zeros: the tail clears those of the vectors that
+  // this round folds into (before the fold; the first round's are run_dense's)
+  ZeroRows pad = pad_rows(xo, yo, Dh);
   View f[2], g[2];
   for (int a = 0; a < 2; ++a) {
     for (int c = 0; c < 6; ++c) {
@@ -696,7 +705,7 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       if ((rc = party_sums(ctx, f[1], g[1], Dh, s.Pmat + 9 * 4096, S11))) return rc;
     }
   }
-  round_tail(ctx, vid, batch, k, z, zo, s, sums, ld, trace);
+  round_tail(ctx, vid, batch, k, z, zo, s, sums, ld, trace, nullptr, nullptr, 0, &pad);
   // f(zeta) = f(0) + zeta (f(1) - f(0)): rows [x_{2i+1} - x_{2i}] times M_zeta, plus x_{2i}.
   // Vectors that sit at one stride (the dense plans put a slot's x vectors, then its y vectors,
   // one after another) go through one launch: segment s of Dh rows (padded to whole tiles); all
@@ -793,6 +802,8 @@ int run_dense(mpc_ctx* ctx, u64 vid, u32 batch, Dense& dv, long long D, const u6
   int zi = 0;
   const bool tc = ctx->gemm_path == MPC_GEMM_LIMB_TC;
   int k = k0;
+  if (k <= R && (D & 1) && !(tc && D <= SMALL_MAX))
+    launch_zero_rows(ctx->st, pad_rows(dv.x[dv.cur], dv.y[dv.cur], D));
   for (; k <= R && !(tc && D <= SMALL_MAX); ++k) {
     Vec& x = dv.x[dv.cur];
     Vec& y = dv.y[dv.cur];

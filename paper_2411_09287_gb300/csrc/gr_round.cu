@@ -33,7 +33,7 @@ constexpr int REC_ROWS = 7;
 // One Pi_Reduce round after its party sums (Fig. Reduce): h(0) and h(p2) by secure GR inner
 // products, zeta' drawn and opened, the next claim z' = L0 h(0) + L1 (z - h(0)) + L2 h(p2), the
 // fold element f and its multiplication matrix.  Block c < 6 computes component c of h(0), h(p2)
-// and z'; block 6 the matrix, the Pi_Rec messages and the next round's cleared sums; in a round over
+// and z'; block 6 the matrix, the Pi_Rec messages and the next round's cleared sums and zero rows; in a round over
 // a matrix S (nvw > 0) the blocks from 7 on take the weights V_j, W_j, two each: times 1 - f or f by
 // bit vwbit of j.  Every block derives zeta' from its streams, so that no block waits for another.
 //
@@ -111,6 +111,8 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
     __syncthreads();
     for (int i = tid; i < 4096; i += 512) a.MM[i] = gr_mulmat_at(fe, i >> 6, i & 63);
     for (long long i = tid; i < a.nzero; i += 512) a.zero[i] = 0ull;
+    for (int i = tid; i < 12 * 64; i += 512)
+      if (a.pad[i >> 6]) a.pad[i >> 6][i & 63] = 0ull;
     return;
   }
   if (blk > 6) {
@@ -549,7 +551,16 @@ k_weighted_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64*
   }
 }
 
+// 64 words of zeros at each of the 12 rows (null: none)
+__global__ void __launch_bounds__(768) k_zero_rows(const ZeroRows r) {
+  grid_dep();
+  u64* p = r.p[threadIdx.x >> 6];
+  if (p) p[threadIdx.x & 63] = 0ull;
+}
+
 }  // namespace
+
+void launch_zero_rows(cudaStream_t st, const ZeroRows& r) { launch_dep(k_zero_rows, 1, 768, 0, st, r); }
 
 void launch_round_tail(cudaStream_t st, const RoundTail& a) {
   launch_dep(k_round_tail, 7 + a.nvw, 512, 0, st, a);

@@ -157,7 +157,12 @@ struct RoundTail {
   u64* trace;           // zeta' | h(0) | h(p2) of the round, or null
   u64 *V, *W;           // nvw elements each (nvw = 0: none), times f or 1 - f by bit vwbit of j
   int nvw, vwbit;
+  u64* pad[12];         // rows of 64 words to clear (null: none): past the folded vectors' odd ends
 };
+struct ZeroRows {
+  u64* p[12];
+};
+void launch_zero_rows(cudaStream_t st, const ZeroRows& r);
 void launch_round_tail(cudaStream_t st, const RoundTail& a);
 // A random GR element of the streams of (purpose, obj), opened into out; record in rec.
 void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
