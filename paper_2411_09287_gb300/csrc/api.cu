@@ -1,6 +1,6 @@
 // libmpc3: the C-ABI and the protocol driver.  Every protocol step runs in the kernels of this
 // library; the host code here only sequences them, moves messages between the three simulated
-// parties (device-to-device copies counted in the ledger) and carves the caller's workspace.
+// parties (counted in the ledger) and carves the caller's workspace.
 //
 // Paper map: mpc_share_input = Pi_<.>^{l,0} (Sec. 2); mpc_mult = Pi_Mult (Fig. MultP);
 // mpc_matmul = Pi_Inner per output (Fig. DPP, Sec. 4.1) + Pi_Trunc (Fig. trunc);
@@ -291,7 +291,13 @@ void apply_fault(mpc_ctx* ctx, int site, u64* dst, long long n) {
   }
 }
 
-int deliver(mpc_ctx* ctx, int phase, int proto, const u64* src, u64* dst, long long n, int site) {
+void count_msgs(mpc_ctx* ctx, int phase, int proto, int count, u64 bytes_each) {
+  ctx->ledger[phase][proto] += (u64)count * bytes_each;
+  ctx->nmsg += (u64)count;
+}
+
+
+int deliver_copy(mpc_ctx* ctx, int phase, int proto, const u64* src, u64* dst, long long n, int site) {
   if (n > 0) CK(cudaMemcpyAsync(dst, src, (size_t)n * 8, cudaMemcpyDeviceToDevice, ctx->st));
   ctx->ledger[phase][proto] += (u64)n * 8;
   ctx->nmsg += 1;
@@ -299,9 +305,15 @@ int deliver(mpc_ctx* ctx, int phase, int proto, const u64* src, u64* dst, long l
   return MPC_OK;
 }
 
-void count_msgs(mpc_ctx* ctx, int phase, int proto, int count, u64 bytes_each) {
-  ctx->ledger[phase][proto] += (u64)count * bytes_each;
-  ctx->nmsg += (u64)count;
+// The message src to a receiver that only reads it: it is handed over in place (dst becomes src), and
+// copied only to be corrupted by an armed fault.  A copy of a small message is a launch of 4 us.
+int deliver(mpc_ctx* ctx, int phase, int proto, u64* src, u64*& dst, long long n, int site) {
+  if (site >= 0 && n > 0 &&
+      (ctx->fault[site].armed || (site == MPC_SITE_GAMMA2 && ctx->fault[MPC_SITE_HIGH_BIT].armed)))
+    return deliver_copy(ctx, phase, proto, src, dst, n, site);
+  count_msgs(ctx, phase, proto, 1, (u64)n * 8);
+  dst = src;
+  return MPC_OK;
 }
 
 int read_status(mpc_ctx* ctx, u32* out) {
@@ -2054,11 +2066,11 @@ int mpc_share_input_from(mpc_ctx* ctx, uint64_t call_id, int owner, const uint64
   u64* m2 = (u64*)xs + 4 * n;
   if (owner == 1)
     CK(cudaMemcpyAsync(m1, mout, (size_t)n * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  else if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m1, n, MPC_SITE_MX_COPY_P1)))
+  else if ((rc = deliver_copy(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m1, n, MPC_SITE_MX_COPY_P1)))
     return rc;
   if (owner == 2)
     CK(cudaMemcpyAsync(m2, mout, (size_t)n * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  else if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m2, n, -1)))
+  else if ((rc = deliver_copy(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m2, n, -1)))
     return rc;
   return cuda_check(ctx, "share_input");
 }
