@@ -263,7 +263,7 @@ def rooflines(phases, steps, peaks, clk, M, N, K, E, gemm_path):
     """Roofline records of the dominant kernels: CUDA-event time of each kernel inside the step
     and the algorithmic u64 multiply-accumulates the library attributes to it.  Tensor kernels
     count the digit products they form (36 f16 digit pairs per u64 MAC for the 8-bit balanced
-    digits, 8 where one operand is a bit; 16 e4m3 limbs per bit-times-u64 MAC for the S matrix;
+    digits, 8 where one operand is a bit; 13 e4m3 limbs per bit-times-u64 MAC for the S matrix;
     the library reports the work in 36-pair units), 2 FLOP each, against
     the measured cuBLAS bf16 rate (sustained: they run inside a long step) or twice it for e4m3
     (the nominal fp8 : bf16 ratio).  CUDA-core kernels count 3 IMAD per u64 MAC."""
@@ -286,8 +286,8 @@ def rooflines(phases, steps, peaks, clk, M, N, K, E, gemm_path):
                      "frac": ach / peak, "traffic": tr * E / NCU_TRAFFIC_E if tr else None,
                      "ms_per_step": ms, "u64_macs_per_step": w, "peak_source": src, "note": note}
 
-    rec("k_trunc_s", 2 * 16, 2 * bf16, "TFLOP/s", "tensor",
-        "tcgen05 kind::f8f6f4, 16 e4m3 limbs per MAC; peak = 2 x measured bf16 (sustained)")
+    rec("k_trunc_s", 2 * 13, 2 * bf16, "TFLOP/s", "tensor",
+        "tcgen05 kind::f8f6f4, 13 e4m3 limbs per MAC; peak = 2 x measured bf16 (sustained)")
     if gemm_path == "tc":
         for k, what in (("k_limb_gemm", "limb-split products"), ("k_gr_matmul", "GR-matrix products"),
                         ("k_gram", "Gram sums")):

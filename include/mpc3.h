@@ -17,6 +17,8 @@
  *     with m = x + [r]_1 + [r]_2 (Sec. 2 Notation).  Matrices are row-major inside a component.
  *   - Every call enqueues work on the context's stream and returns once it is enqueued, except
  *     mpc_verify_* and mpc_reconstruct with a host output, which synchronise to read the result.
+ *     (Independent verification batches run on streams of the context's own, which its stream waits
+ *     for before the call returns.)
  *   - Buffers passed in are borrowed for the duration of the enqueued work; the caller owns them.
  *     `workspace` is caller-owned device scratch of at least mpc_workspace_size(...) bytes,
  *     256-byte aligned; its contents are undefined after the call.
