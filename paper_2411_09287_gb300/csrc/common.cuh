@@ -136,25 +136,6 @@ __host__ __device__ inline u64 gr_hg(const u64* h, int s) {   // (H g)_s, h has 
   return v;
 }
 
-// Serial reduction (one thread): out[c] for c < 64 from p[0..126].
-__host__ __device__ inline void gr_reduce_serial(const u64* p, u64* out) {
-  const u64* h = p + 64;
-  u64 h2[3];
-  for (int m = 0; m < 3; ++m) h2[m] = gr_hg(h, 64 + m);
-  for (int c = 0; c < 64; ++c) {
-    u64 v = p[c] - gr_hg(h, c);
-    if (c < 7) {
-      u64 g = 0;
-      if (c < 3) g += h2[c];
-      if (c - 1 >= 0 && c - 1 < 3) g += h2[c - 1];
-      if (c - 3 >= 0 && c - 3 < 3) g += h2[c - 3];
-      if (c - 4 >= 0 && c - 4 < 3) g += h2[c - 4];
-      v += g;
-    }
-    out[c] = v;
-  }
-}
-
 // Block-cooperative product out = a * b (64 threads of the block participate with tid < 64;
 // other threads idle).  `scratch` holds 128 words of shared memory.  a, b, out may alias.
 __device__ inline void gr_mul_block(const u64* a, const u64* b, u64* out, u64* scratch) {
@@ -186,27 +167,6 @@ __device__ inline void gr_mul_block(const u64* a, const u64* b, u64* out, u64* s
   __syncthreads();
   if (t < 64) out[t] = lo;
   __syncthreads();
-}
-
-// Multiplication matrix of a constant a: M[b][c] = coefficient c of a * x^b (block-cooperative,
-// 64 threads).  Row b+1 = x * row b: shift up one coefficient, the top coefficient u wraps as
-// x^64 = -(1 + x + x^3 + x^4).
-__device__ inline void gr_mulmat_block(const u64* a, u64* M /*64x64 row-major*/) {
-  const int t = threadIdx.x;
-  if (t < 64) M[t] = a[t];
-  __syncthreads();
-  for (int b = 1; b < 64; ++b) {
-    u64 v = 0;
-    if (t < 64) {
-      const u64* prev = M + (b - 1) * 64;
-      const u64 u = prev[63];
-      v = (t > 0) ? prev[t - 1] : 0;
-      if (t == 0 || t == 1 || t == 3 || t == 4) v -= u;
-    }
-    __syncthreads();
-    if (t < 64) M[b * 64 + t] = v;
-    __syncthreads();
-  }
 }
 
 // ---------------------------------------------------------------------------------------------
