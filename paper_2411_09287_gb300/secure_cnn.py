@@ -146,7 +146,7 @@ def _concat(ctx, parts):
 
 
 # Comparisons per non-linear call: each call (a ReLU chunk, or whole channel planes of a max-pool)
-# is verified on its own; 2^16 comparisons take about 37 GB of workspace.
+# is verified on its own; 2^16 comparisons take about 4 GB of workspace.
 NL_CHUNK = 1 << 16
 
 
