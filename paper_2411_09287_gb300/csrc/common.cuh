@@ -17,9 +17,16 @@ typedef uint32_t u32;
 // ---------------------------------------------------------------------------------------------
 // Launches.  A protocol call is a chain of 50 to 400 kernels of 2 to 20 us, each of which needs its
 // predecessor's results, so what passes between two kernels counts as much as a kernel: launch_dep
-// lets a kernel's blocks be set up while its predecessor runs, and grid_dep, the first statement of
+// lets a kernel's blocks be set up while its predecessor runs, and grid_dep, called by every thread of
 // every kernel launched this way, waits for the predecessor's end (its writes visible, and through
 // its own grid_dep those of everything before it) and allows the successor's set-up in turn.
+//   - Before grid_dep a kernel touches nothing that another kernel of a chain writes: kernel
+//     parameters, constants of the context and its own shared memory only (k_round_tail, k_reveal and
+//     k_inner_verify draw their streams there; everywhere else grid_dep is the first statement).
+//   - A block can be resident while its inputs are still being written, so they are not read-only for
+//     the kernel's lifetime, which is what the non-coherent loads of a const __restrict__ pointer or
+//     of __ldg presume (and lets the compiler move them past the wait): inputs are plain const
+//     pointers and plain loads.
 // A kernel that takes tensor memory calls grid_dep before it allocates: a block that held it while it
 // waited could keep a block of its predecessor, on the same SM, from getting any.
 // Verified product of 64 x 64 x 128: 1.26 ms without, 1.05 ms with it; ReLU of 128: 1.30, 1.09 ms.

@@ -33,7 +33,7 @@ __device__ __forceinline__ void mult1(const u64 (&x)[6], const u64 (&y)[6], u64 
   z[4] = p2 + (p1 ^ p1x);
 }
 
-__device__ __forceinline__ u64 bit_of(const u64* __restrict__ w, long long i) {
+__device__ __forceinline__ u64 bit_of(const u64* w, long long i) {
   return (w[i >> 6] >> (i & 63)) & 1ull;
 }
 

@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(256) k_gf_vectors(const GfVerify a, const Coef
 // a_2i+1), and takes round k's sums of them.  A thread makes two folded elements: 24 products for
 // the folds and 16 for the sums.
 __global__ void __launch_bounds__(128)
-k_gf_round(const GfVerify a, const Coef cf, int k, long long D, const u64* __restrict__ x,
-           const u64* __restrict__ y, long long ld, u64* __restrict__ xo, u64* __restrict__ yo,
+k_gf_round(const GfVerify a, const Coef cf, int k, long long D, const u64* x,
+           const u64* y, long long ld, u64* __restrict__ xo, u64* __restrict__ yo,
            long long ldo) {
   grid_dep();
   const long long Dh = (D + 1) / 2, np = (Dh + 1) / 2;

@@ -41,7 +41,7 @@ struct BlkRows {
 
 template <int B, bool FULL>
 __global__ void __launch_bounds__(512)
-k_blk_sums(const BlkIn in, long long nb, int sh, const u64* __restrict__ R, u64* __restrict__ out) {
+k_blk_sums(const BlkIn in, long long nb, int sh, const u64* R, u64* __restrict__ out) {
   grid_dep();
   using Rows = BlkRows<B, FULL>;
   constexpr int NB = 8;
@@ -114,7 +114,7 @@ k_blk_sums(const BlkIn in, long long nb, int sh, const u64* __restrict__ R, u64*
 // out[c][j] += sum_w R[w] Z_c[64 w + j] for the 6 components (the claim of a bit batch): 384 rows,
 // 48 a group, as above.
 __global__ void __launch_bounds__(512)
-k_words_sums(const u64* __restrict__ z, long long ldz, long long nw, const u64* __restrict__ R,
+k_words_sums(const u64* z, long long ldz, long long nw, const u64* R,
              u64* __restrict__ out) {
   grid_dep();
   constexpr int NB = 8, G = 48;
@@ -152,7 +152,7 @@ k_words_sums(const u64* __restrict__ z, long long ldz, long long nw, const u64* 
 
 // z_c += sum_j T_j Zr[c n + j] over the eight j of block (c, y): the claim from its row sums.
 __global__ void __launch_bounds__(256)
-k_blk_claim(const u64* __restrict__ T, const u64* __restrict__ Zr, int n, u64* __restrict__ z) {
+k_blk_claim(const u64* T, const u64* Zr, int n, u64* __restrict__ z) {
   grid_dep();
   __shared__ u64 a[8][64], b[8][64], scr[4 * 128];
   const int tid = threadIdx.x, c = blockIdx.x, j0 = blockIdx.y * 8;
@@ -177,7 +177,7 @@ k_blk_claim(const u64* __restrict__ T, const u64* __restrict__ Zr, int n, u64* _
 template <int B, bool ROWS, bool VEC>
 __global__ void __launch_bounds__(256)
 k_blk_combine(const BlkVec in, const BlkOut out, long long D, long long nb, int sh,
-              const u64* __restrict__ Gt) {
+              const u64* Gt) {
   grid_dep();
   const int t = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * 8;
@@ -203,13 +203,13 @@ k_blk_combine(const BlkVec in, const BlkOut out, long long D, long long nb, int 
       if (VEC && whole) {
 #pragma unroll
         for (int j = 0; j < B; j += 2) {
-          const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(w + j));
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(w + j);
           s[j] = v.x;
           s[j + 1 < B ? j + 1 : j] = v.y;
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < B; ++j) s[j] = (whole || b * B + j < D) ? __ldg(w + j) : 0ull;
+        for (int j = 0; j < B; ++j) s[j] = (whole || b * B + j < D) ? w[j] : 0ull;
       }
       u64 v0 = 0, v1 = 0;
 #pragma unroll

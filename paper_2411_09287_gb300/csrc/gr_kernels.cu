@@ -28,7 +28,7 @@ inline unsigned grid_for(long long n) {
 // rows (16.3 with 256 threads).
 constexpr int POW_ROWS = 16, POW_LG = 4;
 __global__ void __launch_bounds__(512)
-k_gr_powers(const u64* __restrict__ a, long long n, u64* __restrict__ table) {
+k_gr_powers(const u64* a, long long n, u64* __restrict__ table) {
   grid_dep();
   __shared__ u64 rows[POW_ROWS][64], P[64], Pk[POW_LG][64], scr[8 * 128];
   const int tid = threadIdx.x, t = tid & 63;
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256) k_gr_mul1(const u64* a, const u64* b, u64
 
 // out_c = a_c + r b_c, one block per c
 __global__ void __launch_bounds__(256)
-k_gr_axpy(const u64* __restrict__ r, const u64* __restrict__ a, const u64* __restrict__ b,
+k_gr_axpy(const u64* r, const u64* a, const u64* b,
           u64* __restrict__ out) {
   grid_dep();
   __shared__ u64 x[64], y[64], scr[4 * 128];
@@ -121,7 +121,7 @@ __global__ void k_word_transpose(long long rows, long long cols, long long n, co
 }
 
 // out[i] = src[idx(i)] for rows of 64 words, idx(i) = ((i mul) / div) mod m (m = 0: no mod).
-__global__ void k_gather_rows_affine(long long n, const u64* __restrict__ src, long long mul,
+__global__ void k_gather_rows_affine(long long n, const u64* src, long long mul,
                                      long long div, long long m, u64* __restrict__ out) {
   grid_dep();
   for (long long i = blockIdx.x; i < n; i += gridDim.x) {
@@ -133,7 +133,7 @@ __global__ void k_gather_rows_affine(long long n, const u64* __restrict__ src, l
 
 // out[i] = sum_{h < n} in[h ld + i] for i < m words.
 __global__ void __launch_bounds__(256)
-k_sum_blocks(long long m, long long n, long long ld, const u64* __restrict__ in,
+k_sum_blocks(long long m, long long n, long long ld, const u64* in,
              u64* __restrict__ out) {
   grid_dep();
   const long long i = blockIdx.x * 256ll + threadIdx.x;
@@ -145,7 +145,7 @@ k_sum_blocks(long long m, long long n, long long ld, const u64* __restrict__ in,
 }
 
 // out[c] = sum_{h < nper} in[c nper + h] for c < ncomp (rows of 64 words).
-__global__ void k_block_rowsum(long long nper, const u64* __restrict__ in, u64* __restrict__ out) {
+__global__ void k_block_rowsum(long long nper, const u64* in, u64* __restrict__ out) {
   grid_dep();
   const long long c = blockIdx.x;
   u64 v = 0;
@@ -205,7 +205,7 @@ __global__ void k_gr_inverses(u64* out) {
 
 // ---- fold of Gram sums ------------------------------------------------------------------------
 // P: n matrices of 64x64 (P[a][b] = sum u_a v_b); out: n reduced GR elements.
-__global__ void k_gr_fold_reduce(const u64* __restrict__ P, u64* __restrict__ out) {
+__global__ void k_gr_fold_reduce(const u64* P, u64* __restrict__ out) {
   grid_dep();
   __shared__ u64 prod[128];
   const u64* M = P + (long long)blockIdx.x * 4096;
@@ -235,7 +235,7 @@ __global__ void k_gr_fold_reduce(const u64* __restrict__ P, u64* __restrict__ ou
   }
 }
 
-__global__ void k_neg_copy(const u64* __restrict__ a, long long n, u64* __restrict__ out) {
+__global__ void k_neg_copy(const u64* a, long long n, u64* __restrict__ out) {
   grid_dep();
   for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < n;
        w += (long long)gridDim.x * blockDim.x)
@@ -244,7 +244,7 @@ __global__ void k_neg_copy(const u64* __restrict__ a, long long n, u64* __restri
 
 // ---- truncation-pair batch --------------------------------------------------------------------
 // u_j = c_j + r c'_j with c_j = -2^(j+1), c'_j = -2 w_j (w_j the weight of bit j in >>_arith t).
-__global__ void k_trunc_u(const u64* __restrict__ r, int t, u64* __restrict__ u) {
+__global__ void k_trunc_u(const u64* r, int t, u64* __restrict__ u) {
   grid_dep();
   const int j = blockIdx.x;
   const int c = threadIdx.x;
@@ -267,8 +267,8 @@ __global__ void k_trunc_u(const u64* __restrict__ r, int t, u64* __restrict__ u)
 // R_i X_{(t-i) mod 64} to the low coefficient t (i <= t) or to the high coefficient 64 + t
 // (i > t), followed by the reduction mod f.  VW in shared memory; R (optional) holds r^(2e).
 __global__ void __launch_bounds__(256)
-k_trunc_materialize(long long E, const u64* __restrict__ words, const u64* __restrict__ VW,
-                    const u64* __restrict__ R, int kd, u64* __restrict__ out) {
+k_trunc_materialize(long long E, const u64* words, const u64* VW,
+                    const u64* R, int kd, u64* __restrict__ out) {
   grid_dep();
   __shared__ u64 vw[64 * 64];
   __shared__ u64 xs[4][64], rr[4][64], hp[4][64];
@@ -330,7 +330,7 @@ k_trunc_materialize(long long E, const u64* __restrict__ words, const u64* __res
 __device__ __forceinline__ int padj(int j) { return j + (j >> 3); }
 
 __global__ void __launch_bounds__(256)
-k_gr_mul_rows(long long n, const u64* __restrict__ a, const u64* __restrict__ b, u64* out) {
+k_gr_mul_rows(long long n, const u64* a, const u64* b, u64* out) {
   grid_dep();
   __shared__ u64 sa[8][64], sbp[8][216], sc[8][128];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -395,8 +395,8 @@ k_gr_mul_rows(long long n, const u64* __restrict__ a, const u64* __restrict__ b,
 // block for the smallest batches and 256 for 2^20 (361 and 413 us).
 template <int NR>
 __global__ void __launch_bounds__(256)
-k_scalar_gr_sum(long long n, const u64* __restrict__ A, long long lda, int nrows,
-                const u64* __restrict__ R, u64* __restrict__ out) {
+k_scalar_gr_sum(long long n, const u64* A, long long lda, int nrows,
+                const u64* R, u64* __restrict__ out) {
   grid_dep();
   __shared__ __align__(16) u64 as[256][NR];
   const int t = threadIdx.x & 63, grp = threadIdx.x >> 6;

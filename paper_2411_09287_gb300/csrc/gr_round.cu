@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
 // constants) of all 6 x 9 blocks first, by one thread each, then six threads run the rounds, whose
 // dependent chain is what the launch takes.
 __global__ void __launch_bounds__(64)
-k_rec_hash(const u64* __restrict__ log, u32* status, u32 flag) {
+k_rec_hash(const u64* log, u32* status, u32 flag) {
   grid_dep();
   constexpr int LD = 55;             // words of one schedule step, 54 used
   __shared__ u32 wk[64 * LD];
@@ -515,7 +515,7 @@ k_rec_hash(const u64* __restrict__ log, u32* status, u32 flag) {
 // dependent products' latency.  One thread group per j ran 2^k + 5 products one after another:
 // 201 us for k = 6, 461 us for the six rounds of a bit batch.
 __global__ void __launch_bounds__(256)
-k_weighted_sums(const u64* __restrict__ V, const u64* __restrict__ W, const u64* __restrict__ S,
+k_weighted_sums(const u64* V, const u64* W, const u64* S,
                 int n, int k, u64* __restrict__ out) {
   grid_dep();
   __shared__ u64 w[8][64], s[8][64], T[2][64], v[64], scr[4 * 128];

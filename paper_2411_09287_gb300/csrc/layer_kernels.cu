@@ -23,7 +23,7 @@ inline unsigned lgrid(long long n) {
 // floor(x 2^k) as a two's-complement word; x 2^k outside [-2^63, 2^63) saturates, NaN gives 0.
 // Scaling by 2^k is exact in binary floating point (short of overflow, which saturates), and so
 // is floor; the conversion is exact inside the range.
-__global__ void k_encode_fixed(const double* __restrict__ x, long long n, int k,
+__global__ void k_encode_fixed(const double* x, long long n, int k,
                                u64* __restrict__ out) {
   grid_dep();
   const double lo = -9223372036854775808.0, hi = 9223372036854775808.0;
@@ -40,7 +40,7 @@ __global__ void k_encode_fixed(const double* __restrict__ x, long long n, int k,
 }
 
 // the signed value of a word divided by 2^k
-__global__ void k_decode_fixed(const u64* __restrict__ v, long long n, int k,
+__global__ void k_decode_fixed(const u64* v, long long n, int k,
                                double* __restrict__ out) {
   grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -59,7 +59,7 @@ struct ImCol {
   int off;        // (ch H + di) W + dj
   short di, dj;
 };
-__global__ void __launch_bounds__(LTPB) k_im2col(const u64* __restrict__ x, ConvGeom g, u64* __restrict__ cols) {
+__global__ void __launch_bounds__(LTPB) k_im2col(const u64* x, ConvGeom g, u64* __restrict__ cols) {
   grid_dep();
   __shared__ ImCol tab[IM_COLS];
   __shared__ long long base[IM_ROWS];
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(LTPB) k_im2col(const u64* __restrict__ x, Conv
 
 // d1 = [r_x]_1 - [r]_1 and d2 = [r_x]_2 - [r]_2, as P1 and P2 compute them (components 3, 5)
 // and as P0 does (components 0, 1); rx holds the pairs' mask shares in the same components.
-__global__ void k_trunc_remask(const u64* __restrict__ xs, const u64* __restrict__ rx, long long n,
+__global__ void k_trunc_remask(const u64* xs, const u64* rx, long long n,
                                u64* __restrict__ d1_p1, u64* __restrict__ d2_p2,
                                u64* __restrict__ d1_p0, u64* __restrict__ d2_p0) {
   grid_dep();
@@ -122,9 +122,9 @@ __global__ void k_trunc_remask(const u64* __restrict__ xs, const u64* __restrict
 
 // m' = m + d1 + d2 = x + r_x at P1 (own d1, received d2) and P2 (received d1, own d2);
 // m_z = m' >>_arith t into the m components of out (its masks are the pairs' r_z).
-__global__ void k_trunc_online(const u64* __restrict__ xs, long long n, const u64* __restrict__ d1,
-                               const u64* __restrict__ d2_at_p1, const u64* __restrict__ d1_at_p2,
-                               const u64* __restrict__ d2, int t, u64* __restrict__ out) {
+__global__ void k_trunc_online(const u64* xs, long long n, const u64* d1,
+                               const u64* d2_at_p1, const u64* d1_at_p2,
+                               const u64* d2, int t, u64* __restrict__ out) {
   grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {

@@ -1603,8 +1603,8 @@ k_gram_tc(long long Dh, const GramJobs jobs, unsigned* __restrict__ err, unsigne
   volatile int* abort = &abort_flag;
 
   const GramJob& J = jobs.j[blockIdx.z];
-  const u64* __restrict__ x = J.a0;
-  const u64* __restrict__ y = J.b0;
+  const u64* x = J.a0;
+  const u64* y = J.b0;
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const int par = blockIdx.y;                      // parity of y in this CTA's tile
@@ -1652,8 +1652,8 @@ k_gram_tc(long long Dh, const GramJobs jobs, unsigned* __restrict__ err, unsigne
     bool ok = true;
     u64 cv[NQ][8], nv[NQ][8];
     u64 cv2[NQ2][8], nv2[NQ2][8];
-    const u64* __restrict__ x1 = GEN ? J.a1 : nullptr;
-    const u64* __restrict__ y1 = GEN ? J.b1 : nullptr;
+    const u64* x1 = GEN ? J.a1 : nullptr;
+    const u64* y1 = GEN ? J.b1 : nullptr;
     auto issue = [&](long long k, u64 (&v)[NQ][8], u64 (&v2)[NQ2][8]) {
       const long long u = k / RPU;
       const int r = (int)(k - u * RPU);

@@ -16,7 +16,7 @@ inline unsigned grid_for(long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
 
 // out = a - b (sub = 1) or a + b (sub = 0) over n words
-__global__ void k_addsub(long long n, const u64* __restrict__ a, const u64* __restrict__ b, int sub,
+__global__ void k_addsub(long long n, const u64* a, const u64* b, int sub,
                          u64* __restrict__ out) {
   grid_dep();
   GRID_STRIDE(i, n) { out[i] = sub ? a[i] - b[i] : a[i] + b[i]; }
@@ -28,8 +28,8 @@ __global__ void k_addsub(long long n, const u64* __restrict__ a, const u64* __re
 // shared products.  The sources are plane-major: a 64 x 32 tile goes through shared memory, so that
 // reads run along e and writes along i.
 __global__ void __launch_bounds__(TPB)
-k_eda_words(const u64* __restrict__ b1, const u64* __restrict__ b2, const u64* __restrict__ mbits,
-            const u64* __restrict__ eprod, long long np, long long e0, long long ldy,
+k_eda_words(const u64* b1, const u64* b2, const u64* mbits,
+            const u64* eprod, long long np, long long e0, long long ldy,
             u64* __restrict__ xm, u64* __restrict__ y) {
   grid_dep();
   __shared__ u64 tile[64][33];
@@ -51,7 +51,7 @@ k_eda_words(const u64* __restrict__ b1, const u64* __restrict__ b2, const u64* _
 // 2x2 max-pool operands: for every window w = (b, ch, i, j) of a (B C, H, W) tensor (one
 // component of n = B C H W words), left = [a ; c], right = [b ; d] with a = [2i][2j],
 // b = [2i][2j+1], c = [2i+1][2j], d = [2i+1][2j+1]; nw windows, stage width np.
-__global__ void k_window_gather(const u64* __restrict__ x, long long BC, long long H, long long W,
+__global__ void k_window_gather(const u64* x, long long BC, long long H, long long W,
                                 long long np, u64* __restrict__ left, u64* __restrict__ right) {
   grid_dep();
   const long long H2 = H / 2, W2 = W / 2, nw = BC * H2 * W2, n = BC * H * W;
@@ -68,7 +68,7 @@ __global__ void k_window_gather(const u64* __restrict__ x, long long BC, long lo
 }
 
 // out[c][k] = idx[k] >= 0 ? xs[c][idx[k]] : 0 for the six components (a local linear map)
-__global__ void k_gather(const u64* __restrict__ xs, long long n_in, const long long* __restrict__ idx,
+__global__ void k_gather(const u64* xs, long long n_in, const long long* idx,
                          long long n_out, u64* __restrict__ out) {
   grid_dep();
   GRID_STRIDE(t, 6 * n_out) {

@@ -35,7 +35,7 @@ __device__ __forceinline__ u64 asr64(u64 v, int t) { return (u64)(((long long)v)
 // the stream (tag, row_keys[e / N]), so that a row draws the same bits whatever batch it is in;
 // words past E are 0.
 __device__ __forceinline__ void bits_block8(const Key& key, u32 tag, u64 obj, u64 blk,
-                                            const u64* __restrict__ row_keys, long long N,
+                                            const u64* row_keys, long long N,
                                             long long E, u64 w[8]) {
   if (!row_keys) {
     prf_block8(key, tag, obj, blk, w);
@@ -80,7 +80,7 @@ __device__ __forceinline__ void store8w(u64* __restrict__ out, long long e0, lon
   }
   __syncwarp();
 }
-__device__ __forceinline__ void load8w(const u64* __restrict__ in, long long e0, long long n,
+__device__ __forceinline__ void load8w(const u64* in, long long e0, long long n,
                                        u64 v[8], u64* st) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -97,7 +97,7 @@ __device__ __forceinline__ void load8w(const u64* __restrict__ in, long long e0,
 // Pi_<.>^{l,0}(x): [r]_1 from eta01 (P0, P1), [r]_2 from eta02 (P0, P2); P0 forms
 // m = x + [r]_1 + [r]_2 (its outgoing message to P1 and P2).
 __global__ void __launch_bounds__(TPB)
-k_share_input(const u64* __restrict__ x, long long n, Key k01, Key k02, u32 tag1, u32 tag2,
+k_share_input(const u64* x, long long n, Key k01, Key k02, u32 tag1, u32 tag2,
               u64 obj, u64* __restrict__ s, u64* __restrict__ m_out) {
   grid_dep();
   __shared__ u64 stage[TPB / 32][32 * 9];
@@ -146,7 +146,7 @@ k_fill_masks(long long n, Key k01, Key k02, u32 tag1, u32 tag2, u64 obj, u64* __
 
 // Pi_Mult preprocessing (P0): [r_z] <- Pi_[.]; Gamma = r_x r_y + r_z; [Gamma]_1 = PRG(eta01);
 // the message to P2 is [Gamma]_2 = Gamma - [Gamma]_1.
-__global__ void k_mult_offline(const u64* __restrict__ xs, const u64* __restrict__ ys,
+__global__ void k_mult_offline(const u64* xs, const u64* ys,
                                long long n, Key k01, Key k02, u32 tr1, u32 tr2, u32 tg1, u64 obj,
                                u64* __restrict__ zs, u64* __restrict__ g2_out) {
   grid_dep();
@@ -176,9 +176,9 @@ __global__ void k_mult_offline(const u64* __restrict__ xs, const u64* __restrict
 
 // Pi_Mult online: P1: [m_z]_1 = -m_x [r_y]_1 - m_y [r_x]_1 + [Gamma]_1;
 //                 P2: [m_z]_2 = m_x m_y - m_x [r_y]_2 - m_y [r_x]_2 + [Gamma]_2 (received).
-__global__ void k_mult_online(const u64* __restrict__ xs, const u64* __restrict__ ys,
+__global__ void k_mult_online(const u64* xs, const u64* ys,
                               long long n, Key k01, u32 tg1, u64 obj,
-                              const u64* __restrict__ g2_in, u64* __restrict__ p1_out,
+                              const u64* g2_in, u64* __restrict__ p1_out,
                               u64* __restrict__ p2_out) {
   grid_dep();
   const long long nb = (n + 7) / 8;
@@ -203,9 +203,9 @@ __global__ void k_mult_online(const u64* __restrict__ xs, const u64* __restrict_
 
 // After the exchange: P1 holds m = own + received, P2 likewise.  With t >= 0 the truncated
 // output's m is m >>_arith t (Fig. trunc, online), written into outs (P1.m, P2.m components).
-__global__ void k_exchange_finish(long long n, const u64* __restrict__ p1_own,
-                                  const u64* __restrict__ p1_in, const u64* __restrict__ p2_own,
-                                  const u64* __restrict__ p2_in, u64* __restrict__ zs, int t,
+__global__ void k_exchange_finish(long long n, const u64* p1_own,
+                                  const u64* p1_in, const u64* p2_own,
+                                  const u64* p2_in, u64* __restrict__ zs, int t,
                                   u64* __restrict__ outs) {
   grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -230,7 +230,7 @@ __global__ void k_exchange_finish(long long n, const u64* __restrict__ p1_own,
 // r_z with asr(b1, t), asr(b2, t), Gamma_q, r_q).
 // pq layout: <p> at pq[0..6E), <q> at pq[6E..12E).
 __global__ void __launch_bounds__(TPB, 1)
-k_trunc_p0(long long E, Key k01, Key k02, u64 obj, const u64* __restrict__ row_keys, long long N,
+k_trunc_p0(long long E, Key k01, Key k02, u64 obj, const u64* row_keys, long long N,
            int t, u32 ttb1, u32 ttb2,
            u32 tp1, u32 tp2, u32 tpg, u32 tq1, u32 tq2, u32 tqg,
            u64* __restrict__ zpre, u64* __restrict__ zout, u64* __restrict__ pq,
@@ -305,13 +305,13 @@ k_trunc_p0(long long E, Key k01, Key k02, u64 obj, const u64* __restrict__ row_k
 // Pi_Trunc^t preprocessing, P1's and P2's part after the messages: m_p = [m_p]_1 + [m_p]_2 at each
 // of P1, P2; [r_x]_1 := m_{r_x} - [r_{r_x}]_1 at P1, [r_x]_2 := -[r_{r_x}]_2 at P2 (same for r_z).
 __global__ void __launch_bounds__(TPB, 2)
-k_trunc_finish(long long E, Key k01, Key k02, u64 obj, const u64* __restrict__ row_keys,
+k_trunc_finish(long long E, Key k01, Key k02, u64 obj, const u64* row_keys,
                long long N, int t, u32 ttb1,
-               u32 ttb2, const u64* __restrict__ p1_in_mp,
-               const u64* __restrict__ p1_in_mq, const u64* __restrict__ p2_in_mp,
-               const u64* __restrict__ p2_in_mq, const u64* __restrict__ p2_gp2,
-               const u64* __restrict__ p2_gq2, const u64* __restrict__ p1_mp1,
-               const u64* __restrict__ p1_mq1, u64* __restrict__ zpre,
+               u32 ttb2, const u64* p1_in_mp,
+               const u64* p1_in_mq, const u64* p2_in_mp,
+               const u64* p2_in_mq, const u64* p2_gp2,
+               const u64* p2_gq2, const u64* p1_mp1,
+               const u64* p1_mq1, u64* __restrict__ zpre,
                u64* __restrict__ zout, u64* __restrict__ pq) {
   grid_dep();
   __shared__ u64 stage[TPB / 32][32 * 9];
@@ -373,7 +373,7 @@ __global__ void k_xor_one(u64* p, u64 mask) {
 
 // words off .. off + n - 1 of a row-keyed truncation-bit stream (see bits_block8) into out
 __global__ void k_prf_words_keyed(long long n, long long off, Key key, u32 tag,
-                                  const u64* __restrict__ row_keys, long long N,
+                                  const u64* row_keys, long long N,
                                   u64* __restrict__ out) {
   grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -408,7 +408,7 @@ __global__ void k_prf_words(long long n, long long off, Key key, u32 tag, u64 ob
 }
 
 // The three messages of Pi_Rec and P1's opening in one pass (the hashes read the copies).
-__global__ void k_rec_messages(const u64* __restrict__ xs, long long n, long long xidx, u64 xmask,
+__global__ void k_rec_messages(const u64* xs, long long n, long long xidx, u64 xmask,
                                int boolean, u64* __restrict__ in_p2_r1, u64* __restrict__ in_p1_r2,
                                u64* __restrict__ in_p0_m, u64* __restrict__ out) {
   grid_dep();

@@ -35,7 +35,7 @@ __device__ __forceinline__ void node_hash(const u32* l, const u32* r, u32 h[8]) 
 __global__ void __launch_bounds__(HB)
 k_hash_leaves(const HashJobs jobs, long long n, long long nleaves) {
   grid_dep();
-  const u64* __restrict__ data = jobs.data[blockIdx.y];
+  const u64* data = jobs.data[blockIdx.y];
   u32* __restrict__ out = gridDim.x == 1 ? jobs.digest[blockIdx.y] : jobs.scratch[blockIdx.y];
   __shared__ u32 dg[HB][8];
   const long long leaf = blockIdx.x * (long long)HB + threadIdx.x;

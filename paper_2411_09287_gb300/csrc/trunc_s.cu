@@ -75,7 +75,7 @@ __device__ __forceinline__ unsigned nibble_bytes(unsigned nib) {
 // Bound by the writes.  (Each thread gathering its 16 words with a stride of 512 bytes and a table in
 // constant memory, indexed per thread: 231 us for L = 2^16, now 33-43 us.)
 __global__ void __launch_bounds__(256)
-k_limb_table(const u64* __restrict__ Tlo, long long L, unsigned char* __restrict__ TL8) {
+k_limb_table(const u64* Tlo, long long L, unsigned char* __restrict__ TL8) {
   grid_dep();
   __shared__ u64 tile[64][65];
   const long long e0 = (long long)blockIdx.x * 64;   // L is a multiple of 64
@@ -116,7 +116,7 @@ k_limb_table(const u64* __restrict__ Tlo, long long L, unsigned char* __restrict
 // a row: 318 us for 2^24 words, now 84 us.)
 constexpr int BT_W = 16;
 __global__ void __launch_bounds__(32 * BT_W)
-k_bit_transpose(const u64* __restrict__ words, long long nw, u64* __restrict__ BT) {
+k_bit_transpose(const u64* words, long long nw, u64* __restrict__ BT) {
   grid_dep();
   __shared__ u64 rows[64][BT_W + 1];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
@@ -151,8 +151,8 @@ k_bit_transpose(const u64* __restrict__ words, long long nw, u64* __restrict__ B
 }
 
 __global__ void __launch_bounds__(S_THREADS, 1)
-k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* __restrict__ B1T,
-             const u64* __restrict__ B2T, long long nw, long long L, u64* __restrict__ S_hi,
+k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* B1T,
+             const u64* B2T, long long nw, long long L, u64* __restrict__ S_hi,
              unsigned* __restrict__ err, unsigned err_flag) {
   grid_dep();
   extern __shared__ unsigned char dsm[];
