@@ -244,17 +244,26 @@ k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* B1T,
     const int r7 = tid & 7;
     const int roff = (tid >> 3) * 1024 + r7 * 128;
     const long long w0 = ehi * (L / 64);
+    // A chunk's words (two of each row, 16-byte aligned: nw and L / 64 are even) are loaded while the
+    // chunk before is written: loaded after the wait for a free stage, they put a load's latency into
+    // every chunk (4096^2 outputs: 44.3 ms, 39.4 with them ahead).
+    ulonglong2 nb2 = make_ulonglong2(0, 0), nb10 = nb2, nb11 = nb2;
+    auto load_words = [&](int c) {
+      const long long w = w0 + 2 * c;
+      nb2 = *reinterpret_cast<const ulonglong2*>(b2row + w);
+      nb10 = *reinterpret_cast<const ulonglong2*>(b1row0 + w);
+      nb11 = *reinterpret_cast<const ulonglong2*>(b1row1 + w);
+    };
+    if (nchunks > 0) load_words(0);
     bool ok = true;
     for (int c = 0; c < nchunks && ok; ++c) {
       const int st = c % S_NST;
+      const u64 m[2][2] = {{nb10.x & nb2.x, nb10.y & nb2.y}, {nb11.x & nb2.x, nb11.y & nb2.y}};
+      if (c + 1 < nchunks) load_words(c + 1);
       if (c >= S_NST) {
         ok = __all_sync(0xffffffffu, mbar_wait(&empty[st], (unsigned)(((c / S_NST) + 1) & 1), abort));
         if (!ok) break;
       }
-      const long long w = w0 + 2 * c;
-      const u64 m2lo = b2row[w], m2hi = b2row[w + 1];
-      const u64 m[2][2] = {{b1row0[w] & m2lo, b1row0[w + 1] & m2hi},
-                           {b1row1[w] & m2lo, b1row1[w + 1] & m2hi}};
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
         unsigned char* row = base + st * S_STAGE + a * S_ATILE + roff;
