@@ -100,6 +100,8 @@ struct Arena {
     return p;
   }
   bool ok() const { return dry || off <= cap; }
+  // room for `bytes` from offset `from` on, under what was taken since
+  void reserve(size_t from, size_t bytes) { off = std::max(off, from + ((bytes + 255) & ~size_t(255))); }
 };
 
 struct Fault {
@@ -1032,6 +1034,7 @@ struct BlkPlan {
   bool full;              // all components and the claim's sums; else x has 2 and 4 only
   PowPlan pp;
   u64 *T, *Rw, *S, *V, *W, *Vm, *G;
+  void* planes;           // the sums' digit planes (tc), under G and dv, which come after the rounds
   Dense dv;
 };
 
@@ -1056,8 +1059,11 @@ BlkPlan plan_blk(Arena& a, long long D, int R, int wlog, bool full, const bool x
   p.V = p.T;   // the claim is taken from T before the rounds fold it
   p.W = a.take<u64>(p.B * 64);
   p.Vm = a.take<u64>(p.B * 4096);
+  const size_t at = a.off;
   p.G = a.take<u64>(p.nwp * p.B * 64);
+  p.planes = p.G;
   p.dv = plan_dense(a, p.nb, xc, yc);
+  if (p.tc) a.reserve(at, blk_sums_tc_bytes(full, p.nw));
   return p;
 }
 
@@ -1087,10 +1093,8 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
   // parties 1 and 2 only: their matrices sit where those of a full batch's first two would
   const int np = p.full ? 3 : 2, p0 = p.full ? 0 : 1;
   if (p.tc) {
-    // the digit planes (14848 bytes a block of a full batch, 2304 of the edaBits') lie where the
-    // products R_b V_j and the vectors come after the rounds (17408 and 8192)
     g_launches += 3;
-    if (blk_sums_tc(st, in, p.full, p.nw, p.Rw, p.S, p.G, ctx->status, ST_TIMEOUT,
+    if (blk_sums_tc(st, in, p.full, p.nw, p.Rw, p.S, p.planes, ctx->status, ST_TIMEOUT,
                     ctx->tune.gemm_split_min))
       return fail(ctx, MPC_ERR_CUDA, "block sums: tensor maps");
   } else if (p.full || p.kap > 0) {
