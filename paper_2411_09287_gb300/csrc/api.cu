@@ -21,60 +21,6 @@
 
 using namespace mpc3;
 
-// ---- kernel launch accounting: every launcher called from this file is counted ----------------
-namespace {
-unsigned long long g_launches = 0;
-template <class F, class... A>
-inline void counted(int k, F f, A... a) {
-  g_launches += (unsigned long long)k;
-  f(a...);
-}
-}  // namespace
-#define gemm_u64(...) counted(1, mpc3::gemm_u64, __VA_ARGS__)
-#define launch_share_input(...) counted(1, mpc3::launch_share_input, __VA_ARGS__)
-#define launch_fill_masks(...) counted(1, mpc3::launch_fill_masks, __VA_ARGS__)
-#define launch_mult_offline(...) counted(1, mpc3::launch_mult_offline, __VA_ARGS__)
-#define launch_mult_online(...) counted(1, mpc3::launch_mult_online, __VA_ARGS__)
-#define launch_exchange_finish(...) counted(1, mpc3::launch_exchange_finish, __VA_ARGS__)
-#define launch_trunc_p0(...) counted(1, mpc3::launch_trunc_p0, __VA_ARGS__)
-#define launch_trunc_finish(...) counted(1, mpc3::launch_trunc_finish, __VA_ARGS__)
-#define launch_xor_one(...) counted(1, mpc3::launch_xor_one, __VA_ARGS__)
-#define launch_rec_messages(...) counted(1, mpc3::launch_rec_messages, __VA_ARGS__)
-#define launch_hash_jobs(...) counted(2, mpc3::launch_hash_jobs, __VA_ARGS__)
-#define launch_hash_u64(...) counted(2, mpc3::launch_hash_u64, __VA_ARGS__)
-#define launch_digest_check(...) counted(1, mpc3::launch_digest_check, __VA_ARGS__)
-#define launch_gr_powers(...) counted(1, mpc3::launch_gr_powers, __VA_ARGS__)
-#define launch_gr_mul1(...) counted(1, mpc3::launch_gr_mul1, __VA_ARGS__)
-#define launch_gr_axpy(...) counted(1, mpc3::launch_gr_axpy, __VA_ARGS__)
-#define launch_gr_inverses(...) counted(1, mpc3::launch_gr_inverses, __VA_ARGS__)
-#define launch_gr_fold_reduce(...) counted(1, mpc3::launch_gr_fold_reduce, __VA_ARGS__)
-#define launch_neg_copy(...) counted(1, mpc3::launch_neg_copy, __VA_ARGS__)
-#define launch_round_tail(...) counted(1, mpc3::launch_round_tail, __VA_ARGS__)
-#define launch_zero_rows(...) counted(1, mpc3::launch_zero_rows, __VA_ARGS__)
-#define launch_small_round(...) counted(1, mpc3::launch_small_round, __VA_ARGS__)
-#define launch_inner_verify(...) counted(1, mpc3::launch_inner_verify, __VA_ARGS__)
-#define launch_reveal(...) counted(1, mpc3::launch_reveal, __VA_ARGS__)
-#define launch_rec_hash(...) counted(1, mpc3::launch_rec_hash, __VA_ARGS__)
-#define launch_weighted_sums(...) counted(1, mpc3::launch_weighted_sums, __VA_ARGS__)
-#define launch_blk_sums(...) counted(1, mpc3::launch_blk_sums, __VA_ARGS__)
-#define launch_words_sums(...) counted(1, mpc3::launch_words_sums, __VA_ARGS__)
-#define launch_blk_claim(...) counted(1, mpc3::launch_blk_claim, __VA_ARGS__)
-#define launch_blk_combine(...) counted(1, mpc3::launch_blk_combine, __VA_ARGS__)
-#define launch_ones(...) counted(1, mpc3::launch_ones, __VA_ARGS__)
-#define launch_trunc_u(...) counted(1, mpc3::launch_trunc_u, __VA_ARGS__)
-#define launch_trunc_materialize(...) counted(1, mpc3::launch_trunc_materialize, __VA_ARGS__)
-#define launch_gr_mul_rows(...) counted(1, mpc3::launch_gr_mul_rows, __VA_ARGS__)
-#define launch_gather_rows_affine(...) counted(1, mpc3::launch_gather_rows_affine, __VA_ARGS__)
-#define launch_sum_blocks(...) counted(1, mpc3::launch_sum_blocks, __VA_ARGS__)
-#define launch_block_rowsum(...) counted(1, mpc3::launch_block_rowsum, __VA_ARGS__)
-#define launch_gr_mulmat_batch(...) counted(1, mpc3::launch_gr_mulmat_batch, __VA_ARGS__)
-#define launch_word_transpose(...) counted(1, mpc3::launch_word_transpose, __VA_ARGS__)
-#define launch_scalar_gr_sum(...) counted(1, mpc3::launch_scalar_gr_sum, __VA_ARGS__)
-#define launch_prf_words(...) counted(1, mpc3::launch_prf_words, __VA_ARGS__)
-#define launch_prf_words_keyed(...) counted(1, mpc3::launch_prf_words_keyed, __VA_ARGS__)
-#define launch_trunc_limb_table(...) counted(1, mpc3::launch_trunc_limb_table, __VA_ARGS__)
-#define launch_trunc_bit_transpose(...) counted(1, mpc3::launch_trunc_bit_transpose, __VA_ARGS__)
-
 namespace {
 
 constexpr u32 ST_ABORT = 1u;    // a Pi_Rec check failed
@@ -113,6 +59,7 @@ struct Fault {
 __global__ void k_derive_keys(Key master, u32* out) {
   // eta_{0,1}, eta_{0,2}, eta_{1,2}: first 32 bytes of ChaCha20(master, counter 0,
   // nonce (0x0059454B, pair, 0)), pair = 1, 2, 3
+  grid_dep();
   const int pair = threadIdx.x + 1;
   if (pair > 3) return;
   u32 o[16];
@@ -381,7 +328,6 @@ int gr_matmul(mpc_ctx* ctx, long long R, const u64* p0, const u64* p1, u64 s1, l
               const u64* Mmat, const u64* add0, long long ld_add0, u64* out, long long ldc) {
   if (R <= 0) return MPC_OK;
   if (ctx->gemm_path == MPC_GEMM_LIMB_TC) {
-    g_launches += 1;
     Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)R * 4096);
     GrMMArgs g = grargs(ctx);
     g.R = R;
@@ -395,7 +341,7 @@ int gr_matmul(mpc_ctx* ctx, long long R, const u64* p0, const u64* p1, u64 s1, l
     g.out = out;
     g.om = GrRowMap{0, ldc, 0};
     if (gr_matmul_tc_ex(ctx->st, g, ctx->status, ST_TIMEOUT) == 0) return MPC_OK;
-    g_launches -= 1;   // misaligned view: fall through to the CUDA-core GEMM
+    // misaligned view: fall through to the CUDA-core GEMM
   }
   GemmTerm T;
   T.A = p1 ? op(p0, lda, 0, p1, s1) : op(p0, lda);
@@ -412,7 +358,6 @@ int gr_matmul(mpc_ctx* ctx, long long R, const u64* p0, const u64* p1, u64 s1, l
 int dense_gemm(mpc_ctx* ctx, long long M, long long N, long long K, const GemmTerm& T,
                const Epi& e, void* scratch, const GemmGroups& groups = GemmGroups{}) {
   if (scratch && !e.atomic) {
-    g_launches += 4;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->prof) {
       e0 = prof_event(ctx);
@@ -465,7 +410,6 @@ int party_sums(mpc_ctx* ctx, const View& u, const View& v, long long count, u64*
   gb.add(Pmat + 8192, u.c[4], nullptr, 1, u.ld, v.c[4], v.c[5], M1, v.ld, 1);
   gb.add(Pmat + 8192, v.c[4], nullptr, 1, v.ld, u.c[5], nullptr, 1, u.ld, M1);
   if (count > 0 && gb.n > 0) {
-    g_launches += 1;
     gemm_u64_gram_batch(ctx->st, count, gb.n, gb.T, gb.e, nsplit_for(count));
   }
   launch_gr_fold_reduce(ctx->st, Pmat, 3, S);
@@ -647,7 +591,6 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
     bool done = false;
     if (ctx->gemm_path == MPC_GEMM_LIMB_TC) {
       // tensor cores: G00, G11 and the cross sum G01 + G10 directly
-      g_launches += 1;
       {
         Phase kp(ctx, MPC_PROF_K_GRAM, 4.0 * Dh * 4096);
         done = gram3_tc(st, Dh, x.c[0], y.c[1], U, ctx->status, ST_TIMEOUT,
@@ -656,8 +599,6 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       if (done) {
         sums = U;
         ld = 128;
-      } else {
-        g_launches -= 1;
       }
     }
     if (!done) {
@@ -672,7 +613,6 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       CK(cudaMemcpyAsync(S11, s.aux + 64, 512, cudaMemcpyDeviceToDevice, st));
       launch_addsub(st, 64, s.aux + 128, s.aux, 1, s.aux + 192);
       launch_addsub(st, 64, s.aux + 192, s.aux + 64, 1, S01);
-      g_launches += 2;
     }
   } else {
     bool done = false;
@@ -697,10 +637,6 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       add(1, y.c[2], nullptr, 0, x.c[3], nullptr, 0, M1);
       add(2, x.c[4], nullptr, 0, y.c[4], y.c[5], M1, 1);
       add(2, y.c[4], nullptr, 0, x.c[5], nullptr, 0, M1);
-      int nl = 0;
-      for (int q = 0; q < jobs.n; ++q) nl |= (jobs.j[q].a1 || jobs.j[q].b1) ? 2 : 1;
-      nl = (nl & 1) + (nl >> 1);   // one launch for the single-source jobs, one for the others
-      g_launches += nl;
       {
         Phase kp(ctx, MPC_PROF_K_GRAM, 4.0 * Dh * 4096 * jobs.n);
         done = gram_jobs_tc(st, Dh, jobs, ctx->status, ST_TIMEOUT, ctx->tune.gram_split) == 0;
@@ -708,8 +644,6 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
       if (done) {
         sums = U;   // S00 | S01 + S10 | 0 | S11
         ld = 128;
-      } else {
-        g_launches -= nl;
       }
     }
     if (!done) {
@@ -745,10 +679,8 @@ int reduce_round_dense(mpc_ctx* ctx, u64 vid, u32 batch, int k, const Vec& x, co
     g.add0_in = 1;
     g.out = outs[0];
     g.om = GrRowMap{Rp, 64, sout};
-    g_launches += 1;
     Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)n * Dh * 4096);
     if (gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT) == 0) return true;
-    g_launches -= 1;
     return false;
   };
   const u64* ins[12];
@@ -1011,10 +943,8 @@ int power_table(mpc_ctx* ctx, const u64* r, const PowPlan& p, u64* table, u64* a
   g.out = table + p.L * 64;
   g.om = GrRowMap{0, 64, 0};
   g.out_lim = (p.n - p.L) * 64;
-  g_launches += 1;
   Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)(p.n - p.L) * 4096);
   if (gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT) == 0) return MPC_OK;
-  g_launches -= 1;
   launch_gr_powers(st, r, p.n, table);
   return MPC_OK;
 }
@@ -1093,7 +1023,6 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
   // parties 1 and 2 only: their matrices sit where those of a full batch's first two would
   const int np = p.full ? 3 : 2, p0 = p.full ? 0 : 1;
   if (p.tc) {
-    g_launches += 3;
     if (blk_sums_tc(st, in, p.full, p.nw, p.Rw, p.S, p.planes, ctx->status, ST_TIMEOUT,
                     ctx->tune.gemm_split_min))
       return fail(ctx, MPC_ERR_CUDA, "block sums: tensor maps");
@@ -1125,10 +1054,8 @@ int run_blk(mpc_ctx* ctx, u64 vid, u32 batch, BlkPlan& p, const Vec& xw, const V
     g.mrows = p.nwp;
     g.out = p.G;
     g.om = GrRowMap{p.nwp, 64ll * B, 64};
-    g_launches += 1;
     Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)g.R * 4096);
     done = gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT) == 0;
-    if (!done) g_launches -= 1;
   }
   for (int j = 0; j < B && !done; ++j)
     if ((rc = gr_matmul(ctx, p.nw, p.Rw, nullptr, 1, 64, p.Vm + j * 4096, nullptr, 0, p.G + j * 64,
@@ -1459,10 +1386,8 @@ int bit_tables(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* rho) {
       g.mrows = p.L;
       g.out = p.Rtab + p.L * 64;
       g.om = GrRowMap{0, 64, 0};
-      g_launches += 1;
       Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)g.R * 4096);
       done = gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT) == 0;
-      if (!done) g_launches -= 1;
     }
     for (long long h = 1; h < p.nhi && !done; ++h)
       if ((rc = gr_matmul(ctx, p.L, p.Rtab, nullptr, 1, 64, p.Mhi + (h - 1) * 4096, nullptr, 0,
@@ -1487,7 +1412,6 @@ int bit_batch(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* z0, u64 ver
     launch_trunc_bit_transpose(st, p.b2, p.Epad, p.B2T);
     {
       Phase kphase(ctx, MPC_PROF_K_TRUNC_S, 4096.0 * 64 * E);
-      g_launches += 1;
       if (launch_trunc_s_tc(st, p.B1T, p.B2T, p.Epad, p.TL8, p.L, p.nhi, p.S_hi, ctx->status,
                             ST_TIMEOUT))
         return fail(ctx, MPC_ERR_CUDA, "verify_matmul: tensor map of the limb table");
@@ -1506,10 +1430,8 @@ int bit_batch(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* z0, u64 ver
         g.mrows = 4096;
         g.out = blk1;
         g.om = GrRowMap{0, 64, 0};
-        g_launches += 1;
         Phase kp(ctx, MPC_PROF_K_GR_MATMUL, (double)g.R * 4096);
         done = gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT) == 0;
-        if (!done) g_launches -= 1;
       }
       for (long long h = 1; h < p.nhi && !done; ++h) {
         // block h into S (used as scratch), then back: the CUDA-core product is not in place
@@ -1549,7 +1471,6 @@ int bit_batch(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* z0, u64 ver
     const u64* mats[4] = {nV, nV, nW, nW};
     u64* outs[4] = {tx.c[0], tx.c[3], ty.c[1], ty.c[5]};
     auto grmm = [&](const GrMMArgs& g, double work) {
-      g_launches += 1;
       Phase kp(ctx, MPC_PROF_K_GR_MATMUL, work);
       return gr_matmul_tc_ex(st, g, ctx->status, ST_TIMEOUT);
     };
@@ -1780,7 +1701,7 @@ int mpc_create(const mpc_config* cfg, mpc_ctx** out) {
   u32* keys_dev = reinterpret_cast<u32*>(reinterpret_cast<char*>(ctx->cst) + CST_WORDS * 8 + 256);
   Key master;
   std::memcpy(master.k, cfg->seed, 32);
-  k_derive_keys<<<1, 32, 0, ctx->st>>>(master, keys_dev);
+  launch_dep(k_derive_keys, 1, 32, 0, ctx->st, master, keys_dev);
   launch_gr_inverses(ctx->st, ctx->cst + CST_INV);
   e = cudaMemsetAsync(ctx->status, 0, sizeof(u32), ctx->st);
   if (e != cudaSuccess) return bail("cudaMemset", e);
@@ -2133,7 +2054,6 @@ int mpc_matmul_keyed(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const u
       gemm_u64(ctx->st, M, N, K, nterms, T, e, 1);
       return MPC_OK;
     }
-    g_launches += 4;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->prof) {
       e0 = prof_event(ctx);
@@ -2372,7 +2292,6 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
     GramBatch gb;
     for (int c = 0; c < 6; ++c)
       gb.add(p.Pz + c * 4096, p.P, nullptr, 1, 64, p.T + c * M * 64, nullptr, 1, 64, 1);
-    g_launches += 1;
     gemm_u64_gram_batch(st, M, gb.n, gb.T, gb.e, nsplit_for(M));
     launch_gr_fold_reduce(st, p.Pz, 6, s.zinit);
   }
@@ -2472,7 +2391,7 @@ int mpc_profile_read(mpc_ctx* ctx, double* ms, uint64_t* count, double* work) {
   return MPC_OK;
 }
 
-uint64_t mpc_launch_count(void) { return g_launches; }
+uint64_t mpc_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 
 // ---- layer-level calls -----------------------------------------------------------------------
@@ -2497,7 +2416,6 @@ int mpc_share_fixed(mpc_ctx* ctx, uint64_t call_id, int owner, const double* x, 
   {
     Phase phase(ctx, MPC_PROF_SHARE);
     launch_encode_fixed(ctx->st, xd, n, frac_bits, enc);
-    g_launches += 1;
   }
   rc = mpc_share_input_from(ctx, call_id, owner, enc, 0, n, xs, (char*)workspace + ar.off,
                             workspace_bytes > ar.off ? workspace_bytes - ar.off : 0);
@@ -2525,7 +2443,6 @@ int mpc_reconstruct_fixed(mpc_ctx* ctx, const uint64_t* xs, int64_t n, int frac_
   {
     Phase phase(ctx, MPC_PROF_REC);
     launch_decode_fixed(ctx->st, v, n, frac_bits, out_on_host ? stage : out);
-    g_launches += 1;
   }
   if (out_on_host) {
     CK(cudaMemcpyAsync(out, stage, (size_t)n * 8, cudaMemcpyDeviceToHost, ctx->st));
@@ -2552,7 +2469,6 @@ int mpc_conv2d(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const uint64_
   g.Ho = (g.H + 2 * g.pad - g.kh) / g.stride + 1;
   g.Wo = (g.W + 2 * g.pad - g.kw) / g.stride + 1;
   launch_im2col(ctx->st, xs, g, cols);
-  g_launches += 1;
   if ((rc = cuda_check(ctx, "conv2d: im2col"))) return rc;
   return mpc_matmul_keyed(ctx, call_id, cols, ws_, g.B * g.Ho * g.Wo, C_out, g.C * g.kh * g.kw,
                           trunc_bits, row_keys, zpre, zout, pq, workspace, workspace_bytes);
@@ -2587,7 +2503,6 @@ int mpc_trunc(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, int64_t n, int
   {  // online: the wire's mask switched to the pairs' r_x (checked by P0's hashes), then m >> t
     Phase phase(ctx, MPC_PROF_EXCHANGE);
     launch_trunc_remask(st, xs, p.rx, n, p.d1, p.d2, p.d1p0, p.d2p0);
-    g_launches += 1;
     const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_TRUNC;
     if ((rc = deliver(ctx, ph, pr, p.d1, p.d1_at_p2, n, MPC_SITE_TRUNC_D1))) return rc;   // P1->P2
     if ((rc = deliver(ctx, ph, pr, p.d2, p.d2_at_p1, n, -1))) return rc;                 // P2->P1
@@ -2604,7 +2519,6 @@ int mpc_trunc(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, int64_t n, int
     launch_digest_check(st, p.dg, p.dg + 16, p.dg + 8, p.dg + 24, p.dg, p.dg + 16, ctx->status,
                         ST_ABORT);
     launch_trunc_online(st, xs, n, p.d1, p.d2_at_p1, p.d1_at_p2, p.d2, t, out);
-    g_launches += 1;
   }
   if ((rc = cuda_check(ctx, "trunc"))) return rc;
   ctx->pending.insert((call_id << 1) | 1);
@@ -2642,7 +2556,6 @@ int mpc_test_wait_expires(mpc_ctx* ctx, int64_t cycles) {
   if (rc) return rc;
   if (cycles < 1 || cycles > 100000000) return fail(ctx, MPC_ERR_ARG, "test_wait_expires: cycles");
   launch_wait_expires(ctx->st, cycles, ctx->status, ST_TIMEOUT);
-  g_launches += 1;
   if ((rc = cuda_check(ctx, "test_wait_expires"))) return rc;
   u32 stv = 0;
   return read_status(ctx, &stv);   // MPC_ERR_TIMEOUT, and the context is aborted
@@ -2745,19 +2658,19 @@ int compare_select(mpc_ctx* ctx, u64 call_id, int stage, CSPlan& p) {
   k.fault[2] = take_fault(ctx, MPC_SITE_MZ2, N);
   k.fault[3] = take_bit_fault(ctx, MPC_SITE_AND_GAMMA2, 64 * W);
   // edaBits (Fig. edabits) and Delta = d - r, d = a - b
-  g_launches += launch_cs_open_delta(st, k);
+  launch_cs_open_delta(st, k);
   count_mult(ctx, N);                                                    // the bit products
   count_msgs(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_INNER, 3, (u64)np * 8);   // the inner products
   rec_core(ctx, k.dd, np, p.reca, p.delta, false);
   // msb(d) by the carry circuit over the bits of Delta + r; daBits; e = [d >= 0] XOR bit
   launch_trunc_bit_transpose(st, p.delta, np, p.dpl);
-  g_launches += launch_cs_open_bit(st, k);
+  launch_cs_open_bit(st, k);
   for (int l = 1; l <= NL_LEVELS; ++l) count_mult(ctx, level_planes(l) * W);
   count_mult(ctx, np);   // the daBits' two products
   count_mult(ctx, np);
   rec_core(ctx, k.e, W, p.recb, p.dbits, true);
   // out = b + (a - b) [a >= b]
-  g_launches += launch_cs_select(st, k);
+  launch_cs_select(st, k);
   count_mult(ctx, np);
   return cuda_check(ctx, "compare_select");
 }
@@ -2811,7 +2724,7 @@ int gf_verify(mpc_ctx* ctx, u64 vid, GfPlan& g, u64* trace) {
   v.status = ctx->status;
   v.flag_verify = ST_VERIFY;
   v.flag_abort = ST_ABORT;
-  g_launches += launch_gf_verify(ctx->st, v);
+  launch_gf_verify(ctx->st, v);
   // Pi_Rec of r, the zetas and Delta (3 words and 3 hashes each); two secure inner products a round,
   // x alpha and the last inner product
   const int ph = MPC_PHASE_VERIFY, pr = MPC_PROTO_VERIFY;
@@ -2930,7 +2843,6 @@ int verify_nl(mpc_ctx* ctx, u64 vid, NLPlan& p, u64* trace) {
       const CompareSelect& c = p.cs[q].k;
       launch_eda_words(st, c.eda, c.eprod, c.np, e0, p.D1, p.Xe, p.Ye);
       launch_scalar_gr_sum(st, c.np, c.ez, c.np, 6, b.Rw + e0 * 64, s.zinit);
-      g_launches += 1;
       e0 += c.np;
     }
     Vec x{}, y;
@@ -3058,7 +2970,6 @@ int mpc_maxpool2(mpc_ctx* ctx, uint64_t call_id, uint64_t verify_id, const uint6
   // stage 0 operands: left = [a ; c], right = [b ; d] of every window; stage 1: the two halves of its
   // result
   launch_window_gather(st, xs, B * C, H, W, np[0], p.a, p.b);
-  g_launches += 1;
   CompareSelect &k0 = p.cs[0].k, &k1 = p.cs[1].k;
   k0.a = {p.a, np[0], 2 * nw};
   k0.b = {p.b, np[0], 2 * nw};
@@ -3103,6 +3014,5 @@ int mpc_gather(mpc_ctx* ctx, const uint64_t* xs, int64_t n_in, const int64_t* id
   if (n_in <= 0 || n_out <= 0) return fail(ctx, MPC_ERR_SHAPE, "gather: bad size");
   if (!xs || !idx || !out) return fail(ctx, MPC_ERR_ARG, "gather: bad argument");
   launch_gather(ctx->st, xs, n_in, reinterpret_cast<const long long*>(idx), n_out, out);
-  g_launches += 1;
   return cuda_check(ctx, "gather");
 }

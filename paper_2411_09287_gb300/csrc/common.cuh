@@ -6,6 +6,7 @@
 //   * SHA-256 (FIPS 180-4), the hash H of Pi_Rec (Sec. 2, verifiable reconstruction).
 // All ring arithmetic is on uint64_t, i.e. exactly mod 2^64.
 #pragma once
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -35,6 +36,8 @@ __device__ __forceinline__ void grid_dep() {
   asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
+inline std::atomic<unsigned long long> g_launches{0};   // kernels launched (mpc_launch_count)
+
 template <class... P, class... A>
 inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        A&&... args) {
@@ -48,7 +51,8 @@ inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   cfg.stream = st;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  if (cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess)
+    g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
 constexpr int GR_D = 64;                 // extension degree d (Sec. 5: d = 64)

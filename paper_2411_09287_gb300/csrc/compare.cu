@@ -317,22 +317,19 @@ inline unsigned grid_for(long long threads) {
 
 }  // namespace
 
-int launch_cs_open_delta(cudaStream_t st, const CompareSelect& a) {
+void launch_cs_open_delta(cudaStream_t st, const CompareSelect& a) {
   launch_dep(k_cs_bits, dim3(grid_for((a.np + 7) / 8), 6), TPB, 0, st, a);
   launch_dep(k_cs_products, grid_for(8 * a.np), TPB, 0, st, a);
   launch_dep(k_cs_inner, (unsigned)(a.np / 32), TPB, 0, st, a);
-  return 3;
 }
 
-int launch_cs_open_bit(cudaStream_t st, const CompareSelect& a) {
+void launch_cs_open_bit(cudaStream_t st, const CompareSelect& a) {
   launch_dep(k_cs_dabits, grid_for(a.np / 8), TPB, 0, st, a);
   launch_dep(k_cs_msb, (unsigned)((a.np / 64 + 3) / 4), TPB, 0, st, a);
-  return 2;
 }
 
-int launch_cs_select(cudaStream_t st, const CompareSelect& a) {
+void launch_cs_select(cudaStream_t st, const CompareSelect& a) {
   launch_dep(k_cs_select, grid_for(a.np / 8), TPB, 0, st, a);
-  return 1;
 }
 
 }  // namespace mpc3

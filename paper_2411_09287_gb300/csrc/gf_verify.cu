@@ -455,12 +455,11 @@ k_gf_last(const GfVerify a, const Coef cf, int k, long long D0, const u64* x, co
 
 }  // namespace
 
-int launch_gf_verify(cudaStream_t st, const GfVerify& a) {
+void launch_gf_verify(cudaStream_t st, const GfVerify& a) {
   static const Coef cf = [] {
     return Coef{gf_inv(gf_mul(GF_X, GF_X ^ 1ull))};
   }();
   const long long nb = 8 * a.nw;
-  int n = 3;
   cudaMemsetAsync(a.w, 0, sizeof(GfWork), st);
   launch_dep(k_gf_setup, (unsigned)((nb + 2047) / 2048), 256, 0, st, a, nb);
   long long g = (a.nw + 15) / 16;
@@ -474,14 +473,12 @@ int launch_gf_verify(cudaStream_t st, const GfVerify& a) {
     const long long Dh = (D + 1) / 2, ldo = Dh;
     g = ((Dh + 1) / 2 + 127) / 128;
     launch_dep(k_gf_round, (unsigned)(g < 2432 ? g : 2432), 128, 0, st, a, cf, k + 1, D, x, y, ld, xo, yo, ldo);
-    ++n;
     u64* t = x; x = xo; xo = t;
     t = y; y = yo; yo = t;
     D = Dh;
     ld = ldo;
   }
   launch_dep(k_gf_last, 1, 512, 0, st, a, cf, k, D, x, y, ld);
-  return n + 1;
 }
 
 }  // namespace mpc3

@@ -168,6 +168,7 @@ __device__ u64 gf2_64_mul(u64 a, u64 b) {   // GF(2)[x]/(x^64 + x^4 + x^3 + x + 
 // out[0..63] = x^-1, out[64..127] = (1 - x)^-1, out[128..191] = (x (x - 1))^-1.
 // GF(2^64) inverse a^(2^64 - 2) of the residue, then Newton steps y <- y (2 - a y).
 __global__ void k_gr_inverses(u64* out) {
+  grid_dep();
   __shared__ u64 a[64], y[64], t1[64], scr[128];
   __shared__ u64 ybits;
   const int t = threadIdx.x;
@@ -482,7 +483,7 @@ void launch_sum_blocks(cudaStream_t st, long long m, long long n, long long ld, 
   launch_dep(k_sum_blocks, (unsigned)((m + 255) / 256), 256, 0, st, m, n, ld, in, out);
 }
 
-void launch_gr_inverses(cudaStream_t st, u64* out) { k_gr_inverses<<<1, 64, 0, st>>>(out); }
+void launch_gr_inverses(cudaStream_t st, u64* out) { launch_dep(k_gr_inverses, 1, 64, 0, st, out); }
 
 void launch_gr_fold_reduce(cudaStream_t st, const u64* P, int n, u64* out) {
   if (n <= 0) return;

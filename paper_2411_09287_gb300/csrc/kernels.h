@@ -376,10 +376,10 @@ struct CompareSelect {
   u64* e;                // 6 np / 64: Boolean sharing to open
   const u64* dbits;      // e opened
 };
-// The three parts around the openings of dd and e; each returns its number of launches.
-int launch_cs_open_delta(cudaStream_t st, const CompareSelect& a);
-int launch_cs_open_bit(cudaStream_t st, const CompareSelect& a);
-int launch_cs_select(cudaStream_t st, const CompareSelect& a);
+// The three parts around the openings of dd and e.
+void launch_cs_open_delta(cudaStream_t st, const CompareSelect& a);
+void launch_cs_open_bit(cudaStream_t st, const CompareSelect& a);
+void launch_cs_select(cudaStream_t st, const CompareSelect& a);
 
 // ---- non-linear layers (nonlinear.cu) -----------------------------------------------------------
 void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int sub, u64* out);
@@ -413,8 +413,7 @@ struct GfVerify {
   u32* status;
   u32 flag_verify, flag_abort;   // Delta != 0; a hash mismatch
 };
-// Returns the number of launches.
-int launch_gf_verify(cudaStream_t st, const GfVerify& a);
+void launch_gf_verify(cudaStream_t st, const GfVerify& a);
 // ---- layer-level calls (layer_kernels.cu) ----------------------------------------------------
 // Geometry of a convolution: NCHW input (B, C, H, W), kh x kw kernel, stride, zero padding; the
 // output is Ho x Wo per image.

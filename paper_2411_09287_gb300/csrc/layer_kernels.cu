@@ -178,6 +178,7 @@ namespace {
 // on an mbarrier that nothing arrives at; on expiry it records err_flag in the status word and
 // returns, exactly as a tensor-core kernel's waiting role does.
 __global__ void k_wait_expires(long long cycles, unsigned* __restrict__ err, unsigned err_flag) {
+  grid_dep();
   __shared__ __align__(8) u64 bar;
   __shared__ int abort_flag;
   if (threadIdx.x != 0) return;
@@ -190,7 +191,7 @@ __global__ void k_wait_expires(long long cycles, unsigned* __restrict__ err, uns
 }  // namespace
 
 void launch_wait_expires(cudaStream_t st, long long cycles, unsigned* err, unsigned err_flag) {
-  k_wait_expires<<<1, 32, 0, st>>>(cycles, err, err_flag);
+  launch_dep(k_wait_expires, 1, 32, 0, st, cycles, err, err_flag);
 }
 
 }  // namespace mpc3
