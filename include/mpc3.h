@@ -302,7 +302,7 @@ int64_t mpc_trace_words(const mpc_ctx* ctx, int op, int64_t a, int64_t b, int64_
 /* Pi_Rec (Sec. 2): P0 sends [r]_1 to P2 and [r]_2 to P1, P1 sends m to P0; P1 sends H([r]_1) to
  * P2, P2 sends H(m) to P0 and H([r]_2) to P1 (H = SHA-256 Merkle root, 1 KiB leaves).  On any
  * mismatch the call returns MPC_ERR_ABORT; otherwise out = m - [r]_1 - [r]_2 (n words, host if
- * out_on_host, else device).  Refused with MPC_ERR_PENDING while products are unverified. */
+ * out_on_host, else device; a device out may be a component of xs).  Refused with MPC_ERR_PENDING while products are unverified. */
 int mpc_reconstruct(mpc_ctx* ctx, const uint64_t* xs, int64_t n, uint64_t* out, int out_on_host,
                     void* workspace, size_t workspace_bytes);
 

@@ -853,10 +853,8 @@ MatmulPlan plan_matmul(Arena& a, long long M, long long N, long long K, bool tru
   return p;
 }
 
-struct RecPlan {
-  u64 *in_p2_r1, *in_p1_r2, *in_p0_m, *out_dev;
-  u32* hs[6];
-  u32* dg;   // 6 x 8
+struct RecPlan : RecBufs {
+  u64* out_dev;
 };
 
 RecPlan plan_rec(Arena& a, long long n, bool need_out) {
@@ -883,23 +881,11 @@ long long take_rec_fault(mpc_ctx* ctx, long long n, u64* mask) {
 // [r]_2 to P1 (fault site REC_MSG, arithmetic sharings), P1 sends m to P0; P1 sends H([r]_1) to P2,
 // P2 H(m) to P0 and H([r]_2) to P1, and every receiver hashes what it received.  out = P1's opening.
 void rec_core(mpc_ctx* ctx, const u64* xs, long long n, const RecPlan& p, u64* out, bool boolean) {
-  cudaStream_t st = ctx->st;
-  const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_REC;
   u64 xmask = 0;
   const long long xidx = boolean ? -1 : take_rec_fault(ctx, n, &xmask);
-  count_msgs(ctx, ph, pr, 3, (u64)n * 8);
-  launch_rec_messages(st, xs, n, xidx, xmask, boolean, p.in_p2_r1, p.in_p1_r2, p.in_p0_m, out);
-  HashJobs j;
-  const u64* data[6] = {xs + 3 * n, xs + 4 * n, xs + 5 * n, p.in_p2_r1, p.in_p0_m, p.in_p1_r2};
-  for (int q = 0; q < 6; ++q) {
-    j.data[q] = data[q];
-    j.scratch[q] = p.hs[q];
-    j.digest[q] = p.dg + 8 * q;
-  }
-  launch_hash_jobs(st, j, 6, n);
-  count_msgs(ctx, ph, pr, 3, 32);
-  u32* d = p.dg;
-  launch_digest_check(st, d, d + 24, d + 8, d + 32, d + 16, d + 40, ctx->status, ST_ABORT);
+  launch_rec(ctx->st, xs, n, xidx, xmask, boolean, p, out, ctx->status, ST_ABORT);
+  count_msgs(ctx, MPC_PHASE_ONLINE, MPC_PROTO_REC, 3, (u64)n * 8);
+  count_msgs(ctx, MPC_PHASE_ONLINE, MPC_PROTO_REC, 3, 32);
 }
 
 // A table of powers r^i, i < n (rows of 64 words): rows below L by repeated multiplication, row

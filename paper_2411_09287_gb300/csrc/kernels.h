@@ -227,11 +227,14 @@ void launch_trunc_finish(cudaStream_t st, long long E, Key k01, Key k02, u64 obj
                          const u64* p1_mp1, const u64* p1_mq1, u64* zpre, u64* zout, u64* pq,
                          const u64* row_keys, long long N);
 void launch_xor_one(cudaStream_t st, u64* p, u64 mask);
-// The messages of Pi_Rec of a sharing xs and P1's opening: in_p2_r1 = P0.[r]_1, in_p1_r2 = P0.[r]_2
-// (word xidx XORed with xmask when xidx >= 0), in_p0_m = P1.m, out = P1.m - P1.[r]_1 - in_p1_r2 (XOR
-// for a Boolean sharing).
+// The messages of Pi_Rec of a sharing xs and (out not null) P1's opening: in_p2_r1 = P0.[r]_1, in_p1_r2
+// = P0.[r]_2 (word xidx XORed with xmask when xidx >= 0), in_p0_m = P1.m, out = P1.m - P1.[r]_1 -
+// in_p1_r2 (XOR for a Boolean sharing).
 void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask,
                          bool boolean, u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out);
+// The opening alone, from the received in_p1_r2.
+void launch_rec_open(cudaStream_t st, const u64* xs, const u64* in_p1_r2, long long n, bool boolean,
+                     u64* out);
 
 // ---- SHA-256 Merkle hash (sha_kernels.cu) ---------------------------------------------------
 // Merkle hash of Pi_Rec: 1024-byte leaves, subtree roots of 64 aligned leaves per CTA.
@@ -257,6 +260,16 @@ void launch_hash_u64(cudaStream_t st, const u64* data, long long n, u32* scratch
 void launch_digest_check(cudaStream_t st, const u32* a0, const u32* b0, const u32* a1,
                          const u32* b1, const u32* a2, const u32* b2, u32* status, u32 flag);
 size_t hash_scratch_words(long long n);
+// Pi_Rec of the sharing xs of n words (arguments as launch_rec_messages): the messages, the opening and
+// the six hashes, of what P1, P2, P2 hold ([r]_1, m, [r]_2) and of what P2, P0, P1 received; a mismatch
+// sets `flag` in *status.  out may lie in xs.
+struct RecBufs {
+  u64 *in_p2_r1, *in_p1_r2, *in_p0_m;   // n words each
+  u32* hs[6];                           // hash_scratch_words(n) 32-bit words each
+  u32* dg;                              // 6 x 8
+};
+void launch_rec(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask, bool boolean,
+                const RecBufs& b, u64* out, u32* status, u32 flag);
 
 // ---- GR(2^64, 64) kernels (gr_kernels.cu) ---------------------------------------------------
 void launch_gr_powers(cudaStream_t st, const u64* a, long long n, u64* table);

@@ -96,18 +96,10 @@ extern "C" int mpc_reconstruct_noalloc(mpc_ctx* ctx, const uint64_t* xs, int64_t
   u64 xmask = 0;
   const long long xidx = ctx_take_rec_fault(ctx, n, &xmask);
   ctx_count(ctx, ph, pr, 3, (u64)n * 8);
-  launch_rec_messages(st, xs, n, xidx, xmask, false, s->in_p2_r1, s->in_p1_r2, s->in_p0_m, out);
-  HashJobs j;   // sent by P1, P2, P2; of what P2, P0, P1 received
-  const u64* data[6] = {xs + 3 * n, xs + 4 * n, xs + 5 * n, s->in_p2_r1, s->in_p0_m, s->in_p1_r2};
-  for (int q = 0; q < 6; ++q) {
-    j.data[q] = data[q];
-    j.scratch[q] = s->hs[q];
-    j.digest[q] = s->dg + 8 * q;
-  }
-  launch_hash_jobs(st, j, 6, n);
   ctx_count(ctx, ph, pr, 3, 32);
-  u32* d = s->dg;
-  launch_digest_check(st, d, d + 24, d + 8, d + 32, d + 16, d + 40, ctx_status_word(ctx), 1u);
+  RecBufs b{s->in_p2_r1, s->in_p1_r2, s->in_p0_m, {}, s->dg};
+  for (int q = 0; q < 6; ++q) b.hs[q] = s->hs[q];
+  launch_rec(st, xs, n, xidx, xmask, false, b, out, ctx_status_word(ctx), 1u);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return ctx_fail(ctx, MPC_ERR_CUDA, cudaGetErrorString(e));
   u32 stv = 0;

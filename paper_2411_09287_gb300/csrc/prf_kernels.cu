@@ -408,17 +408,29 @@ __global__ void k_prf_words(long long n, long long off, Key key, u32 tag, u64 ob
 }
 
 // The three messages of Pi_Rec and P1's opening in one pass (the hashes read the copies).
-__global__ void k_rec_messages(const u64* xs, long long n, long long xidx, u64 xmask,
-                               int boolean, u64* __restrict__ in_p2_r1, u64* __restrict__ in_p1_r2,
-                               u64* __restrict__ in_p0_m, u64* __restrict__ out) {
+__global__ void k_rec_messages(const u64* xs, long long n, long long xidx, u64 xmask, int boolean,
+                               u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out) {
   grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     in_p2_r1[i] = xs[i];
     const u64 r2 = xs[n + i] ^ (i == xidx ? xmask : 0ull);
     in_p1_r2[i] = r2;
-    const u64 m = xs[2 * n + i], r1 = xs[3 * n + i];
+    const u64 m = xs[2 * n + i];
     in_p0_m[i] = m;
+    if (out) {
+      const u64 r1 = xs[3 * n + i];
+      out[i] = boolean ? m ^ r1 ^ r2 : m - r1 - r2;
+    }
+  }
+}
+
+// P1's opening from its own m and [r]_1 and the received [r]_2; out may be a component of xs.
+__global__ void k_rec_open(const u64* xs, const u64* in_p1_r2, long long n, int boolean, u64* out) {
+  grid_dep();
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const u64 m = xs[2 * n + i], r1 = xs[3 * n + i], r2 = in_p1_r2[i];
     out[i] = boolean ? m ^ r1 ^ r2 : m - r1 - r2;
   }
 }
@@ -498,6 +510,12 @@ void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, long long 
   if (n <= 0) return;
   launch_dep(k_rec_messages, grid_for(n), TPB, 0, st, xs, n, xidx, xmask, boolean ? 1 : 0, in_p2_r1,
                                               in_p1_r2, in_p0_m, out);
+}
+
+void launch_rec_open(cudaStream_t st, const u64* xs, const u64* in_p1_r2, long long n, bool boolean,
+                     u64* out) {
+  if (n <= 0) return;
+  launch_dep(k_rec_open, grid_for(n), TPB, 0, st, xs, in_p1_r2, n, boolean ? 1 : 0, out);
 }
 
 }  // namespace mpc3
