@@ -113,8 +113,9 @@ typedef struct {
  *                  multiple of 128; default: the odd multiple of 128 near sqrt(E) that pads least.
  *                  A batch uses at most E rounded up to a multiple of 128; a row_split above
  *                  trunc_block keeps the whole table of powers (no compact table).
- *   tc_combine_min accepted and reported back (default 32) without effect: sum_(e_hi)
- *                  r^(2 L e_hi) S_hi takes the tensor cores from two blocks on.
+ *   tc_combine_min fewest e_hi blocks for which sum_(e_hi) r^(2 L e_hi) S_hi runs on the tensor
+ *                  cores (fewer: one pass on the CUDA cores); default: from two blocks on
+ *                  (mpc_get_tuning reads 32 while the field is unset).
  *   gemm_split_min fewest 32-deep K chunks per split-K slice of a thin tensor-core product;
  *                  default 8.
  *   gram_split     split-K slices of a tensor-core Gram sum (dense rounds); default 76.

@@ -359,6 +359,9 @@ int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long
                       const unsigned char* TL8, long long L, long long nhi, u64* S_hi,
                       unsigned* err, unsigned err_flag);
 
+// out[p] = the reduced product whose terms are P[a ld + 64 p + b] (a, b < 64), for npairs p.
+void launch_fold_reduce_strided(cudaStream_t st, const u64* P, long long ld, int npairs, u64* out);
+
 // ---- compare-select of the non-linear layers (compare.cu) --------------------------------------
 struct CsView {          // component c of element e at p[c stride + e], 0 for e >= valid or p = null
   const u64* p;

@@ -6,7 +6,9 @@
 // six Pi_Reduce rounds (Fig. Reduce) are all linear combinations of S with public GR weights, so
 // S is computed once per layer.  Writing r^(2e) = T_hi[e_hi] T_lo[e_lo] with e = e_hi L + e_lo:
 //   S_hi[e_hi][(j,j')] = sum_{e_lo} T_lo[e_lo] b1_{e,j} b2_{e,j'}     (this file, tensor cores)
-//   S[(j,j')]          = sum_{e_hi} T_hi[e_hi] (x) S_hi[e_hi][(j,j')]  (a u64 GEMM + fold)
+//   S[(j,j')]          = sum_{e_hi} T_hi[e_hi] S_hi[e_hi][(j,j')]
+// The second sum is a GR-matrix product of the blocks in place and a sum over them, or, on the CUDA
+// cores, one u64 GEMM over the blocks and the reduction of its products (k_fold_reduce_strided).
 // Exactness: each u64 coefficient v of T_lo is written as v = sum_l d_l 32^l mod 2^64 with 13 limbs,
 // -16 <= d_l <= 15 (d_12 the top four bits); e4m3 has four significant bits, so every integer from
 // -16 to 16 is exact in it, as are the bits, and an accumulator sums at most L <= 2^16 terms, so
@@ -31,6 +33,7 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
+#include "gr_mul.cuh"
 #include "kernels.h"
 #include "tcgen05.cuh"
 
@@ -313,6 +316,23 @@ k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* B1T,
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
+// out[p][c] = reduce(sum_{a+b=s} P[a*ld + p*64 + b]), one pair p a block.
+__global__ void __launch_bounds__(128) k_fold_reduce_strided(const u64* P, long long ld, u64* out) {
+  grid_dep();
+  __shared__ u64 prod[128];
+  const long long p = blockIdx.x;
+  const int s = threadIdx.x;
+  u64 v = 0;
+  if (s < 127) {
+    const int a0 = (s < 64) ? 0 : s - 63;
+    const int a1 = (s < 64) ? s : 63;
+    for (int a = a0; a <= a1; ++a) v += P[a * ld + p * 64 + (s - a)];
+  }
+  prod[s] = v;
+  __syncthreads();
+  if (s < 64) out[p * 64 + s] = gr_reduce_at(prod, prod + 64, s);
+}
+
 }  // namespace
 
 void launch_trunc_limb_table(cudaStream_t st, const u64* Tlo, long long L, unsigned char* TL8) {
@@ -342,6 +362,10 @@ int launch_trunc_s_tc(cudaStream_t st, const u64* B1T, const u64* B2T, long long
   dim3 grid(4096 / S_TPAIRS, 64 * S_LIMBS / S_TCOLS, (unsigned)nhi);
   launch_dep(k_trunc_s_tc, grid, S_THREADS, S_SMEM, st, mb, B1T, B2T, Epad / 64, L, S_hi, err, err_flag);
   return 0;
+}
+
+void launch_fold_reduce_strided(cudaStream_t st, const u64* P, long long ld, int npairs, u64* out) {
+  launch_dep(k_fold_reduce_strided, npairs, 128, 0, st, P, ld, out);
 }
 
 }  // namespace mpc3
