@@ -442,6 +442,10 @@ void mpc_ledger_reset(mpc_ctx* ctx);
  * (index mod length) XORed with xor_mask (MPC_SITE_HIGH_BIT ignores xor_mask and uses 2^63).
  * Host side only; it never faults the device. */
 int mpc_inject_fault(mpc_ctx* ctx, int site, uint64_t index, uint64_t xor_mask);
+/* The same for the message after the next `skip` messages of the site (skip = 0: mpc_inject_fault), in
+ * the order in which the calls enqueue them: so every opening of a verification can be reached at
+ * MPC_SITE_REC_MSG (Fig. Reduce, Fig. DPV: r, each round's zeta', Delta, batch after batch). */
+int mpc_inject_fault_after(mpc_ctx* ctx, int site, uint64_t skip, uint64_t index, uint64_t xor_mask);
 
 /* Phase timers: with profiling on, the library brackets each phase of its work with CUDA events
  * on the context's stream (no synchronisation).  mpc_profile(ctx, 1) clears and starts,

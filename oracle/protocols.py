@@ -141,8 +141,8 @@ def _gamma_message(sess: Session, gamma_p0, g1, proto: str, phase: str):
     [Gamma]_2 = Gamma - [Gamma]_1 to P2.  The HIGH_BIT site models the ring attack e = 2^(l-1)."""
     g2 = (gamma_p0 - g1) & sess.mask
     if "HIGH_BIT" in sess.faults:
-        idx, _ = sess.faults.pop("HIGH_BIT")
-        sess.faults["GAMMA2"] = (idx, 1 << (sess.gr.ell - 1))
+        idx, _, skip = sess.faults.pop("HIGH_BIT")
+        sess.faults["GAMMA2"] = (idx, 1 << (sess.gr.ell - 1), skip)
     return sess.send(0, 2, phase, proto, g2, site="GAMMA2")
 
 

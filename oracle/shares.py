@@ -132,9 +132,10 @@ class Session:
         return np.asarray(arr, dtype=np.uint64)
 
     # ---- messages ----------------------------------------------------------------------------
-    def arm_fault(self, site: str, index: int, xor_mask: int):
+    def arm_fault(self, site: str, index: int, xor_mask: int, skip: int = 0):
+        """One-shot fault of the message at `site` after the next `skip` ones."""
         assert site in FAULT_SITES
-        self.faults[site] = (int(index), int(xor_mask))
+        self.faults[site] = (int(index), int(xor_mask), int(skip))
 
     def send(self, src: int, dst: int, phase: str, proto: str, arr, site: str = None,
              nbytes: int = None) -> np.ndarray:
@@ -143,10 +144,13 @@ class Session:
             nbytes = arr.size * 8 * self.gr.ell // 64 if self.gr.ell < 64 else arr.size * 8
         self.ledger.append(LedgerEntry(src, dst, phase, proto, nbytes))
         if site is not None and site in self.faults:
-            idx, m = self.faults.pop(site)
-            flat = arr.reshape(-1)
-            flat[idx % max(flat.size, 1)] ^= np.uint64(m)
-            arr = (flat & self.mask).reshape(arr.shape)
+            idx, m, skip = self.faults.pop(site)
+            if skip:
+                self.faults[site] = (idx, m, skip - 1)
+            else:
+                flat = arr.reshape(-1)
+                flat[idx % max(flat.size, 1)] ^= np.uint64(m)
+                arr = (flat & self.mask).reshape(arr.shape)
         return arr
 
     def send_hash(self, src: int, dst: int, phase: str, proto: str, digest: bytes) -> bytes:

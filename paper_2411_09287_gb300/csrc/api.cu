@@ -54,6 +54,7 @@ struct Fault {
   bool armed = false;
   u64 index = 0;
   u64 mask = 0;
+  u64 skip = 0;   // messages of the site that pass before it
 };
 
 __global__ void k_derive_keys(Key master, u32* out) {
@@ -233,16 +234,20 @@ int guard(mpc_ctx* ctx) {
 bool id_ok(u64 id) { return id < (1ull << 44); }
 
 // ---- messages -----------------------------------------------------------------------------------
-void apply_fault(mpc_ctx* ctx, int site, u64* dst, long long n) {
-  if (site == MPC_SITE_GAMMA2 && ctx->fault[MPC_SITE_HIGH_BIT].armed) {
-    ctx->fault[MPC_SITE_HIGH_BIT].armed = false;
-    ctx->fault[MPC_SITE_GAMMA2] = {true, ctx->fault[MPC_SITE_HIGH_BIT].index, 1ull << 63};
-  }
+// The fault that is due at this message of n words of `site`, disarmed (HIGH_BIT is a fault of the
+// [Gamma]_2 messages, in place of GAMMA2's).
+MsgFault take_fault(mpc_ctx* ctx, int site, long long n) {
+  if (site < 0 || n <= 0) return {};
+  if (site == MPC_SITE_GAMMA2 && ctx->fault[MPC_SITE_HIGH_BIT].armed) site = MPC_SITE_HIGH_BIT;
   Fault& f = ctx->fault[site];
-  if (f.armed && n > 0) {
-    launch_xor_one(ctx->st, dst + (f.index % (u64)n), f.mask);
-    f.armed = false;
+  if (!f.armed) return {};
+  if (f.skip) {
+    --f.skip;
+    return {};
   }
+  f.armed = false;
+  if (site == MPC_SITE_HIGH_BIT) ctx->fault[MPC_SITE_GAMMA2].armed = false;
+  return {(long long)(f.index % (u64)n), f.mask};
 }
 
 void count_msgs(mpc_ctx* ctx, int phase, int proto, int count, u64 bytes_each) {
@@ -250,21 +255,19 @@ void count_msgs(mpc_ctx* ctx, int phase, int proto, int count, u64 bytes_each) {
   ctx->nmsg += (u64)count;
 }
 
-
-int deliver_copy(mpc_ctx* ctx, int phase, int proto, const u64* src, u64* dst, long long n, int site) {
+int deliver_copy(mpc_ctx* ctx, int phase, int proto, const u64* src, u64* dst, long long n,
+                 const MsgFault& f) {
   if (n > 0) CK(cudaMemcpyAsync(dst, src, (size_t)n * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  ctx->ledger[phase][proto] += (u64)n * 8;
-  ctx->nmsg += 1;
-  if (site >= 0) apply_fault(ctx, site, dst, n);
+  count_msgs(ctx, phase, proto, 1, (u64)n * 8);
+  if (f.idx >= 0) launch_xor_one(ctx->st, dst + f.idx, f.mask);
   return MPC_OK;
 }
 
 // The message src to a receiver that only reads it: it is handed over in place (dst becomes src), and
-// copied only to be corrupted by an armed fault.  A copy of a small message is a launch of 4 us.
+// copied only to be corrupted by a fault.  A copy of a small message is a launch of 4 us.
 int deliver(mpc_ctx* ctx, int phase, int proto, u64* src, u64*& dst, long long n, int site) {
-  if (site >= 0 && n > 0 &&
-      (ctx->fault[site].armed || (site == MPC_SITE_GAMMA2 && ctx->fault[MPC_SITE_HIGH_BIT].armed)))
-    return deliver_copy(ctx, phase, proto, src, dst, n, site);
+  const MsgFault f = take_fault(ctx, site, n);
+  if (f.idx >= 0) return deliver_copy(ctx, phase, proto, src, dst, n, f);
   count_msgs(ctx, phase, proto, 1, (u64)n * 8);
   dst = src;
   return MPC_OK;
@@ -476,23 +479,17 @@ void flush_recs(mpc_ctx* ctx, const Small& s) {
   s.nrec = 0;
 }
 
-// Pi_Rec of one shared GR element (3 shares + 3 hashes): the record its messages go to, and an
-// armed REC_MSG fault, which corrupts the P0 -> P1 share, as for any other Pi_Rec.
+// Pi_Rec of one shared GR element (3 shares + 3 hashes): the record its messages go to, and the
+// REC_MSG fault that is due, which corrupts the P0 -> P1 share, as for any other Pi_Rec.
 struct Rec1 {
   u64* rec;
-  u64 mask = 0;
-  int idx = -1;
+  MsgFault fault;
 };
 Rec1 begin_rec(mpc_ctx* ctx, const Small& s) {
   if (s.nrec == REC_SLOTS) flush_recs(ctx, s);
   Rec1 r;
   r.rec = s.rec + (long long)s.nrec++ * REC_WORDS;
-  Fault& f = ctx->fault[MPC_SITE_REC_MSG];
-  if (f.armed) {
-    r.mask = f.mask;
-    r.idx = (int)(f.index % 64);
-    f.armed = false;
-  }
+  r.fault = take_fault(ctx, MPC_SITE_REC_MSG, 64);
   count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);
   count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 32);
   return r;
@@ -501,7 +498,7 @@ Rec1 begin_rec(mpc_ctx* ctx, const Small& s) {
 // <v> random GR element, revealed with Pi_Rec.
 void reveal(mpc_ctx* ctx, u32 purpose, u64 obj, const Small& s, u64* out) {
   const Rec1 r = begin_rec(ctx, s);
-  launch_reveal(ctx->st, ctx->k01, ctx->k02, ctx->k12, purpose, obj, r.mask, r.idx, out, r.rec);
+  launch_reveal(ctx->st, ctx->k01, ctx->k02, ctx->k12, purpose, obj, r.fault, out, r.rec);
 }
 
 // Clears both halves of the round sums and Pi_InnerVerify's; a round adds into cur_sums, and its tail clears the other
@@ -545,8 +542,7 @@ void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, 
   count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 6, 512);   // two secure inner products
   const Rec1 r = begin_rec(ctx, s);
   a.rec = r.rec;
-  a.xmask = r.mask;
-  a.xidx = r.idx;
+  a.fault = r.fault;
   launch_round_tail(ctx->st, a);
   s.uc ^= 1;
 }
@@ -730,8 +726,7 @@ int inner_verify_dense(mpc_ctx* ctx, u64 vid, u32 batch, const Vec& x, const Vec
   count_msgs(ctx, MPC_PHASE_VERIFY, MPC_PROTO_VERIFY, 3, 512);            // the inner product
   const Rec1 r = begin_rec(ctx, s);
   a.rec = r.rec;
-  a.xmask = r.mask;
-  a.xidx = r.idx;
+  a.fault = r.fault;
   a.trace = trace ? trace + (long long)R * TRACE_ROUND : nullptr;
   a.status = ctx->status;
   a.flag = ST_VERIFY;
@@ -873,22 +868,12 @@ RecPlan plan_rec(Arena& a, long long n, bool need_out) {
   return p;
 }
 
-// The armed REC_MSG fault of a Pi_Rec of n words, disarmed: its word index (-1: none) and mask.
-long long take_rec_fault(mpc_ctx* ctx, long long n, u64* mask) {
-  Fault& f = ctx->fault[MPC_SITE_REC_MSG];
-  if (!f.armed) return -1;
-  f.armed = false;
-  *mask = f.mask;
-  return (long long)(f.index % (u64)n);
-}
-
 // Pi_Rec of n words up to the hash comparison (into the status word): P0 sends [r]_1 to P2 and
 // [r]_2 to P1 (fault site REC_MSG, arithmetic sharings), P1 sends m to P0; P1 sends H([r]_1) to P2,
 // P2 H(m) to P0 and H([r]_2) to P1, and every receiver hashes what it received.  out = P1's opening.
 void rec_core(mpc_ctx* ctx, const u64* xs, long long n, const RecPlan& p, u64* out, bool boolean) {
-  u64 xmask = 0;
-  const long long xidx = boolean ? -1 : take_rec_fault(ctx, n, &xmask);
-  launch_rec(ctx->st, xs, n, xidx, xmask, boolean, p, out, ctx->status, ST_ABORT);
+  const MsgFault f = take_fault(ctx, boolean ? -1 : MPC_SITE_REC_MSG, n);
+  launch_rec(ctx->st, xs, n, f, boolean, p, out, ctx->status, ST_ABORT);
   count_msgs(ctx, MPC_PHASE_ONLINE, MPC_PROTO_REC, 3, (u64)n * 8);
   count_msgs(ctx, MPC_PHASE_ONLINE, MPC_PROTO_REC, 3, 32);
 }
@@ -1990,11 +1975,12 @@ int mpc_share_input_from(mpc_ctx* ctx, uint64_t call_id, int owner, const uint64
   u64* m2 = (u64*)xs + 4 * n;
   if (owner == 1)
     CK(cudaMemcpyAsync(m1, mout, (size_t)n * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  else if ((rc = deliver_copy(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m1, n, MPC_SITE_MX_COPY_P1)))
+  else if ((rc = deliver_copy(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m1, n,
+                              take_fault(ctx, MPC_SITE_MX_COPY_P1, n))))
     return rc;
   if (owner == 2)
     CK(cudaMemcpyAsync(m2, mout, (size_t)n * 8, cudaMemcpyDeviceToDevice, ctx->st));
-  else if ((rc = deliver_copy(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m2, n, -1)))
+  else if ((rc = deliver_copy(ctx, MPC_PHASE_ONLINE, MPC_PROTO_SHARE, mout, m2, n, MsgFault{})))
     return rc;
   return cuda_check(ctx, "share_input");
 }
@@ -2353,8 +2339,12 @@ void mpc_ledger_reset(mpc_ctx* ctx) {
 }
 
 int mpc_inject_fault(mpc_ctx* ctx, int site, uint64_t index, uint64_t xor_mask) {
+  return mpc_inject_fault_after(ctx, site, 0, index, xor_mask);
+}
+
+int mpc_inject_fault_after(mpc_ctx* ctx, int site, uint64_t skip, uint64_t index, uint64_t xor_mask) {
   if (!ctx || site < 0 || site >= MPC_NSITE) return MPC_ERR_ARG;
-  ctx->fault[site] = {true, index, site == MPC_SITE_HIGH_BIT ? (1ull << 63) : xor_mask};
+  ctx->fault[site] = {true, index, site == MPC_SITE_HIGH_BIT ? (1ull << 63) : xor_mask, skip};
   return MPC_OK;
 }
 
@@ -2566,8 +2556,7 @@ namespace mpc3 {
 namespace internal {
 int ctx_guard(mpc_ctx* c) { return guard(c); }
 int ctx_fail(mpc_ctx* c, int code, const char* msg) { return fail(c, code, msg); }
-// The armed REC_MSG fault of a Pi_Rec of n words, disarmed: its word index (-1: none) and mask.
-long long ctx_take_rec_fault(mpc_ctx* c, long long n, u64* mask) { return take_rec_fault(c, n, mask); }
+MsgFault ctx_take_rec_fault(mpc_ctx* c, long long n) { return take_fault(c, MPC_SITE_REC_MSG, n); }
 void ctx_count(mpc_ctx* c, int phase, int proto, int count, u64 bytes_each) {
   count_msgs(c, phase, proto, count, bytes_each);
 }
@@ -2582,23 +2571,11 @@ void ctx_set_aborted(mpc_ctx* c) { c->aborted = true; }
 // ---- non-linear layers (Sec. 4.3) -------------------------------------------------------------
 namespace {
 
-// The fault armed at `site` for a message of n words, disarmed.
-MsgFault take_fault(mpc_ctx* ctx, int site, long long n) {
-  if (site == MPC_SITE_GAMMA2 && ctx->fault[MPC_SITE_HIGH_BIT].armed) {
-    ctx->fault[MPC_SITE_HIGH_BIT].armed = false;
-    ctx->fault[MPC_SITE_GAMMA2] = {true, ctx->fault[MPC_SITE_HIGH_BIT].index, 1ull << 63};
-  }
-  Fault& f = ctx->fault[site];
-  if (!f.armed) return {-1, 0};
-  f.armed = false;
-  return {(long long)(f.index % (u64)n), f.mask};
-}
-
-// The same for a Boolean message of nw words: the AND_GAMMA2 site flips bit `index` of it (when mask
+// take_fault for a Boolean message of nw words: the AND_GAMMA2 site flips bit `index` of it (when mask
 // & 1), the Boolean counterpart of an element fault; HIGH_BIT at l = 1 is the same bit flip.
 MsgFault take_bit_fault(mpc_ctx* ctx, int site, long long nw) {
   const MsgFault f = take_fault(ctx, site, 64 * nw);
-  if (f.idx < 0 || !(f.mask & 1ull)) return {-1, 0};
+  if (f.idx < 0 || !(f.mask & 1ull)) return {};
   return {f.idx / 64, 1ull << (f.idx % 64)};
 }
 
@@ -2723,6 +2700,14 @@ int gf_verify(mpc_ctx* ctx, u64 vid, GfPlan& g, u64* trace) {
   v.status = ctx->status;
   v.flag_verify = ST_VERIFY;
   v.flag_abort = ST_ABORT;
+  v.xrec = -1;
+  v.xmask = 0;
+  for (int i = 0; i < g.R + 2; ++i) {   // the openings: r, the zetas, Delta
+    const MsgFault f = take_fault(ctx, MPC_SITE_REC_MSG, 1);
+    if (f.idx < 0) continue;
+    v.xrec = i;
+    v.xmask = f.mask;
+  }
   launch_gf_verify(ctx->st, v);
   // Pi_Rec of r, the zetas and Delta (3 words and 3 hashes each); two secure inner products a round,
   // x alpha and the last inner product

@@ -47,7 +47,7 @@ __device__ __forceinline__ u64 round_stream(const GfVerify& a, int k, int q) {
 // h(0)) with L2 = (zeta^2 + zeta) / (x (x + 1)), L1 = (zeta^2 + x zeta) / (1 + x) = x L2 + zeta.
 __device__ __forceinline__ void gf_tail(const GfVerify& a, int k, const u64* s, const u64* st, u64* z,
                                         u64* zeta_out, const Coef cf, int c) {
-  const u64 zeta = st[8] ^ st[6] ^ st[7];
+  const u64 zeta = st[8] ^ st[6] ^ st[7] ^ (k == a.xrec ? a.xmask : 0ull);   // P1's opening
   u64 h[2];
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_gf_setup(const GfVerify a, long long nb
   if (tid < 3) st[tid] = round_stream(a, 0, tid);
   __syncthreads();
   if (tid == 0) {
-    u64 r = st[2] ^ st[0] ^ st[1];
+    u64 r = st[2] ^ st[0] ^ st[1] ^ (a.xrec == 0 ? a.xmask : 0ull);
     if (blockIdx.x == 0) a.w->r = r;
     r = gf_mul(r, r);
     r = gf_mul(r, r);
@@ -430,18 +430,20 @@ k_gf_last(const GfVerify a, const Coef cf, int k, long long D0, const u64* x, co
   if (tid == 0) {
     const u64 m1 = sd[1] ^ dg, m2 = sd[2] ^ (sd[0] ^ d1 ^ d2 ^ dg);
     dl = m1 ^ m2;                        // m of Delta
-    const u64 delta = dl ^ d1 ^ d2;      // P1's opening
+    const u64 delta = dl ^ d1 ^ d2 ^ (a.xrec == a.R + 1 ? a.xmask : 0ull);   // P1's opening
     if (a.trace) a.trace[(long long)a.R * a.trace_ld] = delta;
     if (delta) atomicOr(a.status, a.flag_verify);
   }
   __syncthreads();
-  // The hashes of every Pi_Rec (r, the zetas, Delta): thread 2 h hashes what was sent for message h,
-  // thread 2 h + 1 what arrived (the same words: these openings have no fault site).
+  // The hashes of every Pi_Rec (r, the zetas, Delta): of message h thread 2 h hashes what its hasher
+  // holds, thread 2 h + 1 what the receiver got, which is the same word unless a fault corrupts it
+  // ([r]_2 at P1).
   for (int i0 = 0; i0 < 6 * (a.R + 2); i0 += 512) {
     const int i = i0 + tid, rec = i / 6, msg = (i % 6) >> 1;
     u64 w = 0;
     if (rec <= a.R) w = a.st[rec == 0 ? msg : 9 * rec + 6 + msg];
     else if (rec == a.R + 1) w = msg == 0 ? d1 : msg == 1 ? d2 : dl;
+    if (rec == a.xrec && msg == 1 && (i & 1)) w ^= a.xmask;
     u32 h[8];
     sha256_word(w, h);
     bool diff = false;

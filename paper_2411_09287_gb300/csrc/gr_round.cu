@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
   }
   __syncthreads();
   if (tid < 64) {   // P1's opening: m - [r]_1 - [r]_2 as received
-    const u64 r2 = st[7][t] ^ (t == a.xidx ? a.xmask : 0ull);
+    const u64 r2 = st[7][t] ^ (t == a.fault.idx ? a.fault.mask : 0ull);
     zt[t] = st[8][t] - st[6][t] - r2;
   }
   __syncthreads();
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
       l[192 + t] = st[6][t];       // [r]_1 held by P1
       l[256 + t] = st[7][t];       // [r]_2 held by P2
       l[320 + t] = st[8][t];       // m held by P2
-      l[384 + t] = st[7][t] ^ (t == a.xidx ? a.xmask : 0ull);   // [r]_2 received by P1
+      l[384 + t] = st[7][t] ^ (t == a.fault.idx ? a.fault.mask : 0ull);   // [r]_2 received by P1
     }
     __syncthreads();
     for (int i = tid; i < 4096; i += 512) a.MM[i] = gr_mulmat_at(fe, i >> 6, i & 63);
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(512) k_round_tail(const RoundTail a) {
 
 // <v> random GR element (streams of `purpose`), opened with Pi_Rec; its messages go to rec.
 __global__ void __launch_bounds__(64)
-k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u64* __restrict__ out,
+k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, const MsgFault fault, u64* __restrict__ out,
          u64* __restrict__ rec) {
   __shared__ u64 st[3][64];
   const int t = threadIdx.x;
@@ -199,7 +199,7 @@ k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask, int xidx, u
   __syncthreads();
   grid_dep();   // the streams come from the keys alone
   const u64 r1 = st[0][t], r2 = st[1][t], m = st[2][t];
-  const u64 r2in = r2 ^ (t == xidx ? xmask : 0ull);
+  const u64 r2in = r2 ^ (t == fault.idx ? fault.mask : 0ull);
   rec[t] = r1;
   rec[64 + t] = r2;
   rec[128 + t] = m;
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
   const u64 r1 = st[0][t], r2 = st[1][t], g1 = st[2][t];
   const u64 g2 = __ldcg(a.acc + t) + r1 + r2 - g1;                          // P0 -> P2
   const u64 m = (__ldcg(a.acc + 64 + t) + g1) + (__ldcg(a.acc + 128 + t) + g2);   // P1 <-> P2
-  const u64 r2in = r2 ^ (t == a.xidx ? a.xmask : 0ull);
+  const u64 r2in = r2 ^ (t == a.fault.idx ? a.fault.mask : 0ull);
   a.rec[t] = r1;
   a.rec[64 + t] = r2;
   a.rec[128 + t] = m;
@@ -566,9 +566,9 @@ void launch_round_tail(cudaStream_t st, const RoundTail& a) {
   launch_dep(k_round_tail, 7 + a.nvw, 512, 0, st, a);
 }
 
-void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
-                   int xidx, u64* out, u64* rec) {
-  launch_dep(k_reveal, 1, 64, 0, st, k01, k02, k12, purpose, obj, xmask, xidx, out, rec);
+void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj,
+                   const MsgFault& fault, u64* out, u64* rec) {
+  launch_dep(k_reveal, 1, 64, 0, st, k01, k02, k12, purpose, obj, fault, out, rec);
 }
 
 void launch_small_round(cudaStream_t st, const SmallRound& a) {

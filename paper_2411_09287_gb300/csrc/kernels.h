@@ -134,6 +134,12 @@ int gram_jobs_tc(cudaStream_t st, long long Dh, const GramJobs& jobs, unsigned* 
 int gram3_tc(cudaStream_t st, long long Dh, const u64* x, const u64* y, u64* P, unsigned* err,
              unsigned err_flag, int nsplit = 0);
 
+// A fault of one message: word idx XORed with mask where it arrives (idx < 0: none).
+struct MsgFault {
+  long long idx = -1;
+  u64 mask = 0;
+};
+
 // ---- single-element steps of the verification (gr_round.cu) ---------------------------------
 // Words of one opened element's record: the copies that Pi_Rec's hashes compare.
 constexpr int REC_WORDS = 7 * 64;
@@ -150,8 +156,7 @@ struct RoundTail {
   u64* MM;              // the multiplication matrix of f
   u64* zp;              // the opened zeta'
   u64* rec;             // this Pi_Rec's record (REC_WORDS)
-  u64 xmask;            // fault: word xidx of the P0 -> P1 message is XORed with xmask
-  int xidx;
+  MsgFault fault;       // of the opening's P0 -> P1 message
   u64* zero;            // nzero words cleared for the next round
   long long nzero;
   u64* trace;           // zeta' | h(0) | h(p2) of the round, or null
@@ -165,8 +170,8 @@ struct ZeroRows {
 void launch_zero_rows(cudaStream_t st, const ZeroRows& r);
 void launch_round_tail(cudaStream_t st, const RoundTail& a);
 // A random GR element of the streams of (purpose, obj), opened into out; record in rec.
-void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj, u64 xmask,
-                   int xidx, u64* out, u64* rec);
+void launch_reveal(cudaStream_t st, Key k01, Key k02, Key k12, u32 purpose, u64 obj,
+                   const MsgFault& fault, u64* out, u64* rec);
 // A round's fold and party sums on a claim of D elements, for short claims.
 struct SmallRound {
   const u64* in[12];    // x's components, then y's (null = zero)
@@ -188,8 +193,7 @@ struct InnerVerify {
   u64 obj;
   u64* acc;
   u64* rec;             // this Pi_Rec's record (REC_WORDS)
-  u64 xmask;            // fault: word xidx of the P0 -> P1 message is XORed with xmask
-  int xidx;
+  MsgFault fault;       // of the opening's P0 -> P1 message
   u64* trace;
   u32* status;
   u32 flag;
@@ -228,10 +232,10 @@ void launch_trunc_finish(cudaStream_t st, long long E, Key k01, Key k02, u64 obj
                          const u64* row_keys, long long N);
 void launch_xor_one(cudaStream_t st, u64* p, u64 mask);
 // The messages of Pi_Rec of a sharing xs and (out not null) P1's opening: in_p2_r1 = P0.[r]_1, in_p1_r2
-// = P0.[r]_2 (word xidx XORed with xmask when xidx >= 0), in_p0_m = P1.m, out = P1.m - P1.[r]_1 -
-// in_p1_r2 (XOR for a Boolean sharing).
-void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask,
-                         bool boolean, u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out);
+// = P0.[r]_2 (with the fault), in_p0_m = P1.m, out = P1.m - P1.[r]_1 - in_p1_r2 (XOR for a Boolean
+// sharing).
+void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, const MsgFault& fault, bool boolean,
+                         u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out);
 // The opening alone, from the received in_p1_r2.
 void launch_rec_open(cudaStream_t st, const u64* xs, const u64* in_p1_r2, long long n, bool boolean,
                      u64* out);
@@ -268,7 +272,7 @@ struct RecBufs {
   u32* hs[6];                           // hash_scratch_words(n) 32-bit words each
   u32* dg;                              // 6 x 8
 };
-void launch_rec(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask, bool boolean,
+void launch_rec(cudaStream_t st, const u64* xs, long long n, const MsgFault& fault, bool boolean,
                 const RecBufs& b, u64* out, u32* status, u32 flag);
 
 // ---- GR(2^64, 64) kernels (gr_kernels.cu) ---------------------------------------------------
@@ -367,10 +371,6 @@ struct CsView {          // component c of element e at p[c stride + e], 0 for e
   const u64* p;
   long long stride, valid;
 };
-struct MsgFault {        // word idx of a message XORed with mask (idx < 0: none)
-  long long idx;
-  u64 mask;
-};
 // One stage of np elements (a multiple of 64): out = max(a, b).
 struct CompareSelect {
   CsView a, b;
@@ -428,6 +428,8 @@ struct GfVerify {
   long long trace_ld;
   u32* status;
   u32 flag_verify, flag_abort;   // Delta != 0; a hash mismatch
+  int xrec;              // fault: the P0 -> P1 message of opening xrec (0: r, k: zeta of round k, R + 1:
+  u64 xmask;             // Delta; -1: none) is XORed with xmask
 };
 void launch_gf_verify(cudaStream_t st, const GfVerify& a);
 // ---- layer-level calls (layer_kernels.cu) ----------------------------------------------------

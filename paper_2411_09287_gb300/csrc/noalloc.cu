@@ -28,7 +28,7 @@ int ctx_guard(mpc_ctx* c);
 int ctx_fail(mpc_ctx* c, int code, const char* msg);
 void ctx_count(mpc_ctx* c, int phase, int proto, int count, u64 bytes_each);
 int ctx_read_status(mpc_ctx* c, u32* out);
-long long ctx_take_rec_fault(mpc_ctx* c, long long n, u64* mask);
+MsgFault ctx_take_rec_fault(mpc_ctx* c, long long n);
 bool ctx_has_pending(const mpc_ctx* c);
 cudaStream_t ctx_stream(const mpc_ctx* c);
 u32* ctx_status_word(const mpc_ctx* c);
@@ -93,13 +93,11 @@ extern "C" int mpc_reconstruct_noalloc(mpc_ctx* ctx, const uint64_t* xs, int64_t
   if ((rc = scratch_for_current_device(ctx, &s))) return rc;
   cudaStream_t st = ctx_stream(ctx);
   const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_REC;
-  u64 xmask = 0;
-  const long long xidx = ctx_take_rec_fault(ctx, n, &xmask);
   ctx_count(ctx, ph, pr, 3, (u64)n * 8);
   ctx_count(ctx, ph, pr, 3, 32);
   RecBufs b{s->in_p2_r1, s->in_p1_r2, s->in_p0_m, {}, s->dg};
   for (int q = 0; q < 6; ++q) b.hs[q] = s->hs[q];
-  launch_rec(st, xs, n, xidx, xmask, false, b, out, ctx_status_word(ctx), 1u);
+  launch_rec(st, xs, n, ctx_take_rec_fault(ctx, n), false, b, out, ctx_status_word(ctx), 1u);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return ctx_fail(ctx, MPC_ERR_CUDA, cudaGetErrorString(e));
   u32 stv = 0;

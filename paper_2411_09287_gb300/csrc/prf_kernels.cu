@@ -408,13 +408,13 @@ __global__ void k_prf_words(long long n, long long off, Key key, u32 tag, u64 ob
 }
 
 // The three messages of Pi_Rec and P1's opening in one pass (the hashes read the copies).
-__global__ void k_rec_messages(const u64* xs, long long n, long long xidx, u64 xmask, int boolean,
+__global__ void k_rec_messages(const u64* xs, long long n, const MsgFault fault, int boolean,
                                u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out) {
   grid_dep();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     in_p2_r1[i] = xs[i];
-    const u64 r2 = xs[n + i] ^ (i == xidx ? xmask : 0ull);
+    const u64 r2 = xs[n + i] ^ (i == fault.idx ? fault.mask : 0ull);
     in_p1_r2[i] = r2;
     const u64 m = xs[2 * n + i];
     in_p0_m[i] = m;
@@ -505,11 +505,11 @@ void launch_prf_words(cudaStream_t st, long long n, Key key, u32 tag, u64 obj, u
   launch_dep(k_prf_words, grid_for((off + n + 7) / 8 - off / 8), TPB, 0, st, n, off, key, tag, obj, out);
 }
 
-void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask,
-                         bool boolean, u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out) {
+void launch_rec_messages(cudaStream_t st, const u64* xs, long long n, const MsgFault& fault, bool boolean,
+                         u64* in_p2_r1, u64* in_p1_r2, u64* in_p0_m, u64* out) {
   if (n <= 0) return;
-  launch_dep(k_rec_messages, grid_for(n), TPB, 0, st, xs, n, xidx, xmask, boolean ? 1 : 0, in_p2_r1,
-                                              in_p1_r2, in_p0_m, out);
+  launch_dep(k_rec_messages, grid_for(n), TPB, 0, st, xs, n, fault, boolean ? 1 : 0, in_p2_r1, in_p1_r2,
+             in_p0_m, out);
 }
 
 void launch_rec_open(cudaStream_t st, const u64* xs, const u64* in_p1_r2, long long n, bool boolean,

@@ -181,12 +181,12 @@ void launch_digest_check(cudaStream_t st, const u32* a0, const u32* b0, const u3
   launch_dep(k_digest_check, 1, 32, 0, st, a0, b0, a1, b1, a2, b2, status, flag);
 }
 
-void launch_rec(cudaStream_t st, const u64* xs, long long n, long long xidx, u64 xmask, bool boolean,
+void launch_rec(cudaStream_t st, const u64* xs, long long n, const MsgFault& fault, bool boolean,
                 const RecBufs& b, u64* out, u32* status, u32 flag) {
   // The opening rides with the messages unless it would overwrite words that are still to be read: an
   // out inside xs is written after the hashes.
   const bool inside = out < xs + 6 * n && xs < out + n;
-  launch_rec_messages(st, xs, n, xidx, xmask, boolean, b.in_p2_r1, b.in_p1_r2, b.in_p0_m,
+  launch_rec_messages(st, xs, n, fault, boolean, b.in_p2_r1, b.in_p1_r2, b.in_p0_m,
                       inside ? nullptr : out);
   HashJobs j;
   const u64* data[6] = {xs + 3 * n, xs + 4 * n, xs + 5 * n, b.in_p2_r1, b.in_p0_m, b.in_p1_r2};

@@ -466,8 +466,9 @@ class Context:
     def ledger_reset(self):
         self.lib.mpc_ledger_reset(self.h)
 
-    def inject_fault(self, site: str, index: int, xor_mask: int = 1):
-        self._check(self.lib.mpc_inject_fault(self.h, SITES[site], index, xor_mask))
+    def inject_fault(self, site: str, index: int, xor_mask: int = 1, skip: int = 0):
+        """mpc_inject_fault_after: a one-shot fault of the message after the next `skip` ones."""
+        self._check(self.lib.mpc_inject_fault_after(self.h, SITES[site], skip, index, xor_mask))
 
     def status(self) -> int:
         return self.lib.mpc_status(self.h)
