@@ -311,6 +311,41 @@ __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
   }
 }
 
+// The end of Pi_InnerVerify in the block that finishes last: the inner product from the sums in acc, Delta
+// opened, the status.  Every thread of the block calls it; st is 3 x 64 words of shared memory.
+__device__ void inner_verify_open(const InnerVerify& a, u64 (*st)[64]) {
+  __shared__ int last;
+  const int tid = threadIdx.x, t = tid & 63;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0)
+    last = atomicAdd(reinterpret_cast<unsigned long long*>(a.acc + 192), 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (tid < 24) {
+    const int q = tid >> 3;
+    stream64(q == 1 ? a.k02 : a.k01, make_tag(P_VER_DELTA, q == 0 ? C_R1 : q == 1 ? C_R2 : C_G1),
+             a.obj, tid & 7, st[q]);
+  }
+  __syncthreads();
+  if (tid >= 64) return;
+  const u64 r1 = st[0][t], r2 = st[1][t], g1 = st[2][t];
+  const u64 g2 = __ldcg(a.acc + t) + r1 + r2 - g1;                          // P0 -> P2
+  const u64 m = (__ldcg(a.acc + 64 + t) + g1) + (__ldcg(a.acc + 128 + t) + g2);   // P1 <-> P2
+  const u64 r2in = r2 ^ (t == a.fault.idx ? a.fault.mask : 0ull);
+  a.rec[t] = r1;
+  a.rec[64 + t] = r2;
+  a.rec[128 + t] = m;
+  a.rec[192 + t] = r1;
+  a.rec[256 + t] = r2;
+  a.rec[320 + t] = m;
+  a.rec[384 + t] = r2in;
+  const u64 d = m - r1 - r2in;
+  if (a.trace) a.trace[t] = d;
+  if (d != 0ull) atomicOr(a.status, a.flag);
+}
+
 // Pi_InnerVerify (Fig. DPV) on a claim of D elements, in one launch.  Row i < D: x'_i = alpha x_i
 // (alpha random, shared, never opened) by Pi_Mult over GR, whose messages are Gamma_i - [Gamma_i]_1
 // (P0 -> P2) and the two halves of m (P1 <-> P2); row D: alpha against -z.  Every block takes some
@@ -324,7 +359,6 @@ __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
 __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
   __shared__ u64 al[6][64];           // r1, r2, m of alpha; r_a, m - r2
   __shared__ u64 u[6][64], v[6][64], st[3][64], scr[4 * 128];
-  __shared__ int last;
   const int tid = threadIdx.x, t = tid & 63, i0 = (tid >> 6) * 16;
   if (tid < 24) {
     const int q = tid >> 3;
@@ -400,35 +434,141 @@ __global__ void __launch_bounds__(256) k_inner_verify(const InnerVerify a) {
     if (tid < 64)
       atomicAdd(reinterpret_cast<unsigned long long*>(a.acc + q * 64 + t), (unsigned long long)r);
   }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0)
-    last = atomicAdd(reinterpret_cast<unsigned long long*>(a.acc + 192), 1ull) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
+  inner_verify_open(a, st);
+}
+
+// g += a b over the 64 factors (a, b in shared memory, 16-byte aligned), 16 at a time.
+__device__ __forceinline__ void gr_mac_row(const u64* a, const u64* b, int l, Gr2& g) {
+#pragma unroll 1
+  for (int i0 = 0; i0 < 64; i0 += 16) gr_mac2<16>(a, b, l, i0, g);
+}
+
+// The same on long claims (few rounds asked for): a warp takes a row, two coefficients a lane.  Bound by
+// the multiply-adds, where the form above, a row a block, is bound by its barriers and by two
+// shared-memory reads for each multiply-add.  Products with an absent (zero) component are left out, as
+// in the Gram sums.
+constexpr int IVL_WARPS = 4;
+__global__ void __launch_bounds__(IVL_WARPS * 32, 5) k_inner_verify_long(const InnerVerify a) {
+  __shared__ __align__(16) u64 al[5][64];               // r1, r2, m of alpha; r_a, m - r2
+  __shared__ __align__(16) u64 U[IVL_WARPS][5][64];     // r_x, m_x (P1), [r]_1, m_x (P2), [r]_2; x' in its place
+  __shared__ __align__(16) u64 V[IVL_WARPS][5][64];     // r_y, m_y (P1), [r]_1, m_y (P2), m_y - [r]_2
+  __shared__ __align__(16) u64 ST[IVL_WARPS][3][64];
+  const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
   if (tid < 24) {
     const int q = tid >> 3;
-    stream64(q == 1 ? a.k02 : a.k01, make_tag(P_VER_DELTA, q == 0 ? C_R1 : q == 1 ? C_R2 : C_G1),
-             a.obj, tid & 7, st[q]);
+    stream64(q == 0 ? a.k01 : q == 1 ? a.k02 : a.k12,
+             make_tag(P_VER_ALPHA, q == 0 ? C_R1 : q == 1 ? C_R2 : C_M12), a.obj, tid & 7, al[q]);
   }
   __syncthreads();
-  if (tid >= 64) return;
-  const u64 r1 = st[0][t], r2 = st[1][t], g1 = st[2][t];
-  const u64 g2 = __ldcg(a.acc + t) + r1 + r2 - g1;                          // P0 -> P2
-  const u64 m = (__ldcg(a.acc + 64 + t) + g1) + (__ldcg(a.acc + 128 + t) + g2);   // P1 <-> P2
-  const u64 r2in = r2 ^ (t == a.fault.idx ? a.fault.mask : 0ull);
-  a.rec[t] = r1;
-  a.rec[64 + t] = r2;
-  a.rec[128 + t] = m;
-  a.rec[192 + t] = r1;
-  a.rec[256 + t] = r2;
-  a.rec[320 + t] = m;
-  a.rec[384 + t] = r2in;
-  const u64 d = m - r1 - r2in;
-  if (a.trace) a.trace[t] = d;
-  if (d != 0ull) atomicOr(a.status, a.flag);
+  if (tid < 64) {
+    al[3][tid] = al[0][tid] + al[1][tid];
+    al[4][tid] = al[2][tid] - al[1][tid];
+  }
+  __syncthreads();
+  grid_dep();   // alpha comes from the keys alone
+  u64(*u)[64] = U[w], (*v)[64] = V[w], (*st)[64] = ST[w];
+  auto get = [&](const u64* src, long long i) {
+    return src ? reinterpret_cast<const ulonglong2*>(src + i * 64)[l] : make_ulonglong2(0, 0);
+  };
+  auto put = [&](u64* dst, u64 x, u64 y) {
+    *reinterpret_cast<ulonglong2*>(dst + 2 * l) = make_ulonglong2(x, y);
+  };
+  Gr2 acc[3];
+  for (long long i = blockIdx.x * (long long)IVL_WARPS + w; i <= a.D; i += (long long)gridDim.x * IVL_WARPS) {
+    const bool row = i < a.D;   // uniform over the warp; the last one is alpha against -z
+    __syncwarp();
+    ulonglong2 y[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      y[c] = row ? get(a.y[c], i) : get(a.z + c * 64, 0);
+      if (!row) y[c] = make_ulonglong2(0ull - y[c].x, 0ull - y[c].y);
+    }
+    put(v[0], y[0].x + y[1].x, y[0].y + y[1].y);
+    put(v[1], y[2].x, y[2].y);
+    put(v[2], y[3].x, y[3].y);
+    put(v[3], y[4].x, y[4].y);
+    put(v[4], y[4].x - y[5].x, y[4].y - y[5].y);
+    if (row) {
+      const ulonglong2 x0 = get(a.x[0], i), x1 = get(a.x[1], i), x2 = get(a.x[2], i), x3 = get(a.x[3], i),
+                       x4 = get(a.x[4], i), x5 = get(a.x[5], i);
+      put(u[0], x0.x + x1.x, x0.y + x1.y);
+      put(u[1], x2.x, x2.y);
+      put(u[2], x3.x, x3.y);
+      put(u[3], x4.x, x4.y);
+      put(u[4], x5.x, x5.y);
+      if (l < 24) {   // masks and [Gamma]_1, words 64 i .. 64 i + 63 of their streams
+        const int q = l >> 3;
+        u64 o[8];
+        prf_block8(q == 1 ? a.k02 : a.k01, make_tag(P_VER_XA, q == 0 ? C_R1 : q == 1 ? C_R2 : C_G1),
+                   a.obj, (u64)i * 8 + (l & 7), o);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) st[q][(l & 7) * 8 + k] = o[k];
+      }
+      __syncwarp();
+      Gr2 g, n;
+      if (a.x[0] || a.x[1]) gr_mac_row(u[0], al[3], l, g);   // P0: r_x r_a
+      if (a.x[4]) gr_mac_row(u[3], al[4], l, g);             // P2: m_x (m_a - [r_a]_2)
+      if (a.x[2]) gr_mac_row(u[1], al[0], l, n);             // P1: -(m_x [r_a]_1 + m_a [r_x]_1)
+      if (a.x[3]) gr_mac_row(u[2], al[2], l, n);
+      if (a.x[5]) gr_mac_row(u[4], al[2], l, n);             // P2: -[r_x]_2 m_a
+      g.sub(n);
+      __syncwarp();
+      put(u[0], g.hi[0], g.hi[1]);
+      __syncwarp();
+      u64 m[2], r1[2], r2[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        // Gamma = r_x r_a + r1 + r2; [m]_1 + [m]_2 takes [Gamma]_1 + (Gamma - [Gamma]_1)
+        r1[h] = st[0][2 * l + h];
+        r2[h] = st[1][2 * l + h];
+        const u64 g1 = st[2][2 * l + h], g2 = r1[h] + r2[h] - g1;
+        m[h] = g.lo[h] - gr_carry_at(u[0], 2 * l + h) + g1 + g2;
+      }
+      __syncwarp();
+      put(u[0], r1[0] + r2[0], r1[1] + r2[1]);
+      put(u[1], m[0], m[1]);
+      put(u[2], r1[0], r1[1]);
+      put(u[3], m[0], m[1]);
+      put(u[4], r2[0], r2[1]);
+    } else {
+      put(u[0], al[3][2 * l], al[3][2 * l + 1]);
+      put(u[1], al[2][2 * l], al[2][2 * l + 1]);
+      put(u[2], al[0][2 * l], al[0][2 * l + 1]);
+      put(u[3], al[2][2 * l], al[2][2 * l + 1]);
+      put(u[4], al[1][2 * l], al[1][2 * l + 1]);
+    }
+    __syncwarp();
+    auto has = [&](int c) { return !row || a.y[c]; };
+    Gr2 n1, n2;
+    if (has(0) || has(1)) gr_mac_row(u[0], v[0], l, acc[0]);
+    if (has(3)) gr_mac_row(u[1], v[2], l, n1);
+    if (has(2)) gr_mac_row(v[1], u[2], l, n1);
+    if (has(4) || has(5)) gr_mac_row(u[3], v[4], l, acc[2]);
+    if (has(4)) gr_mac_row(v[3], u[4], l, n2);
+    acc[1].sub(n1);
+    acc[2].sub(n2);
+  }
+  // the warps' sums: lo in the rows 0 .. 2 of u, hi in those of v
+  __syncwarp();
+  for (int q = 0; q < 3; ++q) {
+    put(u[q], acc[q].lo[0], acc[q].lo[1]);
+    put(v[q], acc[q].hi[0], acc[q].hi[1]);
+  }
+  __syncthreads();
+  for (int e = tid; e < 2 * 192; e += IVL_WARPS * 32) {
+    u64(*X)[5][64] = e < 192 ? U : V;
+    const int q = (e % 192) >> 6, c = e & 63;
+    u64 r = X[0][q][c];
+    for (int k = 1; k < IVL_WARPS; ++k) r += X[k][q][c];
+    X[0][q][c] = r;
+  }
+  __syncthreads();
+  for (int e = tid; e < 192; e += IVL_WARPS * 32)
+    atomicAdd(reinterpret_cast<unsigned long long*>(a.acc + e),
+              (unsigned long long)gr_reduce_at(U[0][e >> 6], V[0][e >> 6], e & 63));
+  inner_verify_open(a, ST[0]);
 }
+
 
 // The hash comparisons of n Pi_Rec calls of single GR elements (one block each): P1 sends H([r]_1)
 // to P2, P2 sends H(m) to P0 and H([r]_2) to P1, and every receiver hashes what it received; a
@@ -576,7 +716,18 @@ void launch_small_round(cudaStream_t st, const SmallRound& a) {
   launch_dep(k_small_round, (unsigned)((n + 1) / 2), 256, 0, st, a);
 }
 
+// Elements from which a claim takes a warp a row.  A verification of 2^16 products, by the elements that
+// are left for this step: 1024: 444 us with a block a row, 465 with a warp; 2048: 422, 420; 4096: 412,
+// 388; of 2^18 products with all of them left 7.50 ms, 6.35; of 2^19 truncations with 2^22 left (two
+// components a side) 122 ms, 57.
+constexpr long long IV_LONG = 2048;
+
 void launch_inner_verify(cudaStream_t st, const InnerVerify& a) {
+  if (a.D >= IV_LONG) {   // up to five blocks an SM
+    const long long g = (a.D + IVL_WARPS) / IVL_WARPS;
+    launch_dep(k_inner_verify_long, (unsigned)(g < 152 * 5 ? g : 152 * 5), IVL_WARPS * 32, 0, st, a);
+    return;
+  }
   const long long n = a.D + 1;   // four blocks an SM at most: rows beyond that are looped over
   launch_dep(k_inner_verify, (unsigned)(n < 608 ? n : 608), 256, 0, st, a);
 }
