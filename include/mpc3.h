@@ -7,8 +7,12 @@
  * batched verification Pi_MultVerify / Pi_BIVerify (Fig. PPEV, Fig. PBDP) built from Pi_Tran
  * (Fig. MTP), Pi_Reduce (Fig. Reduce) and Pi_InnerVerify (Fig. DPV) over GR(2^64, 64), and
  * Pi_Rec (Sec. 2).  All three parties P0, P1, P2 are simulated on one GPU: each holds its own
- * device copy of every share it owns, and every protocol message is a device-to-device copy that
- * is counted in a ledger.
+ * device copy of every share it owns.  A message of Pi_Mult, Pi_Inner and Pi_Trunc is handed to its
+ * receiver in place, and where one kernel runs both sides (the comparison's gates, the verification's
+ * single elements) it stays in registers; input sharing, Pi_Rec of a sharing and the openings of the
+ * verification over GR(2^64, 64) write what the receivers get.  A message that an injected fault
+ * corrupts is copied first, so that its sender keeps the honest one.  A ledger counts every message's
+ * bytes, moved or not.
  *
  * Conventions
  *   - All values are uint64_t, i.e. elements of Z_2^64; arithmetic wraps mod 2^64.

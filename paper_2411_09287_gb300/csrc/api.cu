@@ -263,14 +263,28 @@ int deliver_copy(mpc_ctx* ctx, int phase, int proto, const u64* src, u64* dst, l
   return MPC_OK;
 }
 
-// The message src to a receiver that only reads it: it is handed over in place (dst becomes src), and
-// copied only to be corrupted by a fault.  A copy of a small message is a launch of 4 us.
-int deliver(mpc_ctx* ctx, int phase, int proto, u64* src, u64*& dst, long long n, int site) {
+// The message src to a receiver that only reads it is handed over in place (a copy of a small message
+// is a launch of 4 us); one that a fault corrupts is copied first, into `copy` (n words).  dst: what the
+// receiver reads.
+int deliver(mpc_ctx* ctx, int phase, int proto, const u64* src, const u64*& dst, long long n, int site,
+            u64* copy) {
   const MsgFault f = take_fault(ctx, site, n);
-  if (f.idx >= 0) return deliver_copy(ctx, phase, proto, src, dst, n, f);
+  dst = f.idx < 0 ? src : copy;
+  if (f.idx >= 0) return deliver_copy(ctx, phase, proto, src, copy, n, f);
   count_msgs(ctx, phase, proto, 1, (u64)n * 8);
-  dst = src;
   return MPC_OK;
+}
+
+// Room for the messages of a call that faults corrupt, at most one a site (a fault fires once).
+struct FaultCopies {
+  u64 *g2, *mz1, *mz2;   // GAMMA2 (HIGH_BIT), MZ1, MZ2
+};
+FaultCopies plan_copies(Arena& a, long long n) {
+  FaultCopies c;
+  c.g2 = a.take<u64>(n);
+  c.mz1 = a.take<u64>(n);
+  c.mz2 = a.take<u64>(n);
+  return c;
 }
 
 int read_status(mpc_ctx* ctx, u32* out) {
@@ -831,8 +845,9 @@ int finish_verify(mpc_ctx* ctx, u64 pend_key) {
 
 // ---- plans ----------------------------------------------------------------------------------
 struct MatmulPlan {
-  u64 *g2o, *g2i, *mz1, *mz2, *mz1i, *mz2i;
-  u64 *gp2, *gq2, *gp2i, *gq2i, *mp1, *mq1, *mpi1, *mqi1, *mpi2, *mqi2;
+  u64 *g2, *mz1, *mz2;             // the product's messages
+  u64 *gp2, *gq2, *mp1, *mq1;      // the truncation pairs' messages
+  FaultCopies fc;
   void* tc;   // digit planes of the tensor-core path (null on the u64 path)
 };
 
@@ -840,16 +855,12 @@ MatmulPlan plan_matmul(Arena& a, long long M, long long N, long long K, bool tru
   const long long E = M * N;
   MatmulPlan p{};
   p.tc = tc ? (void*)a.take<unsigned char>((long long)limb_tc_scratch_bytes(M, N, K, 2)) : nullptr;
-  p.g2o = a.take<u64>(E); p.g2i = a.take<u64>(E);
-  p.mz1 = a.take<u64>(E); p.mz2 = a.take<u64>(E);
-  p.mz1i = a.take<u64>(E); p.mz2i = a.take<u64>(E);
-  if (trunc) {
-    p.gp2 = a.take<u64>(E); p.gq2 = a.take<u64>(E);
-    p.gp2i = a.take<u64>(E); p.gq2i = a.take<u64>(E);
-    p.mp1 = a.take<u64>(E); p.mq1 = a.take<u64>(E);
-    p.mpi1 = a.take<u64>(E); p.mqi1 = a.take<u64>(E);
-    p.mpi2 = a.take<u64>(E); p.mqi2 = a.take<u64>(E);
-  }
+  p.g2 = a.take<u64>(E);
+  p.mz1 = a.take<u64>(E);
+  p.mz2 = a.take<u64>(E);
+  if (trunc)
+    for (u64** b : {&p.gp2, &p.gq2, &p.mp1, &p.mq1}) *b = a.take<u64>(E);
+  p.fc = plan_copies(a, E);
   return p;
 }
 
@@ -1591,11 +1602,30 @@ int verify_trunc_chunk(mpc_ctx* ctx, TruncPlan& p, const Small& s, void* tcs, co
   return bit_batch(ctx, p, s, z0, verify_id, batch, tr);
 }
 
+// The messages of the truncation pairs' two inner products (Fig. trunc), as their receivers read them.
+struct PairMsgs {
+  const u64 *gp2, *gq2;             // P2: [Gamma]_2
+  const u64 *mp1, *mq1, *mp2, *mq2; // P1: from P2; P2: from P1
+};
+int deliver_pairs(mpc_ctx* ctx, const u64* gp2, const u64* gq2, const u64* mp1, const u64* mq1, long long n,
+                  const FaultCopies& fc, PairMsgs& m) {
+  const int ph = MPC_PHASE_OFFLINE, pr = MPC_PROTO_TRUNC;
+  int rc;
+  if ((rc = deliver(ctx, ph, pr, gp2, m.gp2, n, MPC_SITE_GAMMA2, fc.g2))) return rc;
+  if ((rc = deliver(ctx, ph, pr, mp1, m.mp2, n, MPC_SITE_MZ1, fc.mz1))) return rc;
+  if ((rc = deliver(ctx, ph, pr, m.gp2, m.mp1, n, MPC_SITE_MZ2, fc.mz2))) return rc;
+  if ((rc = deliver(ctx, ph, pr, gq2, m.gq2, n, MPC_SITE_GAMMA2, fc.g2))) return rc;
+  if ((rc = deliver(ctx, ph, pr, mq1, m.mq2, n, MPC_SITE_MZ1, fc.mz1))) return rc;
+  return deliver(ctx, ph, pr, m.gq2, m.mq1, n, MPC_SITE_MZ2, fc.mz2);
+}
+
 // workspace of a standalone truncation (mpc_trunc)
 struct TruncCallPlan {
   u64* rx;   // 6n: the pairs' r_x shares in the mask components
-  u64 *gp2, *gq2, *gp2i, *gq2i, *mp1, *mq1, *mpi1, *mqi1, *mpi2, *mqi2;   // pair messages
-  u64 *d1, *d2, *d1p0, *d2p0, *d1_at_p2, *d2_at_p1;                      // mask switch
+  u64 *gp2, *gq2, *mp1, *mq1;      // pair messages
+  u64 *d1, *d2, *d1p0, *d2p0;      // mask switch
+  FaultCopies fc;
+  u64* d1x;                        // d1 as a fault corrupts it
   u32* hs[4];
   u32* dg;   // 4 x 8 digest words
 };
@@ -1603,9 +1633,9 @@ struct TruncCallPlan {
 TruncCallPlan plan_trunc_call(Arena& a, long long n) {
   TruncCallPlan p;
   p.rx = a.take<u64>(6 * n);
-  u64** bufs[] = {&p.gp2, &p.gq2, &p.gp2i, &p.gq2i, &p.mp1, &p.mq1, &p.mpi1, &p.mqi1, &p.mpi2,
-                  &p.mqi2, &p.d1, &p.d2, &p.d1p0, &p.d2p0, &p.d1_at_p2, &p.d2_at_p1};
-  for (u64** b : bufs) *b = a.take<u64>(n);
+  for (u64** b : {&p.gp2, &p.gq2, &p.mp1, &p.mq1, &p.d1, &p.d2, &p.d1p0, &p.d2p0, &p.d1x})
+    *b = a.take<u64>(n);
+  p.fc = plan_copies(a, n);
   for (int i = 0; i < 4; ++i) p.hs[i] = a.take<u32>((long long)hash_scratch_words(n));
   p.dg = a.take<u32>(32);
   return p;
@@ -1992,21 +2022,20 @@ int mpc_mult(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const uint64_t*
   if (n <= 0) return fail(ctx, MPC_ERR_SHAPE, "mult: n <= 0");
   if (!xs || !ys || !zs || !id_ok(call_id)) return fail(ctx, MPC_ERR_ARG, "mult: bad argument");
   Arena ar{(char*)workspace, workspace_bytes, 0, false};
-  u64* g2o = ar.take<u64>(n);
-  u64* g2i = ar.take<u64>(n);
-  u64* p1o = ar.take<u64>(n);
-  u64* p2o = ar.take<u64>(n);
-  u64* p1i = ar.take<u64>(n);
-  u64* p2i = ar.take<u64>(n);
+  u64* g2 = ar.take<u64>(n);
+  u64* p1 = ar.take<u64>(n);
+  u64* p2 = ar.take<u64>(n);
+  const FaultCopies fc = plan_copies(ar, n);
   if (!workspace || !ar.ok()) return fail(ctx, MPC_ERR_WORKSPACE, "mult: workspace too small");
   Phase phase(ctx, MPC_PROF_MULT);
   const u64 obj = make_obj(call_id, 0, 0);
-  launch_mult_offline(ctx->st, xs, ys, n, ctx->k01, ctx->k02, obj, zs, g2o);
-  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_MULT, g2o, g2i, n, MPC_SITE_GAMMA2))) return rc;
-  launch_mult_online(ctx->st, xs, ys, n, ctx->k01, obj, g2i, p1o, p2o);
-  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, p1o, p2i, n, MPC_SITE_MZ1))) return rc;
-  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, p2o, p1i, n, MPC_SITE_MZ2))) return rc;
-  launch_exchange_finish(ctx->st, n, p1o, p1i, p2o, p2i, zs, -1, nullptr);
+  const u64 *g2_at_p2, *p1_at_p2, *p2_at_p1;
+  launch_mult_offline(ctx->st, xs, ys, n, ctx->k01, ctx->k02, obj, zs, g2);
+  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_MULT, g2, g2_at_p2, n, MPC_SITE_GAMMA2, fc.g2))) return rc;
+  launch_mult_online(ctx->st, xs, ys, n, ctx->k01, obj, g2_at_p2, p1, p2);
+  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, p1, p1_at_p2, n, MPC_SITE_MZ1, fc.mz1))) return rc;
+  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, p2, p2_at_p1, n, MPC_SITE_MZ2, fc.mz2))) return rc;
+  launch_exchange_finish(ctx->st, n, p1, p2_at_p1, p2, p1_at_p2, zs, -1, nullptr);
   ctx->pending.insert((call_id << 1) | 0);
   return cuda_check(ctx, "mult");
 }
@@ -2057,15 +2086,10 @@ int mpc_matmul_keyed(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const u
     Phase phase(ctx, MPC_PROF_TRUNC_PAIRS);
     launch_trunc_p0(st, E, ctx->k01, ctx->k02, obj, trunc_bits, zpre, zout, pq, p.gp2, p.gq2,
                     p.mp1, p.mq1, (const u64*)row_keys, N);
-    const int ph = MPC_PHASE_OFFLINE, pr = MPC_PROTO_TRUNC;
-    if ((rc = deliver(ctx, ph, pr, p.gp2, p.gp2i, E, MPC_SITE_GAMMA2))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.mp1, p.mpi2, E, MPC_SITE_MZ1))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.gp2i, p.mpi1, E, MPC_SITE_MZ2))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.gq2, p.gq2i, E, MPC_SITE_GAMMA2))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.mq1, p.mqi2, E, MPC_SITE_MZ1))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.gq2i, p.mqi1, E, MPC_SITE_MZ2))) return rc;
-    launch_trunc_finish(st, E, ctx->k01, ctx->k02, obj, trunc_bits, p.mpi1, p.mqi1, p.mpi2,
-                        p.mqi2, p.gp2i, p.gq2i, p.mp1, p.mq1, zpre, zout, pq, (const u64*)row_keys, N);
+    PairMsgs m;
+    if ((rc = deliver_pairs(ctx, p.gp2, p.gq2, p.mp1, p.mq1, E, p.fc, m))) return rc;
+    launch_trunc_finish(st, E, ctx->k01, ctx->k02, obj, trunc_bits, m.mp1, m.mq1, m.mp2, m.mq2, m.gp2,
+                        m.gq2, p.mp1, p.mq1, zpre, zout, pq, (const u64*)row_keys, N);
   } else {
     launch_fill_masks(st, E, ctx->k01, ctx->k02, P_INNER, obj, zpre);
   }
@@ -2077,7 +2101,7 @@ int mpc_matmul_keyed(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const u
     GemmTerm T;
     T.A = op(X, K, 0, X + MK, 1);
     T.B = op(W, N, 0, W + KN, 1);
-    Epi e = epi_store(p.g2o, N);
+    Epi e = epi_store(p.g2, N);
     e.add0 = zpre;
     e.add1 = zpre + E;
     e.prf_sign = M1;
@@ -2086,7 +2110,8 @@ int mpc_matmul_keyed(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const u
     e.obj = obj;
     if ((rc = party_gemm(1, &T, e))) return rc;
   }
-  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_INNER, p.g2o, p.g2i, E, MPC_SITE_GAMMA2)))
+  const u64 *g2_at_p2, *mz1_at_p2, *mz2_at_p1;
+  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_INNER, p.g2, g2_at_p2, E, MPC_SITE_GAMMA2, p.fc.g2)))
     return rc;
   {  // P1, online: [m_Z]_1 = -(M_X [R_W]_1 + [R_X]_1 M_W) + [Gamma]_1
     Phase phase(ctx, MPC_PROF_GEMM);
@@ -2111,16 +2136,16 @@ int mpc_matmul_keyed(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const u
     T[1].A = op(X + 5 * MK, K, 0, nullptr, 1, M1);
     T[1].B = op(W + 4 * KN, N);
     Epi e = epi_store(p.mz2, N);
-    e.add0 = p.g2i;
+    e.add0 = g2_at_p2;
     if ((rc = party_gemm(2, T, e))) return rc;
   }
   {
     Phase phase(ctx, MPC_PROF_EXCHANGE);
-    if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_INNER, p.mz1, p.mz1i, E, MPC_SITE_MZ1)))
+    if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_INNER, p.mz1, mz1_at_p2, E, MPC_SITE_MZ1, p.fc.mz1)))
       return rc;
-    if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_INNER, p.mz2, p.mz2i, E, MPC_SITE_MZ2)))
+    if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_INNER, p.mz2, mz2_at_p1, E, MPC_SITE_MZ2, p.fc.mz2)))
       return rc;
-    launch_exchange_finish(st, E, p.mz1, p.mz2i, p.mz2, p.mz1i, zpre, trunc_bits,
+    launch_exchange_finish(st, E, p.mz1, mz2_at_p1, p.mz2, mz1_at_p2, zpre, trunc_bits,
                            trunc ? zout : nullptr);
   }
   if (!trunc && zout && zout != zpre)
@@ -2479,24 +2504,20 @@ int mpc_trunc(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, int64_t n, int
     Phase phase(ctx, MPC_PROF_TRUNC_PAIRS);
     launch_trunc_p0(st, n, ctx->k01, ctx->k02, obj, t, p.rx, out, pq, p.gp2, p.gq2, p.mp1, p.mq1,
                     nullptr, n);
-    const int ph = MPC_PHASE_OFFLINE, pr = MPC_PROTO_TRUNC;
-    if ((rc = deliver(ctx, ph, pr, p.gp2, p.gp2i, n, MPC_SITE_GAMMA2))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.mp1, p.mpi2, n, MPC_SITE_MZ1))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.gp2i, p.mpi1, n, MPC_SITE_MZ2))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.gq2, p.gq2i, n, MPC_SITE_GAMMA2))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.mq1, p.mqi2, n, MPC_SITE_MZ1))) return rc;
-    if ((rc = deliver(ctx, ph, pr, p.gq2i, p.mqi1, n, MPC_SITE_MZ2))) return rc;
-    launch_trunc_finish(st, n, ctx->k01, ctx->k02, obj, t, p.mpi1, p.mqi1, p.mpi2, p.mqi2,
-                        p.gp2i, p.gq2i, p.mp1, p.mq1, p.rx, out, pq, nullptr, n);
+    PairMsgs m;
+    if ((rc = deliver_pairs(ctx, p.gp2, p.gq2, p.mp1, p.mq1, n, p.fc, m))) return rc;
+    launch_trunc_finish(st, n, ctx->k01, ctx->k02, obj, t, m.mp1, m.mq1, m.mp2, m.mq2, m.gp2, m.gq2, p.mp1,
+                        p.mq1, p.rx, out, pq, nullptr, n);
   }
   {  // online: the wire's mask switched to the pairs' r_x (checked by P0's hashes), then m >> t
     Phase phase(ctx, MPC_PROF_EXCHANGE);
     launch_trunc_remask(st, xs, p.rx, n, p.d1, p.d2, p.d1p0, p.d2p0);
     const int ph = MPC_PHASE_ONLINE, pr = MPC_PROTO_TRUNC;
-    if ((rc = deliver(ctx, ph, pr, p.d1, p.d1_at_p2, n, MPC_SITE_TRUNC_D1))) return rc;   // P1->P2
-    if ((rc = deliver(ctx, ph, pr, p.d2, p.d2_at_p1, n, -1))) return rc;                 // P2->P1
+    const u64 *d1_at_p2, *d2_at_p1;
+    if ((rc = deliver(ctx, ph, pr, p.d1, d1_at_p2, n, MPC_SITE_TRUNC_D1, p.d1x))) return rc;   // P1->P2
+    if ((rc = deliver(ctx, ph, pr, p.d2, d2_at_p1, n, -1, nullptr))) return rc;               // P2->P1
     // P0 sends H(d1) to P2 and H(d2) to P1, who hash the d1, d2 they received
-    const u64* data[4] = {p.d1p0, p.d2p0, p.d1_at_p2, p.d2_at_p1};
+    const u64* data[4] = {p.d1p0, p.d2p0, d1_at_p2, d2_at_p1};
     HashJobs hj{};
     for (int q = 0; q < 4; ++q) {
       hj.data[q] = data[q];
@@ -2507,7 +2528,7 @@ int mpc_trunc(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, int64_t n, int
     count_msgs(ctx, ph, pr, 2, 32);
     launch_digest_check(st, p.dg, p.dg + 16, p.dg + 8, p.dg + 24, p.dg, p.dg + 16, ctx->status,
                         ST_ABORT);
-    launch_trunc_online(st, xs, n, p.d1, p.d2_at_p1, p.d1_at_p2, p.d2, t, out);
+    launch_trunc_online(st, xs, n, p.d1, d2_at_p1, d1_at_p2, p.d2, t, out);
   }
   if ((rc = cuda_check(ctx, "trunc"))) return rc;
   ctx->pending.insert((call_id << 1) | 1);

@@ -17,6 +17,28 @@ def test_block_batch_reserves_its_digit_planes():
     assert "blk_sums_tc_bytes(" in body
 
 
+def test_message_buffers_of_a_product():
+    """A product plans its messages (three, and four of the truncation pairs) and one copy a fault site,
+    not a received copy of every message; a standalone truncation likewise."""
+    import ctypes as C
+
+    from paper_2411_09287_gb300 import build
+    if not os.path.exists(build.LIB):
+        try:
+            build.build()
+        except RuntimeError as e:      # no toolkit on this host
+            pytest.skip(str(e))
+    lib = C.CDLL(build.LIB)
+    size = lib.mpc_workspace_size
+    size.restype = C.c_int64
+    size.argtypes = [C.c_void_p, C.c_int] + [C.c_int64] * 3 + [C.c_int] * 3
+    OP_MATMUL, OP_TRUNC = 2, 11
+    E = 300 * 700
+    assert size(None, OP_MATMUL, 300, 700, 50, 13, -1, -1) <= 8 * E * (3 + 4 + 3) + 10 * 256
+    assert size(None, OP_MATMUL, 300, 700, 50, -1, -1, -1) <= 8 * E * (3 + 3) + 6 * 256
+    assert size(None, OP_TRUNC, E, 0, 0, -1, -1, -1) <= 8 * E * (6 + 4 + 4 + 4) + E   # and the hash trees
+
+
 @pytest.fixture(scope="module")
 def mpc():
     torch = pytest.importorskip("torch")
