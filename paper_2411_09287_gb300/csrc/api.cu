@@ -28,8 +28,8 @@ constexpr u32 ST_VERIFY = 2u;   // Delta != 0
 constexpr u32 ST_TIMEOUT = 4u;  // a bounded device wait expired
 
 // device constants block (words)
-constexpr int CST_INV = 0;      // 192: x^-1, (1-x)^-1, (x(x-1))^-1
-constexpr int CST_WORDS = 192;
+constexpr int CST_INV = 0;      // 64: (x(x-1))^-1
+constexpr int CST_WORDS = 64;
 
 constexpr int TRACE_ROUND = 832;  // words per round in a verification trace
 
@@ -544,7 +544,7 @@ void round_tail(mpc_ctx* ctx, u64 vid, u32 batch, int k, const u64* z, u64* zo, 
   a.k02 = ctx->k02;
   a.k12 = ctx->k12;
   a.obj = make_obj(vid, batch, (u32)k);
-  a.inv = ctx->cst + CST_INV + 128;
+  a.inv = ctx->cst + CST_INV;
   a.z = z;
   a.zo = zo;
   a.coef = s.coef;
@@ -1714,7 +1714,7 @@ int mpc_create(const mpc_config* cfg, mpc_ctx** out) {
   Key master;
   std::memcpy(master.k, cfg->seed, 32);
   launch_dep(k_derive_keys, 1, 32, 0, ctx->st, master, keys_dev);
-  launch_gr_inverses(ctx->st, ctx->cst + CST_INV);
+  launch_gr_inverse(ctx->st, ctx->cst + CST_INV);
   e = cudaMemsetAsync(ctx->status, 0, sizeof(u32), ctx->st);
   if (e != cudaSuccess) return bail("cudaMemset", e);
   u32 kh[24];

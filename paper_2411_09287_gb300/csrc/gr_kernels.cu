@@ -154,7 +154,7 @@ __global__ void k_block_rowsum(long long nper, const u64* in, u64* __restrict__ 
   out[c * 64 + threadIdx.x] = v;
 }
 
-// ---- inverses of the interpolation constants (Pi_Reduce with points 0, 1, x) ------------------
+// ---- inverse of the interpolation constant (Pi_Reduce with points 0, 1, x) --------------------
 __device__ u64 gf2_64_mul(u64 a, u64 b) {   // GF(2)[x]/(x^64 + x^4 + x^3 + x + 1)
   u64 r = 0;
   for (int i = 63; i >= 0; --i) {
@@ -165,43 +165,35 @@ __device__ u64 gf2_64_mul(u64 a, u64 b) {   // GF(2)[x]/(x^64 + x^4 + x^3 + x + 
   return r;
 }
 
-// out[0..63] = x^-1, out[64..127] = (1 - x)^-1, out[128..191] = (x (x - 1))^-1.
-// GF(2^64) inverse a^(2^64 - 2) of the residue, then Newton steps y <- y (2 - a y).
-__global__ void k_gr_inverses(u64* out) {
+// out = (x (x - 1))^-1: the GF(2^64) inverse a^(2^64 - 2) of the residue, then Newton steps
+// y <- y (2 - a y).
+__global__ void k_gr_inverse(u64* out) {
   grid_dep();
   __shared__ u64 a[64], y[64], t1[64], scr[128];
   __shared__ u64 ybits;
   const int t = threadIdx.x;
-  for (int which = 0; which < 3; ++which) {
-    // a = x, 1 - x, x^2 - x
-    u64 v = 0;
-    if (which == 0) v = (t == 1) ? 1ull : 0ull;
-    if (which == 1) v = (t == 0) ? 1ull : ((t == 1) ? ~0ull : 0ull);
-    if (which == 2) v = (t == 2) ? 1ull : ((t == 1) ? ~0ull : 0ull);
-    a[t] = v;
-    __syncthreads();
-    if (t == 0) {
-      u64 bits = 0;
-      for (int c = 0; c < 64; ++c) bits |= (a[c] & 1ull) << c;
-      u64 acc = 1, p = bits;
-      for (int k = 1; k < 64; ++k) {
-        p = gf2_64_mul(p, p);
-        acc = gf2_64_mul(acc, p);
-      }
-      ybits = acc;
+  a[t] = t == 2 ? 1ull : t == 1 ? ~0ull : 0ull;   // x^2 - x
+  __syncthreads();
+  if (t == 0) {
+    u64 bits = 0;
+    for (int c = 0; c < 64; ++c) bits |= (a[c] & 1ull) << c;
+    u64 acc = 1, p = bits;
+    for (int k = 1; k < 64; ++k) {
+      p = gf2_64_mul(p, p);
+      acc = gf2_64_mul(acc, p);
     }
-    __syncthreads();
-    y[t] = (ybits >> t) & 1ull;
-    __syncthreads();
-    for (int it = 0; it < 7; ++it) {
-      gr_mul_block(a, y, t1, scr);            // t1 = a y
-      t1[t] = ((t == 0) ? 2ull : 0ull) - t1[t];
-      __syncthreads();
-      gr_mul_block(y, t1, y, scr);            // y = y (2 - a y)
-    }
-    out[which * 64 + t] = y[t];
-    __syncthreads();
+    ybits = acc;
   }
+  __syncthreads();
+  y[t] = (ybits >> t) & 1ull;
+  __syncthreads();
+  for (int it = 0; it < 7; ++it) {
+    gr_mul_block(a, y, t1, scr);            // t1 = a y
+    t1[t] = ((t == 0) ? 2ull : 0ull) - t1[t];
+    __syncthreads();
+    gr_mul_block(y, t1, y, scr);            // y = y (2 - a y)
+  }
+  out[t] = y[t];
 }
 
 // ---- fold of Gram sums ------------------------------------------------------------------------
@@ -483,7 +475,7 @@ void launch_sum_blocks(cudaStream_t st, long long m, long long n, long long ld, 
   launch_dep(k_sum_blocks, (unsigned)((m + 255) / 256), 256, 0, st, m, n, ld, in, out);
 }
 
-void launch_gr_inverses(cudaStream_t st, u64* out) { launch_dep(k_gr_inverses, 1, 64, 0, st, out); }
+void launch_gr_inverse(cudaStream_t st, u64* out) { launch_dep(k_gr_inverse, 1, 64, 0, st, out); }
 
 void launch_gr_fold_reduce(cudaStream_t st, const u64* P, int n, u64* out) {
   if (n <= 0) return;

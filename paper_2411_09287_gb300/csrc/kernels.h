@@ -280,7 +280,8 @@ void launch_gr_powers(cudaStream_t st, const u64* a, long long n, u64* table);
 void launch_gr_mul1(cudaStream_t st, const u64* a, const u64* b, u64* out);
 // out_c = a_c + r b_c for n GR elements (rows of 64 words)
 void launch_gr_axpy(cudaStream_t st, int n, const u64* r, const u64* a, const u64* b, u64* out);
-void launch_gr_inverses(cudaStream_t st, u64* out);
+// out = (x (x - 1))^-1, the constant of the Lagrange weights at the points 0, 1, x
+void launch_gr_inverse(cudaStream_t st, u64* out);
 void launch_gr_fold_reduce(cudaStream_t st, const u64* P, int n, u64* out);
 void launch_neg_copy(cudaStream_t st, const u64* a, long long n, u64* out);
 void launch_trunc_u(cudaStream_t st, const u64* r, int t, u64* u);
