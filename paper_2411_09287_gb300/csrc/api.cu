@@ -190,8 +190,7 @@ struct Phase {
 // atomic OR) and the inputs, so they run on streams of their own: on(i) sends what follows to side
 // stream i (i < 0: the context's own), after everything before the fork; join() (or the end of the
 // scope) makes the context's stream wait for all of them, so that a call leaves nothing running that
-// its stream does not cover.  Recorded by a stream capture like any fork and join.  With phase timers
-// on, everything stays on the one stream.
+// its stream does not cover.  With phase timers on, everything stays on the one stream.
 struct Fork {
   mpc_ctx* c;
   cudaStream_t main;
@@ -515,8 +514,8 @@ void reveal(mpc_ctx* ctx, u32 purpose, u64 obj, const Small& s, u64* out) {
   launch_reveal(ctx->st, ctx->k01, ctx->k02, ctx->k12, purpose, obj, r.fault, out, r.rec);
 }
 
-// Clears both halves of the round sums and Pi_InnerVerify's; a round adds into cur_sums, and its tail clears the other
-// half for the next round.
+// Clears both halves of the round sums and Pi_InnerVerify's; a round adds into cur_sums, and its tail
+// clears the other half for the next round.
 int sums_begin(mpc_ctx* ctx, const Small& s) {
   s.uc = 0;
   CK(cudaMemsetAsync(s.U, 0, (2 * SUMS_WORDS + IV_ACC_WORDS) * 8, ctx->st));
@@ -1401,7 +1400,7 @@ int bit_batch(mpc_ctx* ctx, TruncPlan& p, const Small& s, const u64* z0, u64 ver
   int rc;
   Phase* phase = new Phase(ctx, MPC_PROF_TRUNC_S);
   {  // S_{j,j'} = sum_e rho^e b1_{e,j} b2_{e,j'} (P0), with rho^e = rho^(L e_hi) rho^e_lo:
-     // tensor cores for the inner sums over e_lo, then sum_{e_hi} T_hi (x) S_hi as a GEMM + fold
+     // tensor cores for the inner sums over e_lo, then sum_{e_hi} T_hi S_hi
     launch_trunc_limb_table(st, p.Rtab, p.L, p.TL8);
     launch_trunc_bit_transpose(st, p.b1, p.Epad, p.B1T);
     launch_trunc_bit_transpose(st, p.b2, p.Epad, p.B2T);
@@ -2031,10 +2030,11 @@ int mpc_mult(mpc_ctx* ctx, uint64_t call_id, const uint64_t* xs, const uint64_t*
   const u64 obj = make_obj(call_id, 0, 0);
   const u64 *g2_at_p2, *p1_at_p2, *p2_at_p1;
   launch_mult_offline(ctx->st, xs, ys, n, ctx->k01, ctx->k02, obj, zs, g2);
-  if ((rc = deliver(ctx, MPC_PHASE_OFFLINE, MPC_PROTO_MULT, g2, g2_at_p2, n, MPC_SITE_GAMMA2, fc.g2))) return rc;
+  const int off = MPC_PHASE_OFFLINE, on = MPC_PHASE_ONLINE, pr = MPC_PROTO_MULT;
+  if ((rc = deliver(ctx, off, pr, g2, g2_at_p2, n, MPC_SITE_GAMMA2, fc.g2))) return rc;
   launch_mult_online(ctx->st, xs, ys, n, ctx->k01, obj, g2_at_p2, p1, p2);
-  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, p1, p1_at_p2, n, MPC_SITE_MZ1, fc.mz1))) return rc;
-  if ((rc = deliver(ctx, MPC_PHASE_ONLINE, MPC_PROTO_MULT, p2, p2_at_p1, n, MPC_SITE_MZ2, fc.mz2))) return rc;
+  if ((rc = deliver(ctx, on, pr, p1, p1_at_p2, n, MPC_SITE_MZ1, fc.mz1))) return rc;
+  if ((rc = deliver(ctx, on, pr, p2, p2_at_p1, n, MPC_SITE_MZ2, fc.mz2))) return rc;
   launch_exchange_finish(ctx->st, n, p1, p2_at_p1, p2, p1_at_p2, zs, -1, nullptr);
   ctx->pending.insert((call_id << 1) | 0);
   return cuda_check(ctx, "mult");
@@ -2278,10 +2278,12 @@ int mpc_verify_matmul_keyed(mpc_ctx* ctx, uint64_t verify_id, const uint64_t* xs
     GemmTerm T;
     T.A = op(xs, K, 1);
     T.B = op(p.P, 64);
-    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, M, T, epi_store(x.c[0], 64), p.tcs, {K + 1, K, MK}))) return rc;
+    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, M, T, epi_store(x.c[0], 64), p.tcs, {K + 1, K, MK})))
+      return rc;
     T.A = op(ws_, N);
     T.B = op(p.Q, 64);
-    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, N, T, epi_store(y.c[0], 64), p.tcs, {K + 1, K, KN}))) return rc;
+    if ((rc = dense_gemm(ctx, 6 * (K + 1), 64, N, T, epi_store(y.c[0], 64), p.tcs, {K + 1, K, KN})))
+      return rc;
   }
   for (int c = 0; c < 6 && !p.grouped; ++c) {
     GemmTerm T;

@@ -45,7 +45,8 @@ __global__ void __launch_bounds__(TPB) k_cs_bits(const CompareSelect a) {
   u64* out = da ? a.da[q] : a.eda[q];
   const Key& key = q == 0 ? a.k01 : q == 1 ? a.k02 : a.k12;
   const u32 tag = make_tag(da ? P_DABIT : P_EDABIT, q == 0 ? C_R1 : q == 1 ? C_R2 : C_M12);
-  for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < n; b += (long long)gridDim.x * TPB) {
+  const long long stride = (long long)gridDim.x * TPB;
+  for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < n; b += stride) {
     u64 w[8];
     prf_block8(key, tag, a.obj, (u64)b, w);
 #pragma unroll
@@ -64,7 +65,8 @@ __global__ void __launch_bounds__(TPB) k_cs_products(const CompareSelect a) {
     prf_block8(a.k02, make_tag(P_EDA_MULT, C_R2), a.obj, (u64)b, r2);
     prf_block8(a.k01, make_tag(P_EDA_MULT, C_G1), a.obj, (u64)b, g1);
     const long long j0 = b * 8;
-    const unsigned b1 = (unsigned)(a.eda[0][j0 >> 6] >> (j0 & 63)), b2 = (unsigned)(a.eda[1][j0 >> 6] >> (j0 & 63));
+    const unsigned b1 = (unsigned)(a.eda[0][j0 >> 6] >> (j0 & 63));
+    const unsigned b2 = (unsigned)(a.eda[1][j0 >> 6] >> (j0 & 63));
     u64 z[6][8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -154,11 +156,12 @@ __global__ void __launch_bounds__(TPB) k_cs_inner(const CompareSelect a) {
 // The daBits: t = b1 b2, r' = b1 + b2 - 2 t, u = r' b3, r = r' + b3 - 2 u, and the first two triples.
 __global__ void __launch_bounds__(TPB) k_cs_dabits(const CompareSelect a) {
   grid_dep();
-  const long long np = a.np, nm = a.nm;
-  for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < np; b += (long long)gridDim.x * TPB) {
+  const long long np = a.np, nm = a.nm, stride = (long long)gridDim.x * TPB;
+  for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < np; b += stride) {
     const long long e0 = b * 8;
-    const unsigned b1 = (unsigned)(a.da[0][e0 >> 6] >> (e0 & 63)), b2 = (unsigned)(a.da[1][e0 >> 6] >> (e0 & 63)),
-                   b3 = (unsigned)(a.da[2][e0 >> 6] >> (e0 & 63));
+    const unsigned b1 = (unsigned)(a.da[0][e0 >> 6] >> (e0 & 63));
+    const unsigned b2 = (unsigned)(a.da[1][e0 >> 6] >> (e0 & 63));
+    const unsigned b3 = (unsigned)(a.da[2][e0 >> 6] >> (e0 & 63));
     u64 r1[8], r2[8], g1[8], t[6][8];
     prf_block8(a.k01, make_tag(P_DA_MULT1, C_R1), a.obj, (u64)b, r1);
     prf_block8(a.k02, make_tag(P_DA_MULT1, C_R2), a.obj, (u64)b, r2);
@@ -279,8 +282,8 @@ __global__ void __launch_bounds__(TPB) k_cs_msb(const CompareSelect a) {
 // B2A of e (opened: dbits) and the selection out = b + d [a >= b], with the third triple.
 __global__ void __launch_bounds__(TPB) k_cs_select(const CompareSelect a) {
   grid_dep();
-  const long long np = a.np, nm = a.nm;
-  for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < np; b += (long long)gridDim.x * TPB) {
+  const long long np = a.np, nm = a.nm, stride = (long long)gridDim.x * TPB;
+  for (long long b = blockIdx.x * (long long)TPB + threadIdx.x; b * 8 < np; b += stride) {
     const long long e0 = b * 8;
     const unsigned bits = (unsigned)(a.dbits[e0 >> 6] >> (e0 & 63));
     u64 r1[8], r2[8], g1[8];

@@ -219,15 +219,18 @@ void gemm_u64(cudaStream_t st, long long M, long long N, long long K, int nterms
   if (M <= 64 && N <= 64) {   // Gram sums (64 x 64 outputs, long K)
     constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4;
     dim3 grid(1, 1, (unsigned)nsplit);
-    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, nterms, terms[0], t1, epi, kps);
+    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K,
+               nterms, terms[0], t1, epi, kps);
   } else if (N <= 64) {
     constexpr int BM = 128, BN = 64, BK = 8, TM = 8, TN = 4;
     dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)nsplit);
-    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, nterms, terms[0], t1, epi, kps);
+    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K,
+               nterms, terms[0], t1, epi, kps);
   } else {
     constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
     dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)nsplit);
-    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, nterms, terms[0], t1, epi, kps);
+    launch_dep(gemm_u64_kernel<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K,
+               nterms, terms[0], t1, epi, kps);
   }
 }
 

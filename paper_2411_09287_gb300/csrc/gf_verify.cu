@@ -474,7 +474,8 @@ void launch_gf_verify(cudaStream_t st, const GfVerify& a) {
   for (; (D + 1) / 2 > GF_TAIL; ++k) {
     const long long Dh = (D + 1) / 2, ldo = Dh;
     g = ((Dh + 1) / 2 + 127) / 128;
-    launch_dep(k_gf_round, (unsigned)(g < 2432 ? g : 2432), 128, 0, st, a, cf, k + 1, D, x, y, ld, xo, yo, ldo);
+    launch_dep(k_gf_round, (unsigned)(g < 2432 ? g : 2432), 128, 0, st, a, cf, k + 1, D, x, y, ld, xo,
+               yo, ldo);
     u64* t = x; x = xo; xo = t;
     t = y; y = yo; yo = t;
     D = Dh;

@@ -2,8 +2,8 @@
 //
 // After Pi_Tran (Fig. MTP) a batch has x_i = w_i X_i and y_i = lift(Y_i), with X_i, Y_i shares in
 // Z_2^64 and w_i a public GR element (r^i, or r^(i / 64) for the edaBit inner products).  The first
-// K <= 3 rounds of Pi_Reduce fold blocks of B = 2^K elements with public weights, so they need no
-// GR vector at all: with w_i = R_b T_j (i = B b + j) and
+// K rounds of Pi_Reduce (at most 3, or 4 for long batches) fold blocks of B = 2^K elements with public
+// weights, so they need no GR vector at all: with w_i = R_b T_j (i = B b + j) and
 //   S^p_{j,j'} = sum_b R_b word^p_{b,j,j'},
 //   word^0 = (X0 + X1)_j (Y0 + Y1)_j',  word^1 = -(X2_j Y3_j' + X3_j Y2_j'),
 //   word^2 = X4_j (Y4 - Y5)_j' - X5_j Y4_j'   (the parties' cross terms; index = share component)
@@ -16,8 +16,8 @@
 // where materialising and folding takes 9 GR products, 10 Gram terms and 12 x 512 bytes of vectors
 // several times over.  The sums grow with B, what the dense rounds still do shrinks with it: B = 8 on
 // the CUDA cores (this file), B = 16 for long batches, whose sums run on the tensor cores (blk_sums_tc:
-// a product of the blocks' words and R); a batch of 2^20
-// triples: 4.06 ms with B = 8 on the tensor cores, 3.38 ms with 16.
+// a product of the blocks' words and R); a batch of 2^20 triples: 4.06 ms with B = 8 on the tensor
+// cores, 3.38 ms with 16.
 #include "gr_mul.cuh"
 #include "kernels.h"
 
@@ -286,6 +286,8 @@ void launch_blk_combine(cudaStream_t st, const BlkVec& in, const BlkOut& out, in
   }
 }
 
-void launch_ones(cudaStream_t st, int n, u64* out) { launch_dep(k_ones, (n * 64 + 255) / 256, 256, 0, st, n, out); }
+void launch_ones(cudaStream_t st, int n, u64* out) {
+  launch_dep(k_ones, (n * 64 + 255) / 256, 256, 0, st, n, out);
+}
 
 }  // namespace mpc3

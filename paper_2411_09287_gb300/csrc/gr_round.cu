@@ -33,9 +33,9 @@ constexpr int REC_ROWS = 7;
 // One Pi_Reduce round after its party sums (Fig. Reduce): h(0) and h(p2) by secure GR inner
 // products, zeta' drawn and opened, the next claim z' = L0 h(0) + L1 (z - h(0)) + L2 h(p2), the
 // fold element f and its multiplication matrix.  Block c < 6 computes component c of h(0), h(p2)
-// and z'; block 6 the matrix, the Pi_Rec messages and the next round's cleared sums and zero rows; in a round over
-// a matrix S (nvw > 0) the blocks from 7 on take the weights V_j, W_j, two each: times 1 - f or f by
-// bit vwbit of j.  Every block derives zeta' from its streams, so that no block waits for another.
+// and z'; block 6 the matrix, the Pi_Rec messages and the next round's cleared sums and zero rows; in a
+// round over a matrix S (nvw > 0) the blocks from 7 on take the weights V_j, W_j, two each: times 1 - f
+// or f by bit vwbit of j.  Every block derives zeta' from its streams, so that no block waits for another.
 //
 // L0 + L1 + L2 = 1 in both readings of the third point, hence z' = h(0) + L1 (z - 2 h(0)) +
 // L2 (h(p2) - h(0)), with (points 0, 1, x) L2 = (z^2 - z) / (x (x - 1)), L1 = z - (z^2 - z) / x -
@@ -216,8 +216,8 @@ k_reveal(Key k01, Key k02, Key k12, u32 purpose, u64 obj, const MsgFault fault, 
 // + o') - S00 - S11, 127 unreduced coefficients each.  A block takes one pair: its 24 products one a
 // warp, then an eighth of each of the fifteen products of the sums a warp.  Bound by latency; on
 // the tensor cores, whose tiles want 128 rows and whose kernels first split their operands, the two
-// Gram launches and the fold of such a round took 36 us at 512 elements, this 16 us, 13 without the fold (20 and 15 us
-// with a coefficient a thread and a load an operand and multiply-add).
+// Gram launches and the fold of such a round took 36 us at 512 elements, this 16 us, 13 without the fold
+// (20 and 15 us with a coefficient a thread and a load an operand and multiply-add).
 __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
   grid_dep();
   __shared__ __align__(16) u64 f[64], v[2][12][64], d[8][64], red[9][128];
@@ -306,8 +306,9 @@ __global__ void __launch_bounds__(256) k_small_round(const SmallRound a) {
     u64 s = red[q][c];
     if (k == 2) s -= red[p][c] + red[3 + p][c];
     // S00 at 0, the cross sum at 3, S11 at 9 (blocks of 128 words)
-    if (s) atomicAdd(reinterpret_cast<unsigned long long*>(a.sums + ((k == 0 ? 0 : k == 1 ? 9 : 3) + p) * 128 + c),
-                     (unsigned long long)s);
+    const int blk = (k == 0 ? 0 : k == 1 ? 9 : 3) + p;
+    if (s)
+      atomicAdd(reinterpret_cast<unsigned long long*>(a.sums + blk * 128 + c), (unsigned long long)s);
   }
 }
 
@@ -450,7 +451,7 @@ __device__ __forceinline__ void gr_mac_row(const u64* a, const u64* b, int l, Gr
 constexpr int IVL_WARPS = 4;
 __global__ void __launch_bounds__(IVL_WARPS * 32, 5) k_inner_verify_long(const InnerVerify a) {
   __shared__ __align__(16) u64 al[5][64];               // r1, r2, m of alpha; r_a, m - r2
-  __shared__ __align__(16) u64 U[IVL_WARPS][5][64];     // r_x, m_x (P1), [r]_1, m_x (P2), [r]_2; x' in its place
+  __shared__ __align__(16) u64 U[IVL_WARPS][5][64];     // r_x, m_x (P1), [r]_1, m_x (P2), [r]_2; then x'
   __shared__ __align__(16) u64 V[IVL_WARPS][5][64];     // r_y, m_y (P1), [r]_1, m_y (P2), m_y - [r]_2
   __shared__ __align__(16) u64 ST[IVL_WARPS][3][64];
   const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
@@ -474,7 +475,8 @@ __global__ void __launch_bounds__(IVL_WARPS * 32, 5) k_inner_verify_long(const I
     *reinterpret_cast<ulonglong2*>(dst + 2 * l) = make_ulonglong2(x, y);
   };
   Gr2 acc[3];
-  for (long long i = blockIdx.x * (long long)IVL_WARPS + w; i <= a.D; i += (long long)gridDim.x * IVL_WARPS) {
+  const long long stride = (long long)gridDim.x * IVL_WARPS;
+  for (long long i = blockIdx.x * (long long)IVL_WARPS + w; i <= a.D; i += stride) {
     const bool row = i < a.D;   // uniform over the warp; the last one is alpha against -z
     __syncwarp();
     ulonglong2 y[6];
@@ -647,7 +649,7 @@ k_rec_hash(const u64* log, u32* status, u32 flag) {
 
 // One of the first rounds of a batch evaluated from a matrix S_{j,j'}, j, j' < n (the truncation
 // batch's and the edaBits' bit pairs, n = 64: S_{j,j'} = sum_e R_e b1_{e,j} b2_{e,j'}; blocks of
-// ring words, n <= 8, one matrix per party): with V_j, W_j the accumulated weights of the x and y
+// ring words, n <= 16, one matrix per party): with V_j, W_j the accumulated weights of the x and y
 // side, the sums over the pairs (j, j') of one 2^k-block
 //   out[2 a + b] += sum_{bit k-1 of j = a, of j' = b} V_j W_j' S_{j,j'},  192 words apart, party p
 // at 64 p (the round's S00, S01, S10, S11; out must be zero on entry).  Block (j, c, p) takes the

@@ -65,7 +65,8 @@ struct GemmGroups {
 };
 int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nterms,
                  const GemmTerm* terms, const Epi& epi, void* scratch, unsigned* err,
-                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min = 0, const GemmGroups& groups = GemmGroups{});
+                 unsigned err_flag, cudaEvent_t ev0, cudaEvent_t ev1, int split_min = 0,
+                 const GemmGroups& groups = GemmGroups{});
 
 // Row map of a GR matrix product: logical row rho sits at word offset (rho % q) s1 + (rho / q) s2
 // (q = 0: rho s1).  q must be a multiple of 128.

@@ -514,7 +514,8 @@ k_blk_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) 
   }
   __syncthreads();
   for (int u = tid; u < ROWS * 2; u += 256) {
-    const int g = u & 1, row = u >> 1, p = row >> 8, j = g * 136 + ((row >> 4) & 15), k = g * 136 + (row & 15);
+    const int g = u & 1, row = u >> 1, p = row >> 8;
+    const int j = g * 136 + ((row >> 4) & 15), k = g * 136 + (row & 15);
     u64 v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -1580,13 +1581,15 @@ k_gr_matmul_tm(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ 
 
 // ---- Gram sums of the dense Pi_Reduce rounds -------------------------------------------------
 // For vectors u, v of n = 2 Dh GR elements (rows of 64 words, element i at row i) a job adds
-//   P[ee] += s C(u_even, v_even), P[oo] += s C(u_odd, v_odd), P[x] += s (C(u_even, v_odd) + C(u_odd, v_even))
+//   P[ee] += s C(u_even, v_even), P[oo] += s C(u_odd, v_odd),
+//   P[x] += s (C(u_even, v_odd) + C(u_odd, v_even))
 // with G(u, v)[a][b] = sum_i u_i[a] v_i[b] (a 64 x 64 matrix, mod 2^64), C its 127 anti-diagonal
-// sums (the coefficients of sum_i u_i v_i before the reduction mod f) and s the job's sign; u = a0 + sa1 a1 and v = b0 + sb1 b1 (a1, b1 may be absent).  The MMA tile is M = 128
-// (rows a: u_even coefficients, then u_odd) x N = 64 (v of one parity, blockIdx.y) with K = the
-// element pairs i, split across blockIdx.x; blockIdx.z is the job; each CTA adds its partial
-// coefficients atomically.  Producers combine and split the rows into digit planes transposed to K-major; MMA
-// issue and drains as in k_limb_gemm_tc; the drain warps accumulate over all of the CTA's chunks.
+// sums (the coefficients of sum_i u_i v_i before the reduction mod f) and s the job's sign; u = a0 +
+// sa1 a1 and v = b0 + sb1 b1 (a1, b1 may be absent).  The MMA tile is M = 128 (rows a: u_even
+// coefficients, then u_odd) x N = 64 (v of one parity, blockIdx.y) with K = the element pairs i, split
+// across blockIdx.x; blockIdx.z is the job; each CTA adds its partial coefficients atomically.
+// Producers combine and split the rows into digit planes transposed to K-major; MMA issue and drains
+// as in k_limb_gemm_tc; the drain warps accumulate over all of the CTA's chunks.
 constexpr size_t GR_SMEM = (size_t)NSTAGE * STAGE + 1024;   // 2 x (64 KB A + 32 KB B)
 
 template <bool GEN>

@@ -88,13 +88,14 @@ void launch_addsub(cudaStream_t st, long long n, const u64* a, const u64* b, int
 }
 void launch_eda_words(cudaStream_t st, const u64* const bits[3], const u64* eprod, long long np,
                       long long e0, long long ldy, u64* xm, u64* y) {
-  launch_dep(k_eda_words, dim3((unsigned)(np / 32), 7), TPB, 0, st, bits[0], bits[1], bits[2], eprod, np, e0,
-                                                            ldy, xm, y);
+  launch_dep(k_eda_words, dim3((unsigned)(np / 32), 7), TPB, 0, st, bits[0], bits[1], bits[2], eprod, np,
+             e0, ldy, xm, y);
 }
 
 void launch_window_gather(cudaStream_t st, const u64* x, long long BC, long long H, long long W,
                           long long np, u64* left, u64* right) {
-  launch_dep(k_window_gather, grid_for(6 * BC * (H / 2) * (W / 2)), TPB, 0, st, x, BC, H, W, np, left, right);
+  launch_dep(k_window_gather, grid_for(6 * BC * (H / 2) * (W / 2)), TPB, 0, st, x, BC, H, W, np, left,
+             right);
 }
 
 void launch_gather(cudaStream_t st, const u64* xs, long long n_in, const long long* idx,

@@ -369,7 +369,9 @@ k_trunc_finish(long long E, Key k01, Key k02, u64 obj, const u64* row_keys,
 }
 
 __global__ void k_xor_one(u64* p, u64 mask) {
-  grid_dep(); *p ^= mask; }
+  grid_dep();
+  *p ^= mask;
+}
 
 // words off .. off + n - 1 of a row-keyed truncation-bit stream (see bits_block8) into out
 __global__ void k_prf_words_keyed(long long n, long long off, Key key, u32 tag,
@@ -441,28 +443,28 @@ void launch_share_input(cudaStream_t st, const u64* x, long long n, Key k01, Key
                         u64* s6, u64* p0_out_m) {
   if (n <= 0) return;
   launch_dep(k_share_input, grid_for((n + 7) / 8), TPB, 0, st, x, n, k01, k02, make_tag(P_SHARE, C_R1),
-                                                       make_tag(P_SHARE, C_R2), obj, s6, p0_out_m);
+             make_tag(P_SHARE, C_R2), obj, s6, p0_out_m);
 }
 
 void launch_fill_masks(cudaStream_t st, long long n, Key k01, Key k02, u32 purpose, u64 obj,
                        u64* s6) {
   if (n <= 0) return;
   launch_dep(k_fill_masks, grid_for((n + 7) / 8), TPB, 0, st, n, k01, k02, make_tag(purpose, C_R1),
-                                                      make_tag(purpose, C_R2), obj, s6);
+             make_tag(purpose, C_R2), obj, s6);
 }
 
 void launch_mult_offline(cudaStream_t st, const u64* xs, const u64* ys, long long n, Key k01,
                          Key k02, u64 obj, u64* zs, u64* p0_out_g2) {
   if (n <= 0) return;
-  launch_dep(k_mult_offline, grid_for((n + 7) / 8), TPB, 0, st, xs, ys, n, k01, k02, make_tag(P_MULT, C_R1), make_tag(P_MULT, C_R2),
-      make_tag(P_MULT, C_G1), obj, zs, p0_out_g2);
+  launch_dep(k_mult_offline, grid_for((n + 7) / 8), TPB, 0, st, xs, ys, n, k01, k02,
+             make_tag(P_MULT, C_R1), make_tag(P_MULT, C_R2), make_tag(P_MULT, C_G1), obj, zs, p0_out_g2);
 }
 
 void launch_mult_online(cudaStream_t st, const u64* xs, const u64* ys, long long n, Key k01,
                         u64 obj, const u64* p2_in_g2, u64* p1_out, u64* p2_out) {
   if (n <= 0) return;
   launch_dep(k_mult_online, grid_for((n + 7) / 8), TPB, 0, st, xs, ys, n, k01, make_tag(P_MULT, C_G1),
-                                                       obj, p2_in_g2, p1_out, p2_out);
+             obj, p2_in_g2, p1_out, p2_out);
 }
 
 void launch_exchange_finish(cudaStream_t st, long long n, const u64* p1_own, const u64* p1_in,
@@ -475,10 +477,12 @@ void launch_trunc_p0(cudaStream_t st, long long E, Key k01, Key k02, u64 obj, in
                      u64* zout, u64* pq, u64* p0_out_gp2, u64* p0_out_gq2, u64* p1_out_mp,
                      u64* p1_out_mq, const u64* row_keys, long long N) {
   if (E <= 0) return;
-  launch_dep(k_trunc_p0, warp_grid((E + 7) / 8), warp_block((E + 7) / 8), 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2),
-      make_tag(P_TRUNC_P, C_R1), make_tag(P_TRUNC_P, C_R2), make_tag(P_TRUNC_P, C_G1),
-      make_tag(P_TRUNC_Q, C_R1), make_tag(P_TRUNC_Q, C_R2), make_tag(P_TRUNC_Q, C_G1), zpre, zout,
-      pq, p0_out_gp2, p0_out_gq2, p1_out_mp, p1_out_mq);
+  const long long n8 = (E + 7) / 8;
+  launch_dep(k_trunc_p0, warp_grid(n8), warp_block(n8), 0, st, E, k01, k02, obj, row_keys, N, t,
+             make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2), make_tag(P_TRUNC_P, C_R1),
+             make_tag(P_TRUNC_P, C_R2), make_tag(P_TRUNC_P, C_G1), make_tag(P_TRUNC_Q, C_R1),
+             make_tag(P_TRUNC_Q, C_R2), make_tag(P_TRUNC_Q, C_G1), zpre, zout, pq, p0_out_gp2,
+             p0_out_gq2, p1_out_mp, p1_out_mq);
 }
 
 void launch_trunc_finish(cudaStream_t st, long long E, Key k01, Key k02, u64 obj, int t,
@@ -487,8 +491,10 @@ void launch_trunc_finish(cudaStream_t st, long long E, Key k01, Key k02, u64 obj
                          const u64* p1_mp1, const u64* p1_mq1, u64* zpre, u64* zout, u64* pq,
                          const u64* row_keys, long long N) {
   if (E <= 0) return;
-  launch_dep(k_trunc_finish, warp_grid((E + 7) / 8), warp_block((E + 7) / 8), 0, st, E, k01, k02, obj, row_keys, N, t, make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2), p1_in_mp,
-      p1_in_mq, p2_in_mp, p2_in_mq, p2_gp2, p2_gq2, p1_mp1, p1_mq1, zpre, zout, pq);
+  const long long n8 = (E + 7) / 8;
+  launch_dep(k_trunc_finish, warp_grid(n8), warp_block(n8), 0, st, E, k01, k02, obj, row_keys, N, t,
+             make_tag(P_TRUNC_BITS, C_TB1), make_tag(P_TRUNC_BITS, C_TB2), p1_in_mp, p1_in_mq, p2_in_mp,
+             p2_in_mq, p2_gp2, p2_gq2, p1_mp1, p1_mq1, zpre, zout, pq);
 }
 
 void launch_xor_one(cudaStream_t st, u64* p, u64 mask) { launch_dep(k_xor_one, 1, 1, 0, st, p, mask); }

@@ -194,7 +194,7 @@ k_trunc_s_tc(const __grid_constant__ CUtensorMap tmB, const u64* B1T,
   };
 
   if (warp == 4) {
-    // ---- TMA producer: limb-table tile (256 columns x 128 e) per chunk ----
+    // ---- TMA producer: limb-table tile (208 columns x 128 e) per chunk ----
     if (lane == 0) {
       int last = -1;
       for (int c = 0; c < nchunks; ++c) {
