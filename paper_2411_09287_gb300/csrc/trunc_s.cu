@@ -13,9 +13,10 @@
 // -16 <= d_l <= 15 (d_12 the top four bits); e4m3 has four significant bits, so every integer from
 // -16 to 16 is exact in it, as are the bits, and an accumulator sums at most L <= 2^16 terms, so
 // every f32 partial sum is an exact integer of at most 2^20; the limbs are recombined mod 2^64 when
-// the e_lo loop ends.  The limbs' number sets the table's size but hardly the time: 2^20 outputs take
-// 2.51 ms with 16 limbs (N = 256), 2.60 with 13, 2.59 with 12 (radix 43, whose table costs small batches
-// 60 us), 2.19 ms without the stores of A: the pair bits' way through shared memory and the MMAs.
+// the e_lo loop ends.  13 limbs take 39.4 ms for 2^24 outputs, 16
+// unsigned ones of 4 bits (N = 256) 41.2; 12 (radix 43) need divisions that cost small batches 60 us.
+// What bounds it is the pair bits' way through shared memory beside the MMAs' reads: without the stores
+// of A it took 16% less.
 //
 // Operands, both K-major (K = e):
 //   A (M = 128 pairs per accumulator): byte (p, e) = e4m3(b1_{e,j} AND b2_{e,j'}), generated in
