@@ -50,35 +50,35 @@ __global__ void k_decode_fixed(const u64* v, long long n, int k,
 
 // cols[c][row][col] = x[c][b][ch][i s + di - p][j s + dj - p] (0 outside the image) for every
 // share component c = blockIdx.y, row = (b Ho + i) Wo + j, col = (ch kh + di) kw + dj.  A block takes
-// IM_ROWS rows: their places in the image and (up to IM_COLS columns) each column's offset once, in
+// `nrows` rows: their places in the image and (up to IM_COLS columns) each column's offset once, in
 // shared memory; a word is then one 32-bit division, two look-ups, a load and a store.  Bound by the
 // words written; with eight 64-bit divisions a word, 136 us for the 79 MB of 4096 x 400 words (now
 // 26 us).
-constexpr int IM_ROWS = 16, IM_COLS = 1024;
+constexpr int IM_ROWS = 512, IM_COLS = 1024;   // most rows of a block, most columns of the table
 struct ImCol {
   int off;        // (ch H + di) W + dj
   short di, dj;
 };
-__global__ void __launch_bounds__(LTPB) k_im2col(const u64* x, ConvGeom g, u64* __restrict__ cols) {
+__global__ void __launch_bounds__(LTPB)
+k_im2col(const u64* x, ConvGeom g, int nrows, u64* __restrict__ cols) {
   grid_dep();
   __shared__ ImCol tab[IM_COLS];
-  __shared__ long long base[IM_ROWS];
-  __shared__ long long y0[IM_ROWS], z0[IM_ROWS];
+  __shared__ long long base[IM_ROWS], y0[IM_ROWS], z0[IM_ROWS];
   const long long Mr = (long long)g.B * g.Ho * g.Wo, n_in = (long long)g.B * g.C * g.H * g.W;
   const long long Kc = (long long)g.C * g.kh * g.kw;
-  const long long r0 = (long long)blockIdx.x * IM_ROWS;
-  const int rows = (int)(Mr - r0 < IM_ROWS ? Mr - r0 : IM_ROWS);
+  const long long r0 = (long long)blockIdx.x * nrows;
+  const int rows = (int)(Mr - r0 < nrows ? Mr - r0 : nrows);
   const bool small = Kc <= IM_COLS && g.H < 32768 && g.W < 32768 && g.C * g.H * g.W < (1ll << 30);
   if (small)
     for (int c = threadIdx.x; c < (int)Kc; c += LTPB) {
       const int kw = (int)g.kw, kh = (int)g.kh, q = c / kw, dj = c - q * kw, ch = q / kh, di = q - ch * kh;
       tab[c] = ImCol{(ch * (int)g.H + di) * (int)g.W + dj, (short)di, (short)dj};
     }
-  if (threadIdx.x < rows) {
-    const long long row = r0 + threadIdx.x, q = row / g.Wo, j = row - q * g.Wo, b = q / g.Ho, i = q - b * g.Ho;
-    y0[threadIdx.x] = i * g.stride - g.pad;
-    z0[threadIdx.x] = j * g.stride - g.pad;
-    base[threadIdx.x] = b * g.C * g.H * g.W + y0[threadIdx.x] * g.W + z0[threadIdx.x];
+  for (int r = threadIdx.x; r < rows; r += LTPB) {
+    const long long row = r0 + r, q = row / g.Wo, j = row - q * g.Wo, b = q / g.Ho, i = q - b * g.Ho;
+    y0[r] = i * g.stride - g.pad;
+    z0[r] = j * g.stride - g.pad;
+    base[r] = b * g.C * g.H * g.W + y0[r] * g.W + z0[r];
   }
   __syncthreads();
   const u64* src = x + blockIdx.y * n_in;
@@ -149,8 +149,15 @@ void launch_decode_fixed(cudaStream_t st, const u64* v, long long n, int k, doub
 
 void launch_im2col(cudaStream_t st, const u64* x, const ConvGeom& g, u64* cols) {
   const long long Mr = (long long)g.B * g.Ho * g.Wo;
-  if (Mr * g.C * g.kh * g.kw <= 0) return;
-  launch_dep(k_im2col, dim3((unsigned)((Mr + IM_ROWS - 1) / IM_ROWS), 6), LTPB, 0, st, x, g, cols);
+  const long long Kc = g.C * g.kh * g.kw;
+  if (Mr * Kc <= 0) return;
+  // 16 rows a block, and for narrow rows as many as make 2048 words while four blocks an SM remain
+  // (a block of 16 words is mostly set-up: a convolution of 802816 rows of one column took 1.91 ms with
+  // 16 rows a block, 1.32 now; 1.37 with the divisions in every word).
+  long long n = (2048 + Kc - 1) / Kc;
+  if (n > 6 * Mr / (152 * 4)) n = 6 * Mr / (152 * 4);
+  n = n < 16 ? 16 : n > IM_ROWS ? IM_ROWS : n;
+  launch_dep(k_im2col, dim3((unsigned)((Mr + n - 1) / n), 6), LTPB, 0, st, x, g, (int)n, cols);
 }
 
 void launch_trunc_remask(cudaStream_t st, const u64* xs, const u64* rx, long long n, u64* d1_p1,
