@@ -91,14 +91,16 @@ __device__ __forceinline__ u32 rotl32(u32 x, int n) { return __funnelshift_l(x, 
 // One ChaCha20 block: out[0..15] = state after 20 rounds plus the input state.  A loop of ten double
 // rounds, 1.5 KB of code: unrolled, a block is 15 KB, and kernels that draw several streams, or run for a
 // few microseconds with a cold instruction cache, wait for instructions (the truncation pairs of
-// 100003 outputs: 53 us, 11 us with the loop and smaller blocks).
+// 100003 outputs: 53 us, 11 us with the loop and smaller blocks).  U = 10 unrolls it, for long kernels
+// of two streams (sharing 2^26 words: 1018 us with the loop, 997 unrolled).
+template <int U = 1>
 __device__ __forceinline__ void chacha_block(const Key& key, u32 counter, u32 n0, u32 n1, u32 n2,
                                              u32 out[16]) {
   u32 x0 = 0x61707865u, x1 = 0x3320646eu, x2 = 0x79622d32u, x3 = 0x6b206574u;
   u32 x4 = key.k[0], x5 = key.k[1], x6 = key.k[2], x7 = key.k[3];
   u32 x8 = key.k[4], x9 = key.k[5], x10 = key.k[6], x11 = key.k[7];
   u32 x12 = counter, x13 = n0, x14 = n1, x15 = n2;
-#pragma unroll 1
+#pragma unroll U
   for (int i = 0; i < 10; ++i) {
     MPC3_QR(x0, x4, x8, x12) MPC3_QR(x1, x5, x9, x13) MPC3_QR(x2, x6, x10, x14)
     MPC3_QR(x3, x7, x11, x15) MPC3_QR(x0, x5, x10, x15) MPC3_QR(x1, x6, x11, x12)
@@ -112,9 +114,10 @@ __device__ __forceinline__ void chacha_block(const Key& key, u32 counter, u32 n0
 }
 
 // The 8 u64 words of block `blk` of stream (tag, obj).
+template <int U = 1>
 __device__ __forceinline__ void prf_block8(const Key& key, u32 tag, u64 obj, u64 blk, u64 w[8]) {
   u32 o[16];
-  chacha_block(key, (u32)blk, tag, (u32)obj, (u32)(obj >> 32), o);
+  chacha_block<U>(key, (u32)blk, tag, (u32)obj, (u32)(obj >> 32), o);
 #pragma unroll
   for (int i = 0; i < 8; ++i) w[i] = (u64)o[2 * i] | ((u64)o[2 * i + 1] << 32);
 }

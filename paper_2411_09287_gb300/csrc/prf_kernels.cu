@@ -109,8 +109,8 @@ k_share_input(const u64* x, long long n, Key k01, Key k02, u32 tag1, u32 tag2,
     const u64 b = (u64)(bw + lane);
     const long long e0 = bw * 8;
     u64 r1[8], r2[8], xv[8];
-    prf_block8(k01, tag1, obj, b, r1);
-    prf_block8(k02, tag2, obj, b, r2);
+    prf_block8<10>(k01, tag1, obj, b, r1);
+    prf_block8<10>(k02, tag2, obj, b, r2);
     store8w(s, e0, n, r1, st);
     store8w(s + n, e0, n, r2, st);
     store8w(s + 3 * n, e0, n, r1, st);
@@ -135,8 +135,8 @@ k_fill_masks(long long n, Key k01, Key k02, u32 tag1, u32 tag2, u64 obj, u64* __
     const u64 b = (u64)(bw + lane);
     const long long e0 = bw * 8;
     u64 r1[8], r2[8];
-    prf_block8(k01, tag1, obj, b, r1);
-    prf_block8(k02, tag2, obj, b, r2);
+    prf_block8<10>(k01, tag1, obj, b, r1);
+    prf_block8<10>(k02, tag2, obj, b, r2);
     store8w(s, e0, n, r1, st);
     store8w(s + n, e0, n, r2, st);
     store8w(s + 3 * n, e0, n, r1, st);
