@@ -51,9 +51,9 @@ void gemm_u64(cudaStream_t st, long long M, long long N, long long K, int nterms
               const GemmTerm* terms, const Epi& epi, int nsplit);
 
 // ---- exact u64 GEMM on the tcgen05 tensor cores (limb_gemm_tc.cu) ---------------------------
-// Same contract as gemm_u64 without split-K (epi.atomic must be 0; returns -1 otherwise and
-// for terms of different layouts, -2 if
-// the tensor maps cannot be encoded).  scratch: limb_tc_scratch_bytes(M, N, K, nterms) bytes,
+// Same contract as gemm_u64 without split-K (epi.atomic must be 0) and with an epilogue on whole rows
+// only (ldc = N; add0 at out's index); returns -1 otherwise and for terms of different layouts, -2 if
+// the tensor maps cannot be encoded.  scratch: limb_tc_scratch_bytes(M, N, K, nterms) bytes,
 // 256-byte aligned (the bf16 digit planes of both operands).  A bounded wait that expires
 // sets err_flag in *err and leaves the output undefined.
 size_t limb_tc_scratch_bytes(long long M, long long N, long long K, int nterms);

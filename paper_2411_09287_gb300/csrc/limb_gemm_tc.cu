@@ -562,31 +562,38 @@ k_eda_planes(const BlkIn in, long long Kp, unsigned short* __restrict__ planes) 
   }
 }
 
-// out[i] = acc_sign*out[i] + add0 + add1 + prf_sign*PRF(i) (the protocol epilogue of gemm_u64).
-__global__ void k_apply_epilogue(long long M, long long N, Epi epi) {
+// out[i] = acc_sign*out[i] + add0 + add1 + prf_sign*PRF(i) (the protocol epilogue of gemm_u64) over the n
+// words of an output without gaps between its rows.  A warp takes 256 words, lane l words l, l + 32, ...:
+// each lane draws the stream block of eight consecutive words and they change places in shared memory.
+// Bound by memory.  (A thread on eight consecutive words leaves each line to the L1 cache for its other
+// seven loads; set up behind the GEMM, whose shared memory takes most of the L1, it does not find them
+// there: product of 4096 x 16 x 4096 words 1.31 ms, 1.00 now.)
+__global__ void __launch_bounds__(256) k_apply_epilogue(long long n, Epi epi) {
   grid_dep();
-  const long long total = M * N;
-  for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < (total + 7) / 8;
-       w += (long long)gridDim.x * blockDim.x) {
-    const long long i0 = w * 8;
-    u64 pr[8];
-    bool block = epi.prf_sign && (N % 8 == 0) && (epi.ldc == N);
-    if (block) prf_block8(epi.key, epi.tag, epi.obj, (u64)(i0 >> 3), pr);
+  __shared__ u64 stage[8][32 * 9];
+  u64* st = stage[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const long long nb = (n + 7) / 8;
+  for (long long b = blockIdx.x * 256ll + (threadIdx.x & ~31); b < nb; b += (long long)gridDim.x * 256) {
+    if (epi.prf_sign) {
+      u64 pr[8];
+      prf_block8(epi.key, epi.tag, epi.obj, (u64)(b + lane), pr);
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) st[lane * 9 + q] = pr[q];
+      __syncwarp();
+    }
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const long long i = i0 + q;
-      if (i >= total) break;
-      const long long r = i / N, c = i % N;
-      const long long idx = r * epi.ldc + c;
-      u64 v = epi.out[idx];
+      const int w = lane + 32 * q;
+      const long long i = b * 8 + w;
+      if (i >= n) break;
+      u64 v = epi.out[i];
       v = (epi.acc_sign == 1ull) ? v : ((epi.acc_sign == ~0ull) ? 0ull - v : epi.acc_sign * v);
-      if (epi.add0) v += epi.add0[epi.ld_add0 ? r * epi.ld_add0 + c : idx];
-      if (epi.add1) v += epi.add1[idx];
-      if (epi.prf_sign) {
-        const u64 p = block ? pr[q] : prf_word(epi.key, epi.tag, epi.obj, (u64)idx);
-        v += epi.prf_sign * p;
-      }
-      epi.out[idx] = v;
+      if (epi.add0) v += epi.add0[i];
+      if (epi.add1) v += epi.add1[i];
+      if (epi.prf_sign) v += epi.prf_sign * st[(w >> 3) * 9 + (w & 7)];
+      epi.out[i] = v;
     }
   }
 }
@@ -1830,6 +1837,8 @@ size_t limb_tc_scratch_bytes(long long M, long long N, long long K, int nterms) 
   return (size_t)(((a + 255) & ~255ll) + ((b + 255) & ~255ll) + 256);
 }
 
+bool has_epilogue(const Epi& e) { return e.acc_sign != 1 || e.add0 || e.add1 || e.prf_sign; }
+
 // C = A B from digit planes (and the epilogue, when it has any terms)
 int limb_gemm_planes(cudaStream_t st, long long M, long long N, long long Kp, unsigned short* Ap,
                      unsigned short* Bp, const Epi& epi, unsigned* err, unsigned err_flag,
@@ -1857,11 +1866,10 @@ int limb_gemm_planes(cudaStream_t st, long long M, long long N, long long Kp, un
   if (ev0) cudaEventRecord(ev0, st);
   launch_dep(k_limb_gemm_tc, grid, TC_THREADS, smem, st, ma, mb, M, N, Kp, epi.out, epi.ldc, err, err_flag);
   if (ev1) cudaEventRecord(ev1, st);
-  if (epi.acc_sign == 1 && !epi.add0 && !epi.add1 && !epi.prf_sign) return 0;
+  if (!has_epilogue(epi)) return 0;
   long long ge = ((M * N + 7) / 8 + 255) / 256;
   if (ge > (1 << 20)) ge = 1 << 20;
-  if (ge < 1) ge = 1;
-  launch_dep(k_apply_epilogue, (unsigned)ge, 256, 0, st, M, N, epi);
+  launch_dep(k_apply_epilogue, (unsigned)ge, 256, 0, st, M * N, epi);
   return 0;
 }
 
@@ -1873,6 +1881,7 @@ int limb_gemm_tc(cudaStream_t st, long long M, long long N, long long K, int nte
   const GemmTerm& t1 = nterms > 1 ? terms[1] : terms[0];
   // the terms of a product have one layout per side
   if (epi.atomic || t1.A.trans != terms[0].A.trans || t1.B.trans != terms[0].B.trans) return -1;
+  if (has_epilogue(epi) && (epi.ldc != N || (epi.add0 && epi.ld_add0 && epi.ld_add0 != N))) return -1;
   const long long Kp = ((nterms * K + TC_BK - 1) / TC_BK) * TC_BK;
   unsigned short* Ap = reinterpret_cast<unsigned short*>(scratch);
   const long long abytes = (8 * M * Kp * 2 + 255) & ~255ll;
