@@ -31,6 +31,10 @@ typedef uint32_t u32;
 // A kernel that takes tensor memory calls grid_dep before it allocates: a block that held it while it
 // waited could keep a block of its predecessor, on the same SM, from getting any.
 // Verified product of 64 x 64 x 128: 1.26 ms without, 1.05 ms with it; ReLU of 128: 1.30, 1.09 ms.
+// A kernel set up early runs with its predecessor's division of the SM between shared memory and L1, and
+// behind a tensor kernel little L1 is left to hold loads in flight (the digit split of 16384 x 8192 words:
+// 0.80 ms, 0.48 launched alone).  So kernels of more threads than the GPU holds at once, whose set-up is
+// little beside their run, are launched alone, unless they take most of the shared memory themselves.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void grid_dep() {
   asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n" ::: "memory");
@@ -50,7 +54,8 @@ inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  const long long threads = (long long)grid.x * grid.y * grid.z * block.x;
+  cfg.numAttrs = smem > 48 * 1024 || threads < 152ll * 2048 ? 1 : 0;
   if (cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess)
     g_launches.fetch_add(1, std::memory_order_relaxed);
 }
